@@ -231,3 +231,92 @@ def tolerance(case):
     if case.get("y", "fp32") == "bf16":
         return {"rel": 6e-3, "max": 2e-2}
     return {"rel": 8e-5, "max": 3e-4} if case["op"] == "qaf" else {"rel": 1e-6, "max": 1e-5}
+
+
+# ---- the same results in 64 bits, from plain torch -----------------------------------------------------------------
+_GRID = (0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0)
+
+
+def _scale64(x):
+    amax = x.abs().max().float()
+    return torch.where(amax == 0, torch.ones_like(amax), amax / torch.full_like(amax, 2688.0))   # by a tensor: a number's reciprocal would be rounded
+
+
+def _philox(seed, offset, blk):
+    """Philox4x32-10 of the counters (blk, offset) under the key `seed`: four tensors of 32-bit words."""
+    low = 0xFFFFFFFF
+    key = [seed & low, (seed >> 32) & low]
+    c = [blk & low, blk >> 32, torch.full_like(blk, offset & low), torch.full_like(blk, offset >> 32)]
+    for _ in range(10):
+        p, q = c[0] * 0xD2511F53, c[2] * 0xCD9E8D57            # wraps mod 2^64: the shifted word is masked below
+        c = [((q >> 32) & low) ^ c[1] ^ key[0], q & low, ((p >> 32) & low) ^ c[3] ^ key[1], p & low]
+        key = [(key[0] + 0x9E3779B9) & low, (key[1] + 0xBB67AE85) & low]
+    return c
+
+
+def _quantized64(x, g, rounding, block=16):
+    """x, in float64, after the quantization of its rows in blocks: E4M3 scales of 16 (or E8M0 scales of 32), E2M1 values."""
+    out = torch.empty(x.shape, dtype=torch.float64, device=x.device)
+    rows, cols = x.shape
+    bit = torch.arange(16, device=x.device)
+    chunk = max(1, (1 << 26) // cols)
+    for r in range(0, rows, chunk):
+        v = x[r:r + chunk].contiguous().float().reshape(-1, block)
+        a = v.abs().amax(1) * ((torch.ones((), device=x.device) / 6.0) / g)
+        if block == 16:
+            sf = a.clamp(max=448.0).to(torch.float8_e4m3fn).float()
+        else:
+            m, e = torch.frexp(a)
+            sf = torch.where(a > 0, torch.ldexp(torch.ones_like(a), e - (m == 0.5).to(e.dtype)), torch.zeros_like(a))
+        inv = torch.where(sf > 0, 1.0 / (sf * g), torch.zeros_like(sf))
+        y = (v * inv[:, None]).abs().clamp(max=6.0).double()
+        step = torch.where(y < 2, 0.5, torch.where(y < 4, 1.0, 2.0))
+        t = y / step
+        if rounding.mode == nb.SR:
+            blk = torch.arange(r * cols // 16, (r * cols + v.numel()) // 16, device=x.device)
+            draws = []
+            for w in _philox(rounding.seed, rounding.offset, blk):
+                for half in (((w >> 8) & 0xFF00) | (w & 0xFF), ((w >> 16) & 0xFF00) | ((w >> 8) & 0xFF)):
+                    draws += [half, (((half[:, None] >> bit) & 1) << (15 - bit)).sum(1)]
+            u = torch.stack(draws, 1).reshape(y.shape)
+            t = t.floor() + (((t - t.floor()) * 65536).floor() + u >= 65536)
+        else:
+            t = t.round()                                      # half to even: the even code, its mantissa bit being 0
+        out[r:r + chunk] = (torch.copysign(t * step, v.double()) * sf.double()[:, None]).reshape(-1, cols)
+    return out * g.double()
+
+
+def exact(case, seed):
+    """What run() returns, in float64: operands quantized as the number formats and the random streams define it (or taken
+    as they are where the product is a bf16 one), then multiplied in float64."""
+    op, sd = case["op"], int(seed) * 8
+    if op == "quantize":
+        return None                                            # codes and scales are whole values
+    M, K, N, x = case["M"], case["K"], case["N"], case.get("x", "bf16")
+    rtn, sr = nb.Rounding(nb.RTN), [nb.Rounding(nb.SR, int(seed), o) for o in range(3)]
+    if op in ("step", "qaf", "wgrad"):
+        X, dY = _normal((M, K), 1.0, sd, x), _normal((M, N), case.get("grad", 1e-4), sd + 2, x)
+        gx, gdy = _scale64(X), _scale64(dY)
+        if op != "qaf":
+            dW = _quantized64(dY.T, gdy, sr[1]) @ _quantized64(X.T, gx, sr[2]).T
+        if op == "wgrad":
+            return dW
+        W = _normal((N, K), 0.02, sd + 1, x)
+        gw = _scale64(W)
+        Y = _quantized64(X, gx, rtn) @ _quantized64(W, gw, rtn).T
+        if op == "qaf":
+            return Y, dY.double() @ W.double(), dY.double().T @ X.double()
+        return Y, _quantized64(dY, gdy, sr[0]) @ _quantized64(W.T, gw, rtn).T, dW
+    if op == "mx":
+        if case["which"] == "fwd":
+            A, B, ra, rb = _normal((M, K), 1.0, sd), _normal((N, K), 0.02, sd + 1), rtn, rtn
+        else:
+            A, B, ra, rb = _normal((M, N), 1e-4, sd).T, _normal((M, K), 1.0, sd + 1).T, sr[1], sr[2]
+        return _quantized64(A, _scale64(A), ra, 32) @ _quantized64(B, _scale64(B), rb, 32).T
+    X, W = _normal((M, K), 1.0, sd), _normal((N, K), 0.02, sd + 1)
+    Y = _quantized64(X, _scale64(X), rtn) @ _quantized64(W, _scale64(W), rtn).T
+    if op == "kept":
+        return Y
+    W2 = _normal((case["N2"], N), 0.02, sd + 2)
+    gh = _scale64(Y.bfloat16())
+    return _quantized64(Y.float(), gh, rtn) @ _quantized64(W2, _scale64(W2), rtn).T
