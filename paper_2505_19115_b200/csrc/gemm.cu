@@ -371,9 +371,12 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 // the register path keeps up with the tensor cores.)
 //
 // The epilogue goes through shared memory (128-byte swizzle) and leaves as tiled bulk stores.
-// Warps: 0 operand producer, 1 MMA issuer, 2-5 epilogue, 6-9 scale movers, 10 scale producer.
+// Warps: 0 operand producer, 1 MMA issuer, 2 scale producer, 3 idle, 4-7 scale movers, 8-15 epilogue.
+// Registers are split by warpgroup: 16 warps start at 128 each; the two control warpgroups go down to 72 and the two
+// epilogue warpgroups up to 184 (256 x (72 + 184) = 65536, what the CTA was launched with).
 // ------------------------------------------------------------------------------------------------
-constexpr int kGemm2Threads = 352;
+constexpr int kGemm2Threads = 512;
+constexpr int kControlRegs = 72, kEpilogueRegs = 184;
 
 template <int BN>
 struct Cfg2 {
@@ -385,8 +388,8 @@ struct Cfg2 {
   static constexpr int kSfaBytes = 2048;
   static constexpr int kSfbBytes = kSfbTiles * 2048;
   static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;
-  static constexpr int kEpiWarpBytes = 2 * 4096;                   // two 32-row x 128-byte buffers per warp
-  static constexpr int kEpiBytes = 4 * kEpiWarpBytes;
+  static constexpr int kEpiWarpBytes = 4096;                       // one 32-row x 128-byte staging buffer per warp
+  static constexpr int kEpiBytes = 8 * kEpiWarpBytes;
   static constexpr int kSmemBytes = kStages * kStageBytes + kEpiBytes + 1024 /*align*/ + 512 /*barriers*/ + 512 /*reciprocal table*/;
   // tensor memory: accumulators, then kSfBufs scale buffers of (16 columns for A, 16 per B tile)
   static constexpr uint32_t kSfaCol = kAccStages * BN;
@@ -438,7 +441,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
   constexpr bool BF16_OUT = (OUT == 1), Q_OUT = (OUT == 2);
   constexpr bool MN_A = (MN & 1) != 0, MN_B = (MN & 2) != 0;
   static_assert(MN == 0 || (BF16_IN && BN == 256), "MN-major operands exist for the bf16 variant with the 256-wide tile");
-  static_assert(!Q_OUT || BN == 256, "the quantized epilogue stores one 128-byte row of codes per tile row");
+  static_assert(!Q_OUT || BN == 256, "the quantized epilogue stores two 64-byte pieces of codes per tile row");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -471,7 +474,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(sfl_bar(s), 1); mbar_init(empty_bar(s), 1); mbar_init(sfx_bar(s), 4); }
     for (int b = 0; b < C::kSfBufs; ++b) { mbar_init(sfr_bar(b), 8); mbar_init(sfe_bar(b), 1); }
-    for (int a = 0; a < C::kAccStages; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 8); }
+    for (int a = 0; a < C::kAccStages; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 16); }
     *abort_flag = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -485,6 +488,8 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 
   // The producer and issuer warps run their loops with all 32 lanes (so that loop state, addresses and
   // descriptors stay warp-uniform) and predicate only the asynchronous instructions on one lane.
+  if (warp < 8) {
+  regs_release<kControlRegs>();
   if (warp == 0) {
     // ------------------------------- operand producer (both CTAs) -------------------------------
     // One warp can issue a tiled copy every ~75 cycles, so operands and scales have a producer each.
@@ -529,7 +534,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
       const unsigned long long t0 = global_timer_ns();
       while (global_timer_ns() - t0 < 200000ull) {}
     }
-  } else if (warp == 10) {
+  } else if (warp == 2) {
     // ------------------------------- scale producer (both CTAs) -------------------------------
     const bool issuer = elect_one() && !BF16_IN;
     int s = 0;
@@ -629,7 +634,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
       ACCOUNT_STORE(pair == 0 && issuer, 6, a_sf);
       ACCOUNT_STORE(pair == 0 && issuer, 7, a_total + ACCOUNT_NOW());
     }
-  } else if (warp >= 6) {                           // warps 6-9 (warp 10 was taken above)
+  } else if (warp >= 4) {
     // ------------------------------- scale movers (both CTAs) -------------------------------
     // Shared-memory scale tile: row l (16 bytes) = four 32-row groups x four k-blocks.  Tensor
     // memory wants exactly that word in lane l of every 32-lane quarter, one column per group.
@@ -683,19 +688,29 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         if (++b == C::kSfBufs) { b = 0; bph ^= 1u; }
       }
     }
-    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 6 && lane == 0, 8, a_land);
-    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 6 && lane == 0, 9, a_free);
-    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 6 && lane == 0, 10, a_total + ACCOUNT_NOW());
+    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 4 && lane == 0, 8, a_land);
+    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 4 && lane == 0, 9, a_free);
+    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 4 && lane == 0, 10, a_total + ACCOUNT_NOW());
+  }
   } else {
-    // ------------------------------- epilogue (both CTAs, warps 2-5) -------------------------------
-    const int quarter = warp & 3;
+    regs_acquire<kEpilogueRegs>();
+    // ------------------------------- epilogue (both CTAs, warps 8-15) -------------------------------
+    // The MMA issuer cannot start the next tile before this accumulator is read out, so the read-out must be short and
+    // nothing in it may wait for stores: two warps share each 32-lane quarter, every warp moves its whole share (128
+    // columns of a 256-wide tile) into registers, hands the accumulator back, and converts, stages and stores it while
+    // the next tile's MMAs run.
+    // Against four warps that held 3 of 8 chunks and streamed the others through their staging buffers (16384 x 11008 x
+    // 4096 with fp32 output: 366 -> 313 us, input gradient of the same layer 293 -> 259; chained bf16 layers 190 -> 182).
+    const int quarter = warp & 3, half = (warp >> 2) & 1;
     const float alpha = (p.a_g ? __ldg(p.a_g) : 1.0f) * (p.b_g ? __ldg(p.b_g) : 1.0f);
-    const uint32_t my_buf = epi_base + quarter * C::kEpiWarpBytes;
-    constexpr int kChunkCols = BF16_OUT ? 64 : 32;
+    const uint32_t buf = epi_base + (warp - 8) * C::kEpiWarpBytes;
+    constexpr int kChunkCols = BF16_OUT ? 64 : 32;                 // accumulator columns per 128 bytes of output row
     constexpr int kLoads = kChunkCols / 32;
+    constexpr int kChunks = Q_OUT ? BN / 32 : BN / kChunkCols;
+    constexpr int kHeld = (kChunks + 1) / 2;                       // chunks of this warp: [half * kHeld, +kHeld) below kChunks
     const uint32_t lead_tempty0 = map_to_cta(tempty_bar(0), 0);
     int acc = 0;
-    uint32_t acc_ph = 0, chunk_no = 0;
+    uint32_t acc_ph = 0;
     bool ok = true;
     ACCOUNT_VARS(a_tile = 0, a_read = 0, a_total = -ACCOUNT_NOW(), a_read_t0 = 0);
     for (int tile = pair; ok && tile < num_tiles; tile += num_pairs) {
@@ -708,157 +723,113 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 #endif
       tc_fence_after();
       const int row0 = tm * 256 + (int)rank * 128 + quarter * 32;
-      const uint32_t t_row = tmem_base + acc * BN + ((uint32_t)(quarter * 32) << 16);
+      const uint32_t t_row = tmem_base + acc * BN + half * (kHeld * kChunkCols) + ((uint32_t)(quarter * 32) << 16);
+      uint32_t r[kHeld * kLoads][32];
+#pragma unroll
+      for (int l = 0; l < kHeld * kLoads; ++l)
+        if (half * kHeld + l / kLoads < kChunks) tmem_ld32(t_row + 32 * l, r[l]);
+      tmem_ld_wait();
+#pragma unroll
+      for (int l = 0; l < kHeld * kLoads; ++l) tmem_ld_pin(r[l]);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8u * acc);  // accumulator fully read: hand it back to the leader
+#ifdef NVFP4_GEMM_ACCOUNT
+      a_read += clock64() - a_read_t0;
+#endif
       if constexpr (Q_OUT) {
-        // ---- quantized output: this lane's row, the tile's 256 columns = 16 blocks of 16 ----
+        // ---- quantized output: this lane's row, 128 of the tile's 256 columns = 8 blocks of 16 ----
         const float cq = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), p.out_g ? __ldg(p.out_g) : 1.0f);
         const int64_t row = (int64_t)row0 + lane;
-        uint32_t codes[32];                          // 128 bytes of codes
-        uint32_t sfw[4] = {0u, 0u, 0u, 0u};          // 16 scale bytes, four per k-tile
+        const int kb0 = tn * (BN / 16) + half * 8;
+        uint32_t sfw[2] = {0u, 0u};                  // 8 scale bytes, four per k-tile
+        if (lane == 0) tma_store_wait_read<0>();     // the previous tile's codes have left the buffer
+        __syncwarp();
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          uint32_t r[32];
-          tmem_ld32(t_row + 32 * c, r);
-          tmem_ld_wait();
-          tmem_ld_pin(r);
-          if (c == 7) {                              // accumulator fully read: hand it back to the leader
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8u * acc);
-          }
+        for (int c = 0; c < 4; ++c) {                // 32 columns = 2 blocks = 16 bytes of codes
+          uint32_t w[4];
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             float v[16], amax = 0.0f;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              v[j] = __uint_as_float(r[16 * h + j]) * alpha;     // the value the fp32 epilogue would store
+              v[j] = __uint_as_float(r[c][16 * h + j]) * alpha;  // the value the fp32 epilogue would store
               amax = fmaxf(amax, fabsf(v[j]));
             }
-            const int kbl = 2 * c + h;
-            const uint64_t blk = (uint64_t)(row * p.out_nkb + (int64_t)tn * (BN / 16) + kbl);
-            uint32_t lo, hi, sf;
-            if (p.out_sr) encode_block<true>(v, amax, cq, inv_table, p.out_rng, blk, lo, hi, sf);
-            else encode_block<false>(v, amax, cq, inv_table, p.out_rng, blk, lo, hi, sf);
-            codes[2 * kbl] = lo;
-            codes[2 * kbl + 1] = hi;
-            sfw[kbl >> 2] |= sf << (8 * (kbl & 3));
+            const uint64_t blk = (uint64_t)(row * p.out_nkb + kb0 + 2 * c + h);
+            uint32_t sf;
+            if (p.out_sr) encode_block<true>(v, amax, cq, inv_table, p.out_rng, blk, w[2 * h], w[2 * h + 1], sf);
+            else encode_block<false>(v, amax, cq, inv_table, p.out_rng, blk, w[2 * h], w[2 * h + 1], sf);
+            sfw[c >> 1] |= sf << (8 * ((2 * c + h) & 3));
           }
-        }
-        // codes: stage 32 rows x 128 bytes (128-byte swizzle) and store them as one box
-        const uint32_t buf = my_buf + (chunk_no & 1u) * 4096u;
-        if (chunk_no >= 2) {
-          if (lane == 0) tma_store_wait_read<1>();
-          __syncwarp();
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const uint32_t dst = buf + lane * 128 + ((c ^ (lane & 7)) << 4);
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(codes[4 * c]), "r"(codes[4 * c + 1]),
-                       "r"(codes[4 * c + 2]), "r"(codes[4 * c + 3]) : "memory");
+          // rows of 64 bytes, 64-byte swizzle: piece index XOR bits 7-8 of the row's offset
+          const uint32_t dst = buf + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
         }
         fence_async_smem();
         __syncwarp();
         if (lane == 0) {
-          tma_store_2d(&map_d, buf, tn * (BN / 2), row0);
+          tma_store_2d(&map_d, buf, tn * (BN / 2) + half * 64, row0);
           tma_store_commit();
         }
-        ++chunk_no;
         // scales
         if (p.out_swizzled) {
           if ((row >> 7) < (((int64_t)p.M + 127) >> 7)) {
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              const int64_t kt = (int64_t)tn * (BN / 64) + t;
+            for (int t = 0; t < 2; ++t) {
+              const int64_t kt = (int64_t)(kb0 >> 2) + t;
               if (kt < p.out_k_tiles)
                 *reinterpret_cast<uint32_t*>(p.out_scales + sf_swizzled_offset(row, kt * 4, p.out_k_tiles)) = sfw[t];
             }
           }
         } else if (row < p.M) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int64_t kb = (int64_t)tn * (BN / 16) + i;
+          for (int i = 0; i < 8; ++i) {
+            const int64_t kb = (int64_t)kb0 + i;
             if (kb < p.out_nkb) p.out_scales[row * p.out_nkb + kb] = (uint8_t)(sfw[i >> 2] >> (8 * (i & 3)));
           }
         }
-        if (++acc == C::kAccStages) { acc = 0; acc_ph ^= 1u; }
-        continue;
-      }
-      // The MMA issuer cannot start the next tile before this accumulator is read out, so the read-out is
-      // what must finish early, not the stores: the first kHeld chunks are converted and parked in
-      // registers, the others stream through the staging buffers, the accumulator is handed back
-      // as soon as the last of them is read, and the parked chunks are stored after that.
-      constexpr int kChunks = BN / kChunkCols;
-      constexpr int kHeld = (kChunks > 3) ? 3 : kChunks - 1;
-
-      // one chunk: accumulator columns [c0, c0 + kChunkCols) -> 32 output words (scaled, converted)
-      auto read_chunk = [&](int c0, uint32_t (&w)[32]) {
-        uint32_t r[kLoads][32];
+      } else {
+        // one chunk at a time: 32 rows x 128 bytes (row = lane, eight 16-byte pieces, piece index XOR (row & 7): the
+        // 128-byte swizzle), sent off as one tiled store
 #pragma unroll
-        for (int l = 0; l < kLoads; ++l) tmem_ld32(t_row + c0 + 32 * l, r[l]);
-        tmem_ld_wait();
+        for (int i = 0; i < kHeld; ++i) {
+          const int c = half * kHeld + i;
+          if (c >= kChunks) break;
+          uint32_t w[32];
+          if constexpr (BF16_OUT) {
 #pragma unroll
-        for (int l = 0; l < kLoads; ++l) tmem_ld_pin(r[l]);
-        if constexpr (BF16_OUT) {
+            for (int e = 0; e < 32; ++e) {
+              const uint32_t* q = r[i * kLoads + e / 16] + 2 * (e % 16);
+              const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(q[0]) * alpha, __uint_as_float(q[1]) * alpha);
+              w[e] = *reinterpret_cast<const uint32_t*>(&h2);
+            }
+          } else {
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(r[0][2 * e]) * alpha, __uint_as_float(r[0][2 * e + 1]) * alpha);
-            const __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(r[kLoads - 1][2 * e]) * alpha, __uint_as_float(r[kLoads - 1][2 * e + 1]) * alpha);
-            w[e] = *reinterpret_cast<const uint32_t*>(&h0);
-            w[16 + e] = *reinterpret_cast<const uint32_t*>(&h1);
+            for (int e = 0; e < 32; ++e) w[e] = __float_as_uint(__uint_as_float(r[i][e]) * alpha);
           }
-        } else {
-#pragma unroll
-          for (int e = 0; e < 32; ++e) w[e] = __float_as_uint(__uint_as_float(r[0][e]) * alpha);
-        }
-      };
-      // stage 32 rows x 128 bytes (row = lane, eight 16-byte pieces, piece index XOR (row & 7): the
-      // 128-byte swizzle) and send them off as one tiled store
-      auto store_chunk = [&](int c0, const uint32_t (&w)[32]) {
-        const uint32_t buf = my_buf + (chunk_no & 1u) * 4096u;
-        if (chunk_no >= 2) {                        // the store issued two chunks ago has read this buffer
-          if (lane == 0) tma_store_wait_read<1>();
+          if (lane == 0) tma_store_wait_read<0>();  // the chunk stored before this one has left the buffer
           __syncwarp();
-        }
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const uint32_t dst = buf + lane * 128 + ((c ^ (lane & 7)) << 4);
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[4 * c]), "r"(w[4 * c + 1]),
-                       "r"(w[4 * c + 2]), "r"(w[4 * c + 3]) : "memory");
-        }
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          tma_store_2d(&map_d, buf, tn * BN + c0, row0);
-          tma_store_commit();
-        }
-        ++chunk_no;
-      };
-
-      uint32_t held[kHeld][32];
-#pragma unroll
-      for (int h = 0; h < kHeld; ++h) read_chunk(h * kChunkCols, held[h]);
-#pragma unroll 1
-      for (int c = kHeld; c < kChunks; ++c) {
-        uint32_t w[32];
-        read_chunk(c * kChunkCols, w);
-        if (c == kChunks - 1) {                     // accumulator fully read: hand it back to the leader
-          tc_fence_before();
+          for (int e = 0; e < 8; ++e) {
+            const uint32_t dst = buf + lane * 128 + ((e ^ (lane & 7)) << 4);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[4 * e]), "r"(w[4 * e + 1]),
+                         "r"(w[4 * e + 2]), "r"(w[4 * e + 3]) : "memory");
+          }
+          fence_async_smem();
           __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8u * acc);
-#ifdef NVFP4_GEMM_ACCOUNT
-          a_read += clock64() - a_read_t0;
-#endif
+          if (lane == 0) {
+            tma_store_2d(&map_d, buf, tn * BN + c * kChunkCols, row0);
+            tma_store_commit();
+          }
         }
-        store_chunk(c * kChunkCols, w);
       }
-#pragma unroll
-      for (int h = 0; h < kHeld; ++h) store_chunk(h * kChunkCols, held[h]);
       if (++acc == C::kAccStages) { acc = 0; acc_ph ^= 1u; }
     }
     if (lane == 0) tma_store_wait_all();
-    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 2 && lane == 0, 12, a_tile);
-    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 2 && lane == 0, 13, a_read);
-    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 2 && lane == 0, 14, a_total + ACCOUNT_NOW());
+    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 8 && lane == 0, 12, a_tile);
+    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 8 && lane == 0, 13, a_read);
+    ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 8 && lane == 0, 14, a_total + ACCOUNT_NOW());
   }
 
   tc_fence_before();
@@ -938,16 +909,16 @@ struct QuantOut {
   int sf_layout = NVFP4_SF_LINEAR;
 };
 
-// Packed codes of the quantized output [M, N/2 bytes] -> boxes of 32 rows x 128 bytes, 128-byte swizzle.
+// Packed codes of the quantized output [M, N/2 bytes] -> boxes of 32 rows x 64 bytes, 64-byte swizzle.
 bool make_qout_map(CUtensorMap* map, uint8_t* base, int64_t M, int64_t N) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)(N / 2), (cuuint64_t)M};
   const cuuint64_t strides[1] = {(cuuint64_t)(N / 2)};
-  const cuuint32_t box[2] = {128, 32};
+  const cuuint32_t box[2] = {64, 32};
   const cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+            CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0>

@@ -116,6 +116,12 @@ __device__ __forceinline__ void tmem_ld_pin(uint32_t (&r)[32]) {
                       "+r"(r[i + 6]), "+r"(r[i + 7]) :: "memory");
 }
 
+// Register budget of the calling warpgroup (every warp of it executes the same one): give back down to N, or take up to N.
+template <int N>
+__device__ __forceinline__ void regs_release() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void regs_acquire() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+
 // ---- cluster / CTA-pair helpers (cta_group::2 path) ----
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
