@@ -35,6 +35,17 @@ __device__ __forceinline__ void build_inv_table_mx(float* inv_table, float g) {
     inv_table[q] = (q == 0 || q == 255) ? 0.0f : __fdiv_rn(1.0f, __fmul_rn(__uint_as_float((uint32_t)q << 23), g));
 }
 
+// Two products in one instruction (each rounded to nearest by itself, as two __fmul_rn).
+// The stochastic encoders are bound by instruction issue: one multiply less per two values took the row quantizer
+// from 35.7 to 33.3 us and the transposed one from 35.4 to 34.5 on 8192 x 8192.
+__device__ __forceinline__ void mul2(float a0, float a1, float b, float& y0, float& y1) {
+  asm("{\n\t.reg .b64 a, b, y;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\t"
+      "mul.rn.f32x2 y, a, b;\n\t"
+      "mov.b64 {%0, %1}, y;\n\t}"
+      : "=f"(y0), "=f"(y1) : "f"(a0), "f"(a1), "f"(b));
+}
+
 // 16 values (signed, already widened to fp32) scaled by inv -> 8 bytes of codes (lo, hi words).
 // `blk` is the linear index of this group of 16 (Philox counter).
 template <bool SR>
@@ -56,7 +67,7 @@ __device__ __forceinline__ void encode_codes(const float (&v)[16], float inv, co
                                              uint32_t& lo, uint32_t& hi) {
   float y[16];
 #pragma unroll
-  for (int j = 0; j < 16; ++j) y[j] = __fmul_rn(v[j], inv);     // the sign rides along; the conversions clamp at 6
+  for (int j = 0; j < 16; j += 2) mul2(v[j], v[j + 1], inv, y[j], y[j + 1]);   // the sign rides along; the conversions clamp at 6
   if constexpr (!SR) {
     lo = e2m1x8_rn(y, 0);
     hi = e2m1x8_rn(y, 8);
