@@ -34,6 +34,43 @@ inline cudaError_t set_max_dynamic_smem(DeviceFlags& flags, Kernel kernel, int b
   return err;
 }
 
+// Launch whose blocks may become resident while the kernel before it on the stream still runs (programmatic dependent
+// launch): barrier set-up, tensor-memory allocation and descriptor fetches of a kernel then overlap the tail of the one
+// before.  The rules every kernel launched this way keeps:
+//   * it calls grid_dependency_wait() in every block, before its first access to memory that an earlier kernel may
+//     still read or write; when that returns, the kernel before it has finished and its writes are visible;
+//   * it calls grid_dependency_trigger() only after that wait.  A kernel that follows it directly therefore starts when
+//     everything TWO launches back is finished, and may read that without waiting ("late" kernels), as long as it still
+//     waits before it ends, so that "finished" keeps meaning "and all before it".
+// After anything else on the stream (a kernel that does not take part, a copy) the attribute changes nothing.
+// One step of a 256-token layer (11 kernels of 3.5-8 us): 61.3 -> 47.5 us; of a 2080 x 1056 x 2848 one: 85.9 -> 68.6.
+// `overlap` false: an ordinary launch (its waits then return at once).
+template <class... Params, class... Args>
+inline cudaError_t launch_overlapped_if(bool overlap, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                        Args&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <class... Params, class... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+  return launch_overlapped_if(true, kernel, grid, block, smem, s, args...);
+}
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Zeroes up to 32 words (quantize.cu), overlapping the kernel before it.
+cudaError_t zero_words(unsigned int* words, int n, cudaStream_t s);
+
+// nvfp4_gemm for a caller inside the library (gemm.cu).  late: the product before this one on the stream is independent
+// of it and everything else it reads was finished before that one began, so its tiles may fill that one's last wave.
+int gemm_checked(const uint8_t* a_codes, const uint8_t* a_sf, const float* a_g, const uint8_t* b_codes, const uint8_t* b_sf,
+                 const float* b_g, int64_t M, int64_t N, int64_t K, void* d, int d_dtype, int64_t ldd, void* cuda_stream, bool late);
+
 // Tile quantizer (quantize_tile.cu): transposed output, optionally the row output from the same read.
 bool tile_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool dual);
 int tile_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, const float* g, bool dual,
@@ -43,6 +80,7 @@ int tile_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, const f
 int tile_error_word(unsigned int* out);
 
 // Per-tensor scale g = amax/2688 in one launch (quantize.cu); scratch_zeroed: two zeroed 32-bit device words.
+// The kernel reads x before it waits for the one launched before it: x must be older than that.
 int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* g_out,
                          unsigned int* scratch_zeroed, void* cuda_stream);
 

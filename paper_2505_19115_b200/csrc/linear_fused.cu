@@ -87,7 +87,7 @@ int resolve_g(int gscale_mode, const void* x, int dtype, int64_t rows, int64_t c
 
 int zero_scratch(int gscale_mode, void* scratch, void* stream) {
   if (gscale_mode != NVFP4_G_AMAX) return NVFP4_OK;
-  return cudaMemsetAsync(scratch, 0, 64, static_cast<cudaStream_t>(stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  return zero_words(static_cast<unsigned int*>(scratch), 16, static_cast<cudaStream_t>(stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
 }  // namespace
@@ -159,7 +159,8 @@ int run_bwd(const void* dY, int dtype, int64_t M, int64_t N, int64_t K, const fl
     return st;
   if (int st = nvfp4_gemm(ws + bl.dy.codes, ws + bl.dy.sf, g_dy, wt_codes, wt_sf, g_w, M, K, N, dX, dx_dtype, K, stream))
     return st;
-  return nvfp4_gemm(ws + bl.dyt.codes, ws + bl.dyt.sf, g_dy, xt_codes, xt_sf, g_x, N, K, M, dW, dw_dtype, K, stream);
+  // independent of the product before it: its first tiles fill that one's last wave
+  return gemm_checked(ws + bl.dyt.codes, ws + bl.dyt.sf, g_dy, xt_codes, xt_sf, g_x, N, K, M, dW, dw_dtype, K, stream, /*late=*/true);
 }
 }  // namespace
 

@@ -33,6 +33,8 @@ __global__ void __launch_bounds__(kThreads, 3) quantize_row_kernel(const QuantPa
   const int64_t kb = (int64_t)blockIdx.x * 32 + lane;
   const int64_t row0 = (int64_t)blockIdx.y * kRowTileRows;
   const bool kb_ok = kb < p.nkb;
+  grid_dependency_wait();
+  grid_dependency_trigger();
   const float g = p.gptr ? __ldg(p.gptr) : 1.0f;
   const float c = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), g);
   const T* x = static_cast<const T*>(p.x);
@@ -140,6 +142,8 @@ __global__ void __launch_bounds__(kThreads, 3) quantize_transposed_kernel(const 
   const int64_t c0 = (int64_t)blockIdx.x * kTCols;
   const int64_t r0 = (int64_t)blockIdx.y * TT::kRows;
   const T* x = static_cast<const T*>(p.x);
+  grid_dependency_wait();
+  grid_dependency_trigger();
   const float g = p.gptr ? __ldg(p.gptr) : 1.0f;
   const float c = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), g);
   __shared__ float inv_table[128];
@@ -307,6 +311,8 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const T* x, int64_t rows
     acc.add4(q.x, q.y, q.z, q.w);
   }
   const uint32_t bits = acc.warp_bits();
+  grid_dependency_wait();                                      // the accumulator is zero; x is older than the kernel that zeroed it
+  grid_dependency_trigger();
   if ((threadIdx.x & 31) == 0 && bits != 0u) atomicMax(out_bits, bits);
 }
 
@@ -339,6 +345,8 @@ __global__ void __launch_bounds__(kThreads) amax_flat_kernel(const uint32_t* x, 
     for (int u = 0; u < 4; ++u) acc.add8(w[u]);
   }
   const uint32_t bits = acc.warp_bits();
+  grid_dependency_wait();                                      // `out` is zero; x is older than the kernel before this one
+  grid_dependency_trigger();
   if constexpr (!TICKET) {
     if ((threadIdx.x & 31) == 0 && bits != 0u) atomicMax(out, bits);
   } else {
@@ -361,15 +369,22 @@ __global__ void __launch_bounds__(kThreads) amax_flat_kernel(const uint32_t* x, 
 }
 
 __global__ void amax_finalize_kernel(float* out) {
+  grid_dependency_wait();
+  grid_dependency_trigger();
   const float amax = *out;
   *out = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 2688.0f);
+}
+
+__global__ void zero_words_kernel(unsigned int* words, int n) {
+  grid_dependency_wait();
+  grid_dependency_trigger();
+  if ((int)threadIdx.x < n) words[threadIdx.x] = 0u;
 }
 
 template <typename T, bool SR, bool SWZ>
 cudaError_t launch_row(const QuantParams& p, cudaStream_t s) {
   dim3 grid((unsigned)ceil_div(p.nkb, 32), (unsigned)ceil_div(p.rows, kRowTileRows));
-  quantize_row_kernel<T, SR, SWZ><<<grid, kThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(quantize_row_kernel<T, SR, SWZ>, grid, kThreads, 0, s, p);
 }
 
 template <typename T, bool SR, bool SWZ>
@@ -379,8 +394,7 @@ cudaError_t launch_transposed(const QuantParams& p, cudaStream_t s) {
   static DeviceFlags smem_set;   // per instantiation, per device
   if (cudaError_t e = set_max_dynamic_smem(smem_set, quantize_transposed_kernel<T, SR, SWZ>, (int)smem)) return e;
   dim3 grid((unsigned)ceil_div(p.cols, kTCols), (unsigned)ceil_div(p.rows, TT::kRows));
-  quantize_transposed_kernel<T, SR, SWZ><<<grid, kThreads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(quantize_transposed_kernel<T, SR, SWZ>, grid, kThreads, smem, s, p);
 }
 
 template <typename T>
@@ -443,14 +457,10 @@ namespace {
 template <typename T>
 cudaError_t dispatch_row_mx(const QuantParams& p, bool sr, bool swz, cudaStream_t s) {
   dim3 grid((unsigned)ceil_div(p.nkb, 32), (unsigned)ceil_div(p.rows, kRowTileRows));
-  if (sr) {
-    if (swz) quantize_row_kernel<T, true, true, true><<<grid, kThreads, 0, s>>>(p);
-    else quantize_row_kernel<T, true, false, true><<<grid, kThreads, 0, s>>>(p);
-  } else {
-    if (swz) quantize_row_kernel<T, false, true, true><<<grid, kThreads, 0, s>>>(p);
-    else quantize_row_kernel<T, false, false, true><<<grid, kThreads, 0, s>>>(p);
-  }
-  return cudaGetLastError();
+  if (sr) return swz ? launch_overlapped(quantize_row_kernel<T, true, true, true>, grid, kThreads, 0, s, p)
+                     : launch_overlapped(quantize_row_kernel<T, true, false, true>, grid, kThreads, 0, s, p);
+  return swz ? launch_overlapped(quantize_row_kernel<T, false, true, true>, grid, kThreads, 0, s, p)
+             : launch_overlapped(quantize_row_kernel<T, false, false, true>, grid, kThreads, 0, s, p);
 }
 }  // namespace
 }  // namespace nvfp4
@@ -547,11 +557,15 @@ int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, i
   const int64_t n32 = total_bytes / 32;
   int64_t fb = ceil_div(n32, (int64_t)kThreads * 4);
   if (fb > sm_count() * 8) fb = sm_count() * 8;
-  if (dtype == NVFP4_BF16)
-    amax_flat_kernel<__nv_bfloat16, true><<<(unsigned)fb, kThreads, 0, s>>>(static_cast<const uint32_t*>(x), n32, scratch_zeroed, g_out);
-  else
-    amax_flat_kernel<float, true><<<(unsigned)fb, kThreads, 0, s>>>(static_cast<const uint32_t*>(x), n32, scratch_zeroed, g_out);
-  return cudaGetLastError() == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  const uint32_t* xw = static_cast<const uint32_t*>(x);
+  const cudaError_t e = (dtype == NVFP4_BF16)
+      ? launch_overlapped(amax_flat_kernel<__nv_bfloat16, true>, (unsigned)fb, kThreads, 0, s, xw, n32, scratch_zeroed, g_out)
+      : launch_overlapped(amax_flat_kernel<float, true>, (unsigned)fb, kThreads, 0, s, xw, n32, scratch_zeroed, g_out);
+  return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
+
+cudaError_t zero_words(unsigned int* words, int n, cudaStream_t s) {
+  return launch_overlapped(zero_words_kernel, 1, 32, 0, s, words, n);
 }
 }  // namespace nvfp4
 
@@ -563,26 +577,26 @@ extern "C" int nvfp4_tensor_amax_scale(const void* x, int dtype, int64_t rows, i
   if (!aligned16(x) || (ld % 8) != 0 || (reinterpret_cast<uintptr_t>(global_scale_out) & 3u)) return NVFP4_ERR_ALIGN;
   if (int st = check_arch()) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  if (cudaMemsetAsync(global_scale_out, 0, sizeof(float), s) != cudaSuccess) return NVFP4_ERR_CUDA;
-  const int64_t vecs = rows * (cols / (dtype == NVFP4_BF16 ? 8 : 4));
-  int64_t blocks = ceil_div(vecs, (int64_t)kThreads * 4);
-  if (blocks > sm_count() * 16) blocks = sm_count() * 16;
-  if (blocks < 1) blocks = 1;
   unsigned int* bits = reinterpret_cast<unsigned int*>(global_scale_out);
+  if (zero_words(bits, 1, s) != cudaSuccess) return NVFP4_ERR_CUDA;
   const int64_t total_bytes = rows * cols * (dtype == NVFP4_BF16 ? 2 : 4);
+  cudaError_t e;
   if (ld == cols && (reinterpret_cast<uintptr_t>(x) & 31u) == 0 && total_bytes % 32 == 0) {
     const int64_t n32 = total_bytes / 32;
     int64_t fb = ceil_div(n32, (int64_t)kThreads * 4);
     if (fb > sm_count() * 8) fb = sm_count() * 8;
-    if (dtype == NVFP4_BF16)
-      amax_flat_kernel<__nv_bfloat16, false><<<(unsigned)fb, kThreads, 0, s>>>(static_cast<const uint32_t*>(x), n32, bits, nullptr);
-    else
-      amax_flat_kernel<float, false><<<(unsigned)fb, kThreads, 0, s>>>(static_cast<const uint32_t*>(x), n32, bits, nullptr);
-  } else if (dtype == NVFP4_BF16)
-    amax_kernel<__nv_bfloat16><<<(unsigned)blocks, kThreads, 0, s>>>(static_cast<const __nv_bfloat16*>(x), rows, cols, ld, bits);
-  else
-    amax_kernel<float><<<(unsigned)blocks, kThreads, 0, s>>>(static_cast<const float*>(x), rows, cols, ld, bits);
-  if (cudaGetLastError() != cudaSuccess) return NVFP4_ERR_CUDA;
-  amax_finalize_kernel<<<1, 1, 0, s>>>(global_scale_out);
-  return cudaGetLastError() == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+    const uint32_t* xw = static_cast<const uint32_t*>(x);
+    e = (dtype == NVFP4_BF16)
+        ? launch_overlapped(amax_flat_kernel<__nv_bfloat16, false>, (unsigned)fb, kThreads, 0, s, xw, n32, bits, (float*)nullptr)
+        : launch_overlapped(amax_flat_kernel<float, false>, (unsigned)fb, kThreads, 0, s, xw, n32, bits, (float*)nullptr);
+  } else {
+    const int64_t vecs = rows * (cols / (dtype == NVFP4_BF16 ? 8 : 4));
+    int64_t blocks = ceil_div(vecs, (int64_t)kThreads * 4);
+    if (blocks > sm_count() * 16) blocks = sm_count() * 16;
+    e = (dtype == NVFP4_BF16)
+        ? launch_overlapped(amax_kernel<__nv_bfloat16>, (unsigned)blocks, kThreads, 0, s, static_cast<const __nv_bfloat16*>(x), rows, cols, ld, bits)
+        : launch_overlapped(amax_kernel<float>, (unsigned)blocks, kThreads, 0, s, static_cast<const float*>(x), rows, cols, ld, bits);
+  }
+  if (e == cudaSuccess) e = launch_overlapped(amax_finalize_kernel, 1, 1, 0, s, global_scale_out);
+  return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }

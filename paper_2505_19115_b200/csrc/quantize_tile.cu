@@ -101,6 +101,8 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t c0 = (int64_t)blockIdx.x * kTileCols;
   const int64_t r0 = (int64_t)blockIdx.y * kTileRows;
+  grid_dependency_wait();
+  grid_dependency_trigger();
   const float g = p.gptr ? __ldg(p.gptr) : 1.0f;
   const float c = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), g);
 
@@ -365,8 +367,7 @@ cudaError_t launch_tile(const CUtensorMap& mx, const CUtensorMap& mct, const CUt
   static DeviceFlags smem_set;   // per instantiation, per device
   if (cudaError_t e = set_max_dynamic_smem(smem_set, quantize_tile_kernel<SR_T, DUAL, SR_R, SWZ, MX_T>, kTileSmem)) return e;
   dim3 grid((unsigned)ceil_div(p.cols, kTileCols), (unsigned)ceil_div(p.rows, kTileRows));
-  quantize_tile_kernel<SR_T, DUAL, SR_R, SWZ, MX_T><<<grid, kThreads, kTileSmem, s>>>(mx, mct, mcr, p);
-  return cudaGetLastError();
+  return launch_overlapped(quantize_tile_kernel<SR_T, DUAL, SR_R, SWZ, MX_T>, grid, kThreads, kTileSmem, s, mx, mct, mcr, p);
 }
 
 template <bool DUAL, bool SWZ>
