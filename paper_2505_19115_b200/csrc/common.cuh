@@ -73,7 +73,7 @@ int gemm_checked(const uint8_t* a_codes, const uint8_t* a_sf, const float* a_g, 
 
 // Tile quantizer (quantize_tile.cu): transposed output, optionally the row output from the same read.
 bool tile_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool dual);
-int tile_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, const float* g, bool dual,
+int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, const float* g, bool dual,
                   const nvfp4_rounding* rt, uint8_t* codes_t, uint8_t* scales_t,
                   const nvfp4_rounding* rr, uint8_t* codes_r, uint8_t* scales_r, int sf_layout, cudaStream_t s,
                   bool mx_t = false);   // mx_t: MXFP4 (blocks of 32, E8M0 scales) for the transposed output, no row output

@@ -444,7 +444,7 @@ extern "C" int nvfp4_quantize(const void* x, int dtype, int64_t rows, int64_t co
   if (ceil_div(rows, 128) > 65535) return NVFP4_ERR_SHAPE;  // grid.y limit
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   if (transposed && tile_quantizer_eligible(dtype, rows, cols, false))
-    return tile_quantize(x, rows, cols, ld, global_scale, false, rounding, codes, scales, nullptr, nullptr, nullptr,
+    return tile_quantize(x, dtype, rows, cols, ld, global_scale, false, rounding, codes, scales, nullptr, nullptr, nullptr,
                          sf_layout, s);
   const bool sr = rounding->mode == NVFP4_SR, swz = sf_layout == NVFP4_SF_SWIZZLED_128x4;
   cudaError_t e = (dtype == NVFP4_BF16) ? dispatch<__nv_bfloat16>(p, transposed != 0, sr, swz, s)
@@ -496,7 +496,7 @@ extern "C" int nvfp4_quantize_mx(const void* x, int dtype, int64_t rows, int64_t
   if (int st = check_arch()) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   if (tile_path)
-    return tile_quantize(x, rows, cols, ld, global_scale, false, rounding, codes, scales, nullptr, nullptr, nullptr, sf_layout, s,
+    return tile_quantize(x, dtype, rows, cols, ld, global_scale, false, rounding, codes, scales, nullptr, nullptr, nullptr, sf_layout, s,
                          /*mx_t=*/true);
   const void* src = x;
   int64_t src_ld = ld;
@@ -533,7 +533,7 @@ extern "C" int nvfp4_quantize_dual(const void* x, int dtype, int64_t rows, int64
     return NVFP4_ERR_ALIGN;
   if (int st = check_arch()) return st;
   if (tile_quantizer_eligible(dtype, rows, cols, true))
-    return tile_quantize(x, rows, cols, ld, global_scale, true, rounding_t, codes_t, scales_t, rounding_row, codes_row,
+    return tile_quantize(x, dtype, rows, cols, ld, global_scale, true, rounding_t, codes_t, scales_t, rounding_row, codes_row,
                          scales_row, sf_layout, static_cast<cudaStream_t>(cuda_stream));
   // shapes or types the tile kernel does not take: the two single-output kernels, two reads
   if (int st = nvfp4_quantize(x, dtype, rows, cols, ld, 0, global_scale, rounding_row, codes_row, scales_row, sf_layout,

@@ -62,9 +62,9 @@ __device__ __forceinline__ void encode_block(const float (&v)[16], float amax, f
   encode_codes<SR>(v, inv_table[q], rng, blk, lo, hi);
 }
 
+// The same with the random words given (unused when rounding to nearest).
 template <bool SR>
-__device__ __forceinline__ void encode_codes(const float (&v)[16], float inv, const PhiloxStream& rng, uint64_t blk,
-                                             uint32_t& lo, uint32_t& hi) {
+__device__ __forceinline__ void encode_with(const float (&v)[16], float inv, const uint4& r4, uint32_t& lo, uint32_t& hi) {
   float y[16];
 #pragma unroll
   for (int j = 0; j < 16; j += 2) mul2(v[j], v[j + 1], inv, y[j], y[j + 1]);   // the sign rides along; the conversions clamp at 6
@@ -72,10 +72,17 @@ __device__ __forceinline__ void encode_codes(const float (&v)[16], float inv, co
     lo = e2m1x8_rn(y, 0);
     hi = e2m1x8_rn(y, 8);
   } else {
-    const uint4 r4 = philox4x32_10(rng, (uint32_t)blk, (uint32_t)(blk >> 32));
     lo = e2m1x8_rs(y, 0, r4.x, r4.y);
     hi = e2m1x8_rs(y, 8, r4.z, r4.w);
   }
+}
+
+template <bool SR>
+__device__ __forceinline__ void encode_codes(const float (&v)[16], float inv, const PhiloxStream& rng, uint64_t blk,
+                                             uint32_t& lo, uint32_t& hi) {
+  uint4 r4 = make_uint4(0, 0, 0, 0);
+  if constexpr (SR) r4 = philox4x32_10(rng, (uint32_t)blk, (uint32_t)(blk >> 32));
+  encode_with<SR>(v, inv, r4, lo, hi);
 }
 
 // max |.| of two packed bf16 pairs, per half (the sign bits of the result are meaningless)

@@ -1,13 +1,15 @@
-// Tile quantizer for bf16 tensors: one read of x[rows, cols] produces the transposed NVFP4
-// quantization (blocks of 16 along the row axis, output stored [cols, rows/2]) and, optionally, the
-// row quantization (blocks along the column axis) of the same tile.  This is the producer fusion
-// for the operands that Eq. 4-6 need in both orientations: dY as Q(dY) for Eq. 5 and Q(dY^T) for
-// Eq. 6, X as Q(X) for Eq. 4 and Q(X^T) for Eq. 6, W as Q(W) for Eq. 4 and Q(W^T) for Eq. 5.
+// Tile quantizer: one read of x[rows, cols] produces the transposed NVFP4 quantization (blocks of 16 along the row
+// axis, output stored [cols, rows/2]) and, optionally, the row quantization (blocks along the column axis) of the same
+// tile.  This is the producer fusion for the operands that Eq. 4-6 need in both orientations: dY as Q(dY) for Eq. 5 and
+// Q(dY^T) for Eq. 6, X as Q(X) for Eq. 4 and Q(X^T) for Eq. 6, W as Q(W) for Eq. 4 and Q(W^T) for Eq. 5.
 //
-// A CTA takes a tile of 256 rows x 64 columns (32 KB).  One thread fetches it with a tiled bulk
-// copy (128-byte swizzle, zero fill outside the tensor); all threads quantize from shared memory;
-// the packed codes are staged in shared memory and leave as tiled bulk stores (which clip at the
-// tensor edge), the scales as plain stores.
+// Persistent blocks walk over tiles of 128 or 256 rows x 64 columns.  One thread fetches tiles with tiled bulk copies
+// (128-byte swizzle, zero fill outside the tensor); all threads quantize from shared memory; the packed codes are staged
+// in shared memory and leave as tiled bulk stores (which clip at the tensor edge), the scales as plain stores.
+//
+// Bound by instruction issue where it rounds stochastically, by memory otherwise.  Against one 256-row tile per block and,
+// for fp32, two single-output passes (us): fp32 16384 x 4096, both outputs, RtN 101 -> 53 and SR 115 -> 56; bf16 256 x 512
+// 3.1 -> 2.3 and 3.5 -> 2.7; 16384 x 1024 11.4 -> 9.9 and 16.0 -> 15.5; 65536 x 4096 transposed SR 118 -> 115.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -19,19 +21,35 @@
 namespace nvfp4 {
 namespace {
 
-constexpr int kTileRows = 256;
 constexpr int kTileCols = 64;
-constexpr int kTileBytes = kTileRows * kTileCols * 2;                 // 32 KB, rows of 128 bytes
-constexpr int kCodesTBytes = kTileCols * (kTileRows / 2);             // 64 output rows x 128 bytes
-constexpr int kCodesRBytes = kTileRows * (kTileCols / 2);             // 256 output rows x 32 bytes
-constexpr int kSfTBytes = kTileCols * (kTileRows / 16);               // [16 row blocks][64 columns]
-constexpr int kSfRBytes = 2 * 512;                                    // two scale tiles (128 rows x 4 blocks)
-constexpr int kTileSmem = kTileBytes + kCodesTBytes + kCodesRBytes + kSfTBytes + kSfRBytes + 1024 /*align*/;
 constexpr unsigned long long kTileWaitLimitNs = 2000000000ull;
+constexpr int kLoader = kThreads - 32;                                // the thread that issues the bulk copies
+
+// Shared memory of a block, in order: tile slots, code staging, scale staging (two of it, used in turn).
+// Two slots: the tile after next lands while the present one is quantized, codes are staged in turn as well.  One slot:
+// the next tile is fetched when the present one's codes have left their staging buffer; the other blocks of the SM cover.
+template <typename T, int ROWS, bool DUAL, int SLOTS>
+struct TileSmem {
+  static constexpr int kBoxBytes = ROWS * 128;                        // a copy's box is 128 bytes wide: 64 bf16 or 32 fp32 columns
+  static constexpr int kBoxes = kTileCols * (int)sizeof(T) / 128;
+  static constexpr int kTileBytes = kBoxes * kBoxBytes;
+  static constexpr int kCodesTBytes = kTileCols * (ROWS / 2);         // 64 output rows, swizzled over their 64 or 128 bytes
+  static constexpr int kCodesRBytes = DUAL ? ROWS * (kTileCols / 2) : 0;   // ROWS output rows x 32 bytes
+  static constexpr int kCodesBytes = kCodesTBytes + kCodesRBytes;
+  static constexpr int kSfTBytes = kTileCols * (ROWS / 16);           // [row block][64 columns]
+  static constexpr int kSfRBytes = DUAL ? (ROWS / 128) * 512 : 0;     // whole scale tiles (128 rows x 4 blocks)
+  static constexpr int kSfBytes = kSfTBytes + kSfRBytes;
+  static constexpr int kCodesAt = SLOTS * kTileBytes, kSfAt = kCodesAt + SLOTS * kCodesBytes;
+  static constexpr int kBytes = kSfAt + 2 * kSfBytes + 1024 /*align*/;
+  static constexpr int kBlocksPerSm = sizeof(T) == 2 ? 4 : 2;
+  static_assert(kBlocksPerSm * (kBytes + 1024 /*static*/ + 1024 /*reserved*/) <= 228 * 1024, "shared memory of an SM");
+};
 
 struct TileParams {
   const float* gptr;
   int64_t rows, cols;
+  int tiles_x, tiles;         // tiles across the columns, in all
+  int step_x, step_y;         // distance between two tiles of a block: gridDim.x = step_y * tiles_x + step_x
   // transposed output (always): quantized shape (cols, rows)
   PhiloxStream t_rng;
   uint8_t* t_scales;
@@ -47,22 +65,20 @@ __device__ unsigned int g_tile_error_word = 0;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// byte offset of (row, byte) inside a tile of 128-byte rows stored with the 128-byte swizzle
-__device__ __forceinline__ uint32_t swz128(uint32_t row, uint32_t byte) {
-  return row * 128u + ((((byte >> 4) ^ (row & 7u)) << 4) | (byte & 15u));
-}
-
-// MX_T: the transposed output is MXFP4 (Section 3, Table 1): blocks of 32 rows with an E8M0 scale rounded up to a
-// power of two; a warp then takes 32 rows at a time, and the two groups of 16 inside a block keep their own
-// random draws (group index as for NVFP4).
 // Shared-memory accesses with the address split into a register part and a compile-time byte offset, so that
 // the unrolled loops below spend no instructions on addresses.  The loads are plain (not volatile) statements, so
 // that the compiler may schedule them ahead of the arithmetic of the previous block; the tile they read is written
-// once, by the bulk copy, and their base address is taken only after the wait for that copy (tile_base_after_wait).
+// by the bulk copy before the wait, and their base address is taken only after that wait (after_wait).
 template <int IMM>
 __device__ __forceinline__ uint32_t lds32(uint32_t addr) {
   uint32_t v;
   asm("ld.shared.b32 %0, [%1 + %2];" : "=r"(v) : "r"(addr), "n"(IMM));
+  return v;
+}
+template <int IMM>
+__device__ __forceinline__ float2 lds64(uint32_t addr) {
+  float2 v;
+  asm("ld.shared.v2.f32 {%0, %1}, [%2 + %3];" : "=f"(v.x), "=f"(v.y) : "r"(addr), "n"(IMM));
   return v;
 }
 template <int IMM>
@@ -71,10 +87,8 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
   asm("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4 + %5];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr), "n"(IMM));
   return v;
 }
-// The tile's shared-memory address as a value the compiler must consider produced here: every load whose address
-// derives from it stays behind the point of the call.
-__device__ __forceinline__ uint32_t tile_base_after_wait(const void* tile) {
-  uint32_t a = smem_addr(tile);
+// An address the compiler must consider produced here: every load whose address derives from it stays behind the call.
+__device__ __forceinline__ uint32_t after_wait(uint32_t a) {
   asm volatile("" : "+r"(a) :: "memory");
   return a;
 }
@@ -82,271 +96,263 @@ template <int IMM>
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t lo, uint32_t hi) {
   asm volatile("st.shared.v2.b32 [%0 + %3], {%1, %2};" ::"r"(addr), "r"(lo), "r"(hi), "n"(IMM) : "memory");
 }
+template <int I>
+using Const = std::integral_constant<int, I>;
+// f(Const<0>) ... f(Const<N - 1>)
+template <int N, int I = 0, typename F>
+__device__ __forceinline__ void unrolled(F&& f) {
+  if constexpr (I < N) {
+    f(Const<I>{});
+    unrolled<N, I + 1>(f);
+  }
+}
 
-template <bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T = false>
-__global__ void __launch_bounds__(kThreads, 4)
+// Bounded wait for a tile; false (and an error word) when the time ran out.
+__device__ __forceinline__ bool wait_tile(uint32_t bar, uint32_t parity) {
+  unsigned long long t0 = 0;
+  for (uint32_t spin = 0;; ++spin) {
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    if (done) return true;
+    if ((spin & 255u) == 255u) {
+      unsigned long long now;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (t0 == 0) t0 = now;
+      if (now - t0 > kTileWaitLimitNs) {
+        atomicOr(&g_tile_error_word, 0x200u);
+        return false;
+      }
+    }
+  }
+}
+
+// MX_T: the transposed output is MXFP4 (Section 3, Table 1): blocks of 32 rows with an E8M0 scale rounded up to a
+// power of two; the two groups of 16 rows inside a block keep their own random draws (group index as for NVFP4).
+template <typename T, int ROWS, int SLOTS, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T>
+__global__ void __launch_bounds__(kThreads, TileSmem<T, ROWS, DUAL, SLOTS>::kBlocksPerSm)
 quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_ct,
                      const __grid_constant__ CUtensorMap map_cr, const TileParams p) {
+  using S = TileSmem<T, ROWS, DUAL, SLOTS>;
+  static_assert(ROWS == 128 || ROWS == 256, "a staged output row is one swizzle span");
+  static_assert(!(MX_T && DUAL) && !(MX_T && sizeof(T) != 2), "the MXFP4 variant writes the transposed output of bf16 tensors only");
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-  uint8_t* tile = smem;                                   // [256][128 B], swizzled
-  uint8_t* codes_t = tile + kTileBytes;                   // [64][128 B], swizzled
-  uint8_t* codes_r = codes_t + kCodesTBytes;              // [256][32 B]
-  uint8_t* sf_t = codes_r + kCodesRBytes;                 // [16][64]
-  uint8_t* sf_r = sf_t + kSfTBytes;                       // [2][512]
-  static_assert(!(MX_T && DUAL), "the MXFP4 variant writes the transposed output only");
-  __shared__ __align__(8) uint64_t bar;
+  const uint32_t smem = (smem_addr(smem_raw) + 1023u) & ~1023u;
+  uint8_t* const smem_gen = smem_raw + (smem - smem_addr(smem_raw));
+  __shared__ __align__(8) uint64_t bars[SLOTS];
   __shared__ float inv_table[MX_T ? 256 : 128];
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t c0 = (int64_t)blockIdx.x * kTileCols;
-  const int64_t r0 = (int64_t)blockIdx.y * kTileRows;
+  // Tiles are walked from the last to the first: a pass over the tensor that ran just before (its amax) left the end of
+  // it in the level-two cache, not the beginning.
+  const int mine = (p.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  int ty = (p.tiles - 1 - (int)blockIdx.x) / p.tiles_x, tx = (p.tiles - 1 - (int)blockIdx.x) - ty * p.tiles_x;
+  int load_x = tx, load_y = ty;                           // the loader's position, up to two tiles ahead
+  auto step_back = [&](int& x, int& y) {
+    x -= p.step_x;
+    y -= p.step_y;
+    if (x < 0) { x += p.tiles_x; --y; }
+  };
+  auto load_tile = [&](int b) {
+    const uint32_t bar = smem_addr(&bars[b]);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(S::kTileBytes) : "memory");
+#pragma unroll
+    for (int i = 0; i < S::kBoxes; ++i)
+      asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+                   ::"r"(smem + b * S::kTileBytes + i * S::kBoxBytes), "l"(&map_x), "r"(bar),
+                     "r"(load_x * kTileCols + i * (128 / (int)sizeof(T))), "r"(load_y * ROWS) : "memory");
+    step_back(load_x, load_y);
+  };
+
+  if (threadIdx.x == kLoader) {
+    for (int i = 0; i < SLOTS; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bars[i])));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   grid_dependency_wait();
   grid_dependency_trigger();
+  if (threadIdx.x == kLoader) {
+    load_tile(0);
+    if (SLOTS > 1 && mine > 1) load_tile(1);
+  }
   const float g = p.gptr ? __ldg(p.gptr) : 1.0f;
   const float c = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), g);
-
-  if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar)));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&bar)), "r"(kTileBytes) : "memory");
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(smem_addr(tile)), "l"(&map_x), "r"(smem_addr(&bar)), "r"((int)c0), "r"((int)r0) : "memory");
-  }
   if constexpr (MX_T) build_inv_table_mx(inv_table, g); else build_inv_table(inv_table, g);
-  __syncthreads();                                        // barrier initialised, table published
-  {
-    // bounded wait for the tile; on a timeout every thread leaves without storing anything
-    const uint32_t b = smem_addr(&bar);
-    uint32_t done = 0;
-    unsigned long long t0 = 0;
-    for (uint32_t spin = 0; !done; ++spin) {
-      asm volatile("{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-                   : "=r"(done) : "r"(b) : "memory");
-      if (!done && (spin & 255u) == 255u) {
-        unsigned long long now;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-        if (t0 == 0) t0 = now;
-        if (now - t0 > kTileWaitLimitNs) {
-          if (threadIdx.x == 0) atomicOr(&g_tile_error_word, 0x200u);
-          return;
-        }
-      }
-    }
-  }
+  __syncthreads();                                        // barriers initialised, table published
 
-  // ---- transposed output: lane -> columns (2*lane, 2*lane+1), warp -> row blocks ----
-  // Codes are staged as [column][128 bytes] with the 128-byte swizzle the tiled store expects.
-  if constexpr (MX_T) {
-    const int rb = warp;                                      // 8 warps, 8 blocks of 32 rows
-    uint32_t w[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) w[j] = *reinterpret_cast<const uint32_t*>(tile + swz128(rb * 32 + j, 4 * lane));
-    uint32_t m[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) m[j] = absmax_bf16x2(w[2 * j], w[2 * j + 1]);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) m[j] = absmax_bf16x2(m[2 * j], m[2 * j + 1]);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) m[j] = absmax_bf16x2(m[2 * j], m[2 * j + 1]);
-    const uint32_t mm = absmax_bf16x2(absmax_bf16x2(m[0], m[1]), absmax_bf16x2(m[2], m[3])) & 0x7FFF7FFFu;
-    const uint32_t sfa = e8m0_encode_up(__fmul_rn(__uint_as_float(mm << 16), c));
-    const uint32_t sfb = e8m0_encode_up(__fmul_rn(__uint_as_float(mm & 0xFFFF0000u), c));
-    const float inv_a = inv_table[sfa], inv_b = inv_table[sfb];
-    const int64_t ca = c0 + 2 * lane;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float va[16], vb[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        va[j] = __uint_as_float(w[16 * h + j] << 16);
-        vb[j] = __uint_as_float(w[16 * h + j] & 0xFFFF0000u);
-      }
-      const int64_t kb = r0 / 16 + rb * 2 + h;                // group of 16 along the quantized row
-      uint32_t lo, hi;
-      encode_codes<SR_T>(va, inv_a, p.t_rng, (uint64_t)(ca * p.t_nkb + kb), lo, hi);
-      *reinterpret_cast<uint2*>(codes_t + swz128(2 * lane, (rb * 2 + h) * 8)) = make_uint2(lo, hi);
-      encode_codes<SR_T>(vb, inv_b, p.t_rng, (uint64_t)((ca + 1) * p.t_nkb + kb), lo, hi);
-      *reinterpret_cast<uint2*>(codes_t + swz128(2 * lane + 1, (rb * 2 + h) * 8)) = make_uint2(lo, hi);
-    }
-    sf_t[rb * kTileCols + 2 * lane] = (uint8_t)sfa;
-    sf_t[rb * kTileCols + 2 * lane + 1] = (uint8_t)sfb;
-  } else {
-  // Two forms of the same arithmetic.  With stochastic rounding in both outputs the kernel sits at its register limit
-  // (64, for four CTAs per SM) and runs fastest with addresses precomputed and the two columns' Philox calls
-  // interleaved; every other instantiation has registers to spare and runs fastest with the plain loop, which lets
-  // the compiler overlap the two row blocks (same-process A/B: 4.43 against 4.17 TB/s for SR/SR, 5.50 against
-  // 5.08-5.16 for the single SR output, 5.31 against 4.93-5.12 for RtN rows + SR transposed).
-  if constexpr (DUAL && SR_T && SR_R) {
-  {
-    // Row rb*16 + j of the tile, bytes 4*lane..4*lane+3: (row & 7) = j & 7, so the swizzled position inside a
-    // row depends on j & 7 only; eight base addresses serve all loads, the rest is a compile-time offset.
-    const uint32_t tile_s = tile_base_after_wait(tile) + (uint32_t)warp * 2048u;
-    uint32_t rowbase[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) rowbase[q] = tile_s + q * 128 + ((((uint32_t)(lane >> 2) ^ q) << 4) | ((uint32_t)(lane & 3) << 2));
-    // staging position of this lane's two output rows (columns 2*lane, 2*lane+1) for row block `warp`; the second
-    // row block of this warp (warp + 8) sits four 16-byte chunks further, which the swizzle turns into an XOR with 64
-    const uint32_t ct_s = smem_addr(codes_t);
-    const uint32_t ra = 2 * lane, rbw = 2 * lane + 1;
-    const uint32_t st_a = ct_s + ra * 128 + ((((uint32_t)(warp >> 1) ^ (ra & 7)) << 4) | ((uint32_t)(warp & 1) << 3));
-    const uint32_t st_b = ct_s + rbw * 128 + ((((uint32_t)(warp >> 1) ^ (rbw & 7)) << 4) | ((uint32_t)(warp & 1) << 3));
-    const uint64_t blk_a0 = (uint64_t)((c0 + 2 * lane) * p.t_nkb + r0 / 16 + warp);
-    uint8_t* sf_lane = sf_t + warp * kTileCols + 2 * lane;
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {                          // row blocks warp and warp + 8
-      uint32_t w[16];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        w[j] = it ? lds32<16384 + 0>(rowbase[j]) : lds32<0>(rowbase[j]);
-        w[j + 8] = it ? lds32<16384 + 1024>(rowbase[j]) : lds32<1024>(rowbase[j]);
-      }
-      uint32_t m[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) m[j] = absmax_bf16x2(w[2 * j], w[2 * j + 1]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) m[j] = absmax_bf16x2(m[2 * j], m[2 * j + 1]);
-      const uint32_t mm = absmax_bf16x2(absmax_bf16x2(m[0], m[1]), absmax_bf16x2(m[2], m[3])) & 0x7FFF7FFFu;
-      const uint64_t blk_a = blk_a0 + 8u * it, blk_b = blk_a + (uint64_t)p.t_nkb;
-      const uint32_t sfa = e4m3_encode(__fmul_rn(__uint_as_float(mm << 16), c));
-      const uint32_t sfb = e4m3_encode(__fmul_rn(__uint_as_float(mm & 0xFFFF0000u), c));
-      const float inv_a = inv_table[sfa], inv_b = inv_table[sfb];
-      uint4 ra = make_uint4(0, 0, 0, 0), rb = ra;
-      if constexpr (SR_T) philox4x32_10_x2(p.t_rng, blk_a, blk_b, ra, rb);
-      uint32_t lo, hi;
-      {
-        float y[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) y[j] = __fmul_rn(__uint_as_float(w[j] << 16), inv_a);          // column 2*lane
-        if constexpr (SR_T) { lo = e2m1x8_rs(y, 0, ra.x, ra.y); hi = e2m1x8_rs(y, 8, ra.z, ra.w); }
-        else { lo = e2m1x8_rn(y, 0); hi = e2m1x8_rn(y, 8); }
-        if (it) sts64<0>(st_a ^ 64u, lo, hi); else sts64<0>(st_a, lo, hi);
-      }
-      {
-        float y[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) y[j] = __fmul_rn(__uint_as_float(w[j] & 0xFFFF0000u), inv_b);  // column 2*lane + 1
-        if constexpr (SR_T) { lo = e2m1x8_rs(y, 0, rb.x, rb.y); hi = e2m1x8_rs(y, 8, rb.z, rb.w); }
-        else { lo = e2m1x8_rn(y, 0); hi = e2m1x8_rn(y, 8); }
-        if (it) sts64<0>(st_b ^ 64u, lo, hi); else sts64<0>(st_b, lo, hi);
-      }
-      *reinterpret_cast<uint16_t*>(sf_lane + it * 8 * kTileCols) = (uint16_t)(sfa | (sfb << 8));
-    }
-  }
-  } else {
-#pragma unroll
-  for (int rb = warp; rb < kTileRows / 16; rb += kThreads / 32) {
-    uint32_t w[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) w[j] = *reinterpret_cast<const uint32_t*>(tile + swz128(rb * 16 + j, 4 * lane));
-    uint32_t m[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) m[j] = absmax_bf16x2(w[2 * j], w[2 * j + 1]);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) m[j] = absmax_bf16x2(m[2 * j], m[2 * j + 1]);
-    const uint32_t mm = absmax_bf16x2(absmax_bf16x2(m[0], m[1]), absmax_bf16x2(m[2], m[3])) & 0x7FFF7FFFu;
-    float va[16], vb[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      va[j] = __uint_as_float(w[j] << 16);                    // column 2*lane
-      vb[j] = __uint_as_float(w[j] & 0xFFFF0000u);            // column 2*lane + 1
-    }
-    const int64_t kb = r0 / 16 + rb;
-    const int64_t ca = c0 + 2 * lane;
-    uint32_t lo, hi, sf;
-    encode_block<SR_T>(va, __uint_as_float(mm << 16), c, inv_table, p.t_rng, (uint64_t)(ca * p.t_nkb + kb), lo, hi, sf);
-    *reinterpret_cast<uint2*>(codes_t + swz128(2 * lane, rb * 8)) = make_uint2(lo, hi);
-    sf_t[rb * kTileCols + 2 * lane] = (uint8_t)sf;
-    encode_block<SR_T>(vb, __uint_as_float(mm & 0xFFFF0000u), c, inv_table, p.t_rng, (uint64_t)((ca + 1) * p.t_nkb + kb), lo, hi, sf);
-    *reinterpret_cast<uint2*>(codes_t + swz128(2 * lane + 1, rb * 8)) = make_uint2(lo, hi);
-    sf_t[rb * kTileCols + 2 * lane + 1] = (uint8_t)sf;
-  }
-  }
-  }
+  // ---- this thread's part of a tile ----
+  // Transposed: columns (2*cp, 2*cp + 1) of the 16 rows of groups g16 and, in a tile of 256 rows, g16 + 8.
+  const int g16 = MX_T ? (warp >> 1) * 2 + (lane >> 4) : warp;
+  const int cp = MX_T ? (warp & 1) * 16 + (lane & 15) : lane;
+  // Row r of a tile starts at r * 128, its 16-byte piece i sits at i ^ (r & 7): for row j of the group the position is
+  // (base | piece) ^ (j & 7) << 4, plus j * 128 as a compile-time offset.
+  const uint32_t t_in = smem + g16 * 2048 + (sizeof(T) == 2 ? (uint32_t)cp * 4u : (uint32_t)(cp >> 4) * S::kBoxBytes + (cp & 15) * 8u);
+  // Codes of a column: half g16 & 1 of piece g16 / 2 of its staged row, swizzled by the row's index (bits 1-2 of it over
+  // 64 bytes, bits 0-2 over 128).  Group g16 + 8 sits four pieces further, which the swizzle turns into an XOR with 64.
+  const uint32_t codes0 = smem + S::kCodesAt;
+  const uint32_t t_out = codes0 + cp * ROWS + ((((uint32_t)g16 >> 1) ^ (ROWS == 128 ? cp & 3 : (2 * cp) & 7)) << 4) + (g16 & 1) * 8;
+  // Row output: block kbl of the tile's 64 columns, rows t, t + 64, ...
+  const int kbl = threadIdx.x & 3, t = threadIdx.x >> 2;
+  const uint32_t r_piece = sizeof(T) == 2 ? 2u * kbl : 4u * (kbl & 1);
+  const uint32_t r_in = smem + (sizeof(T) == 2 ? 0u : (uint32_t)(kbl >> 1) * S::kBoxBytes) + t * 128 + ((r_piece ^ (t & 7)) << 4);
+  const uint32_t r_out = codes0 + S::kCodesTBytes + t * 32 + kbl * 8;
 
-  // ---- row output: thread -> (row, block of 16 columns); four rows per thread ----
-  if constexpr (DUAL) {
-    const int kbl = threadIdx.x & 3;                          // block within the tile's 64 columns
-    const int t = threadIdx.x >> 2;                           // row within a group of 64; (row & 7) = t & 7 for all four groups
-    const uint32_t ld_a = tile_base_after_wait(tile) + (uint32_t)t * 128u + (((uint32_t)(2 * kbl) ^ (uint32_t)(t & 7)) << 4);
-    const uint32_t ld_b = ld_a ^ 16u;                         // the neighbouring 16-byte chunk
-    const uint32_t st_r = smem_addr(codes_r) + (uint32_t)t * 32u + (uint32_t)kbl * 8u;
-    uint8_t* sf_thread = sf_r + (t & 31) * 16 + (t >> 5) * 4 + kbl;
-    const uint64_t blk_r0 = (uint64_t)((r0 + t) * p.r_nkb + c0 / 16 + kbl);
-    const uint64_t blk_step = (uint64_t)(64 * p.r_nkb);
-    auto row_block = [&](auto I) {
+  for (int k = 0; k < mine; ++k) {
+    const int b = SLOTS == 2 ? k & 1 : 0;
+    const int64_t c0 = (int64_t)tx * kTileCols, r0 = (int64_t)ty * ROWS;
+    if (!wait_tile(smem_addr(&bars[b]), (SLOTS == 2 ? k >> 1 : k) & 1)) break;
+    uint8_t* const sf_t = smem_gen + S::kSfAt + (k & 1) * S::kSfBytes;
+    uint8_t* const sf_r = sf_t + S::kSfTBytes;
+
+    const uint32_t in_t = after_wait(t_in + b * S::kTileBytes);
+    const uint64_t blk0_t = (uint64_t)((c0 + 2 * cp) * p.t_nkb + r0 / 16 + g16);
+    unrolled<ROWS / 128>([&](auto I) {
       constexpr int i = decltype(I)::value;
-      const uint4 a = lds128<i * 8192>(ld_a);
-      const uint4 b = lds128<i * 8192>(ld_b);
-      Block16<__nv_bfloat16> blk;
-      blk.w[0] = a.x; blk.w[1] = a.y; blk.w[2] = a.z; blk.w[3] = a.w;
-      blk.w[4] = b.x; blk.w[5] = b.y; blk.w[6] = b.z; blk.w[7] = b.w;
-      float v[16];
-      const float amax = blk.unpack(v);
-      uint32_t lo, hi, sf;
-      encode_block<SR_R>(v, amax, c, inv_table, p.r_rng, blk_r0 + (uint64_t)i * blk_step, lo, hi, sf);
-      sts64<i * 2048>(st_r, lo, hi);
-      if constexpr (SWZ) {
-        sf_thread[(i >> 1) * 512 + (i & 1) * 8] = (uint8_t)sf;
+      [[maybe_unused]] const uint64_t blk_a = blk0_t + 8 * i, blk_b = blk_a + (uint64_t)p.t_nkb;
+      [[maybe_unused]] uint32_t w[16];                    // bf16: both columns packed
+      float va[16], vb[16], amax_a, amax_b;
+      if constexpr (sizeof(T) == 2) {
+        unrolled<16>([&](auto J) {
+          constexpr int j = decltype(J)::value;
+          w[j] = lds32<i * 16384 + j * 128>(in_t ^ ((j & 7) << 4));
+        });
+        uint32_t m[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) m[j] = absmax_bf16x2(w[2 * j], w[2 * j + 1]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) m[j] = absmax_bf16x2(m[2 * j], m[2 * j + 1]);
+        uint32_t mm = absmax_bf16x2(absmax_bf16x2(m[0], m[1]), absmax_bf16x2(m[2], m[3]));
+        if constexpr (MX_T) mm = absmax_bf16x2(mm, __shfl_xor_sync(0xFFFFFFFFu, mm, 16));   // the block's other 16 rows
+        mm &= 0x7FFF7FFFu;
+        amax_a = __uint_as_float(mm << 16);
+        amax_b = __uint_as_float(mm & 0xFFFF0000u);
       } else {
-        const int rl = i * 64 + t;
-        if (r0 + rl < p.rows && c0 / 16 + kbl < p.r_nkb) p.r_scales[(r0 + rl) * p.r_nkb + c0 / 16 + kbl] = (uint8_t)sf;
+        amax_a = amax_b = 0.0f;
+        unrolled<16>([&](auto J) {
+          constexpr int j = decltype(J)::value;
+          const float2 f = lds64<i * 16384 + j * 128>(in_t ^ ((j & 7) << 4));
+          va[j] = f.x;
+          vb[j] = f.y;
+          amax_a = fmaxf(amax_a, fabsf(f.x));
+          amax_b = fmaxf(amax_b, fabsf(f.y));
+        });
       }
-    };
-    row_block(std::integral_constant<int, 0>{});
-    row_block(std::integral_constant<int, 1>{});
-    row_block(std::integral_constant<int, 2>{});
-    row_block(std::integral_constant<int, 3>{});
-  }
+      uint32_t sfa, sfb;
+      if constexpr (MX_T) { sfa = e8m0_encode_up(__fmul_rn(amax_a, c)); sfb = e8m0_encode_up(__fmul_rn(amax_b, c)); }
+      else { sfa = e4m3_encode(__fmul_rn(amax_a, c)); sfb = e4m3_encode(__fmul_rn(amax_b, c)); }
+      const float inv_a = inv_table[sfa], inv_b = inv_table[sfb];
+      // Two Philox chains in flight; one after the other where the compiler has registers to overlap row blocks instead.
+      constexpr bool kPairDraws = ROWS == 128 || SR_R;
+      uint4 ra = make_uint4(0, 0, 0, 0), rb = ra;
+      if constexpr (SR_T && kPairDraws) philox4x32_10_x2(p.t_rng, blk_a, blk_b, ra, rb);
+      if constexpr (SR_T && !kPairDraws) ra = philox4x32_10(p.t_rng, (uint32_t)blk_a, (uint32_t)(blk_a >> 32));
+      uint32_t lo, hi;
+      if constexpr (sizeof(T) == 2) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) va[j] = __uint_as_float(w[j] << 16);
+      }
+      encode_with<SR_T>(va, inv_a, ra, lo, hi);
+      const uint32_t out = (t_out + b * S::kCodesBytes) ^ (i * 64);
+      sts64<0>(out, lo, hi);
+      if constexpr (SR_T && !kPairDraws) rb = philox4x32_10(p.t_rng, (uint32_t)blk_b, (uint32_t)(blk_b >> 32));
+      if constexpr (sizeof(T) == 2) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) vb[j] = __uint_as_float(w[j] & 0xFFFF0000u);
+      }
+      encode_with<SR_T>(vb, inv_b, rb, lo, hi);
+      if constexpr (ROWS == 128) sts64<64>(out, lo, hi); else sts64<128>(out ^ 16u, lo, hi);
+      if constexpr (MX_T) {
+        if (lane < 16) *reinterpret_cast<uint16_t*>(sf_t + ((g16 >> 1) + 4 * i) * kTileCols + 2 * cp) = (uint16_t)(sfa | (sfb << 8));
+      } else {
+        *reinterpret_cast<uint16_t*>(sf_t + (g16 + 8 * i) * kTileCols + 2 * cp) = (uint16_t)(sfa | (sfb << 8));
+      }
+    });
 
-  // ---- codes out: tiled bulk stores from the staging buffers (clipped at the tensor edge) ----
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
-                 ::"l"(&map_ct), "r"(smem_addr(codes_t)), "r"((int)(r0 / 2)), "r"((int)c0) : "memory");
-    if constexpr (DUAL)
-      asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
-                   ::"l"(&map_cr), "r"(smem_addr(codes_r)), "r"((int)(c0 / 2)), "r"((int)r0) : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  }
-
-  // ---- scales out ----
-  constexpr int kSbRows = MX_T ? 32 : 16;                     // rows per scale block of the transposed output
-  constexpr int kSbPerTile = kTileRows / kSbRows;             // 16 or 8 scale blocks per column
-  constexpr int kKtPerTile = kSbPerTile / 4;                  // 4 or 2 scale tiles per column
-  const int64_t kb0 = r0 / kSbRows;
-  if constexpr (SWZ) {
-    // transposed scales: one 32-bit word = four row blocks of one column
-    const bool fill_upper = ((c0 & 127) == 0) && (c0 + kTileCols >= p.cols);   // nobody else owns rows 64..127
-    for (int id = threadIdx.x; id < kTileCols * kKtPerTile; id += kThreads) {
-      const int cl = id / kKtPerTile, t = id % kKtPerTile;
-      const int64_t kt = kb0 / 4 + t;
-      if (kt >= p.t_k_tiles) continue;
-      const uint8_t* s4 = sf_t + (t * 4) * kTileCols + cl;
-      const uint32_t val = (uint32_t)s4[0] | ((uint32_t)s4[kTileCols] << 8) | ((uint32_t)s4[2 * kTileCols] << 16) |
-                           ((uint32_t)s4[3 * kTileCols] << 24);
-      *reinterpret_cast<uint32_t*>(p.t_scales + sf_swizzled_offset(c0 + cl, kt * 4, p.t_k_tiles)) = val;
-      if (fill_upper)
-        *reinterpret_cast<uint32_t*>(p.t_scales + sf_swizzled_offset(c0 + cl + 64, kt * 4, p.t_k_tiles)) = 0u;
-    }
     if constexpr (DUAL) {
-      // row scales: the tile owns two whole 512-byte scale tiles (128 rows x this k-tile)
-      if (threadIdx.x < 64) {
-        const int h = threadIdx.x >> 5, i = threadIdx.x & 31;
-        if (r0 + h * 128 < p.rows) {
-          const uint4 val = *reinterpret_cast<const uint4*>(sf_r + h * 512 + i * 16);
-          *reinterpret_cast<uint4*>(p.r_scales + ((r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) = val;
+      const uint32_t in = after_wait(r_in + b * S::kTileBytes);
+      const uint32_t out = r_out + b * S::kCodesBytes;
+      uint8_t* const sf_thread = sf_r + (t & 31) * 16 + (t >> 5) * 4 + kbl;
+      const uint64_t blk0 = (uint64_t)((r0 + t) * p.r_nkb + c0 / 16 + kbl);
+      unrolled<ROWS / 64>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        Block16<T> blk;
+        if constexpr (sizeof(T) == 2) {
+          const uint4 a = lds128<i * 8192>(in), d = lds128<i * 8192>(in ^ 16u);
+          blk.w[0] = a.x; blk.w[1] = a.y; blk.w[2] = a.z; blk.w[3] = a.w;
+          blk.w[4] = d.x; blk.w[5] = d.y; blk.w[6] = d.z; blk.w[7] = d.w;
+        } else {
+          unrolled<4>([&](auto Q) {
+            constexpr int q = decltype(Q)::value;
+            const uint4 a = lds128<i * 8192>(in ^ (q << 4));
+            blk.f[q] = make_float4(__uint_as_float(a.x), __uint_as_float(a.y), __uint_as_float(a.z), __uint_as_float(a.w));
+          });
+        }
+        float v[16];
+        const float amax = blk.unpack(v);
+        uint32_t lo, hi, sf;
+        encode_block<SR_R>(v, amax, c, inv_table, p.r_rng, blk0 + (uint64_t)(i * 64 * p.r_nkb), lo, hi, sf);
+        sts64<i * 2048>(out, lo, hi);
+        if constexpr (SWZ) {
+          sf_thread[(i >> 1) * 512 + (i & 1) * 8] = (uint8_t)sf;
+        } else {
+          const int64_t r = r0 + t + i * 64;
+          if (r < p.rows && c0 / 16 + kbl < p.r_nkb) p.r_scales[r * p.r_nkb + c0 / 16 + kbl] = (uint8_t)sf;
+        }
+      });
+    }
+
+    // ---- codes out: tiled bulk stores from this tile's staging buffer; the tile's slot takes the tile after next ----
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (SLOTS == 2 && threadIdx.x == kLoader)             // the previous tile's codes have left the other staging buffer
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == kLoader) {
+      const uint32_t out = codes0 + b * S::kCodesBytes;
+      asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
+                   ::"l"(&map_ct), "r"(out), "r"((int)(r0 / 2)), "r"((int)c0) : "memory");
+      if constexpr (DUAL)
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
+                     ::"l"(&map_cr), "r"(out + S::kCodesTBytes), "r"((int)(c0 / 2)), "r"((int)r0) : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      if constexpr (SLOTS == 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      if (k + SLOTS < mine) load_tile(b);
+    }
+
+    // ---- scales out ----
+    constexpr int kSbRows = MX_T ? 32 : 16;               // rows per scale block of the transposed output
+    constexpr int kSbPerTile = ROWS / kSbRows;       // scale blocks per column
+    constexpr int kKtPerTile = kSbPerTile / 4;            // scale tiles per column
+    const int64_t kb0 = r0 / kSbRows;
+    if constexpr (SWZ) {
+      // transposed scales: one 32-bit word = four row blocks of one column
+      static_assert(kTileCols * kKtPerTile <= kThreads, "one word per thread");
+      if (threadIdx.x < kTileCols * kKtPerTile) {
+        const int cl = threadIdx.x / kKtPerTile, q = threadIdx.x % kKtPerTile;
+        const int64_t kt = kb0 / 4 + q;
+        if (kt < p.t_k_tiles) {
+          const uint8_t* s4 = sf_t + (q * 4) * kTileCols + cl;
+          const uint32_t val = (uint32_t)s4[0] | ((uint32_t)s4[kTileCols] << 8) | ((uint32_t)s4[2 * kTileCols] << 16) |
+                               ((uint32_t)s4[3 * kTileCols] << 24);
+          *reinterpret_cast<uint32_t*>(p.t_scales + sf_swizzled_offset(c0 + cl, kt * 4, p.t_k_tiles)) = val;
+          if (((c0 & 127) == 0) && (c0 + kTileCols >= p.cols))        // nobody else owns rows 64..127 of the scale tile
+            *reinterpret_cast<uint32_t*>(p.t_scales + sf_swizzled_offset(c0 + cl + 64, kt * 4, p.t_k_tiles)) = 0u;
         }
       }
+      if constexpr (DUAL) {
+        // row scales: the tile owns whole 512-byte scale tiles (128 rows x this k-tile)
+        const int h = (threadIdx.x >> 5) - 4, i = threadIdx.x & 31;   // from the fifth warp on
+        if (h >= 0 && h < ROWS / 128 && r0 + h * 128 < p.rows)
+          *reinterpret_cast<uint4*>(p.r_scales + ((r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) =
+              *reinterpret_cast<const uint4*>(sf_r + h * 512 + i * 16);
+      }
+    } else {
+      for (int id = threadIdx.x; id < kTileCols * kSbPerTile; id += kThreads) {
+        const int cl = id / kSbPerTile, u = id % kSbPerTile;
+        if (c0 + cl < p.cols && kb0 + u < p.t_nsb) p.t_scales[(c0 + cl) * p.t_nsb + kb0 + u] = sf_t[u * kTileCols + cl];
+      }
     }
-  } else {
-    for (int id = threadIdx.x; id < kTileCols * kSbPerTile; id += kThreads) {
-      const int cl = id / kSbPerTile, u = id % kSbPerTile;
-      if (c0 + cl < p.cols && kb0 + u < p.t_nsb) p.t_scales[(c0 + cl) * p.t_nsb + kb0 + u] = sf_t[u * kTileCols + cl];
-    }
+    step_back(tx, ty);
   }
-  if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // staging must outlive the stores' reads
+  if (threadIdx.x == kLoader) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // staging must outlive the stores' reads
 }
 
 bool make_map_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* base, uint64_t inner, uint64_t outer,
@@ -361,52 +367,87 @@ bool make_map_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* base, uin
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T = false>
-cudaError_t launch_tile(const CUtensorMap& mx, const CUtensorMap& mct, const CUtensorMap& mcr, const TileParams& p,
-                        cudaStream_t s) {
+// What a launch reads and writes; its tensor maps depend on the tile's height.
+struct TileTensors {
+  const void* x;
+  int64_t ld;
+  uint8_t *codes_t, *codes_r;
+};
+
+template <typename T, int ROWS, int SLOTS, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T>
+cudaError_t launch_rows(const TileTensors& a, TileParams& p, cudaStream_t s) {
+  using S = TileSmem<T, ROWS, DUAL, SLOTS>;
+  CUtensorMap mx, mct, mcr;
+  const uint64_t rows = (uint64_t)p.rows, cols = (uint64_t)p.cols;
+  if (!make_map_2d(&mx, sizeof(T) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.x, cols, rows,
+                   (uint64_t)a.ld * sizeof(T), 128 / (int)sizeof(T), ROWS, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_map_2d(&mct, CU_TENSOR_MAP_DATA_TYPE_UINT8, a.codes_t, rows / 2, cols, rows / 2, ROWS / 2, kTileCols,
+                   ROWS == 128 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B))
+    return cudaErrorInvalidValue;
+  mcr = mct;
+  if (DUAL && !make_map_2d(&mcr, CU_TENSOR_MAP_DATA_TYPE_UINT8, a.codes_r, cols / 2, rows, cols / 2, kTileCols / 2, ROWS,
+                           CU_TENSOR_MAP_SWIZZLE_NONE))
+    return cudaErrorInvalidValue;
   static DeviceFlags smem_set;   // per instantiation, per device
-  if (cudaError_t e = set_max_dynamic_smem(smem_set, quantize_tile_kernel<SR_T, DUAL, SR_R, SWZ, MX_T>, kTileSmem)) return e;
-  dim3 grid((unsigned)ceil_div(p.cols, kTileCols), (unsigned)ceil_div(p.rows, kTileRows));
-  return launch_overlapped(quantize_tile_kernel<SR_T, DUAL, SR_R, SWZ, MX_T>, grid, kThreads, kTileSmem, s, mx, mct, mcr, p);
+  if (cudaError_t e = set_max_dynamic_smem(smem_set, quantize_tile_kernel<T, ROWS, SLOTS, SR_T, DUAL, SR_R, SWZ, MX_T>, S::kBytes)) return e;
+  p.tiles_x = (int)ceil_div(p.cols, kTileCols);
+  p.tiles = (int)(p.tiles_x * ceil_div(p.rows, ROWS));
+  const int slots = sm_count() * S::kBlocksPerSm;
+  const int grid = (SLOTS == 1 || p.tiles < slots) ? p.tiles : slots;   // one slot: a block per tile
+  p.step_x = grid % p.tiles_x;
+  p.step_y = grid / p.tiles_x;
+  return launch_overlapped(quantize_tile_kernel<T, ROWS, SLOTS, SR_T, DUAL, SR_R, SWZ, MX_T>, grid, kThreads, S::kBytes, s, mx, mct, mcr, p);
 }
 
-template <bool DUAL, bool SWZ>
-cudaError_t dispatch_tile(bool sr_t, bool sr_r, const CUtensorMap& mx, const CUtensorMap& mct, const CUtensorMap& mcr,
-                          const TileParams& p, cudaStream_t s) {
+template <typename T, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T = false>
+cudaError_t launch_tile(const TileTensors& a, TileParams& p, cudaStream_t s) {
+  // 128-row tiles under persistent blocks win while blocks are few or the arithmetic is heavy; on large tensors a block per
+  // 256-row tile does, started in order by the hardware where walking blocks drift apart (us, 128-row / 256-row):
+  //   both outputs RtN  16384 x 2816 23.0 / 26.2   x 4096 37.0 / 36.0   x 11008 115 / 91     SR  36.7 / 36.9, 52.1 / 51.0, 136 / 131
+  //   transposed RtN    16384 x 1024 8.7 / 8.6     x 2816 21.1 / 19.9   x 11008 80 / 70      SR  9.9 / 11.0, 22.0 / 24.2, 79 / 84
+  // fp32 tensors are bound by memory with the 128-row tile (16384 x 4096, both outputs: 6.2-6.4 TB/s).
+  constexpr bool can_be_tall = sizeof(T) == 2 && (DUAL || !SR_T);
+  if constexpr (can_be_tall)
+    if (p.rows * p.cols >= (int64_t)1 << (DUAL ? 26 : 25))
+      return launch_rows<T, 256, 1, SR_T, DUAL, SR_R, SWZ, MX_T>(a, p, s);
+  return launch_rows<T, 128, 2, SR_T, DUAL, SR_R, SWZ, MX_T>(a, p, s);
+}
+
+template <typename T, bool DUAL, bool SWZ>
+cudaError_t dispatch_tile(bool sr_t, bool sr_r, const TileTensors& a,
+                          TileParams& p, cudaStream_t s) {
   if constexpr (DUAL) {
-    if (sr_t) return sr_r ? launch_tile<true, true, true, SWZ>(mx, mct, mcr, p, s) : launch_tile<true, true, false, SWZ>(mx, mct, mcr, p, s);
-    return sr_r ? launch_tile<false, true, true, SWZ>(mx, mct, mcr, p, s) : launch_tile<false, true, false, SWZ>(mx, mct, mcr, p, s);
+    if (sr_t) return sr_r ? launch_tile<T, true, true, true, SWZ>(a, p, s) : launch_tile<T, true, true, false, SWZ>(a, p, s);
+    return sr_r ? launch_tile<T, false, true, true, SWZ>(a, p, s) : launch_tile<T, false, true, false, SWZ>(a, p, s);
   } else {
-    return sr_t ? launch_tile<true, false, false, SWZ>(mx, mct, mcr, p, s) : launch_tile<false, false, false, SWZ>(mx, mct, mcr, p, s);
+    return sr_t ? launch_tile<T, true, false, false, SWZ>(a, p, s) : launch_tile<T, false, false, false, SWZ>(a, p, s);
   }
+}
+
+template <typename T>
+cudaError_t dispatch_tile(bool dual, bool swz, bool sr_t, bool sr_r, const TileTensors& a,
+                          TileParams& p, cudaStream_t s) {
+  if (dual) return swz ? dispatch_tile<T, true, true>(sr_t, sr_r, a, p, s) : dispatch_tile<T, true, false>(sr_t, sr_r, a, p, s);
+  return swz ? dispatch_tile<T, false, true>(sr_t, sr_r, a, p, s) : dispatch_tile<T, false, false>(sr_t, sr_r, a, p, s);
 }
 
 }  // namespace
 
-// True when the tile kernel can take the tensor: bf16, rows a multiple of 32 (16-byte pitch of the
-// transposed codes) and, for the row output, columns a multiple of 32 as well.
+// True when the tile kernel can take the tensor: rows a multiple of 32 (16-byte pitch of the transposed codes) and, for
+// the row output, columns a multiple of 32 as well.
 bool tile_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool dual) {
-  if (dtype != NVFP4_BF16 || rows % 32 != 0) return false;
+  if (rows % 32 != 0) return false;
   if (dual && cols % 32 != 0) return false;
-  if (ceil_div(rows, kTileRows) > 65535) return false;      // grid.y limit
-  return true;
+  if (rows > (int64_t)65535 * (dtype == NVFP4_BF16 ? 256 : 128)) return false;       // longer tensors are refused further on
+  return ceil_div(rows, 128) * ceil_div(cols, kTileCols) < (int64_t)1 << 31;   // tiles are counted in 32 bits
 }
 
 // Launches the tile kernel.  r_* arguments are ignored unless `dual`.  Arguments are validated by the callers.
-int tile_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, const float* g, bool dual,
+int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, const float* g, bool dual,
                   const nvfp4_rounding* rt, uint8_t* codes_t, uint8_t* scales_t,
                   const nvfp4_rounding* rr, uint8_t* codes_r, uint8_t* scales_r, int sf_layout, cudaStream_t s, bool mx_t) {
-  CUtensorMap mx, mct, mcr;
-  if (!make_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, x, (uint64_t)cols, (uint64_t)rows, (uint64_t)ld * 2, kTileCols,
-                   kTileRows, CU_TENSOR_MAP_SWIZZLE_128B))
-    return NVFP4_ERR_CUDA;
-  if (!make_map_2d(&mct, CU_TENSOR_MAP_DATA_TYPE_UINT8, codes_t, (uint64_t)rows / 2, (uint64_t)cols, (uint64_t)rows / 2,
-                   kTileRows / 2, kTileCols, CU_TENSOR_MAP_SWIZZLE_128B))
-    return NVFP4_ERR_CUDA;
-  mcr = mct;
-  if (dual && !make_map_2d(&mcr, CU_TENSOR_MAP_DATA_TYPE_UINT8, codes_r, (uint64_t)cols / 2, (uint64_t)rows,
-                           (uint64_t)cols / 2, kTileCols / 2, kTileRows, CU_TENSOR_MAP_SWIZZLE_NONE))
-    return NVFP4_ERR_CUDA;
+  const bool bf16 = dtype == NVFP4_BF16;
+  const TileTensors a = {x, ld, codes_t, codes_r};
   TileParams p;
   p.gptr = g; p.rows = rows; p.cols = cols;
   philox_stream_init(&p.t_rng, rt->seed, rt->offset);
@@ -419,14 +460,15 @@ int tile_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, const f
   const bool swz = sf_layout == NVFP4_SF_SWIZZLED_128x4;
   const bool sr_t = rt->mode == NVFP4_SR, sr_r = dual && rr->mode == NVFP4_SR;
   cudaError_t e;
-  if (mx_t) {                                                 // MXFP4, transposed output only
-    if (dual) return NVFP4_ERR_ENUM;
-    if (sr_t) e = swz ? launch_tile<true, false, false, true, true>(mx, mct, mcr, p, s) : launch_tile<true, false, false, false, true>(mx, mct, mcr, p, s);
-    else e = swz ? launch_tile<false, false, false, true, true>(mx, mct, mcr, p, s) : launch_tile<false, false, false, false, true>(mx, mct, mcr, p, s);
-    return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  if (mx_t) {                                                 // MXFP4, transposed output of a bf16 tensor only
+    if (dual || !bf16) return NVFP4_ERR_ENUM;
+    using B = __nv_bfloat16;
+    if (sr_t) e = swz ? launch_tile<B, true, false, false, true, true>(a, p, s) : launch_tile<B, true, false, false, false, true>(a, p, s);
+    else e = swz ? launch_tile<B, false, false, false, true, true>(a, p, s) : launch_tile<B, false, false, false, false, true>(a, p, s);
+  } else {
+    e = bf16 ? dispatch_tile<__nv_bfloat16>(dual, swz, sr_t, sr_r, a, p, s)
+             : dispatch_tile<float>(dual, swz, sr_t, sr_r, a, p, s);
   }
-  if (dual) e = swz ? dispatch_tile<true, true>(sr_t, sr_r, mx, mct, mcr, p, s) : dispatch_tile<true, false>(sr_t, sr_r, mx, mct, mcr, p, s);
-  else e = swz ? dispatch_tile<false, true>(sr_t, sr_r, mx, mct, mcr, p, s) : dispatch_tile<false, false>(sr_t, sr_r, mx, mct, mcr, p, s);
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 

@@ -136,3 +136,30 @@ def test_dual_heavy_tailed_2p24():
         oc, osf = oracle_quantize(x, transposed, float(g_t.item()), r)
         assert np.array_equal(got_c.cpu().numpy(), oc)
         assert np.array_equal(got_s.cpu().numpy().reshape(-1), ob.sf_swizzle(osf).reshape(-1))
+
+
+# one tile and less, ragged in both directions, and more tiles than two per resident block (the two slots of the ring
+# are reused; 592 blocks for bf16, 296 for fp32): the last block of the walk gets fewer tiles than the first
+@pytest.mark.parametrize("shape", [(32, 32), (128, 64), (160, 96), (2080, 1056), (1056, 8224), (8224, 1760)])
+@pytest.mark.parametrize("modes", [(nb.RTN, nb.SR), (nb.SR, nb.SR)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_dual_tiles_of_a_persistent_block(shape, modes, dtype):
+    from oracle import binding as ob
+    from tests.util import oracle_quantize
+    x = _x(shape, 13, dtype=dtype)
+    g_t = nb.nvfp4_tensor_amax_scale(x)
+    rr, rt = nb.Rounding(modes[0], 3, 1), nb.Rounding(modes[1], 3, 2)
+    cr, sr, ct, st = nb.nvfp4_quantize_dual(x, g_t, rr, rt, nb.SF_SWIZZLED)
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    for got_c, got_s, transposed, r in ((cr, sr, False, rr), (ct, st, True, rt)):
+        oc, osf = oracle_quantize(x, transposed, float(g_t.item()), r)
+        assert np.array_equal(got_c.cpu().numpy(), oc)
+        assert np.array_equal(got_s.cpu().numpy().reshape(-1), ob.sf_swizzle(osf).reshape(-1))
+
+
+@pytest.mark.parametrize("sf_layout", [nb.SF_LINEAR, nb.SF_SWIZZLED])
+@pytest.mark.parametrize("mode", [nb.RTN, nb.SR])
+@pytest.mark.parametrize("shape", [(32, 8), (288, 72), (1056, 328)])
+def test_transposed_fp32_tiles(shape, mode, sf_layout):
+    assert_quantize_parity(_x(shape, 14, dtype=torch.float32), True, True, nb.Rounding(mode, 8, 1), sf_layout)
