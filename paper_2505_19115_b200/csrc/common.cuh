@@ -80,9 +80,11 @@ int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t 
 int tile_error_word(unsigned int* out);
 
 // Per-tensor scale g = amax/2688 in one launch (quantize.cu); scratch_zeroed: two zeroed 32-bit device words.
-// The kernel reads x before it waits for the one launched before it: x must be older than that.
+// The scratch is used, and has to be zeroed, only where amax_needs_scratch() says so; after the kernel that zeroes it, and
+// wherever `late` is given, x is read before the wait for the kernel launched before this one: x must be older than that.
+bool amax_needs_scratch(int dtype, int64_t elements);
 int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* g_out,
-                         unsigned int* scratch_zeroed, void* cuda_stream);
+                         unsigned int* scratch_zeroed, bool late, void* cuda_stream);
 
 // ---------------------------------------------------------------------------------------------
 // Scale-factor layout (128 rows x 4 blocks per 512-byte tile, k-tiles contiguous per row tile)

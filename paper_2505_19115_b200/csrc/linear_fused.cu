@@ -6,6 +6,8 @@
 // the GEMMs of Eq. 5 and Eq. 6.  nvfp4_linear_bwd does the same without saved state (it quantizes
 // W^T and X^T itself).  Every operand is bit-identical to what the separate entry points produce
 // with the same rounding arguments, so the results are too.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace nvfp4 {
@@ -73,10 +75,10 @@ bool buffer_ok(const void* p, size_t have, size_t need) {
 // Per-tensor scale of one operand according to gscale_mode: NULL, computed into `slot` (one launch, with two
 // zeroed scratch words), or given.
 int resolve_g(int gscale_mode, const void* x, int dtype, int64_t rows, int64_t cols, const float* given, float* slot,
-              unsigned int* scratch, void* stream, const float** out) {
+              unsigned int* scratch, bool late, void* stream, const float** out) {
   *out = nullptr;
   if (gscale_mode == NVFP4_G_AMAX) {
-    if (int st = tensor_amax_scale_ws(x, dtype, rows, cols, cols, slot, scratch, stream)) return st;
+    if (int st = tensor_amax_scale_ws(x, dtype, rows, cols, cols, slot, scratch, late, stream)) return st;
     *out = slot;
   } else if (gscale_mode == NVFP4_G_GIVEN) {
     if (!given) return NVFP4_ERR_NULL;
@@ -85,8 +87,11 @@ int resolve_g(int gscale_mode, const void* x, int dtype, int64_t rows, int64_t c
   return NVFP4_OK;
 }
 
-int zero_scratch(int gscale_mode, void* scratch, void* stream) {
-  if (gscale_mode != NVFP4_G_AMAX) return NVFP4_OK;
+// Zeroes the scratch words of the call's amax passes if one of them (the largest tensor's) uses them.  `zeroed` says so:
+// the passes after it may then read their tensors at once.
+int zero_scratch(int gscale_mode, int dtype, int64_t largest, void* scratch, void* stream, bool* zeroed) {
+  *zeroed = gscale_mode == NVFP4_G_AMAX && amax_needs_scratch(dtype, largest);
+  if (!*zeroed) return NVFP4_OK;
   return zero_words(static_cast<unsigned int*>(scratch), 16, static_cast<cudaStream_t>(stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
@@ -128,18 +133,19 @@ extern "C" int nvfp4_linear_fwd_save(const void* X, const void* W, int dtype, in
   float* sgw = reinterpret_cast<float*>(sv + sl.gw);
   const float *g_x, *g_w;
   unsigned int* scratch = reinterpret_cast<unsigned int*>(ws + fl.scratch);
-  if (int st = zero_scratch(gscale_mode, scratch, cuda_stream)) return st;
+  bool zeroed;
+  if (int st = zero_scratch(gscale_mode, dtype, std::max(M, N) * K, scratch, cuda_stream, &zeroed)) return st;
   if (gscale_mode == NVFP4_G_GIVEN) {       // the backward pass reads the scales from `saved`
     if (!gx || !gw) return NVFP4_ERR_NULL;
     if (cudaMemcpyAsync(sgx, gx, sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess) return NVFP4_ERR_CUDA;
     if (cudaMemcpyAsync(sgw, gw, sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess) return NVFP4_ERR_CUDA;
   }
   // W first: amax(W) leaves the (smaller) weight tensor in L2 for the quantizer that follows it
-  if (int st = resolve_g(gscale_mode, W, dtype, N, K, gw, sgw, scratch, cuda_stream, &g_w)) return st;
+  if (int st = resolve_g(gscale_mode, W, dtype, N, K, gw, sgw, scratch, zeroed, cuda_stream, &g_w)) return st;
   if (int st = nvfp4_quantize_dual(W, dtype, N, K, K, g_w, rw, ws + fl.w.codes, ws + fl.w.sf, rwt, sv + sl.wt.codes,
                                    sv + sl.wt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
     return st;
-  if (int st = resolve_g(gscale_mode, X, dtype, M, K, gx, sgx, scratch + 2, cuda_stream, &g_x)) return st;
+  if (int st = resolve_g(gscale_mode, X, dtype, M, K, gx, sgx, scratch + 2, true, cuda_stream, &g_x)) return st;
   if (int st = nvfp4_quantize_dual(X, dtype, M, K, K, g_x, rx, ws + fl.x.codes, ws + fl.x.sf, rxt, sv + sl.xt.codes,
                                    sv + sl.xt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
     return st;
@@ -180,8 +186,9 @@ extern "C" int nvfp4_linear_bwd_saved(const void* dY, int dtype, int64_t M, int6
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   const float* g_dy;
   unsigned int* scratch = reinterpret_cast<unsigned int*>(ws + bl.scratch);
-  if (int st = zero_scratch(gscale_mode, scratch, cuda_stream)) return st;
-  if (int st = resolve_g(gscale_mode, dY, dtype, M, N, gdy, reinterpret_cast<float*>(ws + bl.gdy), scratch, cuda_stream, &g_dy)) return st;
+  bool zeroed;
+  if (int st = zero_scratch(gscale_mode, dtype, M * N, scratch, cuda_stream, &zeroed)) return st;
+  if (int st = resolve_g(gscale_mode, dY, dtype, M, N, gdy, reinterpret_cast<float*>(ws + bl.gdy), scratch, zeroed, cuda_stream, &g_dy)) return st;
   const bool scaled = gscale_mode != NVFP4_G_NONE;     // must match the mode nvfp4_linear_fwd_save ran with
   const float* g_x = scaled ? reinterpret_cast<const float*>(sv + sl.gx) : nullptr;
   const float* g_w = scaled ? reinterpret_cast<const float*>(sv + sl.gw) : nullptr;
@@ -203,10 +210,11 @@ extern "C" int nvfp4_linear_bwd(const void* dY, const void* W, const void* X, in
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   const float *g_dy, *g_w, *g_x;
   unsigned int* scratch = reinterpret_cast<unsigned int*>(ws + bl.scratch);
-  if (int st = zero_scratch(gscale_mode, scratch, cuda_stream)) return st;
-  if (int st = resolve_g(gscale_mode, dY, dtype, M, N, gdy, reinterpret_cast<float*>(ws + bl.gdy), scratch, cuda_stream, &g_dy)) return st;
-  if (int st = resolve_g(gscale_mode, W, dtype, N, K, gw, reinterpret_cast<float*>(ws + bl.gw), scratch + 2, cuda_stream, &g_w)) return st;
-  if (int st = resolve_g(gscale_mode, X, dtype, M, K, gx, reinterpret_cast<float*>(ws + bl.gx), scratch + 4, cuda_stream, &g_x)) return st;
+  bool zeroed;
+  if (int st = zero_scratch(gscale_mode, dtype, std::max(M * N, std::max(M, N) * K), scratch, cuda_stream, &zeroed)) return st;
+  if (int st = resolve_g(gscale_mode, dY, dtype, M, N, gdy, reinterpret_cast<float*>(ws + bl.gdy), scratch, zeroed, cuda_stream, &g_dy)) return st;
+  if (int st = resolve_g(gscale_mode, W, dtype, N, K, gw, reinterpret_cast<float*>(ws + bl.gw), scratch + 2, true, cuda_stream, &g_w)) return st;
+  if (int st = resolve_g(gscale_mode, X, dtype, M, K, gx, reinterpret_cast<float*>(ws + bl.gx), scratch + 4, true, cuda_stream, &g_x)) return st;
   if (int st = nvfp4_quantize(W, dtype, N, K, K, 1, g_w, rwt, ws + bl.wt.codes, ws + bl.wt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
     return st;
   if (int st = nvfp4_quantize(X, dtype, M, K, K, 1, g_x, rxt, ws + bl.xt.codes, ws + bl.xt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))

@@ -4,6 +4,7 @@
 // per-tensor amax scale.  All kernels are HBM-bound streaming kernels.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "quantize_core.cuh"
@@ -265,6 +266,24 @@ __device__ __forceinline__ uint32_t absmax_nan_bf16x2(uint32_t a, uint32_t b) {
   return r;
 }
 
+// g of a tensor whose largest |x| has these bits: amax / 2688, 1 for an all-zero tensor.
+__device__ __forceinline__ float amax_to_scale(uint32_t bits) {
+  const float amax = __uint_as_float(bits);
+  return (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 2688.0f);
+}
+
+// 32 bytes at position j, zeros past the end.
+__device__ __forceinline__ void load_vec32(const uint32_t* x, int64_t j, int64_t n_vec32, uint32_t (&w)[8]) {
+  if (j < n_vec32) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "l"(x + j * 8));
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = 0u;
+  }
+}
+
 // Running maximum of one thread over words of source data (bf16 pairs or fp32 values).
 template <typename T>
 struct AmaxBits {
@@ -297,6 +316,48 @@ struct AmaxBits {
   }
 };
 
+// Small dense tensors: one cluster of eight blocks does it all in one launch.  The block maxima meet in the first block's
+// shared memory, so no accumulator has to be zeroed before and no launch has to finish it after: three launches become one.
+// A 256-token layer step 47.1 -> 42.9 us, 16 tokens through kept weights 34.1 -> 29.8.  The line lies where the eight blocks'
+// own bandwidth shows: 256 x 512 2.5 -> 2.1 us, 2080 x 1056 (4.4 MB) 3.0 either way at best.
+// late: wait for the kernel before this one after the loads (x is older than it), not before them.
+constexpr int kSmallAmaxCluster = 8, kSmallAmaxThreads = 1024;
+constexpr int64_t kSmallAmaxBytes = 2 << 20;
+
+template <typename T>
+__global__ void __cluster_dims__(kSmallAmaxCluster, 1, 1) __launch_bounds__(kSmallAmaxThreads)
+amax_cluster_kernel(const uint32_t* x, int64_t n_vec32, float* g_out, int late) {
+  __shared__ uint32_t warp_max[kSmallAmaxThreads / 32];
+  __shared__ uint32_t block_max[kSmallAmaxCluster];            // the first block's copy is used
+  if (!late) { grid_dependency_wait(); grid_dependency_trigger(); }
+  AmaxBits<T> acc;
+  for (int64_t i = (int64_t)blockIdx.x * kSmallAmaxThreads + threadIdx.x; i < n_vec32; i += 4 * kSmallAmaxCluster * kSmallAmaxThreads) {
+    uint32_t w[4][8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) load_vec32(x, i + u * kSmallAmaxCluster * kSmallAmaxThreads, n_vec32, w[u]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc.add8(w[u]);
+  }
+  uint32_t bits = acc.warp_bits();
+  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = bits;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    bits = __reduce_max_sync(0xFFFFFFFFu, warp_max[threadIdx.x]);
+    if (threadIdx.x == 0) {
+      const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&block_max[blockIdx.x]);
+      asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, 0;\n\tst.shared::cluster.u32 [a], %1;\n\t}" ::"r"(mine), "r"(bits) : "memory");
+    }
+  }
+  if (late) { grid_dependency_wait(); grid_dependency_trigger(); }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int i = 0; i < kSmallAmaxCluster; ++i) m = max(m, block_max[i]);
+    *g_out = amax_to_scale(m);
+  }
+}
+
 // Strided tensors: 16-byte loads, grid-stride.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) amax_kernel(const T* x, int64_t rows, int64_t cols, int64_t ld,
@@ -321,26 +382,19 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const T* x, int64_t rows
 // TICKET = true: one launch does it all.  out = {running max bits, ticket}, both zero on entry; the block that
 // takes the last ticket turns the maximum into g = amax / 2688 (1 for an all-zero tensor), stores it in *g_out
 // and leaves the two words zero again.
+// Two blocks of 512 threads per multiprocessor keep 19 MB of loads in flight, and few blocks end in few atomics on one
+// word: against eight blocks of 256, 16384 x 1024 bf16 10.4 -> 8.4 us, x 4096 27.5 -> 23.7, x 11008 57.4 -> 54.6 (6.6 TB/s).
+constexpr int kAmaxThreads = 512, kAmaxBlocksPerSm = 2;
+
 template <typename T, bool TICKET>
-__global__ void __launch_bounds__(kThreads) amax_flat_kernel(const uint32_t* x, int64_t n_vec32, unsigned int* out, float* g_out) {
-  __shared__ uint32_t warp_max[kThreads / 32];
-  const int64_t stride = (int64_t)gridDim.x * kThreads;
+__global__ void __launch_bounds__(kAmaxThreads, kAmaxBlocksPerSm) amax_flat_kernel(const uint32_t* x, int64_t n_vec32, unsigned int* out, float* g_out) {
+  __shared__ uint32_t warp_max[kAmaxThreads / 32];
+  const int64_t stride = (int64_t)gridDim.x * kAmaxThreads;
   AmaxBits<T> acc;
-  for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n_vec32; i += 4 * stride) {
+  for (int64_t i = (int64_t)blockIdx.x * kAmaxThreads + threadIdx.x; i < n_vec32; i += 4 * stride) {
     uint32_t w[4][8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t j = i + u * stride;
-      if (j < n_vec32) {
-        asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=r"(w[u][0]), "=r"(w[u][1]), "=r"(w[u][2]), "=r"(w[u][3]), "=r"(w[u][4]), "=r"(w[u][5]),
-                       "=r"(w[u][6]), "=r"(w[u][7])
-                     : "l"(x + j * 8));
-      } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) w[u][k] = 0u;
-      }
-    }
+    for (int u = 0; u < 4; ++u) load_vec32(x, i + u * stride, n_vec32, w[u]);
 #pragma unroll
     for (int u = 0; u < 4; ++u) acc.add8(w[u]);
   }
@@ -355,13 +409,12 @@ __global__ void __launch_bounds__(kThreads) amax_flat_kernel(const uint32_t* x, 
     if (threadIdx.x == 0) {
       uint32_t block_bits = bits;
 #pragma unroll
-      for (int w8 = 1; w8 < kThreads / 32; ++w8) block_bits = max(block_bits, warp_max[w8]);
+      for (int w8 = 1; w8 < kAmaxThreads / 32; ++w8) block_bits = max(block_bits, warp_max[w8]);
       if (block_bits != 0u) atomicMax(&out[0], block_bits);
       __threadfence();
       if (atomicAdd(&out[1], 1u) == gridDim.x - 1) {                      // every other block's maximum is in
         __threadfence();
-        const float total = __uint_as_float(atomicExch(&out[0], 0u));
-        *g_out = (total == 0.0f) ? 1.0f : __fdiv_rn(total, 2688.0f);
+        *g_out = amax_to_scale(atomicExch(&out[0], 0u));
         out[1] = 0u;
       }
     }
@@ -371,14 +424,24 @@ __global__ void __launch_bounds__(kThreads) amax_flat_kernel(const uint32_t* x, 
 __global__ void amax_finalize_kernel(float* out) {
   grid_dependency_wait();
   grid_dependency_trigger();
-  const float amax = *out;
-  *out = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 2688.0f);
+  *out = amax_to_scale(__float_as_uint(*out));
 }
 
 __global__ void zero_words_kernel(unsigned int* words, int n) {
   grid_dependency_wait();
   grid_dependency_trigger();
   if ((int)threadIdx.x < n) words[threadIdx.x] = 0u;
+}
+
+// Dense and 32-byte aligned: what the 256-bit sweeps take.
+bool amax_flat_ok(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld) {
+  return ld == cols && (reinterpret_cast<uintptr_t>(x) & 31u) == 0 && (rows * cols * (dtype == NVFP4_BF16 ? 2 : 4)) % 32 == 0;
+}
+cudaError_t launch_amax_cluster(const void* x, int dtype, int64_t n32, float* g_out, bool late, cudaStream_t s) {
+  const uint32_t* xw = static_cast<const uint32_t*>(x);
+  return dtype == NVFP4_BF16
+      ? launch_overlapped(amax_cluster_kernel<__nv_bfloat16>, kSmallAmaxCluster, kSmallAmaxThreads, 0, s, xw, n32, g_out, (int)late)
+      : launch_overlapped(amax_cluster_kernel<float>, kSmallAmaxCluster, kSmallAmaxThreads, 0, s, xw, n32, g_out, (int)late);
 }
 
 template <typename T, bool SR, bool SWZ>
@@ -546,23 +609,24 @@ namespace nvfp4 {
 // Per-tensor scale in one launch where the tensor allows it (dense, 32-byte aligned); `scratch_zeroed` is two
 // zeroed 32-bit words in device memory that the kernel leaves zeroed.  Otherwise the three-step public path.
 int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* g_out,
-                         unsigned int* scratch_zeroed, void* cuda_stream) {
+                         unsigned int* scratch_zeroed, bool late, void* cuda_stream) {
   const int64_t total_bytes = rows * cols * (dtype == NVFP4_BF16 ? 2 : 4);
-  if (!x || !g_out || !scratch_zeroed || rows <= 0 || cols <= 0 || ld != cols || (reinterpret_cast<uintptr_t>(x) & 31u) != 0 ||
-      total_bytes % 32 != 0)
+  if (!x || !g_out || !scratch_zeroed || rows <= 0 || cols <= 0 || !amax_flat_ok(x, dtype, rows, cols, ld))
     return nvfp4_tensor_amax_scale(x, dtype, rows, cols, ld, g_out, cuda_stream);
   if (dtype != NVFP4_BF16 && dtype != NVFP4_FP32) return NVFP4_ERR_ENUM;
   if (int st = check_arch()) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const int64_t n32 = total_bytes / 32;
-  int64_t fb = ceil_div(n32, (int64_t)kThreads * 4);
-  if (fb > sm_count() * 8) fb = sm_count() * 8;
+  if (total_bytes <= kSmallAmaxBytes) return launch_amax_cluster(x, dtype, n32, g_out, late, s) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  const int64_t fb = std::min(ceil_div(n32, (int64_t)kAmaxThreads * 4), (int64_t)sm_count() * kAmaxBlocksPerSm);
   const uint32_t* xw = static_cast<const uint32_t*>(x);
   const cudaError_t e = (dtype == NVFP4_BF16)
-      ? launch_overlapped(amax_flat_kernel<__nv_bfloat16, true>, (unsigned)fb, kThreads, 0, s, xw, n32, scratch_zeroed, g_out)
-      : launch_overlapped(amax_flat_kernel<float, true>, (unsigned)fb, kThreads, 0, s, xw, n32, scratch_zeroed, g_out);
+      ? launch_overlapped(amax_flat_kernel<__nv_bfloat16, true>, (unsigned)fb, kAmaxThreads, 0, s, xw, n32, scratch_zeroed, g_out)
+      : launch_overlapped(amax_flat_kernel<float, true>, (unsigned)fb, kAmaxThreads, 0, s, xw, n32, scratch_zeroed, g_out);
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
+
+bool amax_needs_scratch(int dtype, int64_t elements) { return elements * (dtype == NVFP4_BF16 ? 2 : 4) > kSmallAmaxBytes; }
 
 cudaError_t zero_words(unsigned int* words, int n, cudaStream_t s) {
   return launch_overlapped(zero_words_kernel, 1, 32, 0, s, words, n);
@@ -577,18 +641,20 @@ extern "C" int nvfp4_tensor_amax_scale(const void* x, int dtype, int64_t rows, i
   if (!aligned16(x) || (ld % 8) != 0 || (reinterpret_cast<uintptr_t>(global_scale_out) & 3u)) return NVFP4_ERR_ALIGN;
   if (int st = check_arch()) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  const int64_t total_bytes = rows * cols * (dtype == NVFP4_BF16 ? 2 : 4);
+  const bool flat = amax_flat_ok(x, dtype, rows, cols, ld);
+  if (flat && total_bytes <= kSmallAmaxBytes)
+    return launch_amax_cluster(x, dtype, total_bytes / 32, global_scale_out, false, s) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
   unsigned int* bits = reinterpret_cast<unsigned int*>(global_scale_out);
   if (zero_words(bits, 1, s) != cudaSuccess) return NVFP4_ERR_CUDA;
-  const int64_t total_bytes = rows * cols * (dtype == NVFP4_BF16 ? 2 : 4);
   cudaError_t e;
-  if (ld == cols && (reinterpret_cast<uintptr_t>(x) & 31u) == 0 && total_bytes % 32 == 0) {
+  if (flat) {
     const int64_t n32 = total_bytes / 32;
-    int64_t fb = ceil_div(n32, (int64_t)kThreads * 4);
-    if (fb > sm_count() * 8) fb = sm_count() * 8;
+    const int64_t fb = std::min(ceil_div(n32, (int64_t)kAmaxThreads * 4), (int64_t)sm_count() * kAmaxBlocksPerSm);
     const uint32_t* xw = static_cast<const uint32_t*>(x);
     e = (dtype == NVFP4_BF16)
-        ? launch_overlapped(amax_flat_kernel<__nv_bfloat16, false>, (unsigned)fb, kThreads, 0, s, xw, n32, bits, (float*)nullptr)
-        : launch_overlapped(amax_flat_kernel<float, false>, (unsigned)fb, kThreads, 0, s, xw, n32, bits, (float*)nullptr);
+        ? launch_overlapped(amax_flat_kernel<__nv_bfloat16, false>, (unsigned)fb, kAmaxThreads, 0, s, xw, n32, bits, (float*)nullptr)
+        : launch_overlapped(amax_flat_kernel<float, false>, (unsigned)fb, kAmaxThreads, 0, s, xw, n32, bits, (float*)nullptr);
   } else {
     const int64_t vecs = rows * (cols / (dtype == NVFP4_BF16 ? 8 : 4));
     int64_t blocks = ceil_div(vecs, (int64_t)kThreads * 4);
