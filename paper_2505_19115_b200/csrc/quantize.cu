@@ -510,6 +510,8 @@ extern "C" int nvfp4_quantize(const void* x, int dtype, int64_t rows, int64_t co
     return tile_quantize(x, dtype, rows, cols, ld, global_scale, false, rounding, codes, scales, nullptr, nullptr, nullptr,
                          sf_layout, s);
   const bool sr = rounding->mode == NVFP4_SR, swz = sf_layout == NVFP4_SF_SWIZZLED_128x4;
+  if (!transposed && tile_row_quantizer_eligible(dtype, rows, cols, sr))
+    return tile_quantize_row(x, dtype, rows, cols, ld, global_scale, rounding, codes, scales, sf_layout, s);
   cudaError_t e = (dtype == NVFP4_BF16) ? dispatch<__nv_bfloat16>(p, transposed != 0, sr, swz, s)
                                         : dispatch<float>(p, transposed != 0, sr, swz, s);
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;

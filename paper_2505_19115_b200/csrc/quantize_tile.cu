@@ -1,6 +1,5 @@
 // Tile quantizer: one read of x[rows, cols] produces the transposed NVFP4 quantization (blocks of 16 along the row
-// axis, output stored [cols, rows/2]) and, optionally, the row quantization (blocks along the column axis) of the same
-// tile.  This is the producer fusion for the operands that Eq. 4-6 need in both orientations: dY as Q(dY) for Eq. 5 and
+// axis, output stored [cols, rows/2]), the row quantization (blocks along the column axis), or both.  Both is the producer fusion for the operands that Eq. 4-6 need in both orientations: dY as Q(dY) for Eq. 5 and
 // Q(dY^T) for Eq. 6, X as Q(X) for Eq. 4 and Q(X^T) for Eq. 6, W as Q(W) for Eq. 4 and Q(W^T) for Eq. 5.
 //
 // Persistent blocks walk over tiles of 128 or 256 rows x 64 columns.  One thread fetches tiles with tiled bulk copies
@@ -28,16 +27,16 @@ constexpr int kLoader = kThreads - 32;                                // the thr
 // Shared memory of a block, in order: tile slots, code staging, scale staging (two of it, used in turn).
 // Two slots: the tile after next lands while the present one is quantized, codes are staged in turn as well.  One slot:
 // the next tile is fetched when the present one's codes have left their staging buffer; the other blocks of the SM cover.
-template <typename T, int ROWS, bool DUAL, int SLOTS>
+template <typename T, int ROWS, bool TR, bool ROW, int SLOTS>
 struct TileSmem {
   static constexpr int kBoxBytes = ROWS * 128;                        // a copy's box is 128 bytes wide: 64 bf16 or 32 fp32 columns
   static constexpr int kBoxes = kTileCols * (int)sizeof(T) / 128;
   static constexpr int kTileBytes = kBoxes * kBoxBytes;
-  static constexpr int kCodesTBytes = kTileCols * (ROWS / 2);         // 64 output rows, swizzled over their 64 or 128 bytes
-  static constexpr int kCodesRBytes = DUAL ? ROWS * (kTileCols / 2) : 0;   // ROWS output rows x 32 bytes
+  static constexpr int kCodesTBytes = TR ? kTileCols * (ROWS / 2) : 0;   // 64 output rows, swizzled over their 64 or 128 bytes
+  static constexpr int kCodesRBytes = ROW ? ROWS * (kTileCols / 2) : 0;   // ROWS output rows x 32 bytes
   static constexpr int kCodesBytes = kCodesTBytes + kCodesRBytes;
-  static constexpr int kSfTBytes = kTileCols * (ROWS / 16);           // [row block][64 columns]
-  static constexpr int kSfRBytes = DUAL ? (ROWS / 128) * 512 : 0;     // whole scale tiles (128 rows x 4 blocks)
+  static constexpr int kSfTBytes = TR ? kTileCols * (ROWS / 16) : 0;  // [row block][64 columns]
+  static constexpr int kSfRBytes = ROW ? (ROWS / 128) * 512 : 0;     // whole scale tiles (128 rows x 4 blocks)
   static constexpr int kSfBytes = kSfTBytes + kSfRBytes;
   static constexpr int kCodesAt = SLOTS * kTileBytes, kSfAt = kCodesAt + SLOTS * kCodesBytes;
   static constexpr int kBytes = kSfAt + 2 * kSfBytes + 1024 /*align*/;
@@ -50,12 +49,12 @@ struct TileParams {
   int64_t rows, cols;
   int tiles_x, tiles;         // tiles across the columns, in all
   int step_x, step_y;         // distance between two tiles of a block: gridDim.x = step_y * tiles_x + step_x
-  // transposed output (always): quantized shape (cols, rows)
+  // transposed output: quantized shape (cols, rows)
   PhiloxStream t_rng;
   uint8_t* t_scales;
   int64_t t_nkb, t_k_tiles;   // groups of 16 per quantized row (the unit of the random draws); scale tiles per quantized row
   int64_t t_nsb;              // scale blocks per quantized row: rows / 16 (NVFP4) or rows / 32 (MXFP4)
-  // row output (DUAL only): quantized shape (rows, cols)
+  // row output: quantized shape (rows, cols)
   PhiloxStream r_rng;
   uint8_t* r_scales;
   int64_t r_nkb, r_k_tiles;
@@ -129,13 +128,14 @@ __device__ __forceinline__ bool wait_tile(uint32_t bar, uint32_t parity) {
 
 // MX_T: the transposed output is MXFP4 (Section 3, Table 1): blocks of 32 rows with an E8M0 scale rounded up to a
 // power of two; the two groups of 16 rows inside a block keep their own random draws (group index as for NVFP4).
-template <typename T, int ROWS, int SLOTS, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T>
-__global__ void __launch_bounds__(kThreads, TileSmem<T, ROWS, DUAL, SLOTS>::kBlocksPerSm)
+// TR, ROW: which outputs are written.
+template <typename T, int ROWS, int SLOTS, bool TR, bool SR_T, bool ROW, bool SR_R, bool SWZ, bool MX_T>
+__global__ void __launch_bounds__(kThreads, TileSmem<T, ROWS, TR, ROW, SLOTS>::kBlocksPerSm)
 quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_ct,
                      const __grid_constant__ CUtensorMap map_cr, const TileParams p) {
-  using S = TileSmem<T, ROWS, DUAL, SLOTS>;
+  using S = TileSmem<T, ROWS, TR, ROW, SLOTS>;
   static_assert(ROWS == 128 || ROWS == 256, "a staged output row is one swizzle span");
-  static_assert(!(MX_T && DUAL) && !(MX_T && sizeof(T) != 2), "the MXFP4 variant writes the transposed output of bf16 tensors only");
+  static_assert((TR || ROW) && !(MX_T && ROW) && !(MX_T && sizeof(T) != 2), "the MXFP4 variant writes the transposed output of bf16 tensors only");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem = (smem_addr(smem_raw) + 1023u) & ~1023u;
   uint8_t* const smem_gen = smem_raw + (smem - smem_addr(smem_raw));
@@ -203,6 +203,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     uint8_t* const sf_t = smem_gen + S::kSfAt + (k & 1) * S::kSfBytes;
     uint8_t* const sf_r = sf_t + S::kSfTBytes;
 
+    if constexpr (TR) {
     const uint32_t in_t = after_wait(t_in + b * S::kTileBytes);
     const uint64_t blk0_t = (uint64_t)((c0 + 2 * cp) * p.t_nkb + r0 / 16 + g16);
     unrolled<ROWS / 128>([&](auto I) {
@@ -266,8 +267,9 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
         *reinterpret_cast<uint16_t*>(sf_t + (g16 + 8 * i) * kTileCols + 2 * cp) = (uint16_t)(sfa | (sfb << 8));
       }
     });
+    }
 
-    if constexpr (DUAL) {
+    if constexpr (ROW) {
       const uint32_t in = after_wait(r_in + b * S::kTileBytes);
       const uint32_t out = r_out + b * S::kCodesBytes;
       uint8_t* const sf_thread = sf_r + (t & 31) * 16 + (t >> 5) * 4 + kbl;
@@ -307,9 +309,10 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     __syncthreads();
     if (threadIdx.x == kLoader) {
       const uint32_t out = codes0 + b * S::kCodesBytes;
-      asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
-                   ::"l"(&map_ct), "r"(out), "r"((int)(r0 / 2)), "r"((int)c0) : "memory");
-      if constexpr (DUAL)
+      if constexpr (TR)
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
+                     ::"l"(&map_ct), "r"(out), "r"((int)(r0 / 2)), "r"((int)c0) : "memory");
+      if constexpr (ROW)
         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
                      ::"l"(&map_cr), "r"(out + S::kCodesTBytes), "r"((int)(c0 / 2)), "r"((int)r0) : "memory");
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -325,7 +328,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     if constexpr (SWZ) {
       // transposed scales: one 32-bit word = four row blocks of one column
       static_assert(kTileCols * kKtPerTile <= kThreads, "one word per thread");
-      if (threadIdx.x < kTileCols * kKtPerTile) {
+      if (TR && threadIdx.x < kTileCols * kKtPerTile) {
         const int cl = threadIdx.x / kKtPerTile, q = threadIdx.x % kKtPerTile;
         const int64_t kt = kb0 / 4 + q;
         if (kt < p.t_k_tiles) {
@@ -337,14 +340,14 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
             *reinterpret_cast<uint32_t*>(p.t_scales + sf_swizzled_offset(c0 + cl + 64, kt * 4, p.t_k_tiles)) = 0u;
         }
       }
-      if constexpr (DUAL) {
+      if constexpr (ROW) {
         // row scales: the tile owns whole 512-byte scale tiles (128 rows x this k-tile)
         const int h = (threadIdx.x >> 5) - 4, i = threadIdx.x & 31;   // from the fifth warp on
         if (h >= 0 && h < ROWS / 128 && r0 + h * 128 < p.rows)
           *reinterpret_cast<uint4*>(p.r_scales + ((r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) =
               *reinterpret_cast<const uint4*>(sf_r + h * 512 + i * 16);
       }
-    } else {
+    } else if constexpr (TR) {
       for (int id = threadIdx.x; id < kTileCols * kSbPerTile; id += kThreads) {
         const int cl = id / kSbPerTile, u = id % kSbPerTile;
         if (c0 + cl < p.cols && kb0 + u < p.t_nsb) p.t_scales[(c0 + cl) * p.t_nsb + kb0 + u] = sf_t[u * kTileCols + cl];
@@ -374,29 +377,30 @@ struct TileTensors {
   uint8_t *codes_t, *codes_r;
 };
 
-template <typename T, int ROWS, int SLOTS, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T>
+template <typename T, int ROWS, int SLOTS, bool TR, bool SR_T, bool ROW, bool SR_R, bool SWZ, bool MX_T>
 cudaError_t launch_rows(const TileTensors& a, TileParams& p, cudaStream_t s) {
-  using S = TileSmem<T, ROWS, DUAL, SLOTS>;
+  using S = TileSmem<T, ROWS, TR, ROW, SLOTS>;
   CUtensorMap mx, mct, mcr;
   const uint64_t rows = (uint64_t)p.rows, cols = (uint64_t)p.cols;
   if (!make_map_2d(&mx, sizeof(T) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.x, cols, rows,
-                   (uint64_t)a.ld * sizeof(T), 128 / (int)sizeof(T), ROWS, CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_map_2d(&mct, CU_TENSOR_MAP_DATA_TYPE_UINT8, a.codes_t, rows / 2, cols, rows / 2, ROWS / 2, kTileCols,
+                   (uint64_t)a.ld * sizeof(T), 128 / (int)sizeof(T), ROWS, CU_TENSOR_MAP_SWIZZLE_128B))
+    return cudaErrorInvalidValue;
+  mct = mcr = mx;                                             // the map of an output that is not written is not read either
+  if (TR && !make_map_2d(&mct, CU_TENSOR_MAP_DATA_TYPE_UINT8, a.codes_t, rows / 2, cols, rows / 2, ROWS / 2, kTileCols,
                    ROWS == 128 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
-  mcr = mct;
-  if (DUAL && !make_map_2d(&mcr, CU_TENSOR_MAP_DATA_TYPE_UINT8, a.codes_r, cols / 2, rows, cols / 2, kTileCols / 2, ROWS,
+  if (ROW && !make_map_2d(&mcr, CU_TENSOR_MAP_DATA_TYPE_UINT8, a.codes_r, cols / 2, rows, cols / 2, kTileCols / 2, ROWS,
                            CU_TENSOR_MAP_SWIZZLE_NONE))
     return cudaErrorInvalidValue;
   static DeviceFlags smem_set;   // per instantiation, per device
-  if (cudaError_t e = set_max_dynamic_smem(smem_set, quantize_tile_kernel<T, ROWS, SLOTS, SR_T, DUAL, SR_R, SWZ, MX_T>, S::kBytes)) return e;
+  if (cudaError_t e = set_max_dynamic_smem(smem_set, quantize_tile_kernel<T, ROWS, SLOTS, TR, SR_T, ROW, SR_R, SWZ, MX_T>, S::kBytes)) return e;
   p.tiles_x = (int)ceil_div(p.cols, kTileCols);
   p.tiles = (int)(p.tiles_x * ceil_div(p.rows, ROWS));
   const int slots = sm_count() * S::kBlocksPerSm;
   const int grid = (SLOTS == 1 || p.tiles < slots) ? p.tiles : slots;   // one slot: a block per tile
   p.step_x = grid % p.tiles_x;
   p.step_y = grid / p.tiles_x;
-  return launch_overlapped(quantize_tile_kernel<T, ROWS, SLOTS, SR_T, DUAL, SR_R, SWZ, MX_T>, grid, kThreads, S::kBytes, s, mx, mct, mcr, p);
+  return launch_overlapped(quantize_tile_kernel<T, ROWS, SLOTS, TR, SR_T, ROW, SR_R, SWZ, MX_T>, grid, kThreads, S::kBytes, s, mx, mct, mcr, p);
 }
 
 template <typename T, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T = false>
@@ -409,8 +413,8 @@ cudaError_t launch_tile(const TileTensors& a, TileParams& p, cudaStream_t s) {
   constexpr bool can_be_tall = sizeof(T) == 2 && (DUAL || !SR_T);
   if constexpr (can_be_tall)
     if (p.rows * p.cols >= (int64_t)1 << (DUAL ? 26 : 25))
-      return launch_rows<T, 256, 1, SR_T, DUAL, SR_R, SWZ, MX_T>(a, p, s);
-  return launch_rows<T, 128, 2, SR_T, DUAL, SR_R, SWZ, MX_T>(a, p, s);
+      return launch_rows<T, 256, 1, true, SR_T, DUAL, SR_R, SWZ, MX_T>(a, p, s);
+  return launch_rows<T, 128, 2, true, SR_T, DUAL, SR_R, SWZ, MX_T>(a, p, s);
 }
 
 template <typename T, bool DUAL, bool SWZ>
@@ -469,6 +473,35 @@ int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t 
     e = bf16 ? dispatch_tile<__nv_bfloat16>(dual, swz, sr_t, sr_r, a, p, s)
              : dispatch_tile<float>(dual, swz, sr_t, sr_r, a, p, s);
   }
+  return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
+
+// Row output alone.  True when the kernel takes the tensor (columns a multiple of 32: 16-byte pitch of the codes) and is the
+// better one: everywhere but for large bf16 tensors rounded to nearest, where the plain row kernel streams longer pieces
+// (us, row kernel / this: bf16 RtN 256 x 512 4.1 / 2.0, 2080 x 1056 5.7 / 2.4, 11008 x 4096 20.0 / 20.2, 16384 x 11008
+// 71 / 77; SR 7.2 / 2.9 at 2080 x 1056, 24.0 / 21.3, 80 / 75; fp32 RtN 7.0 / 3.4, 36 / 33, 126 / 122).
+bool tile_row_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool sr) {
+  if (cols % 32 != 0 || ceil_div(rows, 128) * ceil_div(cols, kTileCols) >= (int64_t)1 << 31) return false;
+  return dtype == NVFP4_FP32 || sr || rows * cols < (int64_t)48 << 20;
+}
+
+namespace {
+template <typename T>
+cudaError_t dispatch_tile_row(bool sr, bool swz, const TileTensors& a, TileParams& p, cudaStream_t s) {
+  if (sr) return swz ? launch_rows<T, 128, 2, false, false, true, true, true, false>(a, p, s) : launch_rows<T, 128, 2, false, false, true, true, false, false>(a, p, s);
+  return swz ? launch_rows<T, 128, 2, false, false, true, false, true, false>(a, p, s) : launch_rows<T, 128, 2, false, false, true, false, false, false>(a, p, s);
+}
+}  // namespace
+
+int tile_quantize_row(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, const float* g, const nvfp4_rounding* r,
+                      uint8_t* codes, uint8_t* scales, int sf_layout, cudaStream_t s) {
+  TileParams p = {};
+  p.gptr = g; p.rows = rows; p.cols = cols;
+  philox_stream_init(&p.r_rng, r->seed, r->offset);
+  p.r_scales = scales; p.r_nkb = cols / 16; p.r_k_tiles = ceil_div(p.r_nkb, 4);
+  const TileTensors a = {x, ld, nullptr, codes};
+  const bool sr = r->mode == NVFP4_SR, swz = sf_layout == NVFP4_SF_SWIZZLED_128x4;
+  const cudaError_t e = dtype == NVFP4_BF16 ? dispatch_tile_row<__nv_bfloat16>(sr, swz, a, p, s) : dispatch_tile_row<float>(sr, swz, a, p, s);
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 

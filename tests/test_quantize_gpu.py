@@ -163,3 +163,23 @@ def test_dual_tiles_of_a_persistent_block(shape, modes, dtype):
 @pytest.mark.parametrize("shape", [(32, 8), (288, 72), (1056, 328)])
 def test_transposed_fp32_tiles(shape, mode, sf_layout):
     assert_quantize_parity(_x(shape, 14, dtype=torch.float32), True, True, nb.Rounding(mode, 8, 1), sf_layout)
+
+
+# the row output of the tile kernel: edges of a tile in both directions, and a tensor on either side of 48 Mi elements
+# (bf16 rounded to nearest changes kernels there; the strided case reads rows that do not follow one another)
+@pytest.mark.parametrize("sf_layout", [nb.SF_LINEAR, nb.SF_SWIZZLED])
+@pytest.mark.parametrize("mode", [nb.RTN, nb.SR])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("shape", [(1, 32), (127, 96), (129, 64), (257, 1056), (3001, 608)])
+def test_row_tiles(shape, dtype, mode, sf_layout):
+    assert_quantize_parity(_x(shape, 15, dtype=dtype), False, True, nb.Rounding(mode, 4, 9), sf_layout)
+    base = _x((shape[0], shape[1] + 40), 16, dtype=dtype)
+    assert_quantize_parity(base[:, 16:16 + shape[1]], False, True, nb.Rounding(mode, 4, 9), sf_layout)
+
+
+def test_row_kernels_agree_across_the_size_line():
+    x = _x((12289, 4096), 17)                                    # 48 Mi + 4096 elements: the plain row kernel
+    g = nb.nvfp4_tensor_amax_scale(x)
+    codes, scales = nb.nvfp4_quantize(x, global_scale=g)
+    part_c, part_s = nb.nvfp4_quantize(x[:12000], global_scale=g)  # the tile kernel
+    assert torch.equal(codes[:12000], part_c) and torch.equal(scales[:12000], part_s)
