@@ -983,6 +983,15 @@ int launch_gemm2_dt(const uint8_t* a_codes, const uint8_t* b_codes, const GemmPa
 
 }  // namespace
 
+// Tile width of the CTA-pair kernel for a product: 128 columns where that takes no more waves of pairs than 256 does (with
+// few tiles, or a ragged N), since a narrow tile is done sooner; otherwise 256, which loads fewer operand bytes per
+// operation.  us, 256 / 128: 256 x 512 x 512 fp32 6.6 / 5.3, 128 x 4096 x 4096 bf16 10.0 / 8.7, 768 x 704 x 9888 21.8 /
+// 16.7, 7296 x 576 x 896 10.2 / 8.0; with one wave more 736 x 5600 x 4032 11.3 / 13.5, 3072 x 1024 x 16384 27.7 / 38.3.
+int pair_tile_width(int64_t M, int64_t N) {
+  const int64_t pairs = sm_count() / 2, tiles_m = ceil_div(M, 256);
+  return ceil_div(tiles_m * ceil_div(N, 128), pairs) <= ceil_div(tiles_m * ceil_div(N, 256), pairs) ? 128 : 256;
+}
+
 // 0 = automatic.  128 / 256: single-CTA kernel with that tile width.  2128 / 2192 / 2256: CTA-pair
 // kernel with a 256 x {128,192,256} tile.
 int gemm_tile_n_override = 0;
@@ -1024,7 +1033,7 @@ int nvfp4::gemm_checked(const uint8_t* a_codes, const uint8_t* a_sf, const float
   p.tiles_m = p.tiles_n = 0;
   p.late = late;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  const int bn = gemm_tile_n_override ? gemm_tile_n_override : 2256;
+  const int bn = gemm_tile_n_override ? gemm_tile_n_override : 2000 + pair_tile_width(M, N);
   switch (bn) {
     case 128: return launch_gemm<128>(a_codes, b_codes, p, s);
     case 256: return launch_gemm<256>(a_codes, b_codes, p, s);

@@ -197,3 +197,23 @@ def test_pair_and_single_cta_kernels_agree_on_large_shapes(shape):
     obq = ob.quantize(B.float().cpu().numpy(), g=float(gb.item()))
     ref, T = ob.gemm_sampled(oa[0], oa[1], float(ga.item()), obq[0], obq[1], float(gb.item()), ii, jj)
     assert np.all(np.abs(outs[2256].cpu().numpy()[ii, jj] - ref) <= TOL * T)
+
+
+# either side of the line between the narrow and the wide tile (the narrow one where it takes no more waves of 74 pairs):
+# a ragged first tile, the last column of one, N that fills two narrow tiles but not a wide one, 73 / 75 and 147 / 149 tiles
+@pytest.mark.parametrize("shape", [(1, 8, 32), (256, 128, 320), (257, 136, 512), (300, 392, 96), (256, 9344, 256),
+                                   (256, 9600, 256), (18688, 128, 128), (19200, 200, 128)])
+def test_default_tile_width_agrees_with_the_wide_tile(shape):
+    M, N, K = shape
+    ops, _ = _quantized_pair(M, N, K, seed=77)
+    for dt in (torch.float32, torch.bfloat16):
+        try:
+            nb.nvfp4_gemm_set_tile_n(2256)
+            wide = nb.nvfp4_gemm(*ops, out_dtype=dt)
+            nb.nvfp4_gemm_set_tile_n(0)
+            got = nb.nvfp4_gemm(*ops, out_dtype=dt)
+        finally:
+            nb.nvfp4_gemm_set_tile_n(0)
+        torch.cuda.synchronize()
+        assert nb.nvfp4_device_error_word() == 0
+        assert torch.equal(got, wide)
