@@ -120,21 +120,26 @@ def _check(status, where):
         raise NvFp4Error(status, where)
 
 
+_DTYPE_CODES = {torch.bfloat16: BF16, torch.float32: FP32}
+
+
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.bfloat16:
-        return BF16
-    if t.dtype == torch.float32:
-        return FP32
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    code = _DTYPE_CODES.get(t.dtype)
+    if code is None:
+        raise TypeError(f"unsupported dtype {t.dtype}")
+    return code
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    """Handle of `stream`, or of the current stream of the current device.  The small calls are bound by the host, so
+    the handle is fetched without building a torch.cuda.Stream object (1.3 us of a call)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def nvfp4_sf_bytes(Rq: int, Kq: int, sf_layout: int = SF_SWIZZLED) -> int:
