@@ -50,6 +50,22 @@ Layout make_layout(const Plan& pl) {
   return l;
 }
 
+// Per-tensor scales of a call's one or two operands, into their workspace slots.  One launch each, after one that zeroes
+// the scratch words of the passes that use them (16 bytes in the padding behind the first slot); a call's operands are
+// older than the call, so all passes but a first one without that launch before it read at once.
+struct AmaxOperand { const void* x; int64_t rows, cols; float* g; };
+
+int amax_scales(const AmaxOperand* ops, int n, int dtype, float* first_slot, void* stream) {
+  unsigned int* scratch = reinterpret_cast<unsigned int*>(first_slot) + 16;
+  bool zeroed = false;
+  for (int i = 0; i < n; ++i) zeroed = zeroed || amax_needs_scratch(dtype, ops[i].rows * ops[i].cols);
+  if (zeroed && zero_words(scratch, 2 * n, static_cast<cudaStream_t>(stream)) != cudaSuccess) return NVFP4_ERR_CUDA;
+  for (int i = 0; i < n; ++i)
+    if (int st = tensor_amax_scale_ws(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols, ops[i].g, scratch + 2 * i, zeroed || i > 0, stream))
+      return st;
+  return NVFP4_OK;
+}
+
 int run_linear(int which, const void* a, const void* b, int dtype, int64_t M, int64_t N, int64_t K,
                int gscale_mode, const float* ga, const float* gb, const nvfp4_rounding* ra,
                const nvfp4_rounding* rb, void* out, int out_dtype, void* workspace, size_t workspace_bytes,
@@ -75,8 +91,8 @@ int run_linear(int which, const void* a, const void* b, int dtype, int64_t M, in
   if (gscale_mode == NVFP4_G_AMAX) {
     float* wa = reinterpret_cast<float*>(ws + l.a_g);
     float* wb = reinterpret_cast<float*>(ws + l.b_g);
-    if ((st = nvfp4_tensor_amax_scale(a, dtype, pl.a_rows, pl.a_cols, pl.a_cols, wa, stream))) return st;
-    if ((st = nvfp4_tensor_amax_scale(b, dtype, pl.b_rows, pl.b_cols, pl.b_cols, wb, stream))) return st;
+    const AmaxOperand ops[2] = {{a, pl.a_rows, pl.a_cols, wa}, {b, pl.b_rows, pl.b_cols, wb}};
+    if ((st = amax_scales(ops, 2, dtype, wa, stream))) return st;
     g_a = wa; g_b = wb;
   } else if (gscale_mode == NVFP4_G_GIVEN) {
     g_a = ga; g_b = gb;
@@ -153,8 +169,8 @@ extern "C" int nvfp4_linear_fwd_qout(const void* X, const void* W, int dtype, in
   if (gscale_mode == NVFP4_G_AMAX) {
     float* wa = reinterpret_cast<float*>(ws + l.a_g);
     float* wb = reinterpret_cast<float*>(ws + l.b_g);
-    if ((st = nvfp4_tensor_amax_scale(X, dtype, M, K, K, wa, cuda_stream))) return st;
-    if ((st = nvfp4_tensor_amax_scale(W, dtype, N, K, K, wb, cuda_stream))) return st;
+    const AmaxOperand ops[2] = {{X, M, K, wa}, {W, N, K, wb}};
+    if ((st = amax_scales(ops, 2, dtype, wa, cuda_stream))) return st;
     g_x = wa; g_w = wb;
   } else if (gscale_mode == NVFP4_G_GIVEN) {
     g_x = gx; g_w = gw;
@@ -185,7 +201,8 @@ extern "C" int nvfp4_linear_fwd_qin(const uint8_t* x_codes, const uint8_t* x_sca
   int st;
   if (gscale_mode == NVFP4_G_AMAX) {
     float* wb = reinterpret_cast<float*>(ws + l.b_g);
-    if ((st = nvfp4_tensor_amax_scale(W, dtype, N, K, K, wb, cuda_stream))) return st;
+    const AmaxOperand op = {W, N, K, wb};
+    if ((st = amax_scales(&op, 1, dtype, wb, cuda_stream))) return st;
     g_w = wb;
   } else if (gscale_mode == NVFP4_G_GIVEN) {
     g_w = gw;
