@@ -482,14 +482,17 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     if constexpr (!BF16_IN) { prefetch_map(&map_sfa); prefetch_map(&map_sfb); }
   }
   if (warp == 1) tmem_alloc_pair(smem_u32((const void*)tmem_slot), kTmemCols);
-  if (!p.late) grid_dependency_wait();
-  grid_dependency_trigger();
-  if constexpr (Q_OUT) build_inv_table(inv_table, p.out_g ? __ldg(p.out_g) : 1.0f);
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                               // both CTAs' barriers exist before any remote signal
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (!p.late) grid_dependency_wait();              // all of the above overlaps the kernel before this one
+  grid_dependency_trigger();
+  if constexpr (Q_OUT) {
+    build_inv_table(inv_table, p.out_g ? __ldg(p.out_g) : 1.0f);
+    __syncthreads();
+  }
 
   // The producer and issuer warps run their loops with all 32 lanes (so that loop state, addresses and
   // descriptors stay warp-uniform) and predicate only the asynchronous instructions on one lane.
