@@ -554,7 +554,7 @@ extern "C" int nvfp4_quantize_mx(const void* x, int dtype, int64_t rows, int64_t
   if (ceil_div(Rq, 128) > 65535) return NVFP4_ERR_SHAPE;
   // bf16 tensors whose row count is a multiple of 32 (always true here: Kq = rows) go through the tile kernel, which
   // quantizes along the rows straight from the source; the transpose pass remains for what that kernel does not take
-  const bool tile_path = transposed && rows % 32 == 0 && tile_quantizer_eligible(dtype, rows, cols, false);
+  const bool tile_path = transposed && rows % 32 == 0 && tile_quantizer_eligible(dtype, rows, cols, false, /*mx=*/true);
   if (transposed && !tile_path &&
       (!workspace || workspace_bytes < (size_t)rows * cols * 2 || (reinterpret_cast<uintptr_t>(workspace) & 15u)))
     return NVFP4_ERR_WORKSPACE;

@@ -47,15 +47,15 @@ __device__ __forceinline__ void mul2(float a0, float a1, float b, float& y0, flo
 }
 
 // 16 values (signed, already widened to fp32) scaled by inv -> 8 bytes of codes (lo, hi words).
-// `blk` is the linear index of this group of 16 (Philox counter).
-template <bool SR>
-__device__ __forceinline__ void encode_codes(const float (&v)[16], float inv, const PhiloxStream& rng, uint64_t blk,
+// `blk` is the linear index of this group of 16 (Philox counter), in 64 bits or, where all are known to fit, in 32.
+template <bool SR, typename Blk>
+__device__ __forceinline__ void encode_codes(const float (&v)[16], float inv, const PhiloxStream& rng, Blk blk,
                                              uint32_t& lo, uint32_t& hi);
 
 // 16 values and their amax -> codes and one E4M3 scale byte.  c = (1/6)/g.
-template <bool SR>
+template <bool SR, typename Blk>
 __device__ __forceinline__ void encode_block(const float (&v)[16], float amax, float c, const float* inv_table,
-                                             const PhiloxStream& rng, uint64_t blk,
+                                             const PhiloxStream& rng, Blk blk,
                                              uint32_t& lo, uint32_t& hi, uint32_t& sf) {
   const uint32_t q = e4m3_encode(__fmul_rn(amax, c));
   sf = q;
@@ -77,11 +77,11 @@ __device__ __forceinline__ void encode_with(const float (&v)[16], float inv, con
   }
 }
 
-template <bool SR>
-__device__ __forceinline__ void encode_codes(const float (&v)[16], float inv, const PhiloxStream& rng, uint64_t blk,
+template <bool SR, typename Blk>
+__device__ __forceinline__ void encode_codes(const float (&v)[16], float inv, const PhiloxStream& rng, Blk blk,
                                              uint32_t& lo, uint32_t& hi) {
   uint4 r4 = make_uint4(0, 0, 0, 0);
-  if constexpr (SR) r4 = philox4x32_10(rng, (uint32_t)blk, (uint32_t)(blk >> 32));
+  if constexpr (SR) r4 = philox4x32_10(rng, blk);
   encode_with<SR>(v, inv, r4, lo, hi);
 }
 

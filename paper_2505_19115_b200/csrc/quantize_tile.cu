@@ -35,7 +35,7 @@ struct TileSmem {
   static constexpr int kCodesTBytes = TR ? kTileCols * (ROWS / 2) : 0;   // 64 output rows, swizzled over their 64 or 128 bytes
   static constexpr int kCodesRBytes = ROW ? ROWS * (kTileCols / 2) : 0;   // ROWS output rows x 32 bytes
   static constexpr int kCodesBytes = kCodesTBytes + kCodesRBytes;
-  static constexpr int kSfTBytes = TR ? kTileCols * (ROWS / 16) : 0;  // [row block][64 columns]
+  static constexpr int kSfTBytes = TR ? kTileCols * (ROWS / 16) : 0;  // [four row blocks][64 columns][4]: words as scale tiles hold them
   static constexpr int kSfRBytes = ROW ? (ROWS / 128) * 512 : 0;     // whole scale tiles (128 rows x 4 blocks)
   static constexpr int kSfBytes = kSfTBytes + kSfRBytes;
   static constexpr int kCodesAt = SLOTS * kTileBytes, kSfAt = kCodesAt + SLOTS * kCodesBytes;
@@ -180,6 +180,8 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
   __syncthreads();                                        // barriers initialised, table published
 
   // ---- this thread's part of a tile ----
+  // Block indices (the random draws' counters) in 32 bits: the launch has fewer than 2^32 of them.  MXFP4 takes any size.
+  using Blk = std::conditional_t<MX_T, uint64_t, uint32_t>;
   // Transposed: columns (2*cp, 2*cp + 1) of the 16 rows of groups g16 and, in a tile of 256 rows, g16 + 8.
   const int g16 = MX_T ? (warp >> 1) * 2 + (lane >> 4) : warp;
   const int cp = MX_T ? (warp & 1) * 16 + (lane & 15) : lane;
@@ -198,17 +200,17 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
 
   for (int k = 0; k < mine; ++k) {
     const int b = SLOTS == 2 ? k & 1 : 0;
-    const int64_t c0 = (int64_t)tx * kTileCols, r0 = (int64_t)ty * ROWS;
+    const int c0 = tx * kTileCols, r0 = ty * ROWS;          // below 2^31, as rows and columns are
     if (!wait_tile(smem_addr(&bars[b]), (SLOTS == 2 ? k >> 1 : k) & 1)) break;
     uint8_t* const sf_t = smem_gen + S::kSfAt + (k & 1) * S::kSfBytes;
     uint8_t* const sf_r = sf_t + S::kSfTBytes;
 
     if constexpr (TR) {
     const uint32_t in_t = after_wait(t_in + b * S::kTileBytes);
-    const uint64_t blk0_t = (uint64_t)((c0 + 2 * cp) * p.t_nkb + r0 / 16 + g16);
+    const Blk blk0_t = (Blk)((Blk)(c0 + 2 * cp) * (Blk)p.t_nkb + (Blk)(r0 / 16 + g16));
     unrolled<ROWS / 128>([&](auto I) {
       constexpr int i = decltype(I)::value;
-      [[maybe_unused]] const uint64_t blk_a = blk0_t + 8 * i, blk_b = blk_a + (uint64_t)p.t_nkb;
+      [[maybe_unused]] const Blk blk_a = blk0_t + 8 * i, blk_b = blk_a + (Blk)p.t_nkb;
       [[maybe_unused]] uint32_t w[16];                    // bf16: both columns packed
       float va[16], vb[16], amax_a, amax_b;
       if constexpr (sizeof(T) == 2) {
@@ -245,7 +247,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       constexpr bool kPairDraws = ROWS == 128 || SR_R;
       uint4 ra = make_uint4(0, 0, 0, 0), rb = ra;
       if constexpr (SR_T && kPairDraws) philox4x32_10_x2(p.t_rng, blk_a, blk_b, ra, rb);
-      if constexpr (SR_T && !kPairDraws) ra = philox4x32_10(p.t_rng, (uint32_t)blk_a, (uint32_t)(blk_a >> 32));
+      if constexpr (SR_T && !kPairDraws) ra = philox4x32_10(p.t_rng, blk_a);
       uint32_t lo, hi;
       if constexpr (sizeof(T) == 2) {
 #pragma unroll
@@ -254,7 +256,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       encode_with<SR_T>(va, inv_a, ra, lo, hi);
       const uint32_t out = (t_out + b * S::kCodesBytes) ^ (i * 64);
       sts64<0>(out, lo, hi);
-      if constexpr (SR_T && !kPairDraws) rb = philox4x32_10(p.t_rng, (uint32_t)blk_b, (uint32_t)(blk_b >> 32));
+      if constexpr (SR_T && !kPairDraws) rb = philox4x32_10(p.t_rng, blk_b);
       if constexpr (sizeof(T) == 2) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) vb[j] = __uint_as_float(w[j] & 0xFFFF0000u);
@@ -262,9 +264,15 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       encode_with<SR_T>(vb, inv_b, rb, lo, hi);
       if constexpr (ROWS == 128) sts64<64>(out, lo, hi); else sts64<128>(out ^ 16u, lo, hi);
       if constexpr (MX_T) {
-        if (lane < 16) *reinterpret_cast<uint16_t*>(sf_t + ((g16 >> 1) + 4 * i) * kTileCols + 2 * cp) = (uint16_t)(sfa | (sfb << 8));
+        if (lane < 16) {
+          uint8_t* const dst = sf_t + i * (4 * kTileCols) + 8 * cp + (g16 >> 1);
+          dst[0] = (uint8_t)sfa;
+          dst[4] = (uint8_t)sfb;
+        }
       } else {
-        *reinterpret_cast<uint16_t*>(sf_t + (g16 + 8 * i) * kTileCols + 2 * cp) = (uint16_t)(sfa | (sfb << 8));
+        uint8_t* const dst = sf_t + ((g16 >> 2) + 2 * i) * (4 * kTileCols) + 8 * cp + (g16 & 3);
+        dst[0] = (uint8_t)sfa;
+        dst[4] = (uint8_t)sfb;
       }
     });
     }
@@ -273,7 +281,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       const uint32_t in = after_wait(r_in + b * S::kTileBytes);
       const uint32_t out = r_out + b * S::kCodesBytes;
       uint8_t* const sf_thread = sf_r + (t & 31) * 16 + (t >> 5) * 4 + kbl;
-      const uint64_t blk0 = (uint64_t)((r0 + t) * p.r_nkb + c0 / 16 + kbl);
+      const Blk blk0 = (Blk)(r0 + t) * (Blk)p.r_nkb + (Blk)(c0 / 16 + kbl);
       unrolled<ROWS / 64>([&](auto I) {
         constexpr int i = decltype(I)::value;
         Block16<T> blk;
@@ -291,12 +299,12 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
         float v[16];
         const float amax = blk.unpack(v);
         uint32_t lo, hi, sf;
-        encode_block<SR_R>(v, amax, c, inv_table, p.r_rng, blk0 + (uint64_t)(i * 64 * p.r_nkb), lo, hi, sf);
+        encode_block<SR_R>(v, amax, c, inv_table, p.r_rng, blk0 + (Blk)(i * 64) * (Blk)p.r_nkb, lo, hi, sf);
         sts64<i * 2048>(out, lo, hi);
         if constexpr (SWZ) {
           sf_thread[(i >> 1) * 512 + (i & 1) * 8] = (uint8_t)sf;
         } else {
-          const int64_t r = r0 + t + i * 64;
+          const int64_t r = (int64_t)r0 + t + i * 64;
           if (r < p.rows && c0 / 16 + kbl < p.r_nkb) p.r_scales[r * p.r_nkb + c0 / 16 + kbl] = (uint8_t)sf;
         }
       });
@@ -311,10 +319,10 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       const uint32_t out = codes0 + b * S::kCodesBytes;
       if constexpr (TR)
         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
-                     ::"l"(&map_ct), "r"(out), "r"((int)(r0 / 2)), "r"((int)c0) : "memory");
+                     ::"l"(&map_ct), "r"(out), "r"(r0 / 2), "r"(c0) : "memory");
       if constexpr (ROW)
         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
-                     ::"l"(&map_cr), "r"(out + S::kCodesTBytes), "r"((int)(c0 / 2)), "r"((int)r0) : "memory");
+                     ::"l"(&map_cr), "r"(out + S::kCodesTBytes), "r"(c0 / 2), "r"(r0) : "memory");
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
       if constexpr (SLOTS == 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       if (k + SLOTS < mine) load_tile(b);
@@ -324,33 +332,32 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     constexpr int kSbRows = MX_T ? 32 : 16;               // rows per scale block of the transposed output
     constexpr int kSbPerTile = ROWS / kSbRows;       // scale blocks per column
     constexpr int kKtPerTile = kSbPerTile / 4;            // scale tiles per column
-    const int64_t kb0 = r0 / kSbRows;
+    const int kb0 = r0 / kSbRows;
     if constexpr (SWZ) {
       // transposed scales: one 32-bit word = four row blocks of one column
       static_assert(kTileCols * kKtPerTile <= kThreads, "one word per thread");
       if (TR && threadIdx.x < kTileCols * kKtPerTile) {
-        const int cl = threadIdx.x / kKtPerTile, q = threadIdx.x % kKtPerTile;
-        const int64_t kt = kb0 / 4 + q;
-        if (kt < p.t_k_tiles) {
-          const uint8_t* s4 = sf_t + (q * 4) * kTileCols + cl;
-          const uint32_t val = (uint32_t)s4[0] | ((uint32_t)s4[kTileCols] << 8) | ((uint32_t)s4[2 * kTileCols] << 16) |
-                               ((uint32_t)s4[3 * kTileCols] << 24);
-          *reinterpret_cast<uint32_t*>(p.t_scales + sf_swizzled_offset(c0 + cl, kt * 4, p.t_k_tiles)) = val;
-          if (((c0 & 127) == 0) && (c0 + kTileCols >= p.cols))        // nobody else owns rows 64..127 of the scale tile
-            *reinterpret_cast<uint32_t*>(p.t_scales + sf_swizzled_offset(c0 + cl + 64, kt * 4, p.t_k_tiles)) = 0u;
+        // sf_swizzled_offset(c0 + cl, 4 * (kt0 + q), t_k_tiles) taken apart: the tile's part and this thread's
+        const int cl = threadIdx.x / kKtPerTile, q = threadIdx.x % kKtPerTile, kt0 = kb0 / 4;
+        if (kt0 + q < p.t_k_tiles) {
+          uint8_t* dst = p.t_scales + ((int64_t)(c0 >> 7) * p.t_k_tiles + kt0) * 512 + ((c0 & 64) >> 3) +
+                         (q * 512 + (cl & 31) * 16 + (cl >> 5) * 4);
+          *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(sf_t + q * (4 * kTileCols) + cl * 4);
+          if (((c0 & 127) == 0) && ((int64_t)c0 + kTileCols >= p.cols))        // nobody else owns rows 64..127 of the scale tile
+            *reinterpret_cast<uint32_t*>(dst + 8) = 0u;
         }
       }
       if constexpr (ROW) {
         // row scales: the tile owns whole 512-byte scale tiles (128 rows x this k-tile)
         const int h = (threadIdx.x >> 5) - 4, i = threadIdx.x & 31;   // from the fifth warp on
-        if (h >= 0 && h < ROWS / 128 && r0 + h * 128 < p.rows)
-          *reinterpret_cast<uint4*>(p.r_scales + ((r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) =
+        if (h >= 0 && h < ROWS / 128 && (int64_t)r0 + h * 128 < p.rows)
+          *reinterpret_cast<uint4*>(p.r_scales + ((int64_t)(r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) =
               *reinterpret_cast<const uint4*>(sf_r + h * 512 + i * 16);
       }
     } else if constexpr (TR) {
       for (int id = threadIdx.x; id < kTileCols * kSbPerTile; id += kThreads) {
         const int cl = id / kSbPerTile, u = id % kSbPerTile;
-        if (c0 + cl < p.cols && kb0 + u < p.t_nsb) p.t_scales[(c0 + cl) * p.t_nsb + kb0 + u] = sf_t[u * kTileCols + cl];
+        if (c0 + cl < p.cols && kb0 + u < p.t_nsb) p.t_scales[(int64_t)(c0 + cl) * p.t_nsb + kb0 + u] = sf_t[(u >> 2) * (4 * kTileCols) + cl * 4 + (u & 3)];
       }
     }
     step_back(tx, ty);
@@ -407,7 +414,7 @@ template <typename T, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T = fal
 cudaError_t launch_tile(const TileTensors& a, TileParams& p, cudaStream_t s) {
   // 128-row tiles under persistent blocks win while blocks are few or the arithmetic is heavy; on large tensors a block per
   // 256-row tile does, started in order by the hardware where walking blocks drift apart (us, 128-row / 256-row):
-  //   both outputs RtN  16384 x 2816 23.0 / 26.2   x 4096 37.0 / 36.0   x 11008 115 / 91     SR  36.7 / 36.9, 52.1 / 51.0, 136 / 131
+  //   both outputs RtN  16384 x 2816 23.0 / 26.2   x 4096 37.0 / 36.0   x 11008 115 / 91     SR  36.7 / 36.9, 52.1 / 51.0, 136 / 129
   //   transposed RtN    16384 x 1024 8.7 / 8.6     x 2816 21.1 / 19.9   x 11008 80 / 70      SR  9.9 / 11.0, 22.0 / 24.2, 79 / 84
   // fp32 tensors are bound by memory with the 128-row tile (16384 x 4096, both outputs: 6.2-6.4 TB/s).
   constexpr bool can_be_tall = sizeof(T) == 2 && (DUAL || !SR_T);
@@ -439,8 +446,9 @@ cudaError_t dispatch_tile(bool dual, bool swz, bool sr_t, bool sr_r, const TileT
 
 // True when the tile kernel can take the tensor: rows a multiple of 32 (16-byte pitch of the transposed codes) and, for
 // the row output, columns a multiple of 32 as well.
-bool tile_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool dual) {
+bool tile_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool dual, bool mx) {
   if (rows % 32 != 0) return false;
+  if (!mx && rows * cols >= (int64_t)1 << 36) return false;                          // block indices in 32 bits
   if (dual && cols % 32 != 0) return false;
   if (rows > (int64_t)65535 * (dtype == NVFP4_BF16 ? 256 : 128)) return false;       // longer tensors are refused further on
   return ceil_div(rows, 128) * ceil_div(cols, kTileCols) < (int64_t)1 << 31;   // tiles are counted in 32 bits
@@ -481,7 +489,7 @@ int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t 
 // (us, row kernel / this: bf16 RtN 256 x 512 4.1 / 2.0, 2080 x 1056 5.7 / 2.4, 11008 x 4096 20.0 / 20.2, 16384 x 11008
 // 71 / 77; SR 7.2 / 2.9 at 2080 x 1056, 24.0 / 21.3, 80 / 75; fp32 RtN 7.0 / 3.4, 36 / 33, 126 / 122).
 bool tile_row_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool sr) {
-  if (cols % 32 != 0 || ceil_div(rows, 128) * ceil_div(cols, kTileCols) >= (int64_t)1 << 31) return false;
+  if (cols % 32 != 0 || rows * cols >= (int64_t)1 << 36 || ceil_div(rows, 128) * ceil_div(cols, kTileCols) >= (int64_t)1 << 31) return false;
   return dtype == NVFP4_FP32 || sr || rows * cols < (int64_t)48 << 20;
 }
 
