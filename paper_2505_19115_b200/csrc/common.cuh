@@ -80,7 +80,7 @@ int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t 
 // The same kernel with the row output alone.
 bool tile_row_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool sr);
 int tile_quantize_row(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, const float* g, const nvfp4_rounding* r,
-                      uint8_t* codes, uint8_t* scales, int sf_layout, cudaStream_t s);
+                      uint8_t* codes, uint8_t* scales, int sf_layout, cudaStream_t s, bool mx = false);
 int tile_error_word(unsigned int* out);
 
 // Per-tensor scale g = amax/2688 in one launch (quantize.cu); scratch_zeroed: two zeroed 32-bit device words.

@@ -563,6 +563,8 @@ extern "C" int nvfp4_quantize_mx(const void* x, int dtype, int64_t rows, int64_t
   if (tile_path)
     return tile_quantize(x, dtype, rows, cols, ld, global_scale, false, rounding, codes, scales, nullptr, nullptr, nullptr, sf_layout, s,
                          /*mx_t=*/true);
+  if (!transposed && tile_row_quantizer_eligible(dtype, rows, cols, rounding->mode == NVFP4_SR))
+    return tile_quantize_row(x, dtype, rows, cols, ld, global_scale, rounding, codes, scales, sf_layout, s, /*mx=*/true);
   const void* src = x;
   int64_t src_ld = ld;
   if (transposed) {

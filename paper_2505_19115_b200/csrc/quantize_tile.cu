@@ -57,7 +57,7 @@ struct TileParams {
   // row output: quantized shape (rows, cols)
   PhiloxStream r_rng;
   uint8_t* r_scales;
-  int64_t r_nkb, r_k_tiles;
+  int64_t r_nkb, r_k_tiles, r_nsb;   // as t_*
 };
 
 __device__ unsigned int g_tile_error_word = 0;
@@ -126,21 +126,21 @@ __device__ __forceinline__ bool wait_tile(uint32_t bar, uint32_t parity) {
   }
 }
 
-// MX_T: the transposed output is MXFP4 (Section 3, Table 1): blocks of 32 rows with an E8M0 scale rounded up to a
-// power of two; the two groups of 16 rows inside a block keep their own random draws (group index as for NVFP4).
+// MX: the output (one of the two) is MXFP4 (Section 3, Table 1): blocks of 32 with an E8M0 scale rounded up to a power
+// of two; the two groups of 16 inside a block keep their own random draws (group index as for NVFP4).
 // TR, ROW: which outputs are written.
-template <typename T, int ROWS, int SLOTS, bool TR, bool SR_T, bool ROW, bool SR_R, bool SWZ, bool MX_T>
+template <typename T, int ROWS, int SLOTS, bool TR, bool SR_T, bool ROW, bool SR_R, bool SWZ, bool MX>
 __global__ void __launch_bounds__(kThreads, TileSmem<T, ROWS, TR, ROW, SLOTS>::kBlocksPerSm)
 quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_ct,
                      const __grid_constant__ CUtensorMap map_cr, const TileParams p) {
   using S = TileSmem<T, ROWS, TR, ROW, SLOTS>;
   static_assert(ROWS == 128 || ROWS == 256, "a staged output row is one swizzle span");
-  static_assert((TR || ROW) && !(MX_T && ROW) && !(MX_T && sizeof(T) != 2), "the MXFP4 variant writes the transposed output of bf16 tensors only");
+  static_assert((TR || ROW) && !(MX && TR && (ROW || sizeof(T) != 2)), "MXFP4: one output, the transposed one of bf16 tensors only");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem = (smem_addr(smem_raw) + 1023u) & ~1023u;
   uint8_t* const smem_gen = smem_raw + (smem - smem_addr(smem_raw));
   __shared__ __align__(8) uint64_t bars[SLOTS];
-  __shared__ float inv_table[MX_T ? 256 : 128];
+  __shared__ float inv_table[MX ? 256 : 128];
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // Tiles are walked from the last to the first: a pass over the tensor that ran just before (its amax) left the end of
@@ -176,15 +176,15 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
   }
   const float g = p.gptr ? __ldg(p.gptr) : 1.0f;
   const float c = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), g);
-  if constexpr (MX_T) build_inv_table_mx(inv_table, g); else build_inv_table(inv_table, g);
+  if constexpr (MX) build_inv_table_mx(inv_table, g); else build_inv_table(inv_table, g);
   __syncthreads();                                        // barriers initialised, table published
 
   // ---- this thread's part of a tile ----
   // Block indices (the random draws' counters) in 32 bits: the launch has fewer than 2^32 of them.  MXFP4 takes any size.
-  using Blk = std::conditional_t<MX_T, uint64_t, uint32_t>;
+  using Blk = std::conditional_t<MX, uint64_t, uint32_t>;
   // Transposed: columns (2*cp, 2*cp + 1) of the 16 rows of groups g16 and, in a tile of 256 rows, g16 + 8.
-  const int g16 = MX_T ? (warp >> 1) * 2 + (lane >> 4) : warp;
-  const int cp = MX_T ? (warp & 1) * 16 + (lane & 15) : lane;
+  const int g16 = MX ? (warp >> 1) * 2 + (lane >> 4) : warp;
+  const int cp = MX ? (warp & 1) * 16 + (lane & 15) : lane;
   // Row r of a tile starts at r * 128, its 16-byte piece i sits at i ^ (r & 7): for row j of the group the position is
   // (base | piece) ^ (j & 7) << 4, plus j * 128 as a compile-time offset.
   const uint32_t t_in = smem + g16 * 2048 + (sizeof(T) == 2 ? (uint32_t)cp * 4u : (uint32_t)(cp >> 4) * S::kBoxBytes + (cp & 15) * 8u);
@@ -224,7 +224,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
 #pragma unroll
         for (int j = 0; j < 4; ++j) m[j] = absmax_bf16x2(m[2 * j], m[2 * j + 1]);
         uint32_t mm = absmax_bf16x2(absmax_bf16x2(m[0], m[1]), absmax_bf16x2(m[2], m[3]));
-        if constexpr (MX_T) mm = absmax_bf16x2(mm, __shfl_xor_sync(0xFFFFFFFFu, mm, 16));   // the block's other 16 rows
+        if constexpr (MX) mm = absmax_bf16x2(mm, __shfl_xor_sync(0xFFFFFFFFu, mm, 16));   // the block's other 16 rows
         mm &= 0x7FFF7FFFu;
         amax_a = __uint_as_float(mm << 16);
         amax_b = __uint_as_float(mm & 0xFFFF0000u);
@@ -240,7 +240,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
         });
       }
       uint32_t sfa, sfb;
-      if constexpr (MX_T) { sfa = e8m0_encode_up(__fmul_rn(amax_a, c)); sfb = e8m0_encode_up(__fmul_rn(amax_b, c)); }
+      if constexpr (MX) { sfa = e8m0_encode_up(__fmul_rn(amax_a, c)); sfb = e8m0_encode_up(__fmul_rn(amax_b, c)); }
       else { sfa = e4m3_encode(__fmul_rn(amax_a, c)); sfb = e4m3_encode(__fmul_rn(amax_b, c)); }
       const float inv_a = inv_table[sfa], inv_b = inv_table[sfb];
       // Two Philox chains in flight; one after the other where the compiler has registers to overlap row blocks instead.
@@ -263,7 +263,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       }
       encode_with<SR_T>(vb, inv_b, rb, lo, hi);
       if constexpr (ROWS == 128) sts64<64>(out, lo, hi); else sts64<128>(out ^ 16u, lo, hi);
-      if constexpr (MX_T) {
+      if constexpr (MX) {
         if (lane < 16) {
           uint8_t* const dst = sf_t + i * (4 * kTileCols) + 8 * cp + (g16 >> 1);
           dst[0] = (uint8_t)sfa;
@@ -280,7 +280,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     if constexpr (ROW) {
       const uint32_t in = after_wait(r_in + b * S::kTileBytes);
       const uint32_t out = r_out + b * S::kCodesBytes;
-      uint8_t* const sf_thread = sf_r + (t & 31) * 16 + (t >> 5) * 4 + kbl;
+      uint8_t* const sf_thread = sf_r + (t & 31) * 16 + (t >> 5) * 4;
       const Blk blk0 = (Blk)(r0 + t) * (Blk)p.r_nkb + (Blk)(c0 / 16 + kbl);
       unrolled<ROWS / 64>([&](auto I) {
         constexpr int i = decltype(I)::value;
@@ -297,15 +297,25 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
           });
         }
         float v[16];
-        const float amax = blk.unpack(v);
+        float amax = blk.unpack(v);
         uint32_t lo, hi, sf;
-        encode_block<SR_R>(v, amax, c, inv_table, p.r_rng, blk0 + (Blk)(i * 64) * (Blk)p.r_nkb, lo, hi, sf);
-        sts64<i * 2048>(out, lo, hi);
-        if constexpr (SWZ) {
-          sf_thread[(i >> 1) * 512 + (i & 1) * 8] = (uint8_t)sf;
+        if constexpr (MX) {
+          amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, 1));   // the block's other half is the neighbouring lane's
+          sf = e8m0_encode_up(__fmul_rn(amax, c));
+          encode_codes<SR_R>(v, inv_table[sf], p.r_rng, blk0 + (Blk)(i * 64) * (Blk)p.r_nkb, lo, hi);
         } else {
-          const int64_t r = (int64_t)r0 + t + i * 64;
-          if (r < p.rows && c0 / 16 + kbl < p.r_nkb) p.r_scales[r * p.r_nkb + c0 / 16 + kbl] = (uint8_t)sf;
+          encode_block<SR_R>(v, amax, c, inv_table, p.r_rng, blk0 + (Blk)(i * 64) * (Blk)p.r_nkb, lo, hi, sf);
+        }
+        sts64<i * 2048>(out, lo, hi);
+        const int sb = MX ? kbl >> 1 : kbl;              // scale block within the tile; MXFP4: the even lane's
+        if (!MX || (kbl & 1) == 0) {
+          if constexpr (SWZ) {
+            sf_thread[(i >> 1) * 512 + (i & 1) * 8 + sb] = (uint8_t)sf;
+          } else {
+            constexpr int kSb = MX ? 32 : 16;
+            const int64_t r = (int64_t)r0 + t + i * 64;
+            if (r < p.rows && c0 / kSb + sb < p.r_nsb) p.r_scales[r * p.r_nsb + c0 / kSb + sb] = (uint8_t)sf;
+          }
         }
       });
     }
@@ -329,7 +339,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     }
 
     // ---- scales out ----
-    constexpr int kSbRows = MX_T ? 32 : 16;               // rows per scale block of the transposed output
+    constexpr int kSbRows = MX ? 32 : 16;               // rows per scale block of the transposed output
     constexpr int kSbPerTile = ROWS / kSbRows;       // scale blocks per column
     constexpr int kKtPerTile = kSbPerTile / 4;            // scale tiles per column
     const int kb0 = r0 / kSbRows;
@@ -347,7 +357,18 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
             *reinterpret_cast<uint32_t*>(dst + 8) = 0u;
         }
       }
-      if constexpr (ROW) {
+      if constexpr (ROW && MX) {
+        // a scale tile holds 128 columns' scales: this tile owns bytes 0-1 or 2-3 of each of its words
+        if (threadIdx.x >= 128) {
+          const int w = threadIdx.x - 128;               // word: row (w & 3) * 32 + w / 4
+          const uint32_t val = *reinterpret_cast<const uint16_t*>(sf_r + w * 4);
+          uint8_t* const dst = p.r_scales + ((int64_t)(r0 / 128) * p.r_k_tiles + c0 / 128) * 512 + w * 4;
+          if (((c0 & 127) == 0) && ((int64_t)c0 + kTileCols >= p.cols))        // nobody else owns the upper half
+            *reinterpret_cast<uint32_t*>(dst) = val;
+          else
+            *reinterpret_cast<uint16_t*>(dst + ((c0 & 64) >> 5)) = (uint16_t)val;
+        }
+      } else if constexpr (ROW) {
         // row scales: the tile owns whole 512-byte scale tiles (128 rows x this k-tile)
         const int h = (threadIdx.x >> 5) - 4, i = threadIdx.x & 31;   // from the fifth warp on
         if (h >= 0 && h < ROWS / 128 && (int64_t)r0 + h * 128 < p.rows)
@@ -384,7 +405,7 @@ struct TileTensors {
   uint8_t *codes_t, *codes_r;
 };
 
-template <typename T, int ROWS, int SLOTS, bool TR, bool SR_T, bool ROW, bool SR_R, bool SWZ, bool MX_T>
+template <typename T, int ROWS, int SLOTS, bool TR, bool SR_T, bool ROW, bool SR_R, bool SWZ, bool MX>
 cudaError_t launch_rows(const TileTensors& a, TileParams& p, cudaStream_t s) {
   using S = TileSmem<T, ROWS, TR, ROW, SLOTS>;
   CUtensorMap mx, mct, mcr;
@@ -400,17 +421,17 @@ cudaError_t launch_rows(const TileTensors& a, TileParams& p, cudaStream_t s) {
                            CU_TENSOR_MAP_SWIZZLE_NONE))
     return cudaErrorInvalidValue;
   static DeviceFlags smem_set;   // per instantiation, per device
-  if (cudaError_t e = set_max_dynamic_smem(smem_set, quantize_tile_kernel<T, ROWS, SLOTS, TR, SR_T, ROW, SR_R, SWZ, MX_T>, S::kBytes)) return e;
+  if (cudaError_t e = set_max_dynamic_smem(smem_set, quantize_tile_kernel<T, ROWS, SLOTS, TR, SR_T, ROW, SR_R, SWZ, MX>, S::kBytes)) return e;
   p.tiles_x = (int)ceil_div(p.cols, kTileCols);
   p.tiles = (int)(p.tiles_x * ceil_div(p.rows, ROWS));
   const int slots = sm_count() * S::kBlocksPerSm;
   const int grid = (SLOTS == 1 || p.tiles < slots) ? p.tiles : slots;   // one slot: a block per tile
   p.step_x = grid % p.tiles_x;
   p.step_y = grid / p.tiles_x;
-  return launch_overlapped(quantize_tile_kernel<T, ROWS, SLOTS, TR, SR_T, ROW, SR_R, SWZ, MX_T>, grid, kThreads, S::kBytes, s, mx, mct, mcr, p);
+  return launch_overlapped(quantize_tile_kernel<T, ROWS, SLOTS, TR, SR_T, ROW, SR_R, SWZ, MX>, grid, kThreads, S::kBytes, s, mx, mct, mcr, p);
 }
 
-template <typename T, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX_T = false>
+template <typename T, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX = false>
 cudaError_t launch_tile(const TileTensors& a, TileParams& p, cudaStream_t s) {
   // 128-row tiles under persistent blocks win while blocks are few or the arithmetic is heavy; on large tensors a block per
   // 256-row tile does, started in order by the hardware where walking blocks drift apart (us, 128-row / 256-row):
@@ -420,8 +441,8 @@ cudaError_t launch_tile(const TileTensors& a, TileParams& p, cudaStream_t s) {
   constexpr bool can_be_tall = sizeof(T) == 2 && (DUAL || !SR_T);
   if constexpr (can_be_tall)
     if (p.rows * p.cols >= (int64_t)1 << (DUAL ? 26 : 25))
-      return launch_rows<T, 256, 1, true, SR_T, DUAL, SR_R, SWZ, MX_T>(a, p, s);
-  return launch_rows<T, 128, 2, true, SR_T, DUAL, SR_R, SWZ, MX_T>(a, p, s);
+      return launch_rows<T, 256, 1, true, SR_T, DUAL, SR_R, SWZ, MX>(a, p, s);
+  return launch_rows<T, 128, 2, true, SR_T, DUAL, SR_R, SWZ, MX>(a, p, s);
 }
 
 template <typename T, bool DUAL, bool SWZ>
@@ -468,7 +489,7 @@ int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t 
   p.t_k_tiles = ceil_div(p.t_nsb, 4);
   const nvfp4_rounding* r2 = dual ? rr : rt;
   philox_stream_init(&p.r_rng, r2->seed, r2->offset);
-  p.r_scales = scales_r; p.r_nkb = cols / 16; p.r_k_tiles = ceil_div(p.r_nkb, 4);
+  p.r_scales = scales_r; p.r_nkb = p.r_nsb = cols / 16; p.r_k_tiles = ceil_div(p.r_nsb, 4);
   const bool swz = sf_layout == NVFP4_SF_SWIZZLED_128x4;
   const bool sr_t = rt->mode == NVFP4_SR, sr_r = dual && rr->mode == NVFP4_SR;
   cudaError_t e;
@@ -487,29 +508,31 @@ int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t 
 // Row output alone.  True when the kernel takes the tensor (columns a multiple of 32: 16-byte pitch of the codes) and is the
 // better one: everywhere but for large bf16 tensors rounded to nearest, where the plain row kernel streams longer pieces
 // (us, row kernel / this: bf16 RtN 256 x 512 4.1 / 2.0, 2080 x 1056 5.7 / 2.4, 11008 x 4096 20.0 / 20.2, 16384 x 11008
-// 71 / 77; SR 7.2 / 2.9 at 2080 x 1056, 24.0 / 21.3, 80 / 75; fp32 RtN 7.0 / 3.4, 36 / 33, 126 / 122).
+// 71 / 77; SR 7.2 / 2.9 at 2080 x 1056, 24.0 / 21.3, 80 / 75; fp32 RtN 7.0 / 3.4, 36 / 33, 126 / 122).  MXFP4 follows the same line:
+// the 16384 x 1024 x 2816 forward in it 57.8 us / 55.9, 2048 x 4096 x 11008 97.7 / 93.3.
 bool tile_row_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool sr) {
   if (cols % 32 != 0 || rows * cols >= (int64_t)1 << 36 || ceil_div(rows, 128) * ceil_div(cols, kTileCols) >= (int64_t)1 << 31) return false;
   return dtype == NVFP4_FP32 || sr || rows * cols < (int64_t)48 << 20;
 }
 
 namespace {
-template <typename T>
+template <typename T, bool MX>
 cudaError_t dispatch_tile_row(bool sr, bool swz, const TileTensors& a, TileParams& p, cudaStream_t s) {
-  if (sr) return swz ? launch_rows<T, 128, 2, false, false, true, true, true, false>(a, p, s) : launch_rows<T, 128, 2, false, false, true, true, false, false>(a, p, s);
-  return swz ? launch_rows<T, 128, 2, false, false, true, false, true, false>(a, p, s) : launch_rows<T, 128, 2, false, false, true, false, false, false>(a, p, s);
+  if (sr) return swz ? launch_rows<T, 128, 2, false, false, true, true, true, MX>(a, p, s) : launch_rows<T, 128, 2, false, false, true, true, false, MX>(a, p, s);
+  return swz ? launch_rows<T, 128, 2, false, false, true, false, true, MX>(a, p, s) : launch_rows<T, 128, 2, false, false, true, false, false, MX>(a, p, s);
 }
 }  // namespace
 
 int tile_quantize_row(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, const float* g, const nvfp4_rounding* r,
-                      uint8_t* codes, uint8_t* scales, int sf_layout, cudaStream_t s) {
+                      uint8_t* codes, uint8_t* scales, int sf_layout, cudaStream_t s, bool mx) {
   TileParams p = {};
   p.gptr = g; p.rows = rows; p.cols = cols;
   philox_stream_init(&p.r_rng, r->seed, r->offset);
-  p.r_scales = scales; p.r_nkb = cols / 16; p.r_k_tiles = ceil_div(p.r_nkb, 4);
+  p.r_scales = scales; p.r_nkb = cols / 16; p.r_nsb = mx ? cols / 32 : cols / 16; p.r_k_tiles = ceil_div(p.r_nsb, 4);
   const TileTensors a = {x, ld, nullptr, codes};
   const bool sr = r->mode == NVFP4_SR, swz = sf_layout == NVFP4_SF_SWIZZLED_128x4;
-  const cudaError_t e = dtype == NVFP4_BF16 ? dispatch_tile_row<__nv_bfloat16>(sr, swz, a, p, s) : dispatch_tile_row<float>(sr, swz, a, p, s);
+  const cudaError_t e = dtype == NVFP4_BF16 ? (mx ? dispatch_tile_row<__nv_bfloat16, true>(sr, swz, a, p, s) : dispatch_tile_row<__nv_bfloat16, false>(sr, swz, a, p, s))
+                                            : (mx ? dispatch_tile_row<float, true>(sr, swz, a, p, s) : dispatch_tile_row<float, false>(sr, swz, a, p, s));
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
