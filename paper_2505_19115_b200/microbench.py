@@ -72,6 +72,8 @@ def gemm_account(m, n, k, bf16_out=False):
     vp, i64, ci = C.c_void_p, C.c_int64, C.c_int
     L.nvfp4_gemm.restype = ci
     L.nvfp4_gemm.argtypes = [vp, vp, vp, vp, vp, vp, i64, i64, i64, vp, ci, i64, vp]
+    L.nvfp4_gemm_set_tile_n.argtypes = [ci]
+    L.nvfp4_gemm_set_tile_n(2256)            # the account is of the 256-wide tile, whatever the shape
     L.nvfp4_debug_gemm_account.restype = ci
     L.nvfp4_debug_gemm_account.argtypes = [C.POINTER(C.c_longlong)]
     dev = torch.device("cuda", torch.cuda.current_device())
