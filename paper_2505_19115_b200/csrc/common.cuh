@@ -83,6 +83,13 @@ int tile_quantize_row(const void* x, int dtype, int64_t rows, int64_t cols, int6
                       uint8_t* codes, uint8_t* scales, int sf_layout, cudaStream_t s, bool mx = false);
 int tile_error_word(unsigned int* out);
 
+// Per-tensor scales of a call's dense [rows, cols] operands (quantize.cu): the scratch words (two per operand, up to three
+// operands) are zeroed first where they are used, then one launch for all operands if amax_merge() says so, else one for each.
+// The operands are older than the call.
+struct AmaxOperand { const void* x; int64_t rows, cols; float* g; };
+bool amax_merge(const AmaxOperand* ops, int n, int dtype);
+int tensor_amax_scales(const AmaxOperand* ops, int n, int dtype, unsigned int* scratch, void* cuda_stream);
+
 // Per-tensor scale g = amax/2688 in one launch (quantize.cu); scratch_zeroed: two zeroed 32-bit device words.
 // The scratch is used, and has to be zeroed, only where amax_needs_scratch() says so; after the kernel that zeroes it, and
 // wherever `late` is given, x is read before the wait for the kernel launched before this one: x must be older than that.

@@ -50,21 +50,8 @@ Layout make_layout(const Plan& pl) {
   return l;
 }
 
-// Per-tensor scales of a call's one or two operands, into their workspace slots.  One launch each, after one that zeroes
-// the scratch words of the passes that use them (16 bytes in the padding behind the first slot); a call's operands are
-// older than the call, so all passes but a first one without that launch before it read at once.
-struct AmaxOperand { const void* x; int64_t rows, cols; float* g; };
-
-int amax_scales(const AmaxOperand* ops, int n, int dtype, float* first_slot, void* stream) {
-  unsigned int* scratch = reinterpret_cast<unsigned int*>(first_slot) + 16;
-  bool zeroed = false;
-  for (int i = 0; i < n; ++i) zeroed = zeroed || amax_needs_scratch(dtype, ops[i].rows * ops[i].cols);
-  if (zeroed && zero_words(scratch, 2 * n, static_cast<cudaStream_t>(stream)) != cudaSuccess) return NVFP4_ERR_CUDA;
-  for (int i = 0; i < n; ++i)
-    if (int st = tensor_amax_scale_ws(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols, ops[i].g, scratch + 2 * i, zeroed || i > 0, stream))
-      return st;
-  return NVFP4_OK;
-}
+// Scratch words of the amax passes: in the padding behind a scale's workspace slot.
+unsigned int* amax_scratch(float* slot) { return reinterpret_cast<unsigned int*>(slot) + 16; }
 
 int run_linear(int which, const void* a, const void* b, int dtype, int64_t M, int64_t N, int64_t K,
                int gscale_mode, const float* ga, const float* gb, const nvfp4_rounding* ra,
@@ -92,7 +79,7 @@ int run_linear(int which, const void* a, const void* b, int dtype, int64_t M, in
     float* wa = reinterpret_cast<float*>(ws + l.a_g);
     float* wb = reinterpret_cast<float*>(ws + l.b_g);
     const AmaxOperand ops[2] = {{a, pl.a_rows, pl.a_cols, wa}, {b, pl.b_rows, pl.b_cols, wb}};
-    if ((st = amax_scales(ops, 2, dtype, wa, stream))) return st;
+    if ((st = tensor_amax_scales(ops, 2, dtype, amax_scratch(wa), stream))) return st;
     g_a = wa; g_b = wb;
   } else if (gscale_mode == NVFP4_G_GIVEN) {
     g_a = ga; g_b = gb;
@@ -170,7 +157,7 @@ extern "C" int nvfp4_linear_fwd_qout(const void* X, const void* W, int dtype, in
     float* wa = reinterpret_cast<float*>(ws + l.a_g);
     float* wb = reinterpret_cast<float*>(ws + l.b_g);
     const AmaxOperand ops[2] = {{X, M, K, wa}, {W, N, K, wb}};
-    if ((st = amax_scales(ops, 2, dtype, wa, cuda_stream))) return st;
+    if ((st = tensor_amax_scales(ops, 2, dtype, amax_scratch(wa), cuda_stream))) return st;
     g_x = wa; g_w = wb;
   } else if (gscale_mode == NVFP4_G_GIVEN) {
     g_x = gx; g_w = gw;
@@ -202,7 +189,7 @@ extern "C" int nvfp4_linear_fwd_qin(const uint8_t* x_codes, const uint8_t* x_sca
   if (gscale_mode == NVFP4_G_AMAX) {
     float* wb = reinterpret_cast<float*>(ws + l.b_g);
     const AmaxOperand op = {W, N, K, wb};
-    if ((st = amax_scales(&op, 1, dtype, wb, cuda_stream))) return st;
+    if ((st = tensor_amax_scales(&op, 1, dtype, amax_scratch(wb), cuda_stream))) return st;
     g_w = wb;
   } else if (gscale_mode == NVFP4_G_GIVEN) {
     g_w = gw;

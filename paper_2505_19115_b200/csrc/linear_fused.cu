@@ -6,8 +6,6 @@
 // the GEMMs of Eq. 5 and Eq. 6.  nvfp4_linear_bwd does the same without saved state (it quantizes
 // W^T and X^T itself).  Every operand is bit-identical to what the separate entry points produce
 // with the same rounding arguments, so the results are too.
-#include <algorithm>
-
 #include "common.cuh"
 
 namespace nvfp4 {
@@ -72,27 +70,9 @@ bool buffer_ok(const void* p, size_t have, size_t need) {
   return p && have >= need && (reinterpret_cast<uintptr_t>(p) & 255u) == 0;
 }
 
-// Per-tensor scale of one operand according to gscale_mode: NULL, computed into `slot` (one launch, with two
-// zeroed scratch words), or given.
-int resolve_g(int gscale_mode, const void* x, int dtype, int64_t rows, int64_t cols, const float* given, float* slot,
-              unsigned int* scratch, bool late, void* stream, const float** out) {
-  *out = nullptr;
-  if (gscale_mode == NVFP4_G_AMAX) {
-    if (int st = tensor_amax_scale_ws(x, dtype, rows, cols, cols, slot, scratch, late, stream)) return st;
-    *out = slot;
-  } else if (gscale_mode == NVFP4_G_GIVEN) {
-    if (!given) return NVFP4_ERR_NULL;
-    *out = given;
-  }
-  return NVFP4_OK;
-}
-
-// Zeroes the scratch words of the call's amax passes if one of them (the largest tensor's) uses them.  `zeroed` says so:
-// the passes after it may then read their tensors at once.
-int zero_scratch(int gscale_mode, int dtype, int64_t largest, void* scratch, void* stream, bool* zeroed) {
-  *zeroed = gscale_mode == NVFP4_G_AMAX && amax_needs_scratch(dtype, largest);
-  if (!*zeroed) return NVFP4_OK;
-  return zero_words(static_cast<unsigned int*>(scratch), 16, static_cast<cudaStream_t>(stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+// Where a scale comes from according to gscale_mode: nowhere, the slot the amax pass fills, or the caller.
+const float* scale_source(int gscale_mode, const float* slot, const float* given) {
+  return gscale_mode == NVFP4_G_AMAX ? slot : gscale_mode == NVFP4_G_GIVEN ? given : nullptr;
 }
 
 }  // namespace
@@ -131,21 +111,28 @@ extern "C" int nvfp4_linear_fwd_save(const void* X, const void* W, int dtype, in
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   float* sgx = reinterpret_cast<float*>(sv + sl.gx);
   float* sgw = reinterpret_cast<float*>(sv + sl.gw);
-  const float *g_x, *g_w;
-  unsigned int* scratch = reinterpret_cast<unsigned int*>(ws + fl.scratch);
-  bool zeroed;
-  if (int st = zero_scratch(gscale_mode, dtype, std::max(M, N) * K, scratch, cuda_stream, &zeroed)) return st;
   if (gscale_mode == NVFP4_G_GIVEN) {       // the backward pass reads the scales from `saved`
     if (!gx || !gw) return NVFP4_ERR_NULL;
     if (cudaMemcpyAsync(sgx, gx, sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess) return NVFP4_ERR_CUDA;
     if (cudaMemcpyAsync(sgw, gw, sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess) return NVFP4_ERR_CUDA;
   }
-  // W first: amax(W) leaves the (smaller) weight tensor in L2 for the quantizer that follows it
-  if (int st = resolve_g(gscale_mode, W, dtype, N, K, gw, sgw, scratch, zeroed, cuda_stream, &g_w)) return st;
+  const float *g_x = scale_source(gscale_mode, sgx, gx), *g_w = scale_source(gscale_mode, sgw, gw);
+  unsigned int* scratch = reinterpret_cast<unsigned int*>(ws + fl.scratch);
+  const AmaxOperand ops[2] = {{W, N, K, sgw}, {X, M, K, sgx}};
+  const bool amax = gscale_mode == NVFP4_G_AMAX;
+  // Large operands one by one, W first: amax(W) leaves the (smaller) weight tensor in L2 for the quantizer that follows it.
+  const bool merged = amax && amax_merge(ops, 2, dtype);
+  if (merged) {
+    if (int st = tensor_amax_scales(ops, 2, dtype, scratch, cuda_stream)) return st;
+  } else if (amax) {
+    if (zero_words(scratch, 4, s) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (int st = tensor_amax_scale_ws(W, dtype, N, K, K, sgw, scratch, true, cuda_stream)) return st;
+  }
   if (int st = nvfp4_quantize_dual(W, dtype, N, K, K, g_w, rw, ws + fl.w.codes, ws + fl.w.sf, rwt, sv + sl.wt.codes,
                                    sv + sl.wt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
     return st;
-  if (int st = resolve_g(gscale_mode, X, dtype, M, K, gx, sgx, scratch + 2, true, cuda_stream, &g_x)) return st;
+  if (amax && !merged)
+    if (int st = tensor_amax_scale_ws(X, dtype, M, K, K, sgx, scratch + 2, true, cuda_stream)) return st;
   if (int st = nvfp4_quantize_dual(X, dtype, M, K, K, g_x, rx, ws + fl.x.codes, ws + fl.x.sf, rxt, sv + sl.xt.codes,
                                    sv + sl.xt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
     return st;
@@ -184,11 +171,12 @@ extern "C" int nvfp4_linear_bwd_saved(const void* dY, int dtype, int64_t M, int6
   if (!buffer_ok(saved, saved_bytes, sl.total) || !buffer_ok(workspace, workspace_bytes, bl.total)) return NVFP4_ERR_WORKSPACE;
   const uint8_t* sv = static_cast<const uint8_t*>(saved);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  const float* g_dy;
-  unsigned int* scratch = reinterpret_cast<unsigned int*>(ws + bl.scratch);
-  bool zeroed;
-  if (int st = zero_scratch(gscale_mode, dtype, M * N, scratch, cuda_stream, &zeroed)) return st;
-  if (int st = resolve_g(gscale_mode, dY, dtype, M, N, gdy, reinterpret_cast<float*>(ws + bl.gdy), scratch, zeroed, cuda_stream, &g_dy)) return st;
+  if (gscale_mode == NVFP4_G_GIVEN && !gdy) return NVFP4_ERR_NULL;
+  float* sgdy = reinterpret_cast<float*>(ws + bl.gdy);
+  const float* g_dy = scale_source(gscale_mode, sgdy, gdy);
+  const AmaxOperand op = {dY, M, N, sgdy};
+  if (gscale_mode == NVFP4_G_AMAX)
+    if (int st = tensor_amax_scales(&op, 1, dtype, reinterpret_cast<unsigned int*>(ws + bl.scratch), cuda_stream)) return st;
   const bool scaled = gscale_mode != NVFP4_G_NONE;     // must match the mode nvfp4_linear_fwd_save ran with
   const float* g_x = scaled ? reinterpret_cast<const float*>(sv + sl.gx) : nullptr;
   const float* g_w = scaled ? reinterpret_cast<const float*>(sv + sl.gw) : nullptr;
@@ -208,13 +196,12 @@ extern "C" int nvfp4_linear_bwd(const void* dY, const void* W, const void* X, in
   const BwdLayout bl = bwd_layout(M, N, K, false);
   if (!buffer_ok(workspace, workspace_bytes, bl.total)) return NVFP4_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  const float *g_dy, *g_w, *g_x;
-  unsigned int* scratch = reinterpret_cast<unsigned int*>(ws + bl.scratch);
-  bool zeroed;
-  if (int st = zero_scratch(gscale_mode, dtype, std::max(M * N, std::max(M, N) * K), scratch, cuda_stream, &zeroed)) return st;
-  if (int st = resolve_g(gscale_mode, dY, dtype, M, N, gdy, reinterpret_cast<float*>(ws + bl.gdy), scratch, zeroed, cuda_stream, &g_dy)) return st;
-  if (int st = resolve_g(gscale_mode, W, dtype, N, K, gw, reinterpret_cast<float*>(ws + bl.gw), scratch + 2, true, cuda_stream, &g_w)) return st;
-  if (int st = resolve_g(gscale_mode, X, dtype, M, K, gx, reinterpret_cast<float*>(ws + bl.gx), scratch + 4, true, cuda_stream, &g_x)) return st;
+  if (gscale_mode == NVFP4_G_GIVEN && (!gdy || !gw || !gx)) return NVFP4_ERR_NULL;
+  float *sgdy = reinterpret_cast<float*>(ws + bl.gdy), *sgw = reinterpret_cast<float*>(ws + bl.gw), *sgx = reinterpret_cast<float*>(ws + bl.gx);
+  const float *g_dy = scale_source(gscale_mode, sgdy, gdy), *g_w = scale_source(gscale_mode, sgw, gw), *g_x = scale_source(gscale_mode, sgx, gx);
+  const AmaxOperand ops[3] = {{dY, M, N, sgdy}, {W, N, K, sgw}, {X, M, K, sgx}};
+  if (gscale_mode == NVFP4_G_AMAX)
+    if (int st = tensor_amax_scales(ops, 3, dtype, reinterpret_cast<unsigned int*>(ws + bl.scratch), cuda_stream)) return st;
   if (int st = nvfp4_quantize(W, dtype, N, K, K, 1, g_w, rwt, ws + bl.wt.codes, ws + bl.wt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
     return st;
   if (int st = nvfp4_quantize(X, dtype, M, K, K, 1, g_x, rxt, ws + bl.xt.codes, ws + bl.xt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))

@@ -325,13 +325,12 @@ constexpr int kSmallAmaxCluster = 8, kSmallAmaxThreads = 1024;
 constexpr int64_t kSmallAmaxBytes = 2 << 20;
 
 template <typename T>
-__global__ void __cluster_dims__(kSmallAmaxCluster, 1, 1) __launch_bounds__(kSmallAmaxThreads)
-amax_cluster_kernel(const uint32_t* x, int64_t n_vec32, float* g_out, int late) {
+__device__ __forceinline__ void amax_cluster(const uint32_t* x, int64_t n_vec32, float* g_out, int late, uint32_t rank) {
   __shared__ uint32_t warp_max[kSmallAmaxThreads / 32];
   __shared__ uint32_t block_max[kSmallAmaxCluster];            // the first block's copy is used
   if (!late) { grid_dependency_wait(); grid_dependency_trigger(); }
   AmaxBits<T> acc;
-  for (int64_t i = (int64_t)blockIdx.x * kSmallAmaxThreads + threadIdx.x; i < n_vec32; i += 4 * kSmallAmaxCluster * kSmallAmaxThreads) {
+  for (int64_t i = (int64_t)rank * kSmallAmaxThreads + threadIdx.x; i < n_vec32; i += 4 * kSmallAmaxCluster * kSmallAmaxThreads) {
     uint32_t w[4][8];
 #pragma unroll
     for (int u = 0; u < 4; ++u) load_vec32(x, i + u * kSmallAmaxCluster * kSmallAmaxThreads, n_vec32, w[u]);
@@ -344,18 +343,41 @@ amax_cluster_kernel(const uint32_t* x, int64_t n_vec32, float* g_out, int late) 
   if (threadIdx.x < 32) {
     bits = __reduce_max_sync(0xFFFFFFFFu, warp_max[threadIdx.x]);
     if (threadIdx.x == 0) {
-      const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&block_max[blockIdx.x]);
+      const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&block_max[rank]);
       asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, 0;\n\tst.shared::cluster.u32 [a], %1;\n\t}" ::"r"(mine), "r"(bits) : "memory");
     }
   }
   if (late) { grid_dependency_wait(); grid_dependency_trigger(); }
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (rank == 0 && threadIdx.x == 0) {
     uint32_t m = 0u;
 #pragma unroll
     for (int i = 0; i < kSmallAmaxCluster; ++i) m = max(m, block_max[i]);
     *g_out = amax_to_scale(m);
   }
+}
+template <typename T>
+__global__ void __cluster_dims__(kSmallAmaxCluster, 1, 1) __launch_bounds__(kSmallAmaxThreads)
+amax_cluster_kernel(const uint32_t* x, int64_t n_vec32, float* g_out, int late) {
+  amax_cluster<T>(x, n_vec32, g_out, late, blockIdx.x);
+}
+
+// Up to three tensors in one launch: each has a cluster, or a run of blocks in proportion to its size, of its own.
+struct AmaxBatch {
+  struct Op {
+    const uint32_t* x;
+    int64_t n_vec32;
+    float* g;
+    unsigned int* scratch;         // two zeroed words (sweep only)
+    int first_block, blocks;       // of the grid (sweep only)
+  } op[3];
+  int n;
+};
+template <typename T>
+__global__ void __cluster_dims__(kSmallAmaxCluster, 1, 1) __launch_bounds__(kSmallAmaxThreads)
+amax_cluster_batch_kernel(const __grid_constant__ AmaxBatch batch) {
+  const AmaxBatch::Op& op = batch.op[blockIdx.x / kSmallAmaxCluster];
+  amax_cluster<T>(op.x, op.n_vec32, op.g, 0, blockIdx.x % kSmallAmaxCluster);
 }
 
 // Strided tensors: 16-byte loads, grid-stride.
@@ -387,11 +409,11 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const T* x, int64_t rows
 constexpr int kAmaxThreads = 512, kAmaxBlocksPerSm = 2;
 
 template <typename T, bool TICKET>
-__global__ void __launch_bounds__(kAmaxThreads, kAmaxBlocksPerSm) amax_flat_kernel(const uint32_t* x, int64_t n_vec32, unsigned int* out, float* g_out) {
+__device__ __forceinline__ void amax_sweep(const uint32_t* x, int64_t n_vec32, unsigned int* out, float* g_out, int block, int blocks) {
   __shared__ uint32_t warp_max[kAmaxThreads / 32];
-  const int64_t stride = (int64_t)gridDim.x * kAmaxThreads;
+  const int64_t stride = (int64_t)blocks * kAmaxThreads;
   AmaxBits<T> acc;
-  for (int64_t i = (int64_t)blockIdx.x * kAmaxThreads + threadIdx.x; i < n_vec32; i += 4 * stride) {
+  for (int64_t i = (int64_t)block * kAmaxThreads + threadIdx.x; i < n_vec32; i += 4 * stride) {
     uint32_t w[4][8];
 #pragma unroll
     for (int u = 0; u < 4; ++u) load_vec32(x, i + u * stride, n_vec32, w[u]);
@@ -409,16 +431,27 @@ __global__ void __launch_bounds__(kAmaxThreads, kAmaxBlocksPerSm) amax_flat_kern
     if (threadIdx.x == 0) {
       uint32_t block_bits = bits;
 #pragma unroll
-      for (int w8 = 1; w8 < kAmaxThreads / 32; ++w8) block_bits = max(block_bits, warp_max[w8]);
+      for (int w = 1; w < kAmaxThreads / 32; ++w) block_bits = max(block_bits, warp_max[w]);
       if (block_bits != 0u) atomicMax(&out[0], block_bits);
       __threadfence();
-      if (atomicAdd(&out[1], 1u) == gridDim.x - 1) {                      // every other block's maximum is in
+      if (atomicAdd(&out[1], 1u) == (uint32_t)blocks - 1) {                // every other block's maximum is in
         __threadfence();
         *g_out = amax_to_scale(atomicExch(&out[0], 0u));
         out[1] = 0u;
       }
     }
   }
+}
+template <typename T, bool TICKET>
+__global__ void __launch_bounds__(kAmaxThreads, kAmaxBlocksPerSm) amax_flat_kernel(const uint32_t* x, int64_t n_vec32, unsigned int* out, float* g_out) {
+  amax_sweep<T, TICKET>(x, n_vec32, out, g_out, blockIdx.x, gridDim.x);
+}
+template <typename T>
+__global__ void __launch_bounds__(kAmaxThreads, kAmaxBlocksPerSm) amax_flat_batch_kernel(const __grid_constant__ AmaxBatch batch) {
+  int which = 0;
+  while (which + 1 < batch.n && (int)blockIdx.x >= batch.op[which + 1].first_block) ++which;
+  const AmaxBatch::Op& op = batch.op[which];
+  amax_sweep<T, true>(op.x, op.n_vec32, op.scratch, op.g, (int)blockIdx.x - op.first_block, op.blocks);
 }
 
 __global__ void amax_finalize_kernel(float* out) {
@@ -627,6 +660,54 @@ int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, i
   const cudaError_t e = (dtype == NVFP4_BF16)
       ? launch_overlapped(amax_flat_kernel<__nv_bfloat16, true>, (unsigned)fb, kAmaxThreads, 0, s, xw, n32, scratch_zeroed, g_out)
       : launch_overlapped(amax_flat_kernel<float, true>, (unsigned)fb, kAmaxThreads, 0, s, xw, n32, scratch_zeroed, g_out);
+  return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
+
+// Together below 64 MB the operands still lie in the level-two cache when their quantizers read them, so nothing is lost by
+// sweeping them all first, and a launch and its latency are saved for each but one: 256-token layer step 36.8 -> 34.9 us,
+// 2080 x 1056 x 2848 62.6 -> 61.7, 3584 x 1440 x 1952 68.6 -> 67.2, 544 x 800 x 8288 fine-tuning step 84.6 -> 81.9; the
+// 350M-class QKV step (39 MB) +-0.5 %.
+bool amax_merge(const AmaxOperand* ops, int n, int dtype) {
+  int64_t total = 0;
+  for (int i = 0; i < n; ++i) {
+    if (!ops[i].x || !amax_flat_ok(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols)) return false;
+    total += ops[i].rows * ops[i].cols * (dtype == NVFP4_BF16 ? 2 : 4);
+  }
+  return n > 1 && total <= (int64_t)64 << 20;
+}
+
+int tensor_amax_scales(const AmaxOperand* ops, int n, int dtype, unsigned int* scratch, void* cuda_stream) {
+  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  if (int st = check_arch()) return st;
+  bool sweep = false;
+  for (int i = 0; i < n; ++i) sweep = sweep || amax_needs_scratch(dtype, ops[i].rows * ops[i].cols);
+  if (sweep && zero_words(scratch, 2 * n, s) != cudaSuccess) return NVFP4_ERR_CUDA;
+  if (!amax_merge(ops, n, dtype)) {
+    for (int i = 0; i < n; ++i)
+      if (int st = tensor_amax_scale_ws(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols, ops[i].g, scratch + 2 * i, sweep || i > 0, cuda_stream))
+        return st;
+    return NVFP4_OK;
+  }
+  AmaxBatch b = {};
+  b.n = n;
+  int64_t total = 0;
+  for (int i = 0; i < n; ++i) {
+    b.op[i] = {static_cast<const uint32_t*>(ops[i].x), ops[i].rows * ops[i].cols * (dtype == NVFP4_BF16 ? 2 : 4) / 32, ops[i].g, scratch + 2 * i, 0, 0};
+    total += b.op[i].n_vec32;
+  }
+  int first = 0;
+  for (int i = 0; i < n; ++i) {                              // blocks in proportion to the sizes, one wave in all
+    const int64_t share = (int64_t)sm_count() * kAmaxBlocksPerSm * b.op[i].n_vec32 / total;
+    b.op[i].first_block = first;
+    b.op[i].blocks = (int)std::min(ceil_div(b.op[i].n_vec32, (int64_t)kAmaxThreads * 4), std::max<int64_t>(share, 1));
+    first += b.op[i].blocks;
+  }
+  const bool bf16 = dtype == NVFP4_BF16;
+  cudaError_t e;
+  if (sweep) e = bf16 ? launch_overlapped(amax_flat_batch_kernel<__nv_bfloat16>, first, kAmaxThreads, 0, s, b)
+                      : launch_overlapped(amax_flat_batch_kernel<float>, first, kAmaxThreads, 0, s, b);
+  else e = bf16 ? launch_overlapped(amax_cluster_batch_kernel<__nv_bfloat16>, n * kSmallAmaxCluster, kSmallAmaxThreads, 0, s, b)
+                : launch_overlapped(amax_cluster_batch_kernel<float>, n * kSmallAmaxCluster, kSmallAmaxThreads, 0, s, b);
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 

@@ -223,3 +223,24 @@ def test_chained_layers_quantize_in_the_producer(shape, mode):
     if mode == nb.RTN:
         Y_unfused = nb.nvfp4_linear_fwd(H, W2.float(), gscale_mode=nb.G_AMAX, rx=rt, rw=rt)   # bf16 -> fp32 is exact
         assert torch.equal(Y, Y_unfused)
+
+
+# scales of a call's operands: one cluster each in one launch, one sweep shared in proportion to the sizes (a tiny operand
+# beside a large one, two like ones), and one launch each above the line
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("shape", [(256, 512, 512), (32, 4096, 2080), (2080, 2848, 1056), (6144, 2048, 2048), (8192, 2048, 4096)])
+def test_scales_computed_together_equal_scales_computed_alone(shape, dtype):
+    M, N, K = shape
+    X, W = synth.normal((M, K), 1.0, 5, device="cuda", dtype=dtype), synth.normal((N, K), 0.02, 6, device="cuda", dtype=dtype)
+    dY = synth.normal((M, N), 1e-3, 7, device="cuda", dtype=dtype)
+    gx, gw, gdy = (nb.nvfp4_tensor_amax_scale(t) for t in (X, W, dY))
+    assert float(gx) == float(np.float32(float(X.abs().max())) / np.float32(2688))
+    want = nb.nvfp4_linear_fwd(X, W, nb.G_GIVEN, gx=gx, gw=gw)
+    assert torch.equal(nb.nvfp4_linear_fwd(X, W), want)
+    Y, saved = nb.nvfp4_linear_fwd_save(X, W)
+    assert torch.equal(Y, want)
+    dX, dW = nb.nvfp4_linear_bwd_saved(dY, saved, K)
+    dX2, dW2 = nb.nvfp4_linear_bwd(dY, W, X)
+    dX3, dW3 = nb.nvfp4_linear_bwd(dY, W, X, nb.G_GIVEN, gdy=gdy, gw=gw, gx=gx)
+    assert torch.equal(dX, dX3) and torch.equal(dW, dW3) and torch.equal(dX2, dX3) and torch.equal(dW2, dW3)
+    assert nb.nvfp4_device_error_word() == 0
