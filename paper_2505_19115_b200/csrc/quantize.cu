@@ -328,6 +328,9 @@ template <typename T>
 __device__ __forceinline__ void amax_cluster(const uint32_t* x, int64_t n_vec32, float* g_out, int late, uint32_t rank) {
   __shared__ uint32_t warp_max[kSmallAmaxThreads / 32];
   __shared__ uint32_t block_max[kSmallAmaxCluster];            // the first block's copy is used
+  // The first block's shared memory may be written only once that block runs: every block arrives here and waits behind its
+  // loads, which hide the rendezvous (256 x 512 in bf16, back to back: 1.85 -> 1.89 us).
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   if (!late) { grid_dependency_wait(); grid_dependency_trigger(); }
   AmaxBits<T> acc;
   for (int64_t i = (int64_t)rank * kSmallAmaxThreads + threadIdx.x; i < n_vec32; i += 4 * kSmallAmaxCluster * kSmallAmaxThreads) {
@@ -340,6 +343,7 @@ __device__ __forceinline__ void amax_cluster(const uint32_t* x, int64_t n_vec32,
   uint32_t bits = acc.warp_bits();
   if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = bits;
   __syncthreads();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (threadIdx.x < 32) {
     bits = __reduce_max_sync(0xFFFFFFFFu, warp_max[threadIdx.x]);
     if (threadIdx.x == 0) {

@@ -183,3 +183,29 @@ def test_row_kernels_agree_across_the_size_line():
     codes, scales = nb.nvfp4_quantize(x, global_scale=g)
     part_c, part_s = nb.nvfp4_quantize(x[:12000], global_scale=g)  # the tile kernel
     assert torch.equal(codes[:12000], part_c) and torch.equal(scales[:12000], part_s)
+
+
+# the per-tensor scale of small dense tensors: one block's share of a load and less (the other blocks of the cluster have
+# nothing to read), a remainder, and both sides of the 2 MB line; the largest value in the first, a middle and the last place
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("shape", [(1, 16), (1, 48), (1, 8192), (3, 5456), (1024, 1024), (1025, 1024)])
+def test_small_scales_on_repeated_calls(shape, dtype):
+    x = _x(shape, 18, dtype=dtype)
+    flat, outs = x.view(-1), torch.zeros(96, dtype=torch.float32, device="cuda")
+    n = flat.numel()
+    for i in range(96):                       # no wait in between: each call overlaps the one before it
+        flat[(0, n // 2, n - 1)[i % 3]] = 64.0 + i
+        nb.nvfp4_tensor_amax_scale(x, out=outs[i:i + 1])
+    assert np.array_equal(outs.cpu().numpy(), (np.arange(96, dtype=np.float32) + 64) / np.float32(2688))
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_small_scales_of_a_call_together(dtype):
+    # operands of 1 KB to 16 KB, a cluster each in one launch
+    M, K, N = 8, 64, 64
+    X, W = _x((M, K), 19, dtype=dtype), _x((N, K), 20, dtype=dtype, std=0.02)
+    for i in range(32):
+        X[i % M, (7 * i) % K] = 8.0 + i
+        W[(5 * i) % N, i % K] = 1.0 + i
+        want = nb.nvfp4_linear_fwd(X, W, nb.G_GIVEN, gx=nb.nvfp4_tensor_amax_scale(X), gw=nb.nvfp4_tensor_amax_scale(W))
+        assert torch.equal(nb.nvfp4_linear_fwd(X, W), want)
