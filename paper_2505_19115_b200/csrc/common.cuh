@@ -63,6 +63,16 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A per-tensor scale that the kernel before this one may have written (1 where there is none): an ordinary load that stays
+// behind the wait.  __ldg is for data that nobody writes while the kernel is resident, and a kernel launched this way is
+// resident before its wait returns; source tensors read behind the wait are loaded the same way.
+__device__ __forceinline__ float load_scale(const float* g) {
+  if (!g) return 1.0f;
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(g) : "memory");
+  return v;
+}
+
 // Zeroes up to 32 words (quantize.cu), overlapping the kernel before it.
 cudaError_t zero_words(unsigned int* words, int n, cudaStream_t s);
 

@@ -490,7 +490,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
   if (!p.late) grid_dependency_wait();              // all of the above overlaps the kernel before this one
   grid_dependency_trigger();
   if constexpr (Q_OUT) {
-    build_inv_table(inv_table, p.out_g ? __ldg(p.out_g) : 1.0f);
+    build_inv_table(inv_table, load_scale(p.out_g));
     __syncthreads();
   }
 
@@ -710,7 +710,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     // Against four warps that held 3 of 8 chunks and streamed the others through their staging buffers (16384 x 11008 x
     // 4096 with fp32 output: 366 -> 313 us, input gradient of the same layer 293 -> 259; chained bf16 layers 190 -> 182).
     const int quarter = warp & 3, half = (warp >> 2) & 1;
-    const float alpha = (p.a_g ? __ldg(p.a_g) : 1.0f) * (p.b_g ? __ldg(p.b_g) : 1.0f);
+    const float alpha = load_scale(p.a_g) * load_scale(p.b_g);
     const uint32_t buf = epi_base + (warp - 8) * C::kEpiWarpBytes;
     constexpr int kChunkCols = BF16_OUT ? 64 : 32;                 // accumulator columns per 128 bytes of output row
     constexpr int kLoads = kChunkCols / 32;
@@ -747,7 +747,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 #endif
       if constexpr (Q_OUT) {
         // ---- quantized output: this lane's row, 128 of the tile's 256 columns = 8 blocks of 16 ----
-        const float cq = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), p.out_g ? __ldg(p.out_g) : 1.0f);
+        const float cq = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), load_scale(p.out_g));
         const int64_t row = (int64_t)row0 + lane;
         const int kb0 = tn * (BN / 16) + half * 8;
         uint32_t sfw[2] = {0u, 0u};                  // 8 scale bytes, four per k-tile

@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(kThreads, 3) quantize_row_kernel(const QuantPa
   const bool kb_ok = kb < p.nkb;
   grid_dependency_wait();
   grid_dependency_trigger();
-  const float g = p.gptr ? __ldg(p.gptr) : 1.0f;
+  const float g = load_scale(p.gptr);
   const float c = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), g);
   const T* x = static_cast<const T*>(p.x);
   const bool aligned32 = ((reinterpret_cast<uintptr_t>(x) | (uintptr_t)(p.ld * (int64_t)sizeof(T))) & 31u) == 0;
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kThreads, 3) quantize_transposed_kernel(const 
   const T* x = static_cast<const T*>(p.x);
   grid_dependency_wait();
   grid_dependency_trigger();
-  const float g = p.gptr ? __ldg(p.gptr) : 1.0f;
+  const float g = load_scale(p.gptr);
   const float c = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), g);
   __shared__ float inv_table[128];
   build_inv_table(inv_table, g);                              // published by the barrier after the tile lands
@@ -275,7 +275,7 @@ __device__ __forceinline__ float amax_to_scale(uint32_t bits) {
 // 32 bytes at position j, zeros past the end.
 __device__ __forceinline__ void load_vec32(const uint32_t* x, int64_t j, int64_t n_vec32, uint32_t (&w)[8]) {
   if (j < n_vec32) {
-    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
                  : "l"(x + j * 8));
   } else {

@@ -92,6 +92,13 @@ __device__ __forceinline__ uint32_t absmax_bf16x2(uint32_t a, uint32_t b) {
   return r;
 }
 
+// 16 bytes of a tensor that the kernel before this one may have written (see load_scale).
+__device__ __forceinline__ uint4 load_vec16(const void* src) {
+  uint4 v;
+  asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(src));
+  return v;
+}
+
 // One block of 16 contiguous source values.
 template <typename T>
 struct Block16;
@@ -101,12 +108,11 @@ struct Block16<__nv_bfloat16> {
   uint32_t w[8];
   __device__ __forceinline__ void load(const __nv_bfloat16* src, bool aligned32) {
     if (aligned32) {
-      asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                    : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
                    : "l"(src));
     } else {
-      const uint4 a = __ldg(reinterpret_cast<const uint4*>(src));
-      const uint4 b = __ldg(reinterpret_cast<const uint4*>(src) + 1);
+      const uint4 a = load_vec16(src), b = load_vec16(src + 8);
       w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
     }
   }
@@ -129,7 +135,10 @@ struct Block16<float> {
   float4 f[4];
   __device__ __forceinline__ void load(const float* src, bool) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) f[i] = __ldg(reinterpret_cast<const float4*>(src) + i);
+    for (int i = 0; i < 4; ++i) {
+      const uint4 q = load_vec16(src + 4 * i);
+      f[i] = make_float4(__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), __uint_as_float(q.w));
+    }
   }
   __device__ __forceinline__ float unpack(float (&v)[16]) const {
     float amax = 0.0f;

@@ -174,7 +174,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     load_tile(0);
     if (SLOTS > 1 && mine > 1) load_tile(1);
   }
-  const float g = p.gptr ? __ldg(p.gptr) : 1.0f;
+  const float g = load_scale(p.gptr);
   const float c = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), g);
   if constexpr (MX) build_inv_table_mx(inv_table, g); else build_inv_table(inv_table, g);
   __syncthreads();                                        // barriers initialised, table published
