@@ -113,6 +113,11 @@ int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, i
 __host__ __device__ inline int64_t sf_swizzled_offset(int64_t r, int64_t kb, int64_t k_tiles) {
   return ((r >> 7) * k_tiles + (kb >> 2)) * 512 + (r & 31) * 16 + ((r >> 5) & 3) * 4 + (kb & 3);
 }
+// Four scale bytes of one quantized row of which the first `left` belong to the tensor, the others being padding: zero also
+// where the per-tensor scale is NaN or so small that a zero block's scale encodes as NaN.
+__device__ __forceinline__ uint32_t scales_inside(uint32_t word, int64_t left) {
+  return left >= 4 ? word : left <= 0 ? 0u : word & ((1u << (8 * (int)left)) - 1u);
+}
 
 // ---------------------------------------------------------------------------------------------
 // Number formats (Section 3 of the paper)

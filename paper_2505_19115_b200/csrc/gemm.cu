@@ -787,7 +787,8 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             for (int t = 0; t < 2; ++t) {
               const int64_t kt = (int64_t)(kb0 >> 2) + t;
               if (kt < p.out_k_tiles)
-                *reinterpret_cast<uint32_t*>(p.out_scales + sf_swizzled_offset(row, kt * 4, p.out_k_tiles)) = sfw[t];
+                *reinterpret_cast<uint32_t*>(p.out_scales + sf_swizzled_offset(row, kt * 4, p.out_k_tiles)) =
+                    scales_inside(sfw[t], row < p.M ? p.out_nkb - kt * 4 : 0);
             }
           }
         } else if (row < p.M) {

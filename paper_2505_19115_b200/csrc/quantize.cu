@@ -237,7 +237,8 @@ __global__ void __launch_bounds__(kThreads, 3) quantize_transposed_kernel(const 
       const uint8_t* s4 = sf_s + (t * 4) * kTCols + srow;
       const uint32_t val = (uint32_t)s4[0] | ((uint32_t)s4[kTCols] << 8) | ((uint32_t)s4[2 * kTCols] << 16) |
                            ((uint32_t)s4[3 * kTCols] << 24);
-      *reinterpret_cast<uint32_t*>(p.scales + sf_swizzled_offset(c0 + cl, kt * 4, p.k_tiles)) = val;
+      *reinterpret_cast<uint32_t*>(p.scales + sf_swizzled_offset(c0 + cl, kt * 4, p.k_tiles)) =
+          scales_inside(val, c0 + cl < p.cols ? p.nkb - kt * 4 : 0);
       if (fill_upper)
         *reinterpret_cast<uint32_t*>(p.scales + sf_swizzled_offset(c0 + cl + 64, kt * 4, p.k_tiles)) = 0u;
     }

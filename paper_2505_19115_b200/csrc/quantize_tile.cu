@@ -344,6 +344,8 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     constexpr int kKtPerTile = kSbPerTile / 4;            // scale tiles per column
     const int kb0 = r0 / kSbRows;
     if constexpr (SWZ) {
+      // a tile that reaches past the tensor also holds padding (rows and columns are below 2^31)
+      [[maybe_unused]] const bool edge = (uint32_t)c0 + kTileCols > (uint32_t)p.cols || (uint32_t)r0 + ROWS > (uint32_t)p.rows;
       // transposed scales: one 32-bit word = four row blocks of one column
       static_assert(kTileCols * kKtPerTile <= kThreads, "one word per thread");
       if (TR && threadIdx.x < kTileCols * kKtPerTile) {
@@ -352,7 +354,9 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
         if (kt0 + q < p.t_k_tiles) {
           uint8_t* dst = p.t_scales + ((int64_t)(c0 >> 7) * p.t_k_tiles + kt0) * 512 + ((c0 & 64) >> 3) +
                          (q * 512 + (cl & 31) * 16 + (cl >> 5) * 4);
-          *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(sf_t + q * (4 * kTileCols) + cl * 4);
+          uint32_t val = *reinterpret_cast<const uint32_t*>(sf_t + q * (4 * kTileCols) + cl * 4);
+          if (edge) val = scales_inside(val, c0 + cl < p.cols ? p.t_nsb - 4 * (kt0 + q) : 0);
+          *reinterpret_cast<uint32_t*>(dst) = val;
           if (((c0 & 127) == 0) && ((int64_t)c0 + kTileCols >= p.cols))        // nobody else owns rows 64..127 of the scale tile
             *reinterpret_cast<uint32_t*>(dst + 8) = 0u;
         }
@@ -371,9 +375,17 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       } else if constexpr (ROW) {
         // row scales: the tile owns whole 512-byte scale tiles (128 rows x this k-tile)
         const int h = (threadIdx.x >> 5) - 4, i = threadIdx.x & 31;   // from the fifth warp on
-        if (h >= 0 && h < ROWS / 128 && (int64_t)r0 + h * 128 < p.rows)
-          *reinterpret_cast<uint4*>(p.r_scales + ((int64_t)(r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) =
-              *reinterpret_cast<const uint4*>(sf_r + h * 512 + i * 16);
+        if (h >= 0 && h < ROWS / 128 && (int64_t)r0 + h * 128 < p.rows) {
+          uint4 val = *reinterpret_cast<const uint4*>(sf_r + h * 512 + i * 16);   // rows i, i + 32, i + 64, i + 96
+          if (edge) {
+            const int64_t rows_left = p.rows - (r0 + h * 128 + i), left = p.r_nsb - c0 / 16;
+            val.x = scales_inside(val.x, rows_left > 0 ? left : 0);
+            val.y = scales_inside(val.y, rows_left > 32 ? left : 0);
+            val.z = scales_inside(val.z, rows_left > 64 ? left : 0);
+            val.w = scales_inside(val.w, rows_left > 96 ? left : 0);
+          }
+          *reinterpret_cast<uint4*>(p.r_scales + ((int64_t)(r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) = val;
+        }
       }
     } else if constexpr (TR) {
       for (int id = threadIdx.x; id < kTileCols * kSbPerTile; id += kThreads) {

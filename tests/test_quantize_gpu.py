@@ -209,3 +209,30 @@ def test_small_scales_of_a_call_together(dtype):
         W[(5 * i) % N, i % K] = 1.0 + i
         want = nb.nvfp4_linear_fwd(X, W, nb.G_GIVEN, gx=nb.nvfp4_tensor_amax_scale(X), gw=nb.nvfp4_tensor_amax_scale(W))
         assert torch.equal(nb.nvfp4_linear_fwd(X, W), want)
+
+
+# Padding of swizzled scale tiles is zero whatever the per-tensor scale: NaN (a diverged tensor), 0 and a subnormal one make
+# the scale of a block of zeros encode as NaN.  Rows and columns that leave padding in both directions, through the tile
+# kernel (multiples of 32), the plain kernels (multiples of 16 only) and the product's quantizing epilogue.
+@pytest.mark.parametrize("g", [float("nan"), 0.0, 1e-40])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("shape", [(96, 96), (160, 352), (48, 80), (272, 1040)])
+def test_padding_scales_are_zero_under_any_global_scale(shape, dtype, g):
+    from oracle import binding as ob
+    rows, cols = shape
+    x, g_t = _x(shape, 21, dtype=dtype), torch.full((1,), g, device="cuda")
+
+    def padding(Rq, Kq):
+        return ob.sf_swizzle(np.ones((Rq, Kq // 16), np.uint8)) == 0
+    for mode in (nb.RTN, nb.SR):
+        r = nb.Rounding(mode, 1, 2)
+        sr = nb.nvfp4_quantize(x, False, g_t, r, nb.SF_SWIZZLED)[1]
+        st = nb.nvfp4_quantize(x, True, g_t, r, nb.SF_SWIZZLED)[1]
+        _, dr, _, dt = nb.nvfp4_quantize_dual(x, g_t, r, r, nb.SF_SWIZZLED)
+        for sf, (Rq, Kq) in ((sr, (rows, cols)), (dr, (rows, cols)), (st, (cols, rows)), (dt, (cols, rows))):
+            assert not sf.cpu().numpy()[:nb.nvfp4_sf_bytes(Rq, Kq)][padding(Rq, Kq)].any()
+    a = nb.nvfp4_quantize(_x((rows, 64), 22), sf_layout=nb.SF_SWIZZLED)
+    b = nb.nvfp4_quantize(_x(((cols + 31) // 32 * 32, 64), 23), sf_layout=nb.SF_SWIZZLED)
+    sf = nb.nvfp4_gemm_quantized(*a, None, *b, None, g_t, sf_layout=nb.SF_SWIZZLED)[1].cpu().numpy()
+    N = b[0].shape[0]
+    assert not sf[:nb.nvfp4_sf_bytes(rows, N)][padding(rows, N)].any()
