@@ -134,12 +134,17 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)     # not part of torch's public interface
+
+
 def _stream(stream=None):
     """Handle of `stream`, or of the current stream of the current device.  The small calls are bound by the host, so
     the handle is fetched without building a torch.cuda.Stream object (1.3 us of a call)."""
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def nvfp4_sf_bytes(Rq: int, Kq: int, sf_layout: int = SF_SWIZZLED) -> int:

@@ -161,3 +161,13 @@ def test_newer_entry_points_reject_bad_arguments_on_the_host():
     assert L.nvfp4_linear_bwd_bf16_workspace_bytes(256, 512, 512) == 0          # operands are read in place
     gx = lambda **kw: L.nvfp4_gemm_bf16_ex(kw.get("a", buf), kw.get("am", 0), buf, kw.get("bm", 0), kw.get("M", 128), 128, 64, buf, 1, 128, None)
     assert gx(a=None) == 1 and gx(am=2) == 4 and gx(am=1, bm=0) == 4 and gx(am=1, bm=1, M=100) == 2
+
+
+def test_stream_handle_without_the_raw_stream_function(monkeypatch):
+    # the quick way to the current stream's handle is private to torch: where it is missing, the public one serves
+    class Stream:
+        cuda_stream = 1234
+    monkeypatch.setattr(nb, "_raw_stream", None)
+    monkeypatch.setattr(nb.torch.cuda, "current_stream", lambda *a: Stream())
+    assert nb._stream() == 1234
+    assert nb._stream(Stream()) == 1234

@@ -45,3 +45,12 @@ def test_operands_written_by_the_call_before(shape, out_dtype):
     assert nb.nvfp4_device_error_word() == 0
     for w, o in zip(want, got):
         assert all(torch.equal(x, y) for x, y in zip(w, o))
+
+
+def test_stream_handle_is_the_current_streams(monkeypatch):
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        assert nb._stream() == side.cuda_stream
+        monkeypatch.setattr(nb, "_raw_stream", None)
+        assert nb._stream() == side.cuda_stream
+    assert nb._stream() == torch.cuda.current_stream().cuda_stream
