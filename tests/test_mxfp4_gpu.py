@@ -158,3 +158,18 @@ def test_three_products_of_a_layer_in_mxfp4():
         ref, T = ob.gemm_mx(oa[0], oa[1], gf[ga], ob_[0], ob_[1], gf[gb])
         assert np.all(np.abs(_h(D) - ref) <= TOL * T), name
         assert float(D.abs().max()) > 0.0
+
+
+# large bf16 tensors rounded to nearest: the 256-row form of the tile kernel (transposed, from 2^25 elements) and the plain
+# row kernel (from 48 Mi elements), sizes that fill neither a tile nor a scale tile
+@pytest.mark.parametrize("sf_layout", [nb.SF_LINEAR, nb.SF_SWIZZLED])
+@pytest.mark.parametrize("transposed,shape", [(True, (8224, 4104)), (False, (12305, 4128))])
+def test_large_tensors_match_the_oracle(transposed, shape, sf_layout):
+    x = synth.normal(shape, 1.0, 8, device="cuda")
+    g_t = nb.nvfp4_tensor_amax_scale(x)
+    codes, scales = nb.nvfp4_quantize_mx(x, transposed, g_t, None, sf_layout)
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    oc, osf = ob.quantize_mx(_h(x), g=float(g_t.item()), transposed=transposed)
+    assert np.array_equal(codes.cpu().numpy(), oc)
+    assert np.array_equal(scales.cpu().numpy().reshape(-1), (_swz(osf) if sf_layout == nb.SF_SWIZZLED else osf).reshape(-1))

@@ -54,3 +54,89 @@ def test_stream_handle_is_the_current_streams(monkeypatch):
         monkeypatch.setattr(nb, "_raw_stream", None)
         assert nb._stream() == side.cuda_stream
     assert nb._stream() == torch.cuda.current_stream().cuda_stream
+
+
+# Two layers that share a workspace, four steps on the same input, saved-operand and output buffers with inputs that change
+# in between, against the same calls on fresh buffers with a wait after each.  256 x 512: the cluster amax; 2080 x 1056: one
+# shared sweep, ragged tiles; 4096 x 1024 x 3072: the weight gradient starts in the input gradient's last wave.
+def _step_buffers(M, K, N, dtype, mode):
+    layers = []
+    for (k, n) in ((K, N), (N, K)):
+        layers.append(dict(X=torch.empty((M, k), dtype=dtype, device="cuda"), W=torch.empty((n, k), dtype=dtype, device="cuda"),
+                           dY=torch.empty((M, n), dtype=dtype, device="cuda"), K=k,
+                           g=[torch.empty(1, device="cuda") if mode == nb.G_GIVEN else None for _ in range(3)],
+                           saved=torch.empty(nb.nvfp4_linear_saved_bytes(M, n, k), dtype=torch.uint8, device="cuda"),
+                           Y=torch.empty((M, n), device="cuda"), dX=torch.empty((M, k), device="cuda"), dW=torch.empty((n, k), device="cuda")))
+    ws = torch.empty(max(nb.nvfp4_linear_fused_workspace_bytes(M, *nk, w) for nk in ((N, K), (K, N))
+                         for w in (nb.FUSED_FWD_SAVE, nb.FUSED_BWD_SAVED)), dtype=torch.uint8, device="cuda")
+    return layers, ws
+
+
+def _fill(layers, step):
+    for i, l in enumerate(layers):
+        for j, (name, std) in enumerate((("X", 1.0), ("W", 0.02), ("dY", 1e-3))):
+            t = l[name]
+            t.amax()                                            # the old contents lie in caches when the new ones are written
+            t.copy_(_x(t.shape, 100 * step + 10 * i + j, std * 2.0 ** ((step + j) % 3), t.dtype))
+            if l["g"][j] is not None:
+                l["g"][j].copy_(t.float().abs().amax() / 2688)
+
+
+def _step(layers, ws, mode, stream=None, fresh=False):
+    def wait():
+        if fresh:
+            torch.cuda.synchronize()
+    sr = [nb.Rounding(nb.SR, 11, o) for o in range(3)]
+    keep = {}
+    for i, l in enumerate(layers):
+        gx, gw, _ = l["g"]
+        kw = {} if fresh else dict(out=l["Y"], saved=l["saved"], workspace=ws)
+        keep[i] = nb.nvfp4_linear_fwd_save(l["X"], l["W"], mode, gx=gx, gw=gw, rxt=sr[2], stream=stream, **kw)
+        wait()
+    for i, l in reversed(list(enumerate(layers))):
+        kw = {} if fresh else dict(dX=l["dX"], dW=l["dW"], workspace=ws)
+        Y, saved = keep[i]
+        keep[i] = (Y, *nb.nvfp4_linear_bwd_saved(l["dY"], saved, l["K"], mode, gdy=l["g"][2], rdy=sr[0], rdyt=sr[1], stream=stream, **kw))
+        wait()
+    return [t for i in sorted(keep) for t in keep[i]]
+
+
+@pytest.mark.parametrize("how", ["current stream", "given stream", "graph"])
+@pytest.mark.parametrize("mode", [nb.G_AMAX, nb.G_GIVEN])
+@pytest.mark.parametrize("shape,dtype", [((256, 512, 512), torch.bfloat16), ((2080, 1056, 2848), torch.bfloat16),
+                                         ((4096, 1024, 3072), torch.bfloat16), ((1056, 544, 1056), torch.float32)])
+def test_steps_on_the_same_buffers(shape, dtype, mode, how):
+    layers, ws = _step_buffers(*shape, dtype, mode)
+    want = []
+    for i in range(4):
+        _fill(layers, i)
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in _step(layers, ws, mode, fresh=True)])
+    side = torch.cuda.Stream()
+    graph = None
+    if how == "graph":
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            _step(layers, ws, mode)
+    outs = [t for l in layers for t in (l["Y"], l["dX"], l["dW"])]
+    got = []
+    torch.cuda.synchronize()
+    for i in range(4):
+        if how == "given stream":
+            with torch.cuda.stream(side):
+                _fill(layers, i)
+            _step(layers, ws, mode, stream=side)
+            with torch.cuda.stream(side):
+                got.append([t.clone() for t in outs])
+        else:
+            _fill(layers, i)
+            if graph is None:
+                _step(layers, ws, mode)
+            else:
+                graph.replay()
+            got.append([t.clone() for t in outs])
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    for i in range(4):
+        for w, g in zip(want[i], got[i]):
+            assert torch.equal(w, g), f"step {i}"

@@ -236,3 +236,51 @@ def test_padding_scales_are_zero_under_any_global_scale(shape, dtype, g):
     sf = nb.nvfp4_gemm_quantized(*a, None, *b, None, g_t, sf_layout=nb.SF_SWIZZLED)[1].cpu().numpy()
     N = b[0].shape[0]
     assert not sf[:nb.nvfp4_sf_bytes(rows, N)][padding(rows, N)].any()
+
+
+# ---------------------------------------------------------------- the 256-row form of the tile kernel
+# Large bf16 tensors take it: from 2^26 elements with both outputs, from 2^25 transposed and rounded to nearest.  Rows and
+# columns that fill neither a tile nor a scale tile, both layouts.
+@pytest.fixture(scope="module")
+def tall_dual():
+    from tests.util import to_host_f32
+    x = _x((8224, 8224), 24)
+    g_t = nb.nvfp4_tensor_amax_scale(x)
+    return x, g_t, {tr: to_host_f32(x.T.contiguous() if tr else x) for tr in (False, True)}, {}
+
+
+def _sf_wanted(osf, sf_layout):
+    from oracle import binding as ob
+    return (ob.sf_swizzle(osf) if sf_layout == nb.SF_SWIZZLED else osf).reshape(-1)
+
+
+@pytest.mark.parametrize("sf_layout", [nb.SF_LINEAR, nb.SF_SWIZZLED])
+@pytest.mark.parametrize("modes", [(nb.RTN, nb.SR), (nb.SR, nb.SR), (nb.RTN, nb.RTN), (nb.SR, nb.RTN)])
+def test_dual_tall_tiles_ragged(tall_dual, modes, sf_layout):
+    from oracle import binding as ob
+    x, g_t, host, known = tall_dual
+    for tr, mode in ((False, modes[0]), (True, modes[1])):
+        if (tr, mode) not in known:
+            known[tr, mode] = ob.quantize(host[tr], g=float(g_t.item()), mode=mode, seed=6, offset=int(tr))
+    cr, sr, ct, st = nb.nvfp4_quantize_dual(x, g_t, nb.Rounding(modes[0], 6, 0), nb.Rounding(modes[1], 6, 1), sf_layout)
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    for got_c, got_s, key in ((cr, sr, (False, modes[0])), (ct, st, (True, modes[1]))):
+        oc, osf = known[key]
+        assert np.array_equal(got_c.cpu().numpy(), oc)
+        assert np.array_equal(got_s.cpu().numpy().reshape(-1), _sf_wanted(osf, sf_layout))
+
+
+@pytest.mark.parametrize("sf_layout", [nb.SF_LINEAR, nb.SF_SWIZZLED])
+def test_transposed_tall_tiles_ragged(sf_layout):
+    assert_quantize_parity(_x((8224, 4104), 25), True, True, nb.Rounding(nb.RTN), sf_layout)
+
+
+def test_padding_scales_of_tall_tiles_are_zero_under_a_nan_scale():
+    from oracle import binding as ob
+    x, nan = _x((8224, 8224), 26), torch.full((1,), float("nan"), device="cuda")
+    _, sr, _, st = nb.nvfp4_quantize_dual(x, nan, nb.Rounding(nb.SR, 1, 1), nb.Rounding(nb.SR, 1, 2), nb.SF_SWIZZLED)
+    sf = nb.nvfp4_quantize(x, True, nan, None, nb.SF_SWIZZLED)[1]
+    padding = ob.sf_swizzle(np.ones((8224, 514), np.uint8)) == 0
+    for s in (sr, st, sf):
+        assert not s.cpu().numpy()[padding].any()
