@@ -2,8 +2,8 @@
 // axis, output stored [cols, rows/2]), the row quantization (blocks along the column axis), or both.  Both is the producer fusion for the operands that Eq. 4-6 need in both orientations: dY as Q(dY) for Eq. 5 and
 // Q(dY^T) for Eq. 6, X as Q(X) for Eq. 4 and Q(X^T) for Eq. 6, W as Q(W) for Eq. 4 and Q(W^T) for Eq. 5.
 //
-// Persistent blocks walk over tiles of 128 or 256 rows x 64 columns.  One thread fetches tiles with tiled bulk copies
-// (128-byte swizzle, zero fill outside the tensor); all threads quantize from shared memory; the packed codes are staged
+// Persistent blocks walk over tiles of 128 rows x 64 columns, or a block of its own takes each tile of 256 rows (launch_tile
+// says which).  One thread fetches tiles with tiled bulk copies (128-byte swizzle, zero fill outside the tensor); all threads quantize from shared memory; the packed codes are staged
 // in shared memory and leave as tiled bulk stores (which clip at the tensor edge), the scales as plain stores.
 //
 // Bound by instruction issue where it rounds stochastically, by memory otherwise.  Against one 256-row tile per block and,
@@ -24,9 +24,9 @@ constexpr int kTileCols = 64;
 constexpr unsigned long long kTileWaitLimitNs = 2000000000ull;
 constexpr int kLoader = kThreads - 32;                                // the thread that issues the bulk copies
 
-// Shared memory of a block, in order: tile slots, code staging, scale staging (two of it, used in turn).
-// Two slots: the tile after next lands while the present one is quantized, codes are staged in turn as well.  One slot:
-// the next tile is fetched when the present one's codes have left their staging buffer; the other blocks of the SM cover.
+// Shared memory of a block, in order: tile slots, code staging, scale staging, SLOTS of each.
+// Two slots, used in turn: the tile after next lands while the present one is quantized.  One slot: the block has one tile,
+// and the other blocks of the SM cover its load and its stores.
 template <typename T, int ROWS, bool TR, bool ROW, int SLOTS>
 struct TileSmem {
   static constexpr int kBoxBytes = ROWS * 128;                        // a copy's box is 128 bytes wide: 64 bf16 or 32 fp32 columns
@@ -39,7 +39,7 @@ struct TileSmem {
   static constexpr int kSfRBytes = ROW ? (ROWS / 128) * 512 : 0;     // whole scale tiles (128 rows x 4 blocks)
   static constexpr int kSfBytes = kSfTBytes + kSfRBytes;
   static constexpr int kCodesAt = SLOTS * kTileBytes, kSfAt = kCodesAt + SLOTS * kCodesBytes;
-  static constexpr int kBytes = kSfAt + 2 * kSfBytes + 1024 /*align*/;
+  static constexpr int kBytes = kSfAt + SLOTS * kSfBytes + 1024 /*align*/;
   static constexpr int kBlocksPerSm = sizeof(T) == 2 ? 4 : 2;
   static_assert(kBlocksPerSm * (kBytes + 1024 /*static*/ + 1024 /*reserved*/) <= 228 * 1024, "shared memory of an SM");
 };
@@ -48,7 +48,7 @@ struct TileParams {
   const float* gptr;
   int64_t rows, cols;
   int tiles_x, tiles;         // tiles across the columns, in all
-  int step_x, step_y;         // distance between two tiles of a block: gridDim.x = step_y * tiles_x + step_x
+  int step_x, step_y;         // two slots: distance between two tiles of a block, gridDim.x = step_y * tiles_x + step_x
   // transposed output: quantized shape (cols, rows)
   PhiloxStream t_rng;
   uint8_t* t_scales;
@@ -145,7 +145,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // Tiles are walked from the last to the first: a pass over the tensor that ran just before (its amax) left the end of
   // it in the level-two cache, not the beginning.
-  const int mine = (p.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int mine = SLOTS == 1 ? 1 : (p.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
   int ty = (p.tiles - 1 - (int)blockIdx.x) / p.tiles_x, tx = (p.tiles - 1 - (int)blockIdx.x) - ty * p.tiles_x;
   int load_x = tx, load_y = ty;                           // the loader's position, up to two tiles ahead
   auto step_back = [&](int& x, int& y) {
@@ -202,7 +202,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     const int b = SLOTS == 2 ? k & 1 : 0;
     const int c0 = tx * kTileCols, r0 = ty * ROWS;          // below 2^31, as rows and columns are
     if (!wait_tile(smem_addr(&bars[b]), (SLOTS == 2 ? k >> 1 : k) & 1)) break;
-    uint8_t* const sf_t = smem_gen + S::kSfAt + (k & 1) * S::kSfBytes;
+    uint8_t* const sf_t = smem_gen + S::kSfAt + b * S::kSfBytes;
     uint8_t* const sf_r = sf_t + S::kSfTBytes;
 
     if constexpr (TR) {
@@ -320,7 +320,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       });
     }
 
-    // ---- codes out: tiled bulk stores from this tile's staging buffer; the tile's slot takes the tile after next ----
+    // ---- codes out: tiled bulk stores from this tile's staging buffer; its slot then takes the tile after next ----
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (SLOTS == 2 && threadIdx.x == kLoader)             // the previous tile's codes have left the other staging buffer
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -334,8 +334,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
                      ::"l"(&map_cr), "r"(out + S::kCodesTBytes), "r"(c0 / 2), "r"(r0) : "memory");
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-      if constexpr (SLOTS == 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      if (k + SLOTS < mine) load_tile(b);
+      if (SLOTS == 2 && k + SLOTS < mine) load_tile(b);
     }
 
     // ---- scales out ----
@@ -393,7 +392,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
         if (c0 + cl < p.cols && kb0 + u < p.t_nsb) p.t_scales[(int64_t)(c0 + cl) * p.t_nsb + kb0 + u] = sf_t[(u >> 2) * (4 * kTileCols) + cl * 4 + (u & 3)];
       }
     }
-    step_back(tx, ty);
+    if constexpr (SLOTS == 2) step_back(tx, ty);
   }
   if (threadIdx.x == kLoader) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // staging must outlive the stores' reads
 }
