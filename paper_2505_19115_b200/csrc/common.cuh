@@ -88,7 +88,7 @@ int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t 
                   const nvfp4_rounding* rr, uint8_t* codes_r, uint8_t* scales_r, int sf_layout, cudaStream_t s,
                   bool mx_t = false);   // mx_t: MXFP4 (blocks of 32, E8M0 scales) for the transposed output, no row output
 // The same kernel with the row output alone.
-bool tile_row_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool sr);
+bool tile_row_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool sr, bool mx = false);
 int tile_quantize_row(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, const float* g, const nvfp4_rounding* r,
                       uint8_t* codes, uint8_t* scales, int sf_layout, cudaStream_t s, bool mx = false);
 int tile_error_word(unsigned int* out);

@@ -557,8 +557,8 @@ extern "C" int nvfp4_quantize(const void* x, int dtype, int64_t rows, int64_t co
 
 namespace nvfp4 {
 namespace {
-template <typename T>
-cudaError_t dispatch_row_mx(const QuantParams& p, bool sr, bool swz, cudaStream_t s) {
+cudaError_t launch_row_mx(const QuantParams& p, bool sr, bool swz, cudaStream_t s) {
+  using T = __nv_bfloat16;
   dim3 grid((unsigned)ceil_div(p.nkb, 32), (unsigned)ceil_div(p.rows, kRowTileRows));
   if (sr) return swz ? launch_overlapped(quantize_row_kernel<T, true, true, true>, grid, kThreads, 0, s, p)
                      : launch_overlapped(quantize_row_kernel<T, true, false, true>, grid, kThreads, 0, s, p);
@@ -601,8 +601,9 @@ extern "C" int nvfp4_quantize_mx(const void* x, int dtype, int64_t rows, int64_t
   if (tile_path)
     return tile_quantize(x, dtype, rows, cols, ld, global_scale, false, rounding, codes, scales, nullptr, nullptr, nullptr, sf_layout, s,
                          /*mx_t=*/true);
-  if (!transposed && tile_row_quantizer_eligible(dtype, rows, cols, rounding->mode == NVFP4_SR))
+  if (!transposed && tile_row_quantizer_eligible(dtype, rows, cols, rounding->mode == NVFP4_SR, /*mx=*/true))
     return tile_quantize_row(x, dtype, rows, cols, ld, global_scale, rounding, codes, scales, sf_layout, s, /*mx=*/true);
+  if (dtype != NVFP4_BF16) return NVFP4_ERR_SHAPE;            // 2^31 tiles of fp32: beyond any memory
   const void* src = x;
   int64_t src_ld = ld;
   if (transposed) {
@@ -617,8 +618,7 @@ extern "C" int nvfp4_quantize_mx(const void* x, int dtype, int64_t rows, int64_t
   p.codes = codes; p.scales = scales;
   p.nkb = Kq / 16; p.nsb = Kq / 32; p.k_tiles = ceil_div(p.nsb, 4);
   const bool sr = rounding->mode == NVFP4_SR, swz = sf_layout == NVFP4_SF_SWIZZLED_128x4;
-  cudaError_t e = (dtype == NVFP4_BF16) ? dispatch_row_mx<__nv_bfloat16>(p, sr, swz, s) : dispatch_row_mx<float>(p, sr, swz, s);
-  return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  return launch_row_mx(p, sr, swz, s) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
 extern "C" int nvfp4_quantize_dual(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld,

@@ -521,8 +521,9 @@ int tile_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t 
 // (us, row kernel / this: bf16 RtN 256 x 512 4.1 / 2.0, 2080 x 1056 5.7 / 2.4, 11008 x 4096 20.0 / 20.2, 16384 x 11008
 // 71 / 77; SR 7.2 / 2.9 at 2080 x 1056, 24.0 / 21.3, 80 / 75; fp32 RtN 7.0 / 3.4, 36 / 33, 126 / 122).  MXFP4 follows the same line:
 // the 16384 x 1024 x 2816 forward in it 57.8 us / 55.9, 2048 x 4096 x 11008 97.7 / 93.3.
-bool tile_row_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool sr) {
-  if (cols % 32 != 0 || rows * cols >= (int64_t)1 << 36 || ceil_div(rows, 128) * ceil_div(cols, kTileCols) >= (int64_t)1 << 31) return false;
+bool tile_row_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool sr, bool mx) {
+  if (!mx && rows * cols >= (int64_t)1 << 36) return false;                          // block indices in 32 bits
+  if (cols % 32 != 0 || ceil_div(rows, 128) * ceil_div(cols, kTileCols) >= (int64_t)1 << 31) return false;
   return dtype == NVFP4_FP32 || sr || rows * cols < (int64_t)48 << 20;
 }
 
