@@ -112,9 +112,9 @@ NVFP4_API int nvfp4_quantize(const void* x, int dtype, int64_t rows, int64_t col
  * output is bit-identical to what the corresponding nvfp4_quantize call writes.
  * rows and cols must both be multiples of 16.  codes_row: rows*cols/2 bytes, scales_row:
  * nvfp4_sf_bytes(rows, cols, sf_layout); codes_t: cols*rows/2 bytes, scales_t:
- * nvfp4_sf_bytes(cols, rows, sf_layout).  bf16 tensors whose rows and cols are multiples of 32 take
- * the fused kernel (one read, 3.125 bytes of traffic per element); others run the two
- * single-output kernels.  Alignment and errors as for nvfp4_quantize.
+ * nvfp4_sf_bytes(cols, rows, sf_layout).  Tensors whose rows and cols are multiples of 32 take the
+ * fused kernel (one read: 3.125 bytes of traffic per element in bf16, 5.125 in fp32); others run the
+ * two single-output kernels.  Alignment and errors as for nvfp4_quantize.
  */
 NVFP4_API int nvfp4_quantize_dual(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld,
                         const float* global_scale,
@@ -294,9 +294,9 @@ NVFP4_API int nvfp4_linear_bwd(const void* dY, const void* W, const void* X, int
  * values); nvfp4_sf_bytes_mx gives the size.  The random integers of SR belong to groups of 16
  * elements exactly as for NVFP4 (group index r*(Kq/16) + k/16).  Kq % 32 == 0.
  * nvfp4_quantize_mx: transposed == 1 (bf16 only) quantizes along the rows straight from the source
- * tile (no transpose pass, `workspace` unused and may be NULL); only a tensor with more than 2^24 rows
- * goes through a transpose into `workspace` (rows*cols*2 bytes, 16-byte aligned) and is rejected with
- * NVFP4_ERR_WORKSPACE without one.
+ * tile (no transpose pass, `workspace` unused and may be NULL); only a tensor with more than 65535*256 rows
+ * is refused, with NVFP4_ERR_WORKSPACE where `workspace` is not rows*cols*2 bytes, 16-byte aligned, and
+ * with NVFP4_ERR_SHAPE where it is.
  * nvfp4_gemm_mx: as nvfp4_gemm on MXFP4 operands (tcgen05 kind::mxf4, scale_vec::2X).
  */
 NVFP4_API size_t nvfp4_sf_bytes_mx(int64_t Rq, int64_t Kq, int sf_layout);

@@ -482,10 +482,10 @@ cudaError_t launch_amax_cluster(const void* x, int dtype, int64_t n32, float* g_
       : launch_overlapped(amax_cluster_kernel<float>, kSmallAmaxCluster, kSmallAmaxThreads, 0, s, xw, n32, g_out, (int)late);
 }
 
-template <typename T, bool SR, bool SWZ>
+template <typename T, bool SR, bool SWZ, bool MX = false>
 cudaError_t launch_row(const QuantParams& p, cudaStream_t s) {
   dim3 grid((unsigned)ceil_div(p.nkb, 32), (unsigned)ceil_div(p.rows, kRowTileRows));
-  return launch_overlapped(quantize_row_kernel<T, SR, SWZ>, grid, kThreads, 0, s, p);
+  return launch_overlapped(quantize_row_kernel<T, SR, SWZ, MX>, grid, kThreads, 0, s, p);
 }
 
 template <typename T, bool SR, bool SWZ>
@@ -555,19 +555,6 @@ extern "C" int nvfp4_quantize(const void* x, int dtype, int64_t rows, int64_t co
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
-namespace nvfp4 {
-namespace {
-cudaError_t launch_row_mx(const QuantParams& p, bool sr, bool swz, cudaStream_t s) {
-  using T = __nv_bfloat16;
-  dim3 grid((unsigned)ceil_div(p.nkb, 32), (unsigned)ceil_div(p.rows, kRowTileRows));
-  if (sr) return swz ? launch_overlapped(quantize_row_kernel<T, true, true, true>, grid, kThreads, 0, s, p)
-                     : launch_overlapped(quantize_row_kernel<T, true, false, true>, grid, kThreads, 0, s, p);
-  return swz ? launch_overlapped(quantize_row_kernel<T, false, true, true>, grid, kThreads, 0, s, p)
-             : launch_overlapped(quantize_row_kernel<T, false, false, true>, grid, kThreads, 0, s, p);
-}
-}  // namespace
-}  // namespace nvfp4
-
 extern "C" size_t nvfp4_sf_bytes_mx(int64_t Rq, int64_t Kq, int sf_layout) {
   if (Rq <= 0 || Kq <= 0 || (Kq % 32) != 0) return 0;
   if (sf_layout == NVFP4_SF_LINEAR) return (size_t)(Rq * (Kq / 32));
@@ -582,7 +569,7 @@ extern "C" int nvfp4_quantize_mx(const void* x, int dtype, int64_t rows, int64_t
   if (!x || !rounding || !codes || !scales) return NVFP4_ERR_NULL;
   if (dtype != NVFP4_BF16 && dtype != NVFP4_FP32) return NVFP4_ERR_ENUM;
   if (transposed != 0 && transposed != 1) return NVFP4_ERR_ENUM;
-  if (transposed && dtype != NVFP4_BF16) return NVFP4_ERR_ENUM;        // the transposed path goes through the bf16 transpose
+  if (transposed && dtype != NVFP4_BF16) return NVFP4_ERR_ENUM;        // the tile kernel's transposed MXFP4 form
   if ((rounding->mode != NVFP4_RTN && rounding->mode != NVFP4_SR) || rounding->reserved != 0) return NVFP4_ERR_ENUM;
   if (sf_layout != NVFP4_SF_LINEAR && sf_layout != NVFP4_SF_SWIZZLED_128x4) return NVFP4_ERR_ENUM;
   if (rows <= 0 || cols <= 0 || ld < cols || cols % 8 != 0) return NVFP4_ERR_SHAPE;
@@ -590,9 +577,8 @@ extern "C" int nvfp4_quantize_mx(const void* x, int dtype, int64_t rows, int64_t
   if (Kq % 32 != 0 || rows >= (int64_t)1 << 31 || cols >= (int64_t)1 << 31) return NVFP4_ERR_SHAPE;
   if (!aligned16(x) || !aligned16(codes) || !aligned16(scales) || (ld % 8) != 0) return NVFP4_ERR_ALIGN;
   if (ceil_div(Rq, 128) > 65535) return NVFP4_ERR_SHAPE;
-  // bf16 tensors whose row count is a multiple of 32 (always true here: Kq = rows) go through the tile kernel, which
-  // quantizes along the rows straight from the source; the transpose pass remains for what that kernel does not take
-  const bool tile_path = transposed && rows % 32 == 0 && tile_quantizer_eligible(dtype, rows, cols, false, /*mx=*/true);
+  // Kq = rows is a multiple of 32: the tile kernel takes every transposed tensor but the longest, and those are refused
+  const bool tile_path = transposed && tile_quantizer_eligible(dtype, rows, cols, false, /*mx=*/true);
   if (transposed && !tile_path &&
       (!workspace || workspace_bytes < (size_t)rows * cols * 2 || (reinterpret_cast<uintptr_t>(workspace) & 15u)))
     return NVFP4_ERR_WORKSPACE;
@@ -603,22 +589,16 @@ extern "C" int nvfp4_quantize_mx(const void* x, int dtype, int64_t rows, int64_t
                          /*mx_t=*/true);
   if (!transposed && tile_row_quantizer_eligible(dtype, rows, cols, rounding->mode == NVFP4_SR, /*mx=*/true))
     return tile_quantize_row(x, dtype, rows, cols, ld, global_scale, rounding, codes, scales, sf_layout, s, /*mx=*/true);
-  if (dtype != NVFP4_BF16) return NVFP4_ERR_SHAPE;            // 2^31 tiles of fp32: beyond any memory
-  const void* src = x;
-  int64_t src_ld = ld;
-  if (transposed) {
-    // Q(x^T) is by definition the row quantization of the materialised transpose
-    if (int st = nvfp4_transpose_bf16(x, rows, cols, ld, workspace, cuda_stream)) return st;
-    src = workspace;
-    src_ld = rows;
-  }
+  // what is left: large bf16 tensors rounded to nearest, and tensors of 2^31 tiles, beyond any memory
+  if (transposed || dtype != NVFP4_BF16 || rounding->mode != NVFP4_RTN) return NVFP4_ERR_SHAPE;
   QuantParams p;
-  p.x = src; p.rows = Rq; p.cols = Kq; p.ld = src_ld; p.gptr = global_scale;
+  p.x = x; p.rows = rows; p.cols = cols; p.ld = ld; p.gptr = global_scale;
   philox_stream_init(&p.rng, rounding->seed, rounding->offset);
   p.codes = codes; p.scales = scales;
-  p.nkb = Kq / 16; p.nsb = Kq / 32; p.k_tiles = ceil_div(p.nsb, 4);
-  const bool sr = rounding->mode == NVFP4_SR, swz = sf_layout == NVFP4_SF_SWIZZLED_128x4;
-  return launch_row_mx(p, sr, swz, s) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  p.nkb = cols / 16; p.nsb = cols / 32; p.k_tiles = ceil_div(p.nsb, 4);
+  using T = __nv_bfloat16;
+  const cudaError_t e = sf_layout == NVFP4_SF_SWIZZLED_128x4 ? launch_row<T, false, true, true>(p, s) : launch_row<T, false, false, true>(p, s);
+  return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
 extern "C" int nvfp4_quantize_dual(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld,
