@@ -972,12 +972,8 @@ int launch_gemm2(const uint8_t* a_codes, const uint8_t* b_codes, const GemmParam
   const int tiles = p.tiles_m * p.tiles_n;
   const int max_pairs = sm_count() / 2;
   const int pairs = tiles < max_pairs ? tiles : max_pairs;
-  // Overlapping the launch saves two to three microseconds, which long products do not notice; and after a quantizer the
-  // longest one was slower for it (11008 x 4096 x 65536, 5.9e12 operations, with its quantizers: 2180 us without, 2262
-  // with; 1.5e12 operations: +-0.4 %; 5.5e11 in bf16: 2 % faster with).  The line lies between.
-  const bool overlap = 2.0 * g.M * g.N * (double)g.K < 1e12;
-  return launch_overlapped_if(overlap, gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN>, 2 * pairs, kGemm2Threads, C::kSmemBytes, s,
-                              map_a, map_b, map_sfa, map_sfb, map_d, p) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  return launch_overlapped(gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN>, 2 * pairs, kGemm2Threads, C::kSmemBytes, s,
+                           map_a, map_b, map_sfa, map_sfb, map_d, p) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
 template <int BN>
