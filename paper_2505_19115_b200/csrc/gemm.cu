@@ -488,7 +488,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   if (!p.late) grid_dependency_wait();              // all of the above overlaps the kernel before this one
-  grid_dependency_trigger();
+  grid_dependency_trigger();                        // a late product has not waited yet: the kernel behind it is never late
   if constexpr (Q_OUT) {
     build_inv_table(inv_table, load_scale(p.out_g));
     __syncthreads();
