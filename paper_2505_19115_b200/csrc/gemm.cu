@@ -711,6 +711,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     // 4096 with fp32 output: 366 -> 313 us, input gradient of the same layer 293 -> 259; chained bf16 layers 190 -> 182).
     const int quarter = warp & 3, half = (warp >> 2) & 1;
     const float alpha = load_scale(p.a_g) * load_scale(p.b_g);
+    [[maybe_unused]] const float cq = Q_OUT ? __fdiv_rn(__fdiv_rn(1.0f, 6.0f), load_scale(p.out_g)) : 0.0f;
     const uint32_t buf = epi_base + (warp - 8) * C::kEpiWarpBytes;
     constexpr int kChunkCols = BF16_OUT ? 64 : 32;                 // accumulator columns per 128 bytes of output row
     constexpr int kLoads = kChunkCols / 32;
@@ -747,7 +748,6 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 #endif
       if constexpr (Q_OUT) {
         // ---- quantized output: this lane's row, 128 of the tile's 256 columns = 8 blocks of 16 ----
-        const float cq = __fdiv_rn(__fdiv_rn(1.0f, 6.0f), load_scale(p.out_g));
         const int64_t row = (int64_t)row0 + lane;
         const int kb0 = tn * (BN / 16) + half * 8;
         uint32_t sfw[2] = {0u, 0u};                  // 8 scale bytes, four per k-tile
@@ -786,9 +786,9 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
               const int64_t kt = (int64_t)(kb0 >> 2) + t;
+              if (tm * 256 + 256 > p.M || tn * BN + BN > p.N) sfw[t] = scales_inside(sfw[t], row < p.M ? p.out_nkb - kt * 4 : 0);   // padding
               if (kt < p.out_k_tiles)
-                *reinterpret_cast<uint32_t*>(p.out_scales + sf_swizzled_offset(row, kt * 4, p.out_k_tiles)) =
-                    scales_inside(sfw[t], row < p.M ? p.out_nkb - kt * 4 : 0);
+                *reinterpret_cast<uint32_t*>(p.out_scales + sf_swizzled_offset(row, kt * 4, p.out_k_tiles)) = sfw[t];
             }
           }
         } else if (row < p.M) {
