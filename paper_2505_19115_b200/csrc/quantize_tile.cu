@@ -446,8 +446,8 @@ template <typename T, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX = false
 cudaError_t launch_tile(const TileTensors& a, TileParams& p, cudaStream_t s) {
   // 128-row tiles under persistent blocks win while blocks are few or the arithmetic is heavy; on large tensors a block per
   // 256-row tile does, started in order by the hardware where walking blocks drift apart (us, 128-row / 256-row):
-  //   both outputs RtN  16384 x 2816 23.0 / 26.2   x 4096 37.0 / 36.0   x 11008 115 / 91     SR  36.7 / 36.9, 52.1 / 51.0, 136 / 129
-  //   transposed RtN    16384 x 1024 8.7 / 8.6     x 2816 21.1 / 19.9   x 11008 80 / 70      SR  9.9 / 11.0, 22.0 / 24.2, 79 / 84
+  //   both outputs RtN  16384 x 2816 23.5 / 25.5   x 4096 37.5 / 35.5   x 11008 117 / 90     SR  35.0 / 35.6, 50.0 / 49.1, 137 / 130
+  //   transposed RtN    16384 x 1024 7.6 / 8.2     x 2816 19.7 / 19.7   x 11008 74 / 70      SR  9.9 / 11.0, 22.0 / 24.2, 79 / 84
   // fp32 tensors are bound by memory with the 128-row tile (16384 x 4096, both outputs: 6.2-6.4 TB/s).
   constexpr bool can_be_tall = sizeof(T) == 2 && (DUAL || !SR_T);
   if constexpr (can_be_tall)
