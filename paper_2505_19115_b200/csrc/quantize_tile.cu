@@ -126,13 +126,39 @@ __device__ __forceinline__ bool wait_tile(uint32_t bar, uint32_t parity) {
   }
 }
 
+// Padding of scale tiles is zero: every thread goes once more over the words it stored for its block's tiles (the loop of
+// quantize_tile_kernel says which).  Out of line and after the loop, since it is hardly ever called: masking the words on their
+// way out, on edge tiles alone, cost 0.3 us of a 2080-token step's 61.7 and 0.4 of 22.8 for both outputs RtN of 11008 x 4096.
+template <int ROWS, bool TR, bool ROW>
+__device__ __noinline__ void zero_scale_padding(const TileParams& p, int mine) {
+  constexpr int kKtPerTile = ROWS / 64;                   // scale tiles per column
+  for (int tile = p.tiles - 1 - (int)blockIdx.x, k = 0; k < mine; ++k, tile -= (int)gridDim.x) {
+    const int64_t r0 = (int64_t)(tile / p.tiles_x) * ROWS, c0 = (int64_t)(tile % p.tiles_x) * kTileCols;
+    if (TR && threadIdx.x < kTileCols * kKtPerTile) {
+      const int64_t col = c0 + threadIdx.x / kKtPerTile, kt = r0 / 64 + threadIdx.x % kKtPerTile;
+      if (kt < p.t_k_tiles) {
+        uint32_t* const w = reinterpret_cast<uint32_t*>(p.t_scales + sf_swizzled_offset(col, kt * 4, p.t_k_tiles));
+        *w = scales_inside(*w, col < p.cols ? p.t_nsb - kt * 4 : 0);
+      }
+    }
+    if (ROW && threadIdx.x >= 128 && threadIdx.x < 128 + ROWS / 4) {
+      // thread 128 + 32 * h + i: the 16 bytes of rows i, i + 32, i + 64, i + 96 of the tile's half h
+      const int64_t half = r0 + ((threadIdx.x - 128) >> 5) * 128, row = half + (threadIdx.x & 31);
+      if (half < p.rows) {
+        uint32_t* const w = reinterpret_cast<uint32_t*>(p.r_scales + sf_swizzled_offset(row, c0 / 16, p.r_k_tiles));
+        for (int j = 0; j < 4; ++j) w[j] = scales_inside(w[j], row + 32 * j < p.rows ? p.r_nsb - c0 / 16 : 0);
+      }
+    }
+  }
+}
+
 // MX: the output (one of the two) is MXFP4 (Section 3, Table 1): blocks of 32 with an E8M0 scale rounded up to a power
 // of two; the two groups of 16 inside a block keep their own random draws (group index as for NVFP4).
 // TR, ROW: which outputs are written.
 template <typename T, int ROWS, int SLOTS, bool TR, bool SR_T, bool ROW, bool SR_R, bool SWZ, bool MX>
 __global__ void __launch_bounds__(kThreads, TileSmem<T, ROWS, TR, ROW, SLOTS>::kBlocksPerSm)
 quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_ct,
-                     const __grid_constant__ CUtensorMap map_cr, const TileParams p) {
+                     const __grid_constant__ CUtensorMap map_cr, const __grid_constant__ TileParams p) {
   using S = TileSmem<T, ROWS, TR, ROW, SLOTS>;
   static_assert(ROWS == 128 || ROWS == 256, "a staged output row is one swizzle span");
   static_assert((TR || ROW) && !(MX && TR && (ROW || sizeof(T) != 2)), "MXFP4: one output, the transposed one of bf16 tensors only");
@@ -343,8 +369,6 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     constexpr int kKtPerTile = kSbPerTile / 4;            // scale tiles per column
     const int kb0 = r0 / kSbRows;
     if constexpr (SWZ) {
-      // a tile that reaches past the tensor also holds padding (rows and columns are below 2^31)
-      [[maybe_unused]] const bool edge = (uint32_t)c0 + kTileCols > (uint32_t)p.cols || (uint32_t)r0 + ROWS > (uint32_t)p.rows;
       // transposed scales: one 32-bit word = four row blocks of one column
       static_assert(kTileCols * kKtPerTile <= kThreads, "one word per thread");
       if (TR && threadIdx.x < kTileCols * kKtPerTile) {
@@ -353,9 +377,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
         if (kt0 + q < p.t_k_tiles) {
           uint8_t* dst = p.t_scales + ((int64_t)(c0 >> 7) * p.t_k_tiles + kt0) * 512 + ((c0 & 64) >> 3) +
                          (q * 512 + (cl & 31) * 16 + (cl >> 5) * 4);
-          uint32_t val = *reinterpret_cast<const uint32_t*>(sf_t + q * (4 * kTileCols) + cl * 4);
-          if (edge) val = scales_inside(val, c0 + cl < p.cols ? p.t_nsb - 4 * (kt0 + q) : 0);
-          *reinterpret_cast<uint32_t*>(dst) = val;
+          *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(sf_t + q * (4 * kTileCols) + cl * 4);
           if (((c0 & 127) == 0) && ((int64_t)c0 + kTileCols >= p.cols))        // nobody else owns rows 64..127 of the scale tile
             *reinterpret_cast<uint32_t*>(dst + 8) = 0u;
         }
@@ -374,17 +396,9 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
       } else if constexpr (ROW) {
         // row scales: the tile owns whole 512-byte scale tiles (128 rows x this k-tile)
         const int h = (threadIdx.x >> 5) - 4, i = threadIdx.x & 31;   // from the fifth warp on
-        if (h >= 0 && h < ROWS / 128 && (int64_t)r0 + h * 128 < p.rows) {
-          uint4 val = *reinterpret_cast<const uint4*>(sf_r + h * 512 + i * 16);   // rows i, i + 32, i + 64, i + 96
-          if (edge) {
-            const int64_t rows_left = p.rows - (r0 + h * 128 + i), left = p.r_nsb - c0 / 16;
-            val.x = scales_inside(val.x, rows_left > 0 ? left : 0);
-            val.y = scales_inside(val.y, rows_left > 32 ? left : 0);
-            val.z = scales_inside(val.z, rows_left > 64 ? left : 0);
-            val.w = scales_inside(val.w, rows_left > 96 ? left : 0);
-          }
-          *reinterpret_cast<uint4*>(p.r_scales + ((int64_t)(r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) = val;
-        }
+        if (h >= 0 && h < ROWS / 128 && (int64_t)r0 + h * 128 < p.rows)
+          *reinterpret_cast<uint4*>(p.r_scales + ((int64_t)(r0 / 128 + h) * p.r_k_tiles + c0 / 64) * 512 + i * 16) =
+              *reinterpret_cast<const uint4*>(sf_r + h * 512 + i * 16);
       }
     } else if constexpr (TR) {
       for (int id = threadIdx.x; id < kTileCols * kSbPerTile; id += kThreads) {
@@ -394,6 +408,10 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
     }
     if constexpr (SLOTS == 2) step_back(tx, ty);
   }
+  // The zeros beyond the tensor encode to zero scales by themselves unless the per-tensor scale is NaN, zero or subnormal (c is
+  // then NaN, or may be infinite).  Asked of g: asked of c, 2080 x 1056 took 2.57 us instead of 2.40 in every form.
+  if constexpr (SWZ && !MX)
+    if (!(g >= 0x1p-126f)) zero_scale_padding<ROWS, TR, ROW>(p, mine);
   if (threadIdx.x == kLoader) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // staging must outlive the stores' reads
 }
 
