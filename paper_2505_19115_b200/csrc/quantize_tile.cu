@@ -464,8 +464,8 @@ template <typename T, bool SR_T, bool DUAL, bool SR_R, bool SWZ, bool MX = false
 cudaError_t launch_tile(const TileTensors& a, TileParams& p, cudaStream_t s) {
   // 128-row tiles under persistent blocks win while blocks are few or the arithmetic is heavy; on large tensors a block per
   // 256-row tile does, started in order by the hardware where walking blocks drift apart (us, 128-row / 256-row):
-  //   both outputs RtN  16384 x 2816 23.5 / 25.5   x 4096 37.5 / 35.5   x 11008 117 / 90     SR  35.0 / 35.6, 50.0 / 49.1, 137 / 130
-  //   transposed RtN    16384 x 1024 7.6 / 8.2     x 2816 19.7 / 19.7   x 11008 74 / 70      SR  9.9 / 11.0, 22.0 / 24.2, 79 / 84
+  //   both outputs RtN  16384 x 2816 22.9 / 25.6   x 4096 37.5 / 35.6   x 11008 115 / 90     SR  35.4 / 35.2, 50.2 / 48.7, 135 / 128
+  //   transposed RtN    16384 x 1024 7.5 / 8.2     x 2816 19.7 / 19.7   x 11008 73 / 70      SR  9.9 / 11.0, 22.0 / 24.2, 79 / 84
   // fp32 tensors are bound by memory with the 128-row tile (16384 x 4096, both outputs: 6.2-6.4 TB/s).
   constexpr bool can_be_tall = sizeof(T) == 2 && (DUAL || !SR_T);
   if constexpr (can_be_tall)
