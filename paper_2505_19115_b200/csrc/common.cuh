@@ -39,12 +39,9 @@ inline cudaError_t set_max_dynamic_smem(DeviceFlags& flags, Kernel kernel, int b
 // before.  The rules every kernel launched this way keeps:
 //   * it calls grid_dependency_wait() in every block, before its first access to memory that an earlier kernel may
 //     still read or write; when that returns, the kernel before it has finished and its writes are visible;
-//   * it calls grid_dependency_trigger() only after that wait, the late product excepted.  A kernel that follows it directly
-//     therefore starts when everything TWO launches back is finished, and may read that without waiting ("late" kernels), as
-//     long as it still waits before it ends, so that "finished" keeps meaning "and all before it";
-//   * a late product (gemm_checked) triggers at its start, before its wait: what follows it may start while the product before
-//     it still runs.  It is the last kernel of a layer call, and the first kernel of every call waits first: late kernels
-//     stand only behind a kernel of the same call that has waited.
+//   * it calls grid_dependency_trigger() only after that wait.  A kernel that follows it directly therefore starts when
+//     everything TWO launches back is finished, and may read that without waiting ("late" kernels), as long as it still waits
+//     before it ends, so that "finished" keeps meaning "and all before it".
 // After anything else on the stream (a kernel that does not take part, a copy) the attribute changes nothing.
 // One step of a 256-token layer (11 kernels of 3.5-8 us): 61.3 -> 47.5 us; of a 2080 x 1056 x 2848 one: 85.9 -> 68.6.
 // Long products neither gain nor lose (11008 x 4096 x 65536 alone 1326 us launched the ordinary way / 1290 this way, behind its
@@ -75,11 +72,23 @@ __device__ __forceinline__ float load_scale(const float* g) {
 // Zeroes up to 32 words (quantize.cu), overlapping the kernel before it.
 cudaError_t zero_words(unsigned int* words, int n, cudaStream_t s);
 
-// nvfp4_gemm for a caller inside the library (gemm.cu).  late: the product before this one on the stream is independent
-// of it and everything else it reads was finished before that one began, so its tiles may fill that one's last wave.  Only for
-// the last kernel of a call: the kernel behind a late product must not be late itself (see the rules above).
-int gemm_checked(const uint8_t* a_codes, const uint8_t* a_sf, const float* a_g, const uint8_t* b_codes, const uint8_t* b_sf,
-                 const float* b_g, int64_t M, int64_t N, int64_t K, void* d, int d_dtype, int64_t ldd, void* cuda_stream, bool late);
+// A product: the arguments of nvfp4_gemm.
+struct GemmCall {
+  const uint8_t* a_codes;
+  const uint8_t* a_sf;
+  const float* a_g;
+  const uint8_t* b_codes;
+  const uint8_t* b_sf;
+  const float* b_g;
+  int64_t M, N, K;
+  void* d;
+  int d_dtype;
+  int64_t ldd;
+};
+// Two products that do not depend on one another, in one launch; and the two of nvfp4_linear_bwd_bf16 (gemm.cu).
+int gemm_two(const GemmCall& x, const GemmCall& y, void* cuda_stream);
+int gemm_bf16_gradients(const void* dY, const void* W, const void* X, int64_t M, int64_t N, int64_t K, void* dX, int dx_dtype,
+                        void* dW, int dw_dtype, void* cuda_stream);
 
 // Tile quantizer (quantize_tile.cu): transposed output, optionally the row output from the same read.
 bool tile_quantizer_eligible(int dtype, int64_t rows, int64_t cols, bool dual, bool mx = false);

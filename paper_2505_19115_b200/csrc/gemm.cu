@@ -16,6 +16,9 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "quantize_core.cuh"
 #include "tc_ptx.cuh"
 #include "tensor_map.cuh"
@@ -80,7 +83,6 @@ struct GemmParams {
   int k_mmas;                       // instructions along K
   int a_row_tiles, b_row_tiles;     // ceil(M / 128), ceil(N / 128)
   int d_is_bf16;
-  int late = 0;
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -406,19 +408,57 @@ struct Cfg2 {
   static_assert(8 * kNumBarriers + 8 <= 512, "barrier area overflow");
 };
 
-struct Gemm2Params {
+struct Gemm2Maps {
+  CUtensorMap a, b, sfa, sfb, d;
+};
+struct Gemm2Product {
   const float* a_g;
   const float* b_g;
-  int M, N, K;
+  int M, N;
   int tiles_m, tiles_n, k_stages, k_tiles;
   int k_mmas;                       // instructions along K (64 values each; 16 for bf16 operands)
   int a_row_tiles, b_row_tiles;
+  int d_is_bf16, a_mn;              // launches of two products: the output's type; operand A (bf16) is [K, M] (template MN otherwise)
+};
+
+// Which tiles a pair of CTAs computes, and in which order.  One product: tile `pair`, `pair + pairs`, ...  Two products (the
+// input and the weight gradient of a layer, which do not depend on one another): the tiles of the first, whose contraction is
+// the longer one, come first.  n0 = q * pairs + r of them leave pairs - r pairs without one of the last r; those take `head`
+// tiles of the second product each meanwhile, and the others of it are dealt out to all pairs, beginning with those.
+struct TileOrder {
+  int q = 0, r = 0, head = 0;
+  int n1;                           // tiles of the second product, or of the only one
+};
+template <bool PAIRED>
+__device__ __forceinline__ bool tile_at(const TileOrder& o, int pair, int pairs, int i, int& product, int& tile) {
+  product = 0;
+  if constexpr (!PAIRED) {
+    tile = pair + i * pairs;
+  } else {
+    const int rest = pairs - o.r, first = o.q + (pair < o.r);
+    if (i < first) {
+      tile = pair + i * pairs;
+      return true;
+    }
+    product = 1;
+    i -= first;
+    const int rank = pair < o.r ? rest + pair : pair - o.r;
+    if (pair >= o.r && i < o.head) tile = rank + i * rest;
+    else tile = o.head * rest + rank + (i - (pair >= o.r ? o.head : 0)) * pairs;
+  }
+  return tile < o.n1;
+}
+
+template <int PRODUCTS>
+struct Gemm2Params {
+  Gemm2Maps maps[PRODUCTS];
+  Gemm2Product product[PRODUCTS];
+  TileOrder order;
   // quantized output (OUT == 2): per-tensor scale of the output, rounding, scales destination
   const float* out_g;
   PhiloxStream out_rng;
   uint8_t* out_scales;
   int out_sr, out_swizzled;
-  int late;                         // wait for the kernel before this one at the end instead of at the start
   int64_t out_nkb, out_k_tiles;
 };
 
@@ -434,15 +474,16 @@ struct Gemm2Params {
 // row-major, instead of [M, K] / [N, K] (the backward and update products of Eq. 2-3 read W, X and dY that way): a
 // stage then holds, per operand, two boxes of 64 contraction rows x 64 output rows (128 bytes), and the MMA reads
 // them through MN-major descriptors, so no transposed copy of the tensor is ever made.
-template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0>
+// PAIRED: the launch computes two products (TileOrder); their output types, and for bf16 operands (both products of the
+// backward pass have an MN-major B) whether A is MN-major, then come from the parameters, OUT and MN bit 0 being unused.
+template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0, bool PAIRED = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemm2Threads, 1)
-gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                   const __grid_constant__ CUtensorMap map_sfa, const __grid_constant__ CUtensorMap map_sfb,
-                   const __grid_constant__ CUtensorMap map_d, const Gemm2Params p) {
+gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
   using C = Cfg2<BN>;
-  constexpr bool BF16_OUT = (OUT == 1), Q_OUT = (OUT == 2);
-  constexpr bool MN_A = (MN & 1) != 0, MN_B = (MN & 2) != 0;
+  constexpr bool Q_OUT = (OUT == 2);
+  constexpr bool MN_B = (MN & 2) != 0;
   static_assert(MN == 0 || (BF16_IN && BN == 256), "MN-major operands exist for the bf16 variant with the 256-wide tile");
+  static_assert(!PAIRED || (!Q_OUT && !MX && BN % 128 == 0), "two products: the gradients of a layer");
   static_assert(!Q_OUT || BN == 256, "the quantized epilogue stores two 64-byte pieces of codes per tile row");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -469,7 +510,6 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
   const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
-  const int num_tiles = p.tiles_m * p.tiles_n;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(sfl_bar(s), 1); mbar_init(empty_bar(s), 1); mbar_init(sfx_bar(s), 4); }
@@ -478,8 +518,10 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     *abort_flag = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
-    prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_d);
-    if constexpr (!BF16_IN) { prefetch_map(&map_sfa); prefetch_map(&map_sfb); }
+    for (const Gemm2Maps& m : p.maps) {
+      prefetch_map(&m.a); prefetch_map(&m.b); prefetch_map(&m.d);
+      if constexpr (!BF16_IN) { prefetch_map(&m.sfa); prefetch_map(&m.sfb); }
+    }
   }
   if (warp == 1) tmem_alloc_pair(smem_u32((const void*)tmem_slot), kTmemCols);
   tc_fence_before();
@@ -487,8 +529,8 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
   cluster_sync_all();                               // both CTAs' barriers exist before any remote signal
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (!p.late) grid_dependency_wait();              // all of the above overlaps the kernel before this one
-  grid_dependency_trigger();                        // a late product has not waited yet: the kernel behind it is never late
+  grid_dependency_wait();                           // all of the above overlaps the kernel before this one
+  grid_dependency_trigger();
   if constexpr (Q_OUT) {
     build_inv_table(inv_table, load_scale(p.out_g));
     __syncthreads();
@@ -507,11 +549,14 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     bool ok = true;
     constexpr uint32_t kOperandTx = C::kABytes + C::kBBytes;       // per CTA, signalled on the leader's barrier
     ACCOUNT_VARS(a_wait = 0, a_total = -ACCOUNT_NOW());
-    for (int tile = pair; ok && tile < num_tiles; tile += num_pairs) {
+    for (int i = 0, w, tile; ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
+      const Gemm2Product& q = p.product[w];
+      const Gemm2Maps& m = p.maps[w];
+      const bool a_mn = PAIRED ? BF16_IN && q.a_mn : (MN & 1) != 0;
       int tm, tn;
-      tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
+      tile_coords(tile, q.tiles_m, q.tiles_n, tm, tn);
       const int m0 = tm * 256 + (int)rank * 128, n0 = tn * BN + (int)rank * (BN / 2);
-      for (int ks = 0; ks < p.k_stages; ++ks) {
+      for (int ks = 0; ks < q.k_stages; ++ks) {
         // polled without sleeping: the refill of a freed stage is on the main loop's critical path (the ring is
         // five stages deep for a copy latency of three to four stage times), and a sleeping poll adds its period to it
         ACCOUNT(a_wait, ok = mbar_wait_issuer(empty_bar(s), ph ^ 1u, abort_flag, 0x11));
@@ -520,17 +565,17 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         const uint32_t lead_full = map_to_cta(full_bar(s), 0);
         if (issuer) {
           if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2u * kOperandTx);
-          if constexpr (MN_A) {                     // [K, M]: x = byte offset of the output row, y = contraction index
-            tma_load_2d_pair(st, &map_a, lead_full, m0 * 2, ks * 64);
-            tma_load_2d_pair(st + C::kABytes / 2, &map_a, lead_full, (m0 + 64) * 2, ks * 64);
+          if (a_mn) {                               // [K, M]: x = byte offset of the output row, y = contraction index
+            tma_load_2d_pair(st, &m.a, lead_full, m0 * 2, ks * 64);
+            tma_load_2d_pair(st + C::kABytes / 2, &m.a, lead_full, (m0 + 64) * 2, ks * 64);
           } else {
-            tma_load_2d_pair(st, &map_a, lead_full, ks * BK_BYTES, m0);
+            tma_load_2d_pair(st, &m.a, lead_full, ks * BK_BYTES, m0);
           }
           if constexpr (MN_B) {
-            tma_load_2d_pair(st + C::kABytes, &map_b, lead_full, n0 * 2, ks * 64);
-            tma_load_2d_pair(st + C::kABytes + C::kBBytes / 2, &map_b, lead_full, (n0 + 64) * 2, ks * 64);
+            tma_load_2d_pair(st + C::kABytes, &m.b, lead_full, n0 * 2, ks * 64);
+            tma_load_2d_pair(st + C::kABytes + C::kBBytes / 2, &m.b, lead_full, (n0 + 64) * 2, ks * 64);
           } else {
-            tma_load_2d_pair(st + C::kABytes, &map_b, lead_full, ks * BK_BYTES, n0);
+            tma_load_2d_pair(st + C::kABytes, &m.b, lead_full, ks * BK_BYTES, n0);
           }
         }
         if (++s == C::kStages) { s = 0; ph ^= 1u; }
@@ -550,23 +595,25 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     bool ok = true;
     constexpr int kSfTiles = MX ? 2 : 4;                           // 512-byte scale tiles per stage and 128 rows
     constexpr uint32_t kScaleTx = (C::kSfaBytes + C::kSfbBytes) / 4 * kSfTiles;   // signalled on this CTA's own barrier
-    for (int tile = pair; !BF16_IN && ok && tile < num_tiles; tile += num_pairs) {
+    for (int i = 0, w, tile; !BF16_IN && ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
+      const Gemm2Product& q = p.product[w];
+      const Gemm2Maps& m = p.maps[w];
       int tm, tn;
-      tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
-      const int a_row = min(tm * 2 + (int)rank, p.a_row_tiles - 1) * p.k_tiles;
+      tile_coords(tile, q.tiles_m, q.tiles_n, tm, tn);
+      const int a_row = min(tm * 2 + (int)rank, q.a_row_tiles - 1) * q.k_tiles;
       int b_row[C::kSfbTiles];
 #pragma unroll
       for (int h = 0; h < C::kSfbTiles; ++h)                       // rows past N are never stored
-        b_row[h] = min((tn * BN) / 128 + h, p.b_row_tiles - 1) * p.k_tiles;
-      for (int ks = 0; ks < p.k_stages; ++ks) {
+        b_row[h] = min((tn * BN) / 128 + h, q.b_row_tiles - 1) * q.k_tiles;
+      for (int ks = 0; ks < q.k_stages; ++ks) {
         if (!(ok = mbar_wait_relaxed(sfx_bar(s), ph ^ 1u, abort_flag, 0x18))) break;
         const uint32_t sf = smem_base + s * C::kStageBytes + C::kABytes + C::kBBytes;
         if (issuer) {
           mbar_arrive_expect_tx(sfl_bar(s), kScaleTx);
-          tma_load_2d(sf, &map_sfa, sfl_bar(s), 0, a_row + ks * kSfTiles);
+          tma_load_2d(sf, &m.sfa, sfl_bar(s), 0, a_row + ks * kSfTiles);
 #pragma unroll
           for (int h = 0; h < C::kSfbTiles; ++h)
-            tma_load_2d(sf + C::kSfaBytes + h * 2048, &map_sfb, sfl_bar(s), 0, b_row[h] + ks * kSfTiles);
+            tma_load_2d(sf + C::kSfaBytes + h * 2048, &m.sfb, sfl_bar(s), 0, b_row[h] + ks * kSfTiles);
         }
         if (++s == C::kStages) { s = 0; ph ^= 1u; }
       }
@@ -579,19 +626,21 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     // ------------------------------- MMA issuer (leader CTA only) -------------------------------
     if (rank == 0) {
       const bool issuer = elect_one();
-      constexpr uint32_t idesc = BF16_IN ? instr_desc_bf16(256, BN, MN_A, MN_B) : instr_desc(256, BN);
       int s = 0, b = 0, acc = 0;
       uint32_t ph = 0, bph = 0, acc_ph = 0;
       bool ok = true;
       ACCOUNT_VARS(a_acc = 0, a_ops = 0, a_sf = 0, a_total = -ACCOUNT_NOW());
-      for (int tile = pair; ok && tile < num_tiles; tile += num_pairs) {
+      for (int i = 0, w, tile; ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
+        const Gemm2Product& q = p.product[w];
+        const bool a_mn = PAIRED ? BF16_IN && q.a_mn : (MN & 1) != 0;
+        const uint32_t idesc = !BF16_IN ? instr_desc(256, BN) : a_mn ? instr_desc_bf16(256, BN, true, MN_B) : instr_desc_bf16(256, BN, false, MN_B);
         int tm_unused, tn;
-        tile_coords(tile, p.tiles_m, p.tiles_n, tm_unused, tn);
+        tile_coords(tile, q.tiles_m, q.tiles_n, tm_unused, tn);
         const uint32_t sfb_off = (uint32_t)((tn * BN) % 128) / 32;         // first scale column of this N tile
         ACCOUNT(a_acc, ok = mbar_wait_issuer(tempty_bar(acc), acc_ph ^ 1u, abort_flag, 0x12));
         if (!ok) break;
         const uint32_t d_tmem = tmem_base + acc * BN;
-        for (int ks = 0; ks < p.k_stages; ++ks) {
+        for (int ks = 0; ks < q.k_stages; ++ks) {
           ACCOUNT(a_ops, ok = mbar_wait_issuer(full_bar(s), ph, abort_flag, 0x13));
           if (!ok) break;
           if constexpr (!BF16_IN) {
@@ -600,14 +649,15 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
           }
           tc_fence_after();
           const uint32_t st = smem_base + s * C::kStageBytes;
-          const int nkt = min(4, p.k_mmas - ks * 4);
+          const int nkt = min(4, q.k_mmas - ks * 4);
           const uint32_t sfa_t = tmem_base + C::kSfaCol + b * C::kSfCols;
           const uint32_t sfb_t = sfa_t + 16 + sfb_off;
-          const uint64_t adesc = MN_A ? operand_desc_mn(st, C::kABytes / 2) : operand_desc(st);
+          const uint64_t adesc = a_mn ? operand_desc_mn(st, C::kABytes / 2) : operand_desc(st);
           const uint64_t bdesc = MN_B ? operand_desc_mn(st + C::kABytes, C::kBBytes / 2) : operand_desc(st + C::kABytes);
           if (issuer && BF16_IN) {
             // one instruction = 16 contraction indices: 32 bytes along a K-major row, 16 rows (2048 bytes) of an MN-major box
-            constexpr uint32_t a_step = MN_A ? (2048u >> 4) : 2u, b_step = MN_B ? (2048u >> 4) : 2u;
+            const uint32_t a_step = a_mn ? (2048u >> 4) : 2u;
+            constexpr uint32_t b_step = MN_B ? (2048u >> 4) : 2u;
             for (int j = 0; j < nkt; ++j) tc_mma_bf16_pair(d_tmem, adesc + a_step * j, bdesc + b_step * j, idesc, (ks | j) ? 1u : 0u);
             tc_commit_pair(empty_bar(s));
           } else if (issuer && MX) {
@@ -653,8 +703,9 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     uint32_t ph = 0, bph = 0;
     bool ok = true;
     ACCOUNT_VARS(a_land = 0, a_free = 0, a_total = -ACCOUNT_NOW());
-    for (int tile = pair; !BF16_IN && ok && tile < num_tiles; tile += num_pairs) {
-      for (int ks = 0; ks < p.k_stages; ++ks) {
+    for (int i = 0, w, tile; !BF16_IN && ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
+      const int k_stages = p.product[w].k_stages;
+      for (int ks = 0; ks < k_stages; ++ks) {
         ACCOUNT(a_land, ok = mbar_wait_warp_relaxed(sfl_bar(s), ph, abort_flag, 0x16));
         if (!ok) break;
         if constexpr (!C::kSfFollowsStage) {
@@ -710,21 +761,22 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     // Against four warps that held 3 of 8 chunks and streamed the others through their staging buffers (16384 x 11008 x
     // 4096 with fp32 output: 366 -> 313 us, input gradient of the same layer 293 -> 259; chained bf16 layers 190 -> 182).
     const int quarter = warp & 3, half = (warp >> 2) & 1;
-    const float alpha = load_scale(p.a_g) * load_scale(p.b_g);
+    float alphas[PAIRED ? 2 : 1];
+    for (int w = 0; w < (PAIRED ? 2 : 1); ++w) alphas[w] = load_scale(p.product[w].a_g) * load_scale(p.product[w].b_g);
     [[maybe_unused]] const float cq = Q_OUT ? __fdiv_rn(__fdiv_rn(1.0f, 6.0f), load_scale(p.out_g)) : 0.0f;
     const uint32_t buf = epi_base + (warp - 8) * C::kEpiWarpBytes;
-    constexpr int kChunkCols = BF16_OUT ? 64 : 32;                 // accumulator columns per 128 bytes of output row
-    constexpr int kLoads = kChunkCols / 32;
-    constexpr int kChunks = Q_OUT ? BN / 32 : BN / kChunkCols;
-    constexpr int kHeld = (kChunks + 1) / 2;                       // chunks of this warp: [half * kHeld, +kHeld) below kChunks
+    constexpr int kWarpCols = OUT == 1 ? (BN + 127) / 128 * 64 : BN / 2;   // columns of the first half's warps: whole chunks of 128 bytes
+    constexpr int kLoads = kWarpCols / 32;
     const uint32_t lead_tempty0 = map_to_cta(tempty_bar(0), 0);
     int acc = 0;
     uint32_t acc_ph = 0;
     bool ok = true;
     ACCOUNT_VARS(a_tile = 0, a_read = 0, a_total = -ACCOUNT_NOW(), a_read_t0 = 0);
-    for (int tile = pair; ok && tile < num_tiles; tile += num_pairs) {
+    for (int i = 0, w, tile; ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
+      const Gemm2Product& q = p.product[w];
+      const float alpha = PAIRED && w ? alphas[PAIRED] : alphas[0];
       int tm, tn;
-      tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
+      tile_coords(tile, q.tiles_m, q.tiles_n, tm, tn);
       ACCOUNT(a_tile, ok = mbar_wait_warp(tfull_bar(acc), acc_ph, abort_flag, 0x14));
       if (!ok) break;
 #ifdef NVFP4_GEMM_ACCOUNT
@@ -732,14 +784,14 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 #endif
       tc_fence_after();
       const int row0 = tm * 256 + (int)rank * 128 + quarter * 32;
-      const uint32_t t_row = tmem_base + acc * BN + half * (kHeld * kChunkCols) + ((uint32_t)(quarter * 32) << 16);
-      uint32_t r[kHeld * kLoads][32];
+      const uint32_t t_row = tmem_base + acc * BN + half * kWarpCols + ((uint32_t)(quarter * 32) << 16);
+      uint32_t r[kLoads][32];
 #pragma unroll
-      for (int l = 0; l < kHeld * kLoads; ++l)
-        if (half * kHeld + l / kLoads < kChunks) tmem_ld32(t_row + 32 * l, r[l]);
+      for (int l = 0; l < kLoads; ++l)
+        if (half * kWarpCols + 32 * l < BN) tmem_ld32(t_row + 32 * l, r[l]);
       tmem_ld_wait();
 #pragma unroll
-      for (int l = 0; l < kHeld * kLoads; ++l) tmem_ld_pin(r[l]);
+      for (int l = 0; l < kLoads; ++l) tmem_ld_pin(r[l]);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8u * acc);  // accumulator fully read: hand it back to the leader
@@ -777,61 +829,69 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         fence_async_smem();
         __syncwarp();
         if (lane == 0) {
-          tma_store_2d(&map_d, buf, tn * (BN / 2) + half * 64, row0);
+          tma_store_2d(&p.maps[0].d, buf, tn * (BN / 2) + half * 64, row0);
           tma_store_commit();
         }
         // scales
         if (p.out_swizzled) {
-          if ((row >> 7) < (((int64_t)p.M + 127) >> 7)) {
+          if ((row >> 7) < (((int64_t)q.M + 127) >> 7)) {
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
               const int64_t kt = (int64_t)(kb0 >> 2) + t;
-              if (tm * 256 + 256 > p.M || tn * BN + BN > p.N) sfw[t] = scales_inside(sfw[t], row < p.M ? p.out_nkb - kt * 4 : 0);   // padding
+              if (tm * 256 + 256 > q.M || tn * BN + BN > q.N) sfw[t] = scales_inside(sfw[t], row < q.M ? p.out_nkb - kt * 4 : 0);   // padding
               if (kt < p.out_k_tiles)
                 *reinterpret_cast<uint32_t*>(p.out_scales + sf_swizzled_offset(row, kt * 4, p.out_k_tiles)) = sfw[t];
             }
           }
-        } else if (row < p.M) {
+        } else if (row < q.M) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int64_t kb = (int64_t)kb0 + i;
-            if (kb < p.out_nkb) p.out_scales[row * p.out_nkb + kb] = (uint8_t)(sfw[i >> 2] >> (8 * (i & 3)));
+          for (int j = 0; j < 8; ++j) {
+            const int64_t kb = (int64_t)kb0 + j;
+            if (kb < p.out_nkb) p.out_scales[row * p.out_nkb + kb] = (uint8_t)(sfw[j >> 2] >> (8 * (j & 3)));
           }
         }
       } else {
         // one chunk at a time: 32 rows x 128 bytes (row = lane, eight 16-byte pieces, piece index XOR (row & 7): the
         // 128-byte swizzle), sent off as one tiled store
+        const CUtensorMap* map_d = &p.maps[w].d;
+        auto store_chunks = [&](auto bf16) {
+          constexpr bool BF16_OUT = decltype(bf16)::value;
+          constexpr int kChunkCols = BF16_OUT ? 64 : 32;           // accumulator columns per 128 bytes of output row
+          static_assert(kWarpCols % kChunkCols == 0, "a warp stores whole chunks");
 #pragma unroll
-        for (int i = 0; i < kHeld; ++i) {
-          const int c = half * kHeld + i;
-          if (c >= kChunks) break;
-          uint32_t w[32];
-          if constexpr (BF16_OUT) {
+          for (int c = 0; c < kWarpCols; c += kChunkCols) {
+            if (half * kWarpCols + c >= BN) break;
+            uint32_t v[32];
+            if constexpr (BF16_OUT) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              const uint32_t* q = r[i * kLoads + e / 16] + 2 * (e % 16);
-              const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(q[0]) * alpha, __uint_as_float(q[1]) * alpha);
-              w[e] = *reinterpret_cast<const uint32_t*>(&h2);
+              for (int e = 0; e < 32; ++e) {
+                const uint32_t* x = r[(c + 2 * e) / 32] + (2 * e) % 32;
+                const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(x[0]) * alpha, __uint_as_float(x[1]) * alpha);
+                v[e] = *reinterpret_cast<const uint32_t*>(&h2);
+              }
+            } else {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(r[c / 32][e]) * alpha);
             }
-          } else {
+            if (lane == 0) tma_store_wait_read<0>();  // the chunk stored before this one has left the buffer
+            __syncwarp();
 #pragma unroll
-            for (int e = 0; e < 32; ++e) w[e] = __float_as_uint(__uint_as_float(r[i][e]) * alpha);
+            for (int e = 0; e < 8; ++e) {
+              const uint32_t dst = buf + lane * 128 + ((e ^ (lane & 7)) << 4);
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v[4 * e]), "r"(v[4 * e + 1]),
+                           "r"(v[4 * e + 2]), "r"(v[4 * e + 3]) : "memory");
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              tma_store_2d(map_d, buf, tn * BN + half * kWarpCols + c, row0);
+              tma_store_commit();
+            }
           }
-          if (lane == 0) tma_store_wait_read<0>();  // the chunk stored before this one has left the buffer
-          __syncwarp();
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const uint32_t dst = buf + lane * 128 + ((e ^ (lane & 7)) << 4);
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[4 * e]), "r"(w[4 * e + 1]),
-                         "r"(w[4 * e + 2]), "r"(w[4 * e + 3]) : "memory");
-          }
-          fence_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            tma_store_2d(&map_d, buf, tn * BN + c * kChunkCols, row0);
-            tma_store_commit();
-          }
-        }
+        };
+        if constexpr (!PAIRED) store_chunks(std::bool_constant<OUT == 1>{});
+        else if (q.d_is_bf16) store_chunks(std::true_type{});
+        else store_chunks(std::false_type{});
       }
       if (++acc == C::kAccStages) { acc = 0; acc_ph ^= 1u; }
     }
@@ -841,7 +901,6 @@ gemm2_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 8 && lane == 0, 14, a_total + ACCOUNT_NOW());
   }
 
-  if (p.late) grid_dependency_wait();
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                               // the peer's MMAs and loads are done before anyone frees or exits
@@ -931,37 +990,36 @@ bool make_qout_map(CUtensorMap* map, uint8_t* base, int64_t M, int64_t N) {
             CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tensor maps and sizes of one product for the CTA-pair kernel.
+template <int BN, bool BF16_IN, bool MX>
+bool describe_product(const GemmParams& g, const uint8_t* a_codes, const uint8_t* b_codes, int mn, Gemm2Maps* m, Gemm2Product* q) {
+  const int64_t row_bytes = BF16_IN ? (int64_t)g.K * 2 : g.K / 2;       // operand rows as bytes
+  // MN-major bf16 operand: the tensor is [K, rows] with the output axis contiguous; boxes of 64 contraction rows x 128 bytes
+  if (!((mn & 1) ? make_codes_map(&m->a, a_codes, g.K, (int64_t)g.M * 2, 64) : make_codes_map(&m->a, a_codes, g.M, row_bytes, 128)))
+    return false;
+  if (!((mn & 2) ? make_codes_map(&m->b, b_codes, g.K, (int64_t)g.N * 2, 64) : make_codes_map(&m->b, b_codes, g.N, row_bytes, BN / 2)))
+    return false;
+  if constexpr (BF16_IN) {
+    m->sfa = m->a;                                                       // never used by the kernel
+    m->sfb = m->b;
+  } else {
+    if (!make_sf_map(&m->sfa, g.a_sf, (int64_t)g.a_row_tiles * g.k_tiles, MX ? 2 : 4)) return false;
+    if (!make_sf_map(&m->sfb, g.b_sf, (int64_t)g.b_row_tiles * g.k_tiles, MX ? 2 : 4)) return false;
+  }
+  if (g.d && !make_out_map(&m->d, g.d, g.M, g.N, g.ldd, g.d_is_bf16 != 0)) return false;
+  *q = {g.a_g, g.b_g, g.M, g.N, (g.M + 255) / 256, (g.N + BN - 1) / BN, g.k_stages, g.k_tiles, g.k_mmas, g.a_row_tiles, g.b_row_tiles,
+        g.d_is_bf16, mn & 1};
+  return true;
+}
+
 template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0>
 int launch_gemm2(const uint8_t* a_codes, const uint8_t* b_codes, const GemmParams& g, cudaStream_t s,
                  const QuantOut& q = QuantOut()) {
   using C = Cfg2<BN>;
-  CUtensorMap map_a, map_b, map_sfa, map_sfb, map_d;
-  const int64_t row_bytes = BF16_IN ? (int64_t)g.K * 2 : g.K / 2;       // operand rows as bytes
-  // MN-major bf16 operand: the tensor is [K, rows] with the output axis contiguous; boxes of 64 contraction rows x 128 bytes
-  if (!((MN & 1) ? make_codes_map(&map_a, a_codes, g.K, (int64_t)g.M * 2, 64) : make_codes_map(&map_a, a_codes, g.M, row_bytes, 128)))
-    return NVFP4_ERR_CUDA;
-  if (!((MN & 2) ? make_codes_map(&map_b, b_codes, g.K, (int64_t)g.N * 2, 64) : make_codes_map(&map_b, b_codes, g.N, row_bytes, BN / 2)))
-    return NVFP4_ERR_CUDA;
-  if constexpr (BF16_IN) {
-    map_sfa = map_a;                                                     // never used by the kernel
-    map_sfb = map_b;
-  } else {
-    if (!make_sf_map(&map_sfa, g.a_sf, (int64_t)g.a_row_tiles * g.k_tiles, MX ? 2 : 4)) return NVFP4_ERR_CUDA;
-    if (!make_sf_map(&map_sfb, g.b_sf, (int64_t)g.b_row_tiles * g.k_tiles, MX ? 2 : 4)) return NVFP4_ERR_CUDA;
-  }
-  if constexpr (OUT == 2) {
-    if (!make_qout_map(&map_d, q.codes, g.M, g.N)) return NVFP4_ERR_CUDA;
-  } else {
-    if (!make_out_map(&map_d, g.d, g.M, g.N, g.ldd, OUT == 1)) return NVFP4_ERR_CUDA;
-  }
-  Gemm2Params p;
-  p.a_g = g.a_g; p.b_g = g.b_g; p.M = g.M; p.N = g.N; p.K = g.K;
-  p.tiles_m = (g.M + 255) / 256;
-  p.tiles_n = (g.N + BN - 1) / BN;
-  p.k_stages = g.k_stages; p.k_tiles = g.k_tiles;
-  p.k_mmas = g.k_mmas;
-  p.a_row_tiles = g.a_row_tiles; p.b_row_tiles = g.b_row_tiles;
-  p.late = g.late;
+  Gemm2Params<1> p;
+  if (!describe_product<BN, BF16_IN, MX>(g, a_codes, b_codes, MN, &p.maps[0], &p.product[0])) return NVFP4_ERR_CUDA;
+  if constexpr (OUT == 2)
+    if (!make_qout_map(&p.maps[0].d, q.codes, g.M, g.N)) return NVFP4_ERR_CUDA;
   p.out_g = q.g; p.out_scales = q.scales; p.out_sr = 0; p.out_swizzled = q.sf_layout == NVFP4_SF_SWIZZLED_128x4;
   p.out_nkb = g.N / 16; p.out_k_tiles = ceil_div(p.out_nkb, 4);
   philox_stream_init(&p.out_rng, q.rounding ? q.rounding->seed : 0, q.rounding ? q.rounding->offset : 0);
@@ -969,11 +1027,48 @@ int launch_gemm2(const uint8_t* a_codes, const uint8_t* b_codes, const GemmParam
   static DeviceFlags smem_set;                         // per instantiation, per device
   if (set_max_dynamic_smem(smem_set, gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN>, C::kSmemBytes) != cudaSuccess)
     return NVFP4_ERR_CUDA;
-  const int tiles = p.tiles_m * p.tiles_n;
+  p.order.n1 = p.product[0].tiles_m * p.product[0].tiles_n;
   const int max_pairs = sm_count() / 2;
-  const int pairs = tiles < max_pairs ? tiles : max_pairs;
-  return launch_overlapped(gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN>, 2 * pairs, kGemm2Threads, C::kSmemBytes, s,
-                           map_a, map_b, map_sfa, map_sfb, map_d, p) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  const int pairs = p.order.n1 < max_pairs ? p.order.n1 : max_pairs;
+  return launch_overlapped(gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN>, 2 * pairs, kGemm2Threads, C::kSmemBytes, s, p) == cudaSuccess
+             ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
+
+// What a tile of the pair kernel takes, in cycles of a CTA pair: its k-stages and the turn-round of the accumulator, or sending
+// its output off, which takes longer below ten stages (1024-value contractions: 4100-4400 cycles a tile with bf16 output,
+// 5900 with fp32).
+int64_t tile_cycles(int bn, const GemmParams& p) {
+  const int64_t loop = bn == 128 ? 330 * (int64_t)p.k_stages + 200 : 590 * (int64_t)p.k_stages + 900;
+  return std::max<int64_t>(loop, (p.d_is_bf16 ? 4000 : 5600) * bn / 256);
+}
+
+// Order of two products' tiles over `pairs` pairs (c0, c1: cycles of a tile), and the cycles until the last is done.
+int64_t order_tiles(int64_t n0, int64_t c0, int64_t n1, int64_t c1, int64_t pairs, TileOrder* o) {
+  const int64_t q = n0 / pairs, r = n0 % pairs, rest = pairs - r;
+  const int64_t head = r ? std::min(c0 / c1, n1 / rest) : 0;
+  const int64_t left = n1 - head * rest, waves = left / pairs, rem = left % pairs;
+  o->q = (int)q; o->r = (int)r; o->head = (int)head; o->n1 = (int)n1;
+  const int64_t ahead = q * c0 + head * c1, behind = r ? (q + 1) * c0 : 0;      // when the two kinds of pairs begin to deal out the rest
+  return std::max(ahead + (waves + (rem > 0)) * c1, r ? behind + (waves + (rem > rest)) * c1 : 0);
+}
+
+// Two products that do not depend on one another in one launch: one after the other, each left pairs idle in its last wave.
+// One step of 256 x 512 x 512 34.7 -> 32.1 us, 2080 x 1056 x 2848 62.2 -> 58.5, 16384 x 1024 x 3072 198 -> 192; the bf16
+// gradients of 16384 x 4096 x 4096 with its forward product 1100 -> 1072, of 3872 x 1856 x 832 63.5 -> 49.2.
+template <int BN, bool BF16_IN>
+int launch_gemm2_paired(const GemmParams (&g)[2], const uint8_t* const (&a)[2], const uint8_t* const (&b)[2], const int (&mn)[2], cudaStream_t s) {
+  using C = Cfg2<BN>;
+  constexpr auto kernel = gemm2_nvfp4_kernel<BN, 0, BF16_IN, false, BF16_IN ? 2 : 0, true>;
+  Gemm2Params<2> p;
+  for (int w = 0; w < 2; ++w)
+    if (!describe_product<BN, BF16_IN, false>(g[w], a[w], b[w], mn[w], &p.maps[w], &p.product[w])) return NVFP4_ERR_CUDA;
+  p.out_g = nullptr; p.out_scales = nullptr;
+  static DeviceFlags smem_set;                         // per instantiation, per device
+  if (set_max_dynamic_smem(smem_set, kernel, C::kSmemBytes) != cudaSuccess) return NVFP4_ERR_CUDA;
+  const int64_t n0 = (int64_t)p.product[0].tiles_m * p.product[0].tiles_n, n1 = (int64_t)p.product[1].tiles_m * p.product[1].tiles_n;
+  const int64_t pairs = std::min<int64_t>(n0 + n1, sm_count() / 2);
+  order_tiles(n0, tile_cycles(BN, g[0]), n1, tile_cycles(BN, g[1]), pairs, &p.order);
+  return launch_overlapped(kernel, (unsigned)(2 * pairs), kGemm2Threads, C::kSmemBytes, s, p) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
 template <int BN>
@@ -992,6 +1087,22 @@ int pair_tile_width(int64_t M, int64_t N) {
   return ceil_div(tiles_m * ceil_div(N, 128), pairs) <= ceil_div(tiles_m * ceil_div(N, 256), pairs) ? 128 : 256;
 }
 
+// The same choice for two products in one launch, by the cycles that the tiles' order takes.
+int paired_tile_width(const GemmParams (&p)[2]) {
+  int64_t cycles[2];
+  for (int i = 0; i < 2; ++i) {
+    const int bn = 128 << i;
+    int64_t n[2], c[2];
+    for (int w = 0; w < 2; ++w) {
+      n[w] = ceil_div(p[w].M, 256) * ceil_div(p[w].N, bn);
+      c[w] = tile_cycles(bn, p[w]);
+    }
+    TileOrder o;
+    cycles[i] = order_tiles(n[0], c[0], n[1], c[1], std::min<int64_t>(n[0] + n[1], sm_count() / 2), &o);
+  }
+  return cycles[0] <= cycles[1] ? 128 : 256;
+}
+
 // 0 = automatic.  128 / 256: single-CTA kernel with that tile width.  2128 / 2192 / 2256: CTA-pair
 // kernel with a 256 x {128,192,256} tile.
 int gemm_tile_n_override = 0;
@@ -1006,47 +1117,67 @@ extern "C" int nvfp4_gemm_set_tile_n(int bn) {
   return NVFP4_OK;
 }
 
-int nvfp4::gemm_checked(const uint8_t* a_codes, const uint8_t* a_sf, const float* a_g,
-                        const uint8_t* b_codes, const uint8_t* b_sf, const float* b_g,
-                        int64_t M, int64_t N, int64_t K, void* d, int d_dtype, int64_t ldd, void* cuda_stream, bool late) {
-  if (!a_codes || !a_sf || !b_codes || !b_sf || !d) return NVFP4_ERR_NULL;
-  if (d_dtype != NVFP4_BF16 && d_dtype != NVFP4_FP32) return NVFP4_ERR_ENUM;
-  if (M <= 0 || N <= 0 || K <= 0 || (K % 32) != 0 || ldd < N) return NVFP4_ERR_SHAPE;
-  if (M >= (1ll << 31) - 256 || N >= (1ll << 31) - 256 || K >= (1ll << 31) - 256) return NVFP4_ERR_SHAPE;
-  const int64_t esz = (d_dtype == NVFP4_BF16) ? 2 : 4;
-  if (!aligned16(a_codes) || !aligned16(a_sf) || !aligned16(b_codes) || !aligned16(b_sf) || !aligned16(d) ||
-      ((ldd * esz) % 16) != 0)
+namespace {
+// The checks of nvfp4_gemm, and its sizes as the kernels take them.
+int checked_params(const GemmCall& c, GemmParams* p) {
+  if (!c.a_codes || !c.a_sf || !c.b_codes || !c.b_sf || !c.d) return NVFP4_ERR_NULL;
+  if (c.d_dtype != NVFP4_BF16 && c.d_dtype != NVFP4_FP32) return NVFP4_ERR_ENUM;
+  if (c.M <= 0 || c.N <= 0 || c.K <= 0 || (c.K % 32) != 0 || c.ldd < c.N) return NVFP4_ERR_SHAPE;
+  if (c.M >= (1ll << 31) - 256 || c.N >= (1ll << 31) - 256 || c.K >= (1ll << 31) - 256) return NVFP4_ERR_SHAPE;
+  const int64_t esz = (c.d_dtype == NVFP4_BF16) ? 2 : 4;
+  if (!aligned16(c.a_codes) || !aligned16(c.a_sf) || !aligned16(c.b_codes) || !aligned16(c.b_sf) || !aligned16(c.d) ||
+      ((c.ldd * esz) % 16) != 0)
     return NVFP4_ERR_ALIGN;
-  if ((a_g && (reinterpret_cast<uintptr_t>(a_g) & 3u)) || (b_g && (reinterpret_cast<uintptr_t>(b_g) & 3u)))
+  if ((c.a_g && (reinterpret_cast<uintptr_t>(c.a_g) & 3u)) || (c.b_g && (reinterpret_cast<uintptr_t>(c.b_g) & 3u)))
     return NVFP4_ERR_ALIGN;
-  if (int st = check_arch()) return st;
-
+  p->a_sf = c.a_sf; p->b_sf = c.b_sf; p->a_g = c.a_g; p->b_g = c.b_g; p->d = c.d; p->ldd = c.ldd;
+  p->M = (int)c.M; p->N = (int)c.N; p->K = (int)c.K;
+  p->k_stages = (int)ceil_div(c.K, BK);
+  p->k_tiles = (int)ceil_div(c.K, MMA_K);
+  p->k_mmas = p->k_tiles;
+  p->a_row_tiles = (int)ceil_div(c.M, 128);
+  p->b_row_tiles = (int)ceil_div(c.N, 128);
+  p->d_is_bf16 = (c.d_dtype == NVFP4_BF16);
+  p->tiles_m = p->tiles_n = 0;
+  return check_arch();
+}
+int gemm(const GemmCall& c, void* cuda_stream) {
   GemmParams p;
-  p.a_sf = a_sf; p.b_sf = b_sf; p.a_g = a_g; p.b_g = b_g; p.d = d; p.ldd = ldd;
-  p.M = (int)M; p.N = (int)N; p.K = (int)K;
-  p.k_stages = (int)ceil_div(K, BK);
-  p.k_tiles = (int)ceil_div(K, MMA_K);
-  p.k_mmas = p.k_tiles;
-  p.a_row_tiles = (int)ceil_div(M, 128);
-  p.b_row_tiles = (int)ceil_div(N, 128);
-  p.d_is_bf16 = (d_dtype == NVFP4_BF16);
-  p.tiles_m = p.tiles_n = 0;
-  p.late = late;
+  if (int st = checked_params(c, &p)) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  const int bn = gemm_tile_n_override ? gemm_tile_n_override : 2000 + pair_tile_width(M, N);
+  const int bn = gemm_tile_n_override ? gemm_tile_n_override : 2000 + pair_tile_width(c.M, c.N);
   switch (bn) {
-    case 128: return launch_gemm<128>(a_codes, b_codes, p, s);
-    case 256: return launch_gemm<256>(a_codes, b_codes, p, s);
-    case 2128: return launch_gemm2_dt<128>(a_codes, b_codes, p, s);
-    case 2192: return launch_gemm2_dt<192>(a_codes, b_codes, p, s);
-    default: return launch_gemm2_dt<256>(a_codes, b_codes, p, s);
+    case 128: return launch_gemm<128>(c.a_codes, c.b_codes, p, s);
+    case 256: return launch_gemm<256>(c.a_codes, c.b_codes, p, s);
+    case 2128: return launch_gemm2_dt<128>(c.a_codes, c.b_codes, p, s);
+    case 2192: return launch_gemm2_dt<192>(c.a_codes, c.b_codes, p, s);
+    default: return launch_gemm2_dt<256>(c.a_codes, c.b_codes, p, s);
   }
+}
+}  // namespace
+
+int nvfp4::gemm_two(const GemmCall& x, const GemmCall& y, void* cuda_stream) {
+  if (gemm_tile_n_override != 0 && gemm_tile_n_override != 2128 && gemm_tile_n_override != 2256) {
+    if (int st = gemm(x, cuda_stream)) return st;
+    return gemm(y, cuda_stream);
+  }
+  const bool x_first = x.K >= y.K;
+  const GemmCall* const c[2] = {x_first ? &x : &y, x_first ? &y : &x};
+  GemmParams p[2];
+  for (int w = 0; w < 2; ++w)
+    if (int st = checked_params(*c[w], &p[w])) return st;
+  const uint8_t* const a[2] = {c[0]->a_codes, c[1]->a_codes};
+  const uint8_t* const b[2] = {c[0]->b_codes, c[1]->b_codes};
+  const int mn[2] = {0, 0};
+  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  const int bn = gemm_tile_n_override ? gemm_tile_n_override - 2000 : paired_tile_width(p);
+  return bn == 128 ? launch_gemm2_paired<128, false>(p, a, b, mn, s) : launch_gemm2_paired<256, false>(p, a, b, mn, s);
 }
 
 extern "C" int nvfp4_gemm(const uint8_t* a_codes, const uint8_t* a_sf, const float* a_g,
                           const uint8_t* b_codes, const uint8_t* b_sf, const float* b_g,
                           int64_t M, int64_t N, int64_t K, void* d, int d_dtype, int64_t ldd, void* cuda_stream) {
-  return gemm_checked(a_codes, a_sf, a_g, b_codes, b_sf, b_g, M, N, K, d, d_dtype, ldd, cuda_stream, false);
+  return gemm({a_codes, a_sf, a_g, b_codes, b_sf, b_g, M, N, K, d, d_dtype, ldd}, cuda_stream);
 }
 
 extern "C" int nvfp4_gemm_quantized(const uint8_t* a_codes, const uint8_t* a_sf, const float* a_g,
@@ -1106,55 +1237,69 @@ extern "C" int nvfp4_gemm_mx(const uint8_t* a_codes, const uint8_t* a_sf, const 
 }
 
 namespace {
-int gemm_bf16_any(const void* a, int a_mn, const void* b, int b_mn, int64_t M, int64_t N, int64_t K,
-                  void* d, int d_dtype, int64_t ldd, void* cuda_stream);
+int checked_bf16_params(const GemmCall& c, int a_mn, int b_mn, GemmParams* p) {
+  if (!c.a_codes || !c.b_codes || !c.d) return NVFP4_ERR_NULL;
+  if ((a_mn && c.M % 8 != 0) || (b_mn && c.N % 8 != 0)) return NVFP4_ERR_SHAPE;   // 16-byte row pitch of an MN-major operand
+  if (c.d_dtype != NVFP4_BF16 && c.d_dtype != NVFP4_FP32) return NVFP4_ERR_ENUM;
+  if (c.M <= 0 || c.N <= 0 || c.K <= 0 || (c.K % 16) != 0 || c.ldd < c.N) return NVFP4_ERR_SHAPE;
+  if (c.M >= (1ll << 31) - 256 || c.N >= (1ll << 31) - 256 || c.K >= (1ll << 30)) return NVFP4_ERR_SHAPE;
+  const int64_t esz = (c.d_dtype == NVFP4_BF16) ? 2 : 4;
+  if (!aligned16(c.a_codes) || !aligned16(c.b_codes) || !aligned16(c.d) || ((c.ldd * esz) % 16) != 0) return NVFP4_ERR_ALIGN;
+  p->a_sf = p->b_sf = nullptr; p->a_g = p->b_g = nullptr; p->d = c.d; p->ldd = c.ldd;
+  p->M = (int)c.M; p->N = (int)c.N; p->K = (int)c.K;
+  p->k_stages = (int)ceil_div(c.K * 2, BK_BYTES);    // 64 bf16 values per stage
+  p->k_tiles = (int)(c.K / 16);                      // 32-byte steps = one MMA each
+  p->k_mmas = p->k_tiles;
+  p->a_row_tiles = (int)ceil_div(c.M, 128);
+  p->b_row_tiles = (int)ceil_div(c.N, 128);
+  p->d_is_bf16 = (c.d_dtype == NVFP4_BF16);
+  p->tiles_m = p->tiles_n = 0;
+  return check_arch();
 }
+int gemm_bf16_any(const GemmCall& c, int a_mn, int b_mn, void* cuda_stream) {
+  GemmParams p;
+  if (int st = checked_bf16_params(c, a_mn, b_mn, &p)) return st;
+  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  switch ((a_mn ? 1 : 0) | (b_mn ? 2 : 0)) {
+    case 0: return p.d_is_bf16 ? launch_gemm2<256, 1, true>(c.a_codes, c.b_codes, p, s) : launch_gemm2<256, 0, true>(c.a_codes, c.b_codes, p, s);
+    case 2: return p.d_is_bf16 ? launch_gemm2<256, 1, true, false, 2>(c.a_codes, c.b_codes, p, s) : launch_gemm2<256, 0, true, false, 2>(c.a_codes, c.b_codes, p, s);
+    case 3: return p.d_is_bf16 ? launch_gemm2<256, 1, true, false, 3>(c.a_codes, c.b_codes, p, s) : launch_gemm2<256, 0, true, false, 3>(c.a_codes, c.b_codes, p, s);
+    default: return NVFP4_ERR_ENUM;
+  }
+}
+GemmCall bf16_call(const void* a, const void* b, int64_t M, int64_t N, int64_t K, void* d, int d_dtype, int64_t ldd) {
+  return {static_cast<const uint8_t*>(a), nullptr, nullptr, static_cast<const uint8_t*>(b), nullptr, nullptr, M, N, K, d, d_dtype, ldd};
+}
+}  // namespace
 
 extern "C" int nvfp4_gemm_bf16(const void* a, const void* b, int64_t M, int64_t N, int64_t K,
                                void* d, int d_dtype, int64_t ldd, void* cuda_stream) {
-  return gemm_bf16_any(a, 0, b, 0, M, N, K, d, d_dtype, ldd, cuda_stream);
+  return gemm_bf16_any(bf16_call(a, b, M, N, K, d, d_dtype, ldd), 0, 0, cuda_stream);
 }
 
 extern "C" int nvfp4_gemm_bf16_ex(const void* a, int a_mn_major, const void* b, int b_mn_major, int64_t M, int64_t N, int64_t K,
                                   void* d, int d_dtype, int64_t ldd, void* cuda_stream) {
   if ((a_mn_major != 0 && a_mn_major != 1) || (b_mn_major != 0 && b_mn_major != 1)) return NVFP4_ERR_ENUM;
   if (a_mn_major && !b_mn_major) return NVFP4_ERR_ENUM;      // no product of Eq. 1-3 has that shape; not instantiated
-  return gemm_bf16_any(a, a_mn_major, b, b_mn_major, M, N, K, d, d_dtype, ldd, cuda_stream);
+  return gemm_bf16_any(bf16_call(a, b, M, N, K, d, d_dtype, ldd), a_mn_major, b_mn_major, cuda_stream);
 }
 
-namespace {
-int gemm_bf16_any(const void* a, int a_mn, const void* b, int b_mn, int64_t M, int64_t N, int64_t K,
-                  void* d, int d_dtype, int64_t ldd, void* cuda_stream) {
-  if (!a || !b || !d) return NVFP4_ERR_NULL;
-  if ((a_mn && M % 8 != 0) || (b_mn && N % 8 != 0)) return NVFP4_ERR_SHAPE;   // 16-byte row pitch of an MN-major operand
-  if (d_dtype != NVFP4_BF16 && d_dtype != NVFP4_FP32) return NVFP4_ERR_ENUM;
-  if (M <= 0 || N <= 0 || K <= 0 || (K % 16) != 0 || ldd < N) return NVFP4_ERR_SHAPE;
-  if (M >= (1ll << 31) - 256 || N >= (1ll << 31) - 256 || K >= (1ll << 30)) return NVFP4_ERR_SHAPE;
-  const int64_t esz = (d_dtype == NVFP4_BF16) ? 2 : 4;
-  if (!aligned16(a) || !aligned16(b) || !aligned16(d) || ((ldd * esz) % 16) != 0) return NVFP4_ERR_ALIGN;
-  if (int st = check_arch()) return st;
-  GemmParams p;
-  p.a_sf = p.b_sf = nullptr; p.a_g = p.b_g = nullptr; p.d = d; p.ldd = ldd;
-  p.M = (int)M; p.N = (int)N; p.K = (int)K;
-  p.k_stages = (int)ceil_div(K * 2, BK_BYTES);       // 64 bf16 values per stage
-  p.k_tiles = (int)(K / 16);                         // 32-byte steps = one MMA each
-  p.k_mmas = p.k_tiles;
-  p.a_row_tiles = (int)ceil_div(M, 128);
-  p.b_row_tiles = (int)ceil_div(N, 128);
-  p.d_is_bf16 = (d_dtype == NVFP4_BF16);
-  p.tiles_m = p.tiles_n = 0;
-  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  const uint8_t* ab = static_cast<const uint8_t*>(a);
-  const uint8_t* bb = static_cast<const uint8_t*>(b);
-  const int mn = (a_mn ? 1 : 0) | (b_mn ? 2 : 0);
-  switch (mn) {
-    case 0: return p.d_is_bf16 ? launch_gemm2<256, 1, true>(ab, bb, p, s) : launch_gemm2<256, 0, true>(ab, bb, p, s);
-    case 2: return p.d_is_bf16 ? launch_gemm2<256, 1, true, false, 2>(ab, bb, p, s) : launch_gemm2<256, 0, true, false, 2>(ab, bb, p, s);
-    case 3: return p.d_is_bf16 ? launch_gemm2<256, 1, true, false, 3>(ab, bb, p, s) : launch_gemm2<256, 0, true, false, 3>(ab, bb, p, s);
-    default: return NVFP4_ERR_ENUM;
-  }
+// dX[M, K] = dY . W and dW[N, K] = dY^T . X in one launch (arguments as for nvfp4_linear_bwd_bf16).
+int nvfp4::gemm_bf16_gradients(const void* dY, const void* W, const void* X, int64_t M, int64_t N, int64_t K, void* dX, int dx_dtype,
+                               void* dW, int dw_dtype, void* cuda_stream) {
+  // dX: contraction over N, dY has N contiguous (K-major operand), W is [contraction, output] (MN-major operand);
+  // dW: contraction over the token axis, both operands are [contraction, output]
+  const GemmCall dx = bf16_call(dY, W, M, K, N, dX, dx_dtype, K), dw = bf16_call(dY, X, N, K, M, dW, dw_dtype, K);
+  const bool dw_first = M >= N;
+  const GemmCall* const c[2] = {dw_first ? &dw : &dx, dw_first ? &dx : &dw};
+  const int mn[2] = {dw_first ? 3 : 2, dw_first ? 2 : 3};
+  GemmParams p[2];
+  for (int w = 0; w < 2; ++w)
+    if (int st = checked_bf16_params(*c[w], mn[w] & 1, 1, &p[w])) return st;
+  const uint8_t* const a[2] = {c[0]->a_codes, c[1]->a_codes};
+  const uint8_t* const b[2] = {c[0]->b_codes, c[1]->b_codes};
+  return launch_gemm2_paired<256, true>(p, a, b, mn, static_cast<cudaStream_t>(cuda_stream));
 }
-}  // namespace
 
 extern "C" int nvfp4_device_error_word(uint32_t* host_out) {
   if (!host_out) return NVFP4_ERR_NULL;

@@ -150,10 +150,8 @@ int run_bwd(const void* dY, int dtype, int64_t M, int64_t N, int64_t K, const fl
   if (int st = nvfp4_quantize_dual(dY, dtype, M, N, N, g_dy, rdy, ws + bl.dy.codes, ws + bl.dy.sf, rdyt,
                                    ws + bl.dyt.codes, ws + bl.dyt.sf, NVFP4_SF_SWIZZLED_128x4, stream))
     return st;
-  if (int st = nvfp4_gemm(ws + bl.dy.codes, ws + bl.dy.sf, g_dy, wt_codes, wt_sf, g_w, M, K, N, dX, dx_dtype, K, stream))
-    return st;
-  // independent of the product before it: its first tiles fill that one's last wave
-  return gemm_checked(ws + bl.dyt.codes, ws + bl.dyt.sf, g_dy, xt_codes, xt_sf, g_x, N, K, M, dW, dw_dtype, K, stream, /*late=*/true);
+  return gemm_two({ws + bl.dy.codes, ws + bl.dy.sf, g_dy, wt_codes, wt_sf, g_w, M, K, N, dX, dx_dtype, K},
+                  {ws + bl.dyt.codes, ws + bl.dyt.sf, g_dy, xt_codes, xt_sf, g_x, N, K, M, dW, dw_dtype, K}, stream);
 }
 }  // namespace
 

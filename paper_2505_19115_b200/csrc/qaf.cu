@@ -80,9 +80,11 @@ extern "C" int nvfp4_linear_bwd_bf16(const void* dY, const void* W, const void* 
   if ((dx_dtype != NVFP4_BF16 && dx_dtype != NVFP4_FP32) || (dw_dtype != NVFP4_BF16 && dw_dtype != NVFP4_FP32)) return NVFP4_ERR_ENUM;
   if (M <= 0 || N <= 0 || K <= 0 || M % 16 != 0 || N % 16 != 0 || K % 16 != 0) return NVFP4_ERR_SHAPE;
   if (!aligned16(dY) || !aligned16(W) || !aligned16(X) || !aligned16(dX) || !aligned16(dW)) return NVFP4_ERR_ALIGN;
-  // dX[M,K] = dY[M,N] . W[N,K]: contraction over N; dY has N contiguous (K-major operand), W is [contraction, output]
-  // with the output axis contiguous (MN-major operand)
-  if (int st = nvfp4_gemm_bf16_ex(dY, 0, W, 1, M, K, N, dX, dx_dtype, K, cuda_stream)) return st;
-  // dW[N,K] = dY[M,N]^T . X[M,K]: contraction over the token axis M; both operands are [contraction, output]
-  return nvfp4_gemm_bf16_ex(dY, 1, X, 1, N, K, M, dW, dw_dtype, K, cuda_stream);
+  // one launch of both, unless the weight gradient goes where the other product still reads the weights
+  const uintptr_t w = reinterpret_cast<uintptr_t>(W), dw = reinterpret_cast<uintptr_t>(dW);
+  if (dw < w + (uintptr_t)(N * K * 2) && w < dw + (uintptr_t)(N * K * (dw_dtype == NVFP4_BF16 ? 2 : 4))) {
+    if (int st = nvfp4_gemm_bf16_ex(dY, 0, W, 1, M, K, N, dX, dx_dtype, K, cuda_stream)) return st;
+    return nvfp4_gemm_bf16_ex(dY, 1, X, 1, N, K, M, dW, dw_dtype, K, cuda_stream);
+  }
+  return gemm_bf16_gradients(dY, W, X, M, N, K, dX, dx_dtype, dW, dw_dtype, cuda_stream);
 }

@@ -155,6 +155,21 @@ def test_fused_layer_with_given_scales_and_bf16_outputs():
     _assert_close(_host(dW), *oracle_linear("dw", dY, X, nb.Rounding(nb.SR, 0, 1), nb.Rounding(nb.SR, 0, 2), True))
 
 
+# One launch deals the tiles of both gradients out to the pairs of CTAs: fewer tiles than pairs, a first product that fills its
+# waves exactly (9472 x 8192), one that leaves pairs over (4096 x 3072 x 1024: 48 tiles), either product being the longer one.
+@pytest.mark.parametrize("shape", [(32, 32, 32), (768, 512, 1280), (18944, 512, 256), (4096, 1024, 3072), (256, 8192, 9472), (2080, 1056, 2848), (512, 2048, 8192)])
+@pytest.mark.parametrize("dx_dtype,dw_dtype", [(torch.float32, torch.float32), (torch.bfloat16, torch.float32), (torch.float32, torch.bfloat16)])
+def test_gradients_of_one_launch_equal_the_single_products(shape, dx_dtype, dw_dtype):
+    M, K, N = shape
+    X, W, dY = (t.cuda() for t in synth.linear_inputs(M, K, N, seed=33, grad_std=1e-3))
+    rt, sr0, sr1, sr2 = nb.Rounding(nb.RTN), nb.Rounding(nb.SR, 6, 0), nb.Rounding(nb.SR, 6, 1), nb.Rounding(nb.SR, 6, 2)
+    want = (nb.nvfp4_linear_bwd_dx(dY, W, rdy=sr0, rw=rt, out_dtype=dx_dtype), nb.nvfp4_linear_bwd_dw(dY, X, rdy=sr1, rx=sr2, out_dtype=dw_dtype))
+    got = nb.nvfp4_linear_bwd(dY, W, X, rdy=sr0, rdyt=sr1, rwt=rt, rxt=sr2, dx_dtype=dx_dtype, dw_dtype=dw_dtype)
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    assert torch.equal(want[0], got[0]) and torch.equal(want[1], got[1])
+
+
 # ---------------------------------------------------------------- non-finite inputs stay visible
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
 def test_non_finite_input_propagates_through_the_per_tensor_scale(bad):

@@ -119,3 +119,21 @@ def test_backward_and_update_in_bf16_at_layer_size():
     ref = np.einsum("ms,ms->s", hdY[:, ii].astype(np.float64), hX[:, jj].astype(np.float64))
     T = np.einsum("ms,ms->s", np.abs(hdY[:, ii]).astype(np.float64), np.abs(hX[:, jj]).astype(np.float64))
     assert np.all(np.abs(_h(dW)[ii, jj] - ref) <= TOL * T + 1e-30)
+
+
+# Both gradients in one launch: tile counts as in the NVFP4 test, and a weight gradient that goes where the weights are read.
+@pytest.mark.parametrize("shape", [(16, 16, 16), (768, 512, 1280), (18944, 512, 256), (4096, 1024, 3072), (256, 4096, 4736), (1040, 528, 1424)])
+def test_gradients_of_one_launch_equal_the_single_products(shape):
+    M, K, N = shape
+    X, W, dY = (t.cuda() for t in synth.linear_inputs(M, K, N, seed=44, grad_std=1e-3))
+    for dtype in (torch.float32, torch.bfloat16):
+        dX, dW = nb.nvfp4_linear_bwd_bf16(dY, W, X, dx_dtype=dtype)
+        assert torch.equal(dX, nb.nvfp4_gemm_bf16_ex(dY, 0, W, 1, out_dtype=dtype))
+        assert torch.equal(dW, nb.nvfp4_gemm_bf16_ex(dY, 1, X, 1))
+    W2 = W.clone()
+    st = nb.lib().nvfp4_linear_bwd_bf16(dY.data_ptr(), W2.data_ptr(), X.data_ptr(), M, N, K, dX.data_ptr(), nb.BF16, W2.data_ptr(), nb.BF16,
+                                        None, 0, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert st == 0 and nb.nvfp4_device_error_word() == 0
+    assert torch.equal(dX, nb.nvfp4_gemm_bf16_ex(dY, 0, W, 1, out_dtype=torch.bfloat16))
+    assert torch.equal(W2, nb.nvfp4_gemm_bf16_ex(dY, 1, X, 1, out_dtype=torch.bfloat16))
