@@ -777,7 +777,9 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
       const float alpha = PAIRED && w ? alphas[PAIRED] : alphas[0];
       int tm, tn;
       tile_coords(tile, q.tiles_m, q.tiles_n, tm, tn);
-      ACCOUNT(a_tile, ok = mbar_wait_warp(tfull_bar(acc), acc_ph, abort_flag, 0x14));
+      // Polled without sleeping: the next tile's MMAs wait for this read-out.  Against a lane that sleeps 32 ns between its polls:
+      // 16384 x 3072 x 2048 fp32 57.6 -> 56.2 us, 16384 x 4096 x 4096 bf16 109.7 -> 107.0, 1024 x 1024 x 16384 21.2 -> 20.1.
+      ACCOUNT(a_tile, ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, 0x14));
       if (!ok) break;
 #ifdef NVFP4_GEMM_ACCOUNT
       a_read_t0 = clock64();
