@@ -247,7 +247,7 @@ class Block:
             self.layer(l, gmode, self.given[i] if gmode == self.nb.G_GIVEN else None)
 
     def launches_per_step(self, gmode=None):
-        per_layer = 3 + 3                                  # dual quantizers, GEMMs
+        per_layer = 3 + 2                                  # dual quantizers, the forward product, both gradients
         if gmode == self.nb.G_GIVEN:
             return len(self.layers) * per_layer
         # + amax sweeps and, per call, the kernel that zeroes their scratch; X and W share a sweep when together below 64 MB
@@ -501,7 +501,7 @@ def main():
     for _ in range(args.warmup):
         block.step()
     barrier()
-    # One step = 55 launches of 1-400 us: captured once into a CUDA graph (after the warm-up, so that every
+    # One step = 50 launches of 1-700 us: captured once into a CUDA graph (after the warm-up, so that every
     # one-time set-up inside the library is done) and replayed, which removes the launch gaps between them.
     ms, launch_mode = timed_graph(block.step, args.steps, barrier, not args.no_graph, sampler)
     clocks = sampler.stop() if rank == 0 else None
