@@ -379,17 +379,21 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 // epilogue warpgroups up to 184 (256 x (72 + 184) = 65536, what the CTA was launched with).
 // ------------------------------------------------------------------------------------------------
 constexpr int kGemm2Threads = 512;
+constexpr int kMnBoxBytes = 64 * 128;             // box of an MN-major operand: 64 contraction rows x 64 values
 constexpr int kControlRegs = 72, kEpilogueRegs = 184;
 
-template <int BN>
+// bf16 operands have no scales: the room goes to another operand stage and a second accumulator.
+// us, five stages, one accumulator and 256 columns only -> this: 16384 x 4096 x 4096 417 -> 404, 2048 x 1024 x 2816 28.3 -> 24.6,
+// 512 x 704 x 9888 50.8 -> 43.3; 2816 x 1024 x 16384 96.7 -> 97.2.
+template <int BN, bool BF16_IN = false>
 struct Cfg2 {
   static constexpr int kSfbTiles = (BN % 128 == 0) ? BN / 128 : BN / 128 + 1;
-  static constexpr int kStages = (BN == 128) ? 6 : 5;
-  static constexpr int kAccStages = (BN == 256) ? 1 : 2;
+  static constexpr int kStages = BF16_IN ? (BN == 128 ? 8 : 6) : (BN == 128) ? 6 : 5;
+  static constexpr int kAccStages = (BN == 256 && !BF16_IN) ? 1 : 2;
   static constexpr int kABytes = 128 * BK_BYTES;
   static constexpr int kBBytes = (BN / 2) * BK_BYTES;
-  static constexpr int kSfaBytes = 2048;
-  static constexpr int kSfbBytes = kSfbTiles * 2048;
+  static constexpr int kSfaBytes = BF16_IN ? 0 : 2048;
+  static constexpr int kSfbBytes = BF16_IN ? 0 : kSfbTiles * 2048;
   static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;
   static constexpr int kEpiWarpBytes = 4096;                       // one 32-row x 128-byte staging buffer per warp
   static constexpr int kEpiBytes = 8 * kEpiWarpBytes;
@@ -398,12 +402,12 @@ struct Cfg2 {
   static constexpr uint32_t kSfaCol = kAccStages * BN;
   static constexpr uint32_t kSfCols = 16 + kSfbTiles * 16;
   static constexpr int kSfBufsFit = (int)((kTmemCols - kSfaCol) / kSfCols);
-  static constexpr int kSfBufs = kSfBufsFit > kStages ? kStages : kSfBufsFit;
+  static constexpr int kSfBufs = BF16_IN ? 0 : kSfBufsFit > kStages ? kStages : kSfBufsFit;
   // with as many scale buffers as stages, buffer b is stage s and needs no barrier of its own
   static constexpr bool kSfFollowsStage = (kSfBufs == kStages);
   static constexpr int kNumBarriers = 4 * kStages + 2 * kSfBufs + 2 * kAccStages;
   static_assert(kStageBytes % 1024 == 0, "stage must keep the 1024-byte swizzle alignment");
-  static_assert(kSfBufs >= 2, "need at least two scale buffers in tensor memory");
+  static_assert(BF16_IN || kSfBufs >= 2, "need at least two scale buffers in tensor memory");
   static_assert(kSmemBytes <= 232448, "shared memory overflow");
   static_assert(8 * kNumBarriers + 8 <= 512, "barrier area overflow");
 };
@@ -479,10 +483,10 @@ struct Gemm2Params {
 template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0, bool PAIRED = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemm2Threads, 1)
 gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
-  using C = Cfg2<BN>;
+  using C = Cfg2<BN, BF16_IN>;
   constexpr bool Q_OUT = (OUT == 2);
   constexpr bool MN_B = (MN & 2) != 0;
-  static_assert(MN == 0 || (BF16_IN && BN == 256), "MN-major operands exist for the bf16 variant with the 256-wide tile");
+  static_assert(MN == 0 || (BF16_IN && BN % 128 == 0), "MN-major operands exist for the bf16 variant");
   static_assert(!PAIRED || (!Q_OUT && !MX && BN % 128 == 0), "two products: the gradients of a layer");
   static_assert(!Q_OUT || BN == 256, "the quantized epilogue stores two 64-byte pieces of codes per tile row");
   extern __shared__ uint8_t smem_raw[];
@@ -567,13 +571,13 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
           if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2u * kOperandTx);
           if (a_mn) {                               // [K, M]: x = byte offset of the output row, y = contraction index
             tma_load_2d_pair(st, &m.a, lead_full, m0 * 2, ks * 64);
-            tma_load_2d_pair(st + C::kABytes / 2, &m.a, lead_full, (m0 + 64) * 2, ks * 64);
+            tma_load_2d_pair(st + kMnBoxBytes, &m.a, lead_full, (m0 + 64) * 2, ks * 64);
           } else {
             tma_load_2d_pair(st, &m.a, lead_full, ks * BK_BYTES, m0);
           }
           if constexpr (MN_B) {
-            tma_load_2d_pair(st + C::kABytes, &m.b, lead_full, n0 * 2, ks * 64);
-            tma_load_2d_pair(st + C::kABytes + C::kBBytes / 2, &m.b, lead_full, (n0 + 64) * 2, ks * 64);
+            for (int h = 0; h < BN / 128; ++h)      // boxes of 64 columns
+              tma_load_2d_pair(st + C::kABytes + h * kMnBoxBytes, &m.b, lead_full, (n0 + 64 * h) * 2, ks * 64);
           } else {
             tma_load_2d_pair(st + C::kABytes, &m.b, lead_full, ks * BK_BYTES, n0);
           }
@@ -652,8 +656,8 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
           const int nkt = min(4, q.k_mmas - ks * 4);
           const uint32_t sfa_t = tmem_base + C::kSfaCol + b * C::kSfCols;
           const uint32_t sfb_t = sfa_t + 16 + sfb_off;
-          const uint64_t adesc = a_mn ? operand_desc_mn(st, C::kABytes / 2) : operand_desc(st);
-          const uint64_t bdesc = MN_B ? operand_desc_mn(st + C::kABytes, C::kBBytes / 2) : operand_desc(st + C::kABytes);
+          const uint64_t adesc = a_mn ? operand_desc_mn(st, kMnBoxBytes) : operand_desc(st);
+          const uint64_t bdesc = MN_B ? operand_desc_mn(st + C::kABytes, kMnBoxBytes) : operand_desc(st + C::kABytes);
           if (issuer && BF16_IN) {
             // one instruction = 16 contraction indices: 32 bytes along a K-major row, 16 rows (2048 bytes) of an MN-major box
             const uint32_t a_step = a_mn ? (2048u >> 4) : 2u;
@@ -1017,7 +1021,7 @@ bool describe_product(const GemmParams& g, const uint8_t* a_codes, const uint8_t
 template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0>
 int launch_gemm2(const uint8_t* a_codes, const uint8_t* b_codes, const GemmParams& g, cudaStream_t s,
                  const QuantOut& q = QuantOut()) {
-  using C = Cfg2<BN>;
+  using C = Cfg2<BN, BF16_IN>;
   Gemm2Params<1> p;
   if (!describe_product<BN, BF16_IN, MX>(g, a_codes, b_codes, MN, &p.maps[0], &p.product[0])) return NVFP4_ERR_CUDA;
   if constexpr (OUT == 2)
@@ -1039,8 +1043,8 @@ int launch_gemm2(const uint8_t* a_codes, const uint8_t* b_codes, const GemmParam
 // What a tile of the pair kernel takes, in cycles of a CTA pair: its k-stages and the turn-round of the accumulator, or sending
 // its output off, which takes longer below ten stages (1024-value contractions: 4100-4400 cycles a tile with bf16 output,
 // 5900 with fp32).
-int64_t tile_cycles(int bn, const GemmParams& p) {
-  const int64_t loop = bn == 128 ? 330 * (int64_t)p.k_stages + 200 : 590 * (int64_t)p.k_stages + 900;
+int64_t tile_cycles(int bn, const GemmParams& p, bool bf16_in) {
+  const int64_t stages = p.k_stages, loop = bn == 128 ? (bf16_in ? 380 : 330) * stages + 200 : bf16_in ? 570 * stages + 300 : 590 * stages + 900;
   return std::max<int64_t>(loop, (p.d_is_bf16 ? 4000 : 5600) * bn / 256);
 }
 
@@ -1059,7 +1063,7 @@ int64_t order_tiles(int64_t n0, int64_t c0, int64_t n1, int64_t c1, int64_t pair
 // gradients of 16384 x 4096 x 4096 with its forward product 1100 -> 1072, of 3872 x 1856 x 832 63.5 -> 49.2.
 template <int BN, bool BF16_IN>
 int launch_gemm2_paired(const GemmParams (&g)[2], const uint8_t* const (&a)[2], const uint8_t* const (&b)[2], const int (&mn)[2], cudaStream_t s) {
-  using C = Cfg2<BN>;
+  using C = Cfg2<BN, BF16_IN>;
   constexpr auto kernel = gemm2_nvfp4_kernel<BN, 0, BF16_IN, false, BF16_IN ? 2 : 0, true>;
   Gemm2Params<2> p;
   for (int w = 0; w < 2; ++w)
@@ -1069,7 +1073,7 @@ int launch_gemm2_paired(const GemmParams (&g)[2], const uint8_t* const (&a)[2], 
   if (set_max_dynamic_smem(smem_set, kernel, C::kSmemBytes) != cudaSuccess) return NVFP4_ERR_CUDA;
   const int64_t n0 = (int64_t)p.product[0].tiles_m * p.product[0].tiles_n, n1 = (int64_t)p.product[1].tiles_m * p.product[1].tiles_n;
   const int64_t pairs = std::min<int64_t>(n0 + n1, sm_count() / 2);
-  order_tiles(n0, tile_cycles(BN, g[0]), n1, tile_cycles(BN, g[1]), pairs, &p.order);
+  order_tiles(n0, tile_cycles(BN, g[0], BF16_IN), n1, tile_cycles(BN, g[1], BF16_IN), pairs, &p.order);
   return launch_overlapped(kernel, (unsigned)(2 * pairs), kGemm2Threads, C::kSmemBytes, s, p) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
@@ -1090,14 +1094,14 @@ int pair_tile_width(int64_t M, int64_t N) {
 }
 
 // The same choice for two products in one launch, by the cycles that the tiles' order takes.
-int paired_tile_width(const GemmParams (&p)[2]) {
+int paired_tile_width(const GemmParams (&p)[2], bool bf16_in) {
   int64_t cycles[2];
   for (int i = 0; i < 2; ++i) {
     const int bn = 128 << i;
     int64_t n[2], c[2];
     for (int w = 0; w < 2; ++w) {
       n[w] = ceil_div(p[w].M, 256) * ceil_div(p[w].N, bn);
-      c[w] = tile_cycles(bn, p[w]);
+      c[w] = tile_cycles(bn, p[w], bf16_in);
     }
     TileOrder o;
     cycles[i] = order_tiles(n[0], c[0], n[1], c[1], std::min<int64_t>(n[0] + n[1], sm_count() / 2), &o);
@@ -1172,7 +1176,7 @@ int nvfp4::gemm_two(const GemmCall& x, const GemmCall& y, void* cuda_stream) {
   const uint8_t* const b[2] = {c[0]->b_codes, c[1]->b_codes};
   const int mn[2] = {0, 0};
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  const int bn = gemm_tile_n_override ? gemm_tile_n_override - 2000 : paired_tile_width(p);
+  const int bn = gemm_tile_n_override ? gemm_tile_n_override - 2000 : paired_tile_width(p, false);
   return bn == 128 ? launch_gemm2_paired<128, false>(p, a, b, mn, s) : launch_gemm2_paired<256, false>(p, a, b, mn, s);
 }
 
@@ -1258,17 +1262,22 @@ int checked_bf16_params(const GemmCall& c, int a_mn, int b_mn, GemmParams* p) {
   p->tiles_m = p->tiles_n = 0;
   return check_arch();
 }
+template <int BN>
+int launch_bf16(const GemmCall& c, const GemmParams& p, int a_mn, int b_mn, cudaStream_t s) {
+  switch ((a_mn ? 1 : 0) | (b_mn ? 2 : 0)) {
+    case 0: return p.d_is_bf16 ? launch_gemm2<BN, 1, true>(c.a_codes, c.b_codes, p, s) : launch_gemm2<BN, 0, true>(c.a_codes, c.b_codes, p, s);
+    case 2: return p.d_is_bf16 ? launch_gemm2<BN, 1, true, false, 2>(c.a_codes, c.b_codes, p, s) : launch_gemm2<BN, 0, true, false, 2>(c.a_codes, c.b_codes, p, s);
+    case 3: return p.d_is_bf16 ? launch_gemm2<BN, 1, true, false, 3>(c.a_codes, c.b_codes, p, s) : launch_gemm2<BN, 0, true, false, 3>(c.a_codes, c.b_codes, p, s);
+    default: return NVFP4_ERR_ENUM;
+  }
+}
 int gemm_bf16_any(const GemmCall& c, int a_mn, int b_mn, void* cuda_stream) {
   GemmParams p;
   if (int st = checked_bf16_params(c, a_mn, b_mn, &p)) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  switch ((a_mn ? 1 : 0) | (b_mn ? 2 : 0)) {
-    case 0: return p.d_is_bf16 ? launch_gemm2<256, 1, true>(c.a_codes, c.b_codes, p, s) : launch_gemm2<256, 0, true>(c.a_codes, c.b_codes, p, s);
-    case 2: return p.d_is_bf16 ? launch_gemm2<256, 1, true, false, 2>(c.a_codes, c.b_codes, p, s) : launch_gemm2<256, 0, true, false, 2>(c.a_codes, c.b_codes, p, s);
-    case 3: return p.d_is_bf16 ? launch_gemm2<256, 1, true, false, 3>(c.a_codes, c.b_codes, p, s) : launch_gemm2<256, 0, true, false, 3>(c.a_codes, c.b_codes, p, s);
-    default: return NVFP4_ERR_ENUM;
-  }
+  return pair_tile_width(c.M, c.N) == 128 ? launch_bf16<128>(c, p, a_mn, b_mn, s) : launch_bf16<256>(c, p, a_mn, b_mn, s);
 }
+
 GemmCall bf16_call(const void* a, const void* b, int64_t M, int64_t N, int64_t K, void* d, int d_dtype, int64_t ldd) {
   return {static_cast<const uint8_t*>(a), nullptr, nullptr, static_cast<const uint8_t*>(b), nullptr, nullptr, M, N, K, d, d_dtype, ldd};
 }
@@ -1300,7 +1309,8 @@ int nvfp4::gemm_bf16_gradients(const void* dY, const void* W, const void* X, int
     if (int st = checked_bf16_params(*c[w], mn[w] & 1, 1, &p[w])) return st;
   const uint8_t* const a[2] = {c[0]->a_codes, c[1]->a_codes};
   const uint8_t* const b[2] = {c[0]->b_codes, c[1]->b_codes};
-  return launch_gemm2_paired<256, true>(p, a, b, mn, static_cast<cudaStream_t>(cuda_stream));
+  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  return paired_tile_width(p, true) == 128 ? launch_gemm2_paired<128, true>(p, a, b, mn, s) : launch_gemm2_paired<256, true>(p, a, b, mn, s);
 }
 
 extern "C" int nvfp4_device_error_word(uint32_t* host_out) {

@@ -137,3 +137,19 @@ def test_gradients_of_one_launch_equal_the_single_products(shape):
     assert st == 0 and nb.nvfp4_device_error_word() == 0
     assert torch.equal(dX, nb.nvfp4_gemm_bf16_ex(dY, 0, W, 1, out_dtype=torch.bfloat16))
     assert torch.equal(W2, nb.nvfp4_gemm_bf16_ex(dY, 1, X, 1, out_dtype=torch.bfloat16))
+
+
+# both tile widths, and last waves of fewer tiles than pairs, on integers: every sum is exact
+@pytest.mark.parametrize("majors", [(0, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("shape", [(256, 128, 64), (264, 136, 208), (9728, 512, 128), (9728, 488, 336), (9496, 264, 1040)])
+def test_gemm_bf16_tile_forms_are_exact(shape, majors):
+    M, N, K = shape
+    A = torch.randint(-4, 5, (M, K), generator=torch.Generator("cuda").manual_seed(1), device="cuda").to(torch.bfloat16)
+    B = torch.randint(-4, 5, (N, K), generator=torch.Generator("cuda").manual_seed(2), device="cuda").to(torch.bfloat16)
+    a, b = (x.t().contiguous() if mn else x for x, mn in zip((A, B), majors))
+    D = nb.nvfp4_gemm_bf16_ex(a, majors[0], b, majors[1])
+    Db = nb.nvfp4_gemm_bf16_ex(a, majors[0], b, majors[1], out_dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    want = A.double() @ B.double().T
+    assert torch.equal(D.double(), want) and torch.equal(Db, want.to(torch.bfloat16))
