@@ -413,7 +413,7 @@ struct Cfg2 {
 };
 
 struct Gemm2Maps {
-  CUtensorMap a, b, sfa, sfb, d;
+  CUtensorMap a, b, b_half, sfa, sfb, d;   // b_half: operand B for half tiles, where there are any
 };
 struct Gemm2Product {
   const float* a_g;
@@ -429,29 +429,42 @@ struct Gemm2Product {
 // input and the weight gradient of a layer, which do not depend on one another): the tiles of the first, whose contraction is
 // the longer one, come first.  n0 = q * pairs + r of them leave pairs - r pairs without one of the last r; those take `head`
 // tiles of the second product each meanwhile, and the others of it are dealt out to all pairs, beginning with those.
+// The last wave, where it would leave half of the pairs idle, has halves of tiles (128 of the 256 columns): items from `split` on.
 struct TileOrder {
   int q = 0, r = 0, head = 0;
-  int n1;                           // tiles of the second product, or of the only one
+  int n1, split;                    // items of the second product, or of the only one; the first that is half a tile
 };
-template <bool PAIRED>
-__device__ __forceinline__ bool tile_at(const TileOrder& o, int pair, int pairs, int i, int& product, int& tile) {
-  product = 0;
+struct TileItem {
+  int product, tile, half;          // half: 0 or 1, or -1 for a whole tile
+};
+template <bool PAIRED, bool HALVES>
+__device__ __forceinline__ bool tile_at(const TileOrder& o, int pair, int pairs, int i, TileItem& t) {
+  t.product = 0;
+  t.half = -1;
+  int item;
   if constexpr (!PAIRED) {
-    tile = pair + i * pairs;
+    item = pair + i * pairs;
   } else {
     const int rest = pairs - o.r, first = o.q + (pair < o.r);
     if (i < first) {
-      tile = pair + i * pairs;
+      t.tile = pair + i * pairs;
       return true;
     }
-    product = 1;
+    t.product = 1;
     i -= first;
     const int rank = pair < o.r ? rest + pair : pair - o.r;
-    if (pair >= o.r && i < o.head) tile = rank + i * rest;
-    else tile = o.head * rest + rank + (i - (pair >= o.r ? o.head : 0)) * pairs;
+    if (pair >= o.r && i < o.head) item = rank + i * rest;
+    else item = o.head * rest + rank + (i - (pair >= o.r ? o.head : 0)) * pairs;
   }
-  return tile < o.n1;
+  t.tile = item;
+  if (HALVES && item >= o.split) {
+    t.tile = o.split + ((item - o.split) >> 1);
+    t.half = (item - o.split) & 1;
+  }
+  return item < o.n1;
 }
+// Launches with half tiles take a kernel of their own (HALVES): the choice costs the others 1-2 % of a short product.
+constexpr bool has_halves(int bn, int out, bool bf16_in, bool paired) { return bn == 256 && out != 2 && (paired || !bf16_in); }
 
 template <int PRODUCTS>
 struct Gemm2Params {
@@ -480,13 +493,14 @@ struct Gemm2Params {
 // them through MN-major descriptors, so no transposed copy of the tensor is ever made.
 // PAIRED: the launch computes two products (TileOrder); their output types, and for bf16 operands (both products of the
 // backward pass have an MN-major B) whether A is MN-major, then come from the parameters, OUT and MN bit 0 being unused.
-template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0, bool PAIRED = false>
+template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0, bool PAIRED = false, bool HALVES = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemm2Threads, 1)
 gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
   using C = Cfg2<BN, BF16_IN>;
   constexpr bool Q_OUT = (OUT == 2);
   constexpr bool MN_B = (MN & 2) != 0;
   static_assert(MN == 0 || (BF16_IN && BN % 128 == 0), "MN-major operands exist for the bf16 variant");
+  static_assert(!HALVES || BN == 256, "a half tile is 128 columns wide");
   static_assert(!PAIRED || (!Q_OUT && !MX && BN % 128 == 0), "two products: the gradients of a layer");
   static_assert(!Q_OUT || BN == 256, "the quantized epilogue stores two 64-byte pieces of codes per tile row");
   extern __shared__ uint8_t smem_raw[];
@@ -551,15 +565,17 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
     int s = 0;
     uint32_t ph = 0;
     bool ok = true;
-    constexpr uint32_t kOperandTx = C::kABytes + C::kBBytes;       // per CTA, signalled on the leader's barrier
     ACCOUNT_VARS(a_wait = 0, a_total = -ACCOUNT_NOW());
-    for (int i = 0, w, tile; ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
-      const Gemm2Product& q = p.product[w];
-      const Gemm2Maps& m = p.maps[w];
+    TileItem t;
+    for (int i = 0; ok && tile_at<PAIRED, HALVES>(p.order, pair, num_pairs, i, t); ++i) {
+      const Gemm2Product& q = p.product[t.product];
+      const Gemm2Maps& m = p.maps[t.product];
       const bool a_mn = PAIRED ? BF16_IN && q.a_mn : (MN & 1) != 0;
       int tm, tn;
-      tile_coords(tile, q.tiles_m, q.tiles_n, tm, tn);
-      const int m0 = tm * 256 + (int)rank * 128, n0 = tn * BN + (int)rank * (BN / 2);
+      tile_coords(t.tile, q.tiles_m, q.tiles_n, tm, tn);
+      const bool whole = !HALVES || t.half < 0;
+      const int m0 = tm * 256 + (int)rank * 128, n0 = whole ? tn * BN + (int)rank * (BN / 2) : tn * BN + t.half * (BN / 2) + (int)rank * (BN / 4);
+      const uint32_t operand_tx = 2u * (C::kABytes + (whole ? C::kBBytes : C::kBBytes / 2));   // of both CTAs, signalled on the leader's barrier
       for (int ks = 0; ks < q.k_stages; ++ks) {
         // polled without sleeping: the refill of a freed stage is on the main loop's critical path (the ring is
         // five stages deep for a copy latency of three to four stage times), and a sleeping poll adds its period to it
@@ -568,7 +584,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
         const uint32_t st = smem_base + s * C::kStageBytes;
         const uint32_t lead_full = map_to_cta(full_bar(s), 0);
         if (issuer) {
-          if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2u * kOperandTx);
+          if (rank == 0) mbar_arrive_expect_tx(full_bar(s), operand_tx);
           if (a_mn) {                               // [K, M]: x = byte offset of the output row, y = contraction index
             tma_load_2d_pair(st, &m.a, lead_full, m0 * 2, ks * 64);
             tma_load_2d_pair(st + kMnBoxBytes, &m.a, lead_full, (m0 + 64) * 2, ks * 64);
@@ -576,10 +592,10 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
             tma_load_2d_pair(st, &m.a, lead_full, ks * BK_BYTES, m0);
           }
           if constexpr (MN_B) {
-            for (int h = 0; h < BN / 128; ++h)      // boxes of 64 columns
+            for (int h = 0; h < (whole ? BN / 128 : 1); ++h)      // boxes of 64 columns
               tma_load_2d_pair(st + C::kABytes + h * kMnBoxBytes, &m.b, lead_full, (n0 + 64 * h) * 2, ks * 64);
           } else {
-            tma_load_2d_pair(st + C::kABytes, &m.b, lead_full, ks * BK_BYTES, n0);
+            tma_load_2d_pair(st + C::kABytes, whole ? &m.b : &m.b_half, lead_full, ks * BK_BYTES, n0);
           }
         }
         if (++s == C::kStages) { s = 0; ph ^= 1u; }
@@ -599,11 +615,12 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
     bool ok = true;
     constexpr int kSfTiles = MX ? 2 : 4;                           // 512-byte scale tiles per stage and 128 rows
     constexpr uint32_t kScaleTx = (C::kSfaBytes + C::kSfbBytes) / 4 * kSfTiles;   // signalled on this CTA's own barrier
-    for (int i = 0, w, tile; !BF16_IN && ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
-      const Gemm2Product& q = p.product[w];
-      const Gemm2Maps& m = p.maps[w];
+    TileItem t;
+    for (int i = 0; !BF16_IN && ok && tile_at<PAIRED, HALVES>(p.order, pair, num_pairs, i, t); ++i) {
+      const Gemm2Product& q = p.product[t.product];
+      const Gemm2Maps& m = p.maps[t.product];
       int tm, tn;
-      tile_coords(tile, q.tiles_m, q.tiles_n, tm, tn);
+      tile_coords(t.tile, q.tiles_m, q.tiles_n, tm, tn);
       const int a_row = min(tm * 2 + (int)rank, q.a_row_tiles - 1) * q.k_tiles;
       int b_row[C::kSfbTiles];
 #pragma unroll
@@ -634,13 +651,17 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
       uint32_t ph = 0, bph = 0, acc_ph = 0;
       bool ok = true;
       ACCOUNT_VARS(a_acc = 0, a_ops = 0, a_sf = 0, a_total = -ACCOUNT_NOW());
-      for (int i = 0, w, tile; ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
-        const Gemm2Product& q = p.product[w];
+      TileItem t;
+      for (int i = 0; ok && tile_at<PAIRED, HALVES>(p.order, pair, num_pairs, i, t); ++i) {
+        const Gemm2Product& q = p.product[t.product];
+        const bool whole = !HALVES || t.half < 0;
         const bool a_mn = PAIRED ? BF16_IN && q.a_mn : (MN & 1) != 0;
-        const uint32_t idesc = !BF16_IN ? instr_desc(256, BN) : a_mn ? instr_desc_bf16(256, BN, true, MN_B) : instr_desc_bf16(256, BN, false, MN_B);
+        constexpr uint32_t kHalfN = ((uint32_t)(BN / 2) >> 3) << 17;       // what the instruction descriptor of half as many columns has less
+        const uint32_t idesc = (!BF16_IN ? instr_desc(256, BN) : a_mn ? instr_desc_bf16(256, BN, true, MN_B) : instr_desc_bf16(256, BN, false, MN_B)) -
+                               (whole ? 0u : kHalfN);
         int tm_unused, tn;
-        tile_coords(tile, q.tiles_m, q.tiles_n, tm_unused, tn);
-        const uint32_t sfb_off = (uint32_t)((tn * BN) % 128) / 32;         // first scale column of this N tile
+        tile_coords(t.tile, q.tiles_m, q.tiles_n, tm_unused, tn);
+        const uint32_t sfb_off = (uint32_t)((tn * BN) % 128) / 32 + (whole ? 0u : 4u * t.half);   // first scale column of this N tile
         ACCOUNT(a_acc, ok = mbar_wait_issuer(tempty_bar(acc), acc_ph ^ 1u, abort_flag, 0x12));
         if (!ok) break;
         const uint32_t d_tmem = tmem_base + acc * BN;
@@ -666,7 +687,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
             tc_commit_pair(empty_bar(s));
           } else if (issuer && MX) {
             for (int j = 0; j < nkt; ++j)
-              tc_mma_mxf4_pair(d_tmem, adesc + 2u * j, bdesc + 2u * j, (j & 1) ? instr_desc_mx(256, BN, 1) : instr_desc_mx(256, BN, 0),
+              tc_mma_mxf4_pair(d_tmem, adesc + 2u * j, bdesc + 2u * j, ((j & 1) ? instr_desc_mx(256, BN, 1) : instr_desc_mx(256, BN, 0)) - (whole ? 0u : kHalfN),
                                sfa_t + 4 * (j >> 1), sfb_t + 4 * C::kSfbTiles * (j >> 1), (ks | j) ? 1u : 0u);
             tc_commit_pair(empty_bar(s));
             if constexpr (!C::kSfFollowsStage) tc_commit_pair(sfe_bar(b));
@@ -707,8 +728,9 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
     uint32_t ph = 0, bph = 0;
     bool ok = true;
     ACCOUNT_VARS(a_land = 0, a_free = 0, a_total = -ACCOUNT_NOW());
-    for (int i = 0, w, tile; !BF16_IN && ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
-      const int k_stages = p.product[w].k_stages;
+    TileItem t;
+    for (int i = 0; !BF16_IN && ok && tile_at<PAIRED, HALVES>(p.order, pair, num_pairs, i, t); ++i) {
+      const int k_stages = p.product[t.product].k_stages;
       for (int ks = 0; ks < k_stages; ++ks) {
         ACCOUNT(a_land, ok = mbar_wait_warp_relaxed(sfl_bar(s), ph, abort_flag, 0x16));
         if (!ok) break;
@@ -776,11 +798,14 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
     uint32_t acc_ph = 0;
     bool ok = true;
     ACCOUNT_VARS(a_tile = 0, a_read = 0, a_total = -ACCOUNT_NOW(), a_read_t0 = 0);
-    for (int i = 0, w, tile; ok && tile_at<PAIRED>(p.order, pair, num_pairs, i, w, tile); ++i) {
-      const Gemm2Product& q = p.product[w];
-      const float alpha = PAIRED && w ? alphas[PAIRED] : alphas[0];
+    TileItem t;
+    for (int i = 0; ok && tile_at<PAIRED, HALVES>(p.order, pair, num_pairs, i, t); ++i) {
+      const Gemm2Product& q = p.product[t.product];
+      const float alpha = PAIRED && t.product ? alphas[PAIRED] : alphas[0];
+      const int warp_cols = HALVES && t.half >= 0 ? BN / 4 : kWarpCols;    // columns of a first half's warp
+      const int tile_cols = HALVES && t.half >= 0 ? BN / 2 : BN;
       int tm, tn;
-      tile_coords(tile, q.tiles_m, q.tiles_n, tm, tn);
+      tile_coords(t.tile, q.tiles_m, q.tiles_n, tm, tn);
       // Polled without sleeping: the next tile's MMAs wait for this read-out.  Against a lane that sleeps 32 ns between its polls:
       // 16384 x 3072 x 2048 fp32 57.6 -> 56.2 us, 16384 x 4096 x 4096 bf16 109.7 -> 107.0, 1024 x 1024 x 16384 21.2 -> 20.1.
       ACCOUNT(a_tile, ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, 0x14));
@@ -790,11 +815,11 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
 #endif
       tc_fence_after();
       const int row0 = tm * 256 + (int)rank * 128 + quarter * 32;
-      const uint32_t t_row = tmem_base + acc * BN + half * kWarpCols + ((uint32_t)(quarter * 32) << 16);
+      const uint32_t t_row = tmem_base + acc * BN + half * warp_cols + ((uint32_t)(quarter * 32) << 16);
       uint32_t r[kLoads][32];
 #pragma unroll
       for (int l = 0; l < kLoads; ++l)
-        if (half * kWarpCols + 32 * l < BN) tmem_ld32(t_row + 32 * l, r[l]);
+        if (32 * l < warp_cols && half * warp_cols + 32 * l < tile_cols) tmem_ld32(t_row + 32 * l, r[l]);
       tmem_ld_wait();
 #pragma unroll
       for (int l = 0; l < kLoads; ++l) tmem_ld_pin(r[l]);
@@ -859,14 +884,15 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
       } else {
         // one chunk at a time: 32 rows x 128 bytes (row = lane, eight 16-byte pieces, piece index XOR (row & 7): the
         // 128-byte swizzle), sent off as one tiled store
-        const CUtensorMap* map_d = &p.maps[w].d;
+        const CUtensorMap* map_d = &p.maps[t.product].d;
+        const int col0 = tn * BN + (HALVES && t.half > 0 ? BN / 2 : 0) + half * warp_cols;
         auto store_chunks = [&](auto bf16) {
           constexpr bool BF16_OUT = decltype(bf16)::value;
           constexpr int kChunkCols = BF16_OUT ? 64 : 32;           // accumulator columns per 128 bytes of output row
           static_assert(kWarpCols % kChunkCols == 0, "a warp stores whole chunks");
 #pragma unroll
           for (int c = 0; c < kWarpCols; c += kChunkCols) {
-            if (half * kWarpCols + c >= BN) break;
+            if (c >= warp_cols || half * warp_cols + c >= tile_cols) break;
             uint32_t v[32];
             if constexpr (BF16_OUT) {
 #pragma unroll
@@ -890,7 +916,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
             fence_async_smem();
             __syncwarp();
             if (lane == 0) {
-              tma_store_2d(map_d, buf, tn * BN + half * kWarpCols + c, row0);
+              tma_store_2d(map_d, buf, col0 + c, row0);
               tma_store_commit();
             }
           }
@@ -996,15 +1022,42 @@ bool make_qout_map(CUtensorMap* map, uint8_t* base, int64_t M, int64_t N) {
             CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// What a tile of the pair kernel takes, in cycles of a CTA pair: its k-stages and the turn-round of the accumulator, or sending
+// its output off, which takes longer below ten stages (1024-value contractions: 4100-4400 cycles a tile with bf16 output,
+// 5900 with fp32).
+int64_t tile_cycles(int bn, const GemmParams& p, bool bf16_in) {
+  const int64_t stages = p.k_stages, loop = bn == 128 ? (bf16_in ? 380 : 330) * stages + 200 : bf16_in ? 570 * stages + 300 : 590 * stages + 900;
+  return std::max<int64_t>(loop, (p.d_is_bf16 ? 4000 : 5600) * bn / 256);
+}
+
+// Order of two products' tiles over `pairs` pairs (c0, c1: cycles of a tile; n0 = 0: one product), and the cycles until the last
+// is done.  halves: the last wave may have half tiles.  They are worth it where one such wave takes all of them (us, without /
+// with: fp32 16384 x 1024 x 2816, 256 tiles, 30.1 / 28.5; bf16 16384 x 1024 x 3072 24.4 / 23.7; fp32 16384 x 3072 x 1024, 768 tiles,
+// 39.9 / 39.5) and the launch is not so long that the kernel's 1 % more for every tile eats it (both gradients of 16384 x 11008 x
+// 4096, 72 waves of the shorter tile: step 1148 / 1154).
+int64_t order_tiles(int64_t n0, int64_t c0, int64_t n1, int64_t c1, int64_t pairs, bool halves, TileOrder* o) {
+  const int64_t q = n0 / pairs, r = n0 % pairs, rest = pairs - r;
+  const int64_t head = r ? std::min(c0 / c1, n1 / rest) : 0;
+  const int64_t left = n1 - head * rest, waves = left / pairs, rem = left % pairs;
+  const bool split = halves && 2 * rem <= pairs && (n0 * c0 + n1 * c1) / pairs < 40 * c1;
+  const int64_t last = split ? 2 * rem : rem, c_last = split ? (c1 * 5 + 7) / 8 : c1;
+  o->q = (int)q; o->r = (int)r; o->head = (int)head;
+  o->n1 = (int)(n1 - rem + last); o->split = (int)(split ? n1 - rem : n1);
+  const int64_t ahead = q * c0 + head * c1, behind = r ? (q + 1) * c0 : 0;      // when the two kinds of pairs begin to deal out the rest
+  return std::max(ahead + waves * c1 + (last > 0 ? c_last : 0), r ? behind + waves * c1 + (last > rest ? c_last : 0) : 0);
+}
+
 // Tensor maps and sizes of one product for the CTA-pair kernel.
 template <int BN, bool BF16_IN, bool MX>
-bool describe_product(const GemmParams& g, const uint8_t* a_codes, const uint8_t* b_codes, int mn, Gemm2Maps* m, Gemm2Product* q) {
+bool describe_product(const GemmParams& g, const uint8_t* a_codes, const uint8_t* b_codes, int mn, bool halves, Gemm2Maps* m, Gemm2Product* q) {
   const int64_t row_bytes = BF16_IN ? (int64_t)g.K * 2 : g.K / 2;       // operand rows as bytes
   // MN-major bf16 operand: the tensor is [K, rows] with the output axis contiguous; boxes of 64 contraction rows x 128 bytes
   if (!((mn & 1) ? make_codes_map(&m->a, a_codes, g.K, (int64_t)g.M * 2, 64) : make_codes_map(&m->a, a_codes, g.M, row_bytes, 128)))
     return false;
   if (!((mn & 2) ? make_codes_map(&m->b, b_codes, g.K, (int64_t)g.N * 2, 64) : make_codes_map(&m->b, b_codes, g.N, row_bytes, BN / 2)))
     return false;
+  m->b_half = m->b;
+  if (halves && !(mn & 2) && !make_codes_map(&m->b_half, b_codes, g.N, row_bytes, BN / 4)) return false;
   if constexpr (BF16_IN) {
     m->sfa = m->a;                                                       // never used by the kernel
     m->sfb = m->b;
@@ -1018,44 +1071,32 @@ bool describe_product(const GemmParams& g, const uint8_t* a_codes, const uint8_t
   return true;
 }
 
+template <auto KERNEL, int BN, bool BF16_IN, int PRODUCTS>
+int launch_pairs(int64_t pairs, const Gemm2Params<PRODUCTS>& p, cudaStream_t s) {
+  using C = Cfg2<BN, BF16_IN>;
+  static DeviceFlags smem_set;                         // per kernel, per device
+  if (set_max_dynamic_smem(smem_set, KERNEL, C::kSmemBytes) != cudaSuccess) return NVFP4_ERR_CUDA;
+  return launch_overlapped(KERNEL, (unsigned)(2 * pairs), kGemm2Threads, C::kSmemBytes, s, p) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
+
 template <int BN, int OUT, bool BF16_IN = false, bool MX = false, int MN = 0>
 int launch_gemm2(const uint8_t* a_codes, const uint8_t* b_codes, const GemmParams& g, cudaStream_t s,
                  const QuantOut& q = QuantOut()) {
-  using C = Cfg2<BN, BF16_IN>;
+  constexpr bool kHalves = has_halves(BN, OUT, BF16_IN, false);
   Gemm2Params<1> p;
-  if (!describe_product<BN, BF16_IN, MX>(g, a_codes, b_codes, MN, &p.maps[0], &p.product[0])) return NVFP4_ERR_CUDA;
+  const int64_t max_pairs = sm_count() / 2;
+  order_tiles(0, 0, ceil_div(g.M, 256) * ceil_div(g.N, BN), 1, max_pairs, kHalves, &p.order);
+  const int64_t pairs = std::min<int64_t>(p.order.n1, max_pairs);
+  if (!describe_product<BN, BF16_IN, MX>(g, a_codes, b_codes, MN, p.order.split < p.order.n1, &p.maps[0], &p.product[0])) return NVFP4_ERR_CUDA;
   if constexpr (OUT == 2)
     if (!make_qout_map(&p.maps[0].d, q.codes, g.M, g.N)) return NVFP4_ERR_CUDA;
   p.out_g = q.g; p.out_scales = q.scales; p.out_sr = 0; p.out_swizzled = q.sf_layout == NVFP4_SF_SWIZZLED_128x4;
   p.out_nkb = g.N / 16; p.out_k_tiles = ceil_div(p.out_nkb, 4);
   philox_stream_init(&p.out_rng, q.rounding ? q.rounding->seed : 0, q.rounding ? q.rounding->offset : 0);
   if (q.rounding) p.out_sr = q.rounding->mode == NVFP4_SR;
-  static DeviceFlags smem_set;                         // per instantiation, per device
-  if (set_max_dynamic_smem(smem_set, gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN>, C::kSmemBytes) != cudaSuccess)
-    return NVFP4_ERR_CUDA;
-  p.order.n1 = p.product[0].tiles_m * p.product[0].tiles_n;
-  const int max_pairs = sm_count() / 2;
-  const int pairs = p.order.n1 < max_pairs ? p.order.n1 : max_pairs;
-  return launch_overlapped(gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN>, 2 * pairs, kGemm2Threads, C::kSmemBytes, s, p) == cudaSuccess
-             ? NVFP4_OK : NVFP4_ERR_CUDA;
-}
-
-// What a tile of the pair kernel takes, in cycles of a CTA pair: its k-stages and the turn-round of the accumulator, or sending
-// its output off, which takes longer below ten stages (1024-value contractions: 4100-4400 cycles a tile with bf16 output,
-// 5900 with fp32).
-int64_t tile_cycles(int bn, const GemmParams& p, bool bf16_in) {
-  const int64_t stages = p.k_stages, loop = bn == 128 ? (bf16_in ? 380 : 330) * stages + 200 : bf16_in ? 570 * stages + 300 : 590 * stages + 900;
-  return std::max<int64_t>(loop, (p.d_is_bf16 ? 4000 : 5600) * bn / 256);
-}
-
-// Order of two products' tiles over `pairs` pairs (c0, c1: cycles of a tile), and the cycles until the last is done.
-int64_t order_tiles(int64_t n0, int64_t c0, int64_t n1, int64_t c1, int64_t pairs, TileOrder* o) {
-  const int64_t q = n0 / pairs, r = n0 % pairs, rest = pairs - r;
-  const int64_t head = r ? std::min(c0 / c1, n1 / rest) : 0;
-  const int64_t left = n1 - head * rest, waves = left / pairs, rem = left % pairs;
-  o->q = (int)q; o->r = (int)r; o->head = (int)head; o->n1 = (int)n1;
-  const int64_t ahead = q * c0 + head * c1, behind = r ? (q + 1) * c0 : 0;      // when the two kinds of pairs begin to deal out the rest
-  return std::max(ahead + (waves + (rem > 0)) * c1, r ? behind + (waves + (rem > rest)) * c1 : 0);
+  if constexpr (kHalves)
+    if (p.order.split < p.order.n1) return launch_pairs<gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN, false, true>, BN, BF16_IN>(pairs, p, s);
+  return launch_pairs<gemm2_nvfp4_kernel<BN, OUT, BF16_IN, MX, MN>, BN, BF16_IN>(pairs, p, s);
 }
 
 // Two products that do not depend on one another in one launch: one after the other, each left pairs idle in its last wave.
@@ -1063,18 +1104,18 @@ int64_t order_tiles(int64_t n0, int64_t c0, int64_t n1, int64_t c1, int64_t pair
 // gradients of 16384 x 4096 x 4096 with its forward product 1100 -> 1072, of 3872 x 1856 x 832 63.5 -> 49.2.
 template <int BN, bool BF16_IN>
 int launch_gemm2_paired(const GemmParams (&g)[2], const uint8_t* const (&a)[2], const uint8_t* const (&b)[2], const int (&mn)[2], cudaStream_t s) {
-  using C = Cfg2<BN, BF16_IN>;
-  constexpr auto kernel = gemm2_nvfp4_kernel<BN, 0, BF16_IN, false, BF16_IN ? 2 : 0, true>;
+  constexpr bool kHalves = has_halves(BN, 0, BF16_IN, true);
+  constexpr int kMn = BF16_IN ? 2 : 0;
   Gemm2Params<2> p;
-  for (int w = 0; w < 2; ++w)
-    if (!describe_product<BN, BF16_IN, false>(g[w], a[w], b[w], mn[w], &p.maps[w], &p.product[w])) return NVFP4_ERR_CUDA;
-  p.out_g = nullptr; p.out_scales = nullptr;
-  static DeviceFlags smem_set;                         // per instantiation, per device
-  if (set_max_dynamic_smem(smem_set, kernel, C::kSmemBytes) != cudaSuccess) return NVFP4_ERR_CUDA;
-  const int64_t n0 = (int64_t)p.product[0].tiles_m * p.product[0].tiles_n, n1 = (int64_t)p.product[1].tiles_m * p.product[1].tiles_n;
+  const int64_t n0 = ceil_div(g[0].M, 256) * ceil_div(g[0].N, BN), n1 = ceil_div(g[1].M, 256) * ceil_div(g[1].N, BN);
   const int64_t pairs = std::min<int64_t>(n0 + n1, sm_count() / 2);
-  order_tiles(n0, tile_cycles(BN, g[0], BF16_IN), n1, tile_cycles(BN, g[1], BF16_IN), pairs, &p.order);
-  return launch_overlapped(kernel, (unsigned)(2 * pairs), kGemm2Threads, C::kSmemBytes, s, p) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  order_tiles(n0, tile_cycles(BN, g[0], BF16_IN), n1, tile_cycles(BN, g[1], BF16_IN), pairs, kHalves, &p.order);
+  for (int w = 0; w < 2; ++w)
+    if (!describe_product<BN, BF16_IN, false>(g[w], a[w], b[w], mn[w], w == 1 && p.order.split < p.order.n1, &p.maps[w], &p.product[w])) return NVFP4_ERR_CUDA;
+  p.out_g = nullptr; p.out_scales = nullptr;
+  if constexpr (kHalves)
+    if (p.order.split < p.order.n1) return launch_pairs<gemm2_nvfp4_kernel<BN, 0, BF16_IN, false, kMn, true, true>, BN, BF16_IN>(pairs, p, s);
+  return launch_pairs<gemm2_nvfp4_kernel<BN, 0, BF16_IN, false, kMn, true>, BN, BF16_IN>(pairs, p, s);
 }
 
 template <int BN>
@@ -1104,7 +1145,7 @@ int paired_tile_width(const GemmParams (&p)[2], bool bf16_in) {
       c[w] = tile_cycles(bn, p[w], bf16_in);
     }
     TileOrder o;
-    cycles[i] = order_tiles(n[0], c[0], n[1], c[1], std::min<int64_t>(n[0] + n[1], sm_count() / 2), &o);
+    cycles[i] = order_tiles(n[0], c[0], n[1], c[1], std::min<int64_t>(n[0] + n[1], sm_count() / 2), bn == 256, &o);
   }
   return cycles[0] <= cycles[1] ? 128 : 256;
 }

@@ -217,3 +217,24 @@ def test_default_tile_width_agrees_with_the_wide_tile(shape):
         torch.cuda.synchronize()
         assert nb.nvfp4_device_error_word() == 0
         assert torch.equal(got, wide)
+
+
+# a last wave of at most half as many tiles as pairs is computed in half tiles: 76 and 111 tiles (2 and 37 over), a half beyond
+# N, one that N ends in, few stages and many; 112 tiles (38 over) stay whole
+@pytest.mark.parametrize("shape", [(9728, 512, 64), (9728, 488, 320), (9500, 264, 1056), (9728, 376, 256), (9472, 768, 96), (9472, 520, 4160), (7168, 1024, 512)])
+def test_half_tiles_of_the_last_wave_agree_with_the_single_cta_kernel(shape):
+    M, N, K = shape
+    A, B = synth.normal((M, K), 1.0, 81, device="cuda"), synth.normal((N, K), 0.02, 82, device="cuda")
+    ga, gb = nb.nvfp4_tensor_amax_scale(A), nb.nvfp4_tensor_amax_scale(B)
+    ops = (*nb.nvfp4_quantize(A, global_scale=ga, sf_layout=nb.SF_SWIZZLED), ga, *nb.nvfp4_quantize(B, global_scale=gb, sf_layout=nb.SF_SWIZZLED), gb)
+    for dt in (torch.float32, torch.bfloat16):
+        outs = []
+        try:
+            for tile in (128, 2256, 0):
+                nb.nvfp4_gemm_set_tile_n(tile)
+                outs.append(nb.nvfp4_gemm(*ops, out_dtype=dt))
+        finally:
+            nb.nvfp4_gemm_set_tile_n(0)
+        torch.cuda.synchronize()
+        assert nb.nvfp4_device_error_word() == 0
+        assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])

@@ -173,3 +173,18 @@ def test_large_tensors_match_the_oracle(transposed, shape, sf_layout):
     oc, osf = ob.quantize_mx(_h(x), g=float(g_t.item()), transposed=transposed)
     assert np.array_equal(codes.cpu().numpy(), oc)
     assert np.array_equal(scales.cpu().numpy().reshape(-1), (_swz(osf) if sf_layout == nb.SF_SWIZZLED else osf).reshape(-1))
+
+
+# the half tiles of a last wave that would leave half of the pairs idle: small integers in, so that every sum is exact
+@pytest.mark.parametrize("shape", [(256, 256, 64), (9728, 512, 128), (9728, 488, 320), (9500, 264, 1056)])
+def test_half_tiles_of_the_last_wave_are_exact(shape):
+    M, N, K = shape
+    A = torch.randint(-2, 3, (M, K), generator=torch.Generator("cuda").manual_seed(1), device="cuda")
+    B = torch.randint(-2, 3, (N, K), generator=torch.Generator("cuda").manual_seed(2), device="cuda")
+    ops = []
+    for x in (A, B):
+        ops += [*nb.nvfp4_quantize_mx(x.to(torch.bfloat16), False, None, None, nb.SF_SWIZZLED), None]
+    D = nb.nvfp4_gemm_mx(*ops)
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    assert torch.equal(D.double(), A.double() @ B.double().T)
