@@ -32,7 +32,8 @@ __global__ void __launch_bounds__(kThreads, 3) quantize_row_kernel(const QuantPa
   __shared__ float inv_table[MX ? 256 : 128];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t kb = (int64_t)blockIdx.x * 32 + lane;
-  const int64_t row0 = (int64_t)blockIdx.y * kRowTileRows;
+  // Row tiles from the last to the first: an amax pass that ran just before left the end of the tensor in the level-two cache.
+  const int64_t row_tile = gridDim.y - 1 - blockIdx.y, row0 = row_tile * kRowTileRows;
   const bool kb_ok = kb < p.nkb;
   grid_dependency_wait();
   grid_dependency_trigger();
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(kThreads, 3) quantize_row_kernel(const QuantPa
     const int64_t kt = (int64_t)blockIdx.x * kTilesPerCta + q;
     if (q < kTilesPerCta && kt < p.k_tiles) {
       const uint4 val = *reinterpret_cast<const uint4*>(sf_s + q * kSfChunkPitch + i * 16);
-      *reinterpret_cast<uint4*>(p.scales + ((int64_t)blockIdx.y * p.k_tiles + kt) * 512 + i * 16) = val;
+      *reinterpret_cast<uint4*>(p.scales + (row_tile * p.k_tiles + kt) * 512 + i * 16) = val;
     }
   }
 }
