@@ -247,12 +247,15 @@ class Block:
             self.layer(l, gmode, self.given[i] if gmode == self.nb.G_GIVEN else None)
 
     def launches_per_step(self, gmode=None):
-        per_layer = 3 + 2                                  # dual quantizers, the forward product, both gradients
-        if gmode == self.nb.G_GIVEN:
-            return len(self.layers) * per_layer
-        # + amax sweeps and, per call, the kernel that zeroes their scratch; X and W share a sweep when together below 64 MB
-        shared = sum((l["X"].numel() + l["W"].numel()) * l["X"].element_size() <= 64 << 20 for l in self.layers)
-        return len(self.layers) * (per_layer + 3 + 2) - shared
+        def quantized(*tensors):                           # operands of one call (the library's quantize_operands)
+            n, elements = len(tensors), sum(t.numel() for t in tensors)
+            size = elements * tensors[0].element_size()
+            if gmode == self.nb.G_GIVEN:
+                return 1 if n == 1 or elements <= 1 << 26 else n + 1      # one launch for all, or the scales' copy and one each
+            if size <= 24 << 20:
+                return 2
+            return 1 + (1 if size <= 64 << 20 else n) + n                 # words zeroed, amax passes, quantizers
+        return sum(quantized(l["W"], l["X"]) + 1 + quantized(l["dY"]) + 1 for l in self.layers)
 
 
 def timed_graph(step, steps, barrier, use_graph=True, sampler=None):

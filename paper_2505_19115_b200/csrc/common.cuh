@@ -69,9 +69,6 @@ __device__ __forceinline__ float load_scale(const float* g) {
   return v;
 }
 
-// Zeroes up to 32 words (quantize.cu), overlapping the kernel before it.
-cudaError_t zero_words(unsigned int* words, int n, cudaStream_t s);
-
 // A product: the arguments of nvfp4_gemm.
 struct GemmCall {
   const uint8_t* a_codes;
@@ -102,19 +99,33 @@ int tile_quantize_row(const void* x, int dtype, int64_t rows, int64_t cols, int6
                       uint8_t* codes, uint8_t* scales, int sf_layout, cudaStream_t s, bool mx = false);
 int tile_error_word(unsigned int* out);
 
-// Per-tensor scales of a call's dense [rows, cols] operands (quantize.cu): the scratch words (two per operand, up to three
-// operands) are zeroed first where they are used, then one launch for all operands if amax_merge() says so, else one for each.
-// The operands are older than the call.
-struct AmaxOperand { const void* x; int64_t rows, cols; float* g; };
-bool amax_merge(const AmaxOperand* ops, int n, int dtype);
-int tensor_amax_scales(const AmaxOperand* ops, int n, int dtype, unsigned int* scratch, void* cuda_stream);
-
-// Per-tensor scale g = amax/2688 in one launch (quantize.cu); scratch_zeroed: two zeroed 32-bit device words.
-// The scratch is used, and has to be zeroed, only where amax_needs_scratch() says so; after the kernel that zeroes it, and
-// wherever `late` is given, x is read before the wait for the kernel launched before this one: x must be older than that.
-bool amax_needs_scratch(int dtype, int64_t elements);
-int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* g_out,
-                         unsigned int* scratch_zeroed, bool late, void* cuda_stream);
+// A dense operand [rows, cols] of a layer call, as its products take it: rows, columns (transposed) or both, with swizzled scales.
+struct LayerOperand {
+  const void* x;
+  int64_t rows, cols;
+  const nvfp4_rounding* rr;       // null: no row output
+  uint8_t *codes_r, *scales_r;
+  const nvfp4_rounding* rt;       // null: no transposed output
+  uint8_t *codes_t, *scales_t;
+  const float* given;             // NVFP4_G_GIVEN: its scale
+  float* slot;                    // its scale in the call's buffers: kScaleSlotBytes, the rest of which the amax passes use; null: not kept
+};
+constexpr int kScaleSlotBytes = 256;
+constexpr int kMaxLayerOperands = 3;
+// Quantizes a layer call's operands (quantize.cu), with their amax passes where the mode asks for it: the operands are older
+// than the call, and this is the first thing that it launches.  g[i]: where the scale of operand i is afterwards.
+int quantize_operands(const LayerOperand* ops, int n, int dtype, int gscale_mode, const float** g, void* cuda_stream);
+// Where a quantizer takes its per-tensor scale from: one stored scale (null = 1), or the maxima that an amax sweep left
+// (n > 0).  keep: where to leave the scale for the kernels behind it (null = nowhere).
+struct ScaleSource {
+  const float* g = nullptr;
+  const uint32_t* maxima = nullptr;
+  int n = 0;
+  float* keep = nullptr;
+};
+// The part of it that one launch of the tile quantizer does for all (quantize_tile.cu).
+bool tile_batch_eligible(const LayerOperand* ops, int n, int dtype);
+int tile_quantize_batch(const LayerOperand* ops, const ScaleSource* scale, int n, int dtype, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------------
 // Scale-factor layout (128 rows x 4 blocks per 512-byte tile, k-tiles contiguous per row tile)

@@ -50,8 +50,14 @@ Layout make_layout(const Plan& pl) {
   return l;
 }
 
-// Scratch words of the amax passes: in the padding behind a scale's workspace slot.
-unsigned int* amax_scratch(float* slot) { return reinterpret_cast<unsigned int*>(slot) + 16; }
+// One operand's quantization in the workspace.
+LayerOperand operand(const void* x, int64_t rows, int64_t cols, int transposed, const nvfp4_rounding* r, uint8_t* codes, uint8_t* scales,
+                     const float* given, uint8_t* slot) {
+  LayerOperand op = {x, rows, cols, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, given, reinterpret_cast<float*>(slot)};
+  if (transposed) { op.rt = r; op.codes_t = codes; op.scales_t = scales; }
+  else { op.rr = r; op.codes_r = codes; op.scales_r = scales; }
+  return op;
+}
 
 int run_linear(int which, const void* a, const void* b, int dtype, int64_t M, int64_t N, int64_t K,
                int gscale_mode, const float* ga, const float* gb, const nvfp4_rounding* ra,
@@ -72,23 +78,13 @@ int run_linear(int which, const void* a, const void* b, int dtype, int64_t M, in
   if (!workspace || workspace_bytes < l.total || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return NVFP4_ERR_WORKSPACE;
 
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  const float* g_a = nullptr;
-  const float* g_b = nullptr;
-  int st;
-  if (gscale_mode == NVFP4_G_AMAX) {
-    float* wa = reinterpret_cast<float*>(ws + l.a_g);
-    float* wb = reinterpret_cast<float*>(ws + l.b_g);
-    const AmaxOperand ops[2] = {{a, pl.a_rows, pl.a_cols, wa}, {b, pl.b_rows, pl.b_cols, wb}};
-    if ((st = tensor_amax_scales(ops, 2, dtype, amax_scratch(wa), stream))) return st;
-    g_a = wa; g_b = wb;
-  } else if (gscale_mode == NVFP4_G_GIVEN) {
-    g_a = ga; g_b = gb;
-  }
-  if ((st = nvfp4_quantize(a, dtype, pl.a_rows, pl.a_cols, pl.a_cols, pl.a_transposed, g_a, ra, ws + l.a_codes,
-                           ws + l.a_sf, NVFP4_SF_SWIZZLED_128x4, stream))) return st;
-  if ((st = nvfp4_quantize(b, dtype, pl.b_rows, pl.b_cols, pl.b_cols, pl.b_transposed, g_b, rb, ws + l.b_codes,
-                           ws + l.b_sf, NVFP4_SF_SWIZZLED_128x4, stream))) return st;
-  return nvfp4_gemm(ws + l.a_codes, ws + l.a_sf, g_a, ws + l.b_codes, ws + l.b_sf, g_b, pl.gemm_m, pl.gemm_n,
+  uint8_t* const slots = gscale_mode == NVFP4_G_AMAX ? ws : nullptr;
+  const LayerOperand ops[2] = {
+      operand(a, pl.a_rows, pl.a_cols, pl.a_transposed, ra, ws + l.a_codes, ws + l.a_sf, ga, slots ? slots + l.a_g : nullptr),
+      operand(b, pl.b_rows, pl.b_cols, pl.b_transposed, rb, ws + l.b_codes, ws + l.b_sf, gb, slots ? slots + l.b_g : nullptr)};
+  const float* g[2];
+  if (int st = quantize_operands(ops, 2, dtype, gscale_mode, g, stream)) return st;
+  return nvfp4_gemm(ws + l.a_codes, ws + l.a_sf, g[0], ws + l.b_codes, ws + l.b_sf, g[1], pl.gemm_m, pl.gemm_n,
                     pl.gemm_k, out, out_dtype, pl.gemm_n, stream);
 }
 
@@ -150,21 +146,12 @@ extern "C" int nvfp4_linear_fwd_qout(const void* X, const void* W, int dtype, in
   const Layout l = make_layout(pl);
   if (!workspace || workspace_bytes < l.total || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return NVFP4_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  const float* g_x = nullptr;
-  const float* g_w = nullptr;
-  int st;
-  if (gscale_mode == NVFP4_G_AMAX) {
-    float* wa = reinterpret_cast<float*>(ws + l.a_g);
-    float* wb = reinterpret_cast<float*>(ws + l.b_g);
-    const AmaxOperand ops[2] = {{X, M, K, wa}, {W, N, K, wb}};
-    if ((st = tensor_amax_scales(ops, 2, dtype, amax_scratch(wa), cuda_stream))) return st;
-    g_x = wa; g_w = wb;
-  } else if (gscale_mode == NVFP4_G_GIVEN) {
-    g_x = gx; g_w = gw;
-  }
-  if ((st = nvfp4_quantize(X, dtype, M, K, K, 0, g_x, rx, ws + l.a_codes, ws + l.a_sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))) return st;
-  if ((st = nvfp4_quantize(W, dtype, N, K, K, 0, g_w, rw, ws + l.b_codes, ws + l.b_sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))) return st;
-  return nvfp4_gemm_quantized(ws + l.a_codes, ws + l.a_sf, g_x, ws + l.b_codes, ws + l.b_sf, g_w, M, N, K, gy, ry, y_codes,
+  uint8_t* const slots = gscale_mode == NVFP4_G_AMAX ? ws : nullptr;
+  const LayerOperand ops[2] = {operand(X, M, K, 0, rx, ws + l.a_codes, ws + l.a_sf, gx, slots ? slots + l.a_g : nullptr),
+                               operand(W, N, K, 0, rw, ws + l.b_codes, ws + l.b_sf, gw, slots ? slots + l.b_g : nullptr)};
+  const float* g[2];
+  if (int st = quantize_operands(ops, 2, dtype, gscale_mode, g, cuda_stream)) return st;
+  return nvfp4_gemm_quantized(ws + l.a_codes, ws + l.a_sf, g[0], ws + l.b_codes, ws + l.b_sf, g[1], M, N, K, gy, ry, y_codes,
                               y_scales, sf_layout, cuda_stream);
 }
 
@@ -184,17 +171,9 @@ extern "C" int nvfp4_linear_fwd_qin(const uint8_t* x_codes, const uint8_t* x_sca
   const Layout l = make_layout(pl);
   if (!workspace || workspace_bytes < l.total || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return NVFP4_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  const float* g_w = nullptr;
-  int st;
-  if (gscale_mode == NVFP4_G_AMAX) {
-    float* wb = reinterpret_cast<float*>(ws + l.b_g);
-    const AmaxOperand op = {W, N, K, wb};
-    if ((st = tensor_amax_scales(&op, 1, dtype, amax_scratch(wb), cuda_stream))) return st;
-    g_w = wb;
-  } else if (gscale_mode == NVFP4_G_GIVEN) {
-    g_w = gw;
-  }
-  if ((st = nvfp4_quantize(W, dtype, N, K, K, 0, g_w, rw, ws + l.b_codes, ws + l.b_sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))) return st;
+  const LayerOperand op = operand(W, N, K, 0, rw, ws + l.b_codes, ws + l.b_sf, gw, gscale_mode == NVFP4_G_AMAX ? ws + l.b_g : nullptr);
+  const float* g_w;
+  if (int st = quantize_operands(&op, 1, dtype, gscale_mode, &g_w, cuda_stream)) return st;
   return nvfp4_gemm(x_codes, x_scales, gx, ws + l.b_codes, ws + l.b_sf, g_w, M, N, K, Y, y_dtype, N, cuda_stream);
 }
 

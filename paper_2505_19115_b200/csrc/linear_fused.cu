@@ -34,17 +34,17 @@ SavedLayout saved_layout(int64_t M, int64_t N, int64_t K) {
   return l;
 }
 
-struct FwdLayout { Operand x, w; size_t scratch, total; };
+struct FwdLayout { Operand x, w; size_t total; };
 FwdLayout fwd_layout(int64_t M, int64_t N, int64_t K) {
   FwdLayout l; size_t off = 0;
   place(off, M, K, &l.x);
   place(off, N, K, &l.w);
-  l.scratch = off; off = align256(off + 64);          // zeroed words of the one-launch amax passes
+  off = align256(off + 64);                // unused; part of the size that callers were told
   l.total = off;
   return l;
 }
 
-struct BwdLayout { Operand dy, dyt, wt, xt; size_t gdy, gw, gx, scratch, total; };
+struct BwdLayout { Operand dy, dyt, wt, xt; size_t gdy, gw, gx, total; };
 BwdLayout bwd_layout(int64_t M, int64_t N, int64_t K, bool with_saved) {
   BwdLayout l; size_t off = 0;
   place(off, M, N, &l.dy);                 // Q(dY): [M, N]
@@ -54,7 +54,7 @@ BwdLayout bwd_layout(int64_t M, int64_t N, int64_t K, bool with_saved) {
   l.gdy = off; off = align256(off + sizeof(float));
   l.gw = off; off = align256(off + sizeof(float));
   l.gx = off; off = align256(off + sizeof(float));
-  l.scratch = off; off = align256(off + 64);
+  off = align256(off + 64);                // unused; part of the size that callers were told
   l.total = off;
   return l;
 }
@@ -70,10 +70,8 @@ bool buffer_ok(const void* p, size_t have, size_t need) {
   return p && have >= need && (reinterpret_cast<uintptr_t>(p) & 255u) == 0;
 }
 
-// Where a scale comes from according to gscale_mode: nowhere, the slot the amax pass fills, or the caller.
-const float* scale_source(int gscale_mode, const float* slot, const float* given) {
-  return gscale_mode == NVFP4_G_AMAX ? slot : gscale_mode == NVFP4_G_GIVEN ? given : nullptr;
-}
+// The slot of a scale, where the mode has one filled.
+float* scale_slot(uint8_t* base, size_t at, bool used) { return used ? reinterpret_cast<float*>(base + at) : nullptr; }
 
 }  // namespace
 }  // namespace nvfp4
@@ -108,48 +106,24 @@ extern "C" int nvfp4_linear_fwd_save(const void* X, const void* W, int dtype, in
   if (!buffer_ok(saved, saved_bytes, sl.total) || !buffer_ok(workspace, workspace_bytes, fl.total)) return NVFP4_ERR_WORKSPACE;
   uint8_t* sv = static_cast<uint8_t*>(saved);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  float* sgx = reinterpret_cast<float*>(sv + sl.gx);
-  float* sgw = reinterpret_cast<float*>(sv + sl.gw);
-  if (gscale_mode == NVFP4_G_GIVEN) {       // the backward pass reads the scales from `saved`
-    if (!gx || !gw) return NVFP4_ERR_NULL;
-    if (cudaMemcpyAsync(sgx, gx, sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess) return NVFP4_ERR_CUDA;
-    if (cudaMemcpyAsync(sgw, gw, sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess) return NVFP4_ERR_CUDA;
-  }
-  const float *g_x = scale_source(gscale_mode, sgx, gx), *g_w = scale_source(gscale_mode, sgw, gw);
-  unsigned int* scratch = reinterpret_cast<unsigned int*>(ws + fl.scratch);
-  const AmaxOperand ops[2] = {{W, N, K, sgw}, {X, M, K, sgx}};
-  const bool amax = gscale_mode == NVFP4_G_AMAX;
-  // Large operands one by one, W first: amax(W) leaves the (smaller) weight tensor in L2 for the quantizer that follows it.
-  const bool merged = amax && amax_merge(ops, 2, dtype);
-  if (merged) {
-    if (int st = tensor_amax_scales(ops, 2, dtype, scratch, cuda_stream)) return st;
-  } else if (amax) {
-    if (zero_words(scratch, 4, s) != cudaSuccess) return NVFP4_ERR_CUDA;
-    if (int st = tensor_amax_scale_ws(W, dtype, N, K, K, sgw, scratch, true, cuda_stream)) return st;
-  }
-  if (int st = nvfp4_quantize_dual(W, dtype, N, K, K, g_w, rw, ws + fl.w.codes, ws + fl.w.sf, rwt, sv + sl.wt.codes,
-                                   sv + sl.wt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
-    return st;
-  if (amax && !merged)
-    if (int st = tensor_amax_scale_ws(X, dtype, M, K, K, sgx, scratch + 2, true, cuda_stream)) return st;
-  if (int st = nvfp4_quantize_dual(X, dtype, M, K, K, g_x, rx, ws + fl.x.codes, ws + fl.x.sf, rxt, sv + sl.xt.codes,
-                                   sv + sl.xt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
-    return st;
-  return nvfp4_gemm(ws + fl.x.codes, ws + fl.x.sf, g_x, ws + fl.w.codes, ws + fl.w.sf, g_w, M, N, K, Y, y_dtype, N,
+  if (gscale_mode == NVFP4_G_GIVEN && (!gx || !gw)) return NVFP4_ERR_NULL;
+  // The backward pass reads the scales from `saved`, given ones too.  W first: its pass leaves the (smaller) weight tensor in
+  // the level-two cache for the quantizer that follows it.
+  const bool kept = gscale_mode != NVFP4_G_NONE;
+  const LayerOperand ops[2] = {
+      {W, N, K, rw, ws + fl.w.codes, ws + fl.w.sf, rwt, sv + sl.wt.codes, sv + sl.wt.sf, gw, scale_slot(sv, sl.gw, kept)},
+      {X, M, K, rx, ws + fl.x.codes, ws + fl.x.sf, rxt, sv + sl.xt.codes, sv + sl.xt.sf, gx, scale_slot(sv, sl.gx, kept)}};
+  const float* g[2];
+  if (int st = quantize_operands(ops, 2, dtype, gscale_mode, g, cuda_stream)) return st;
+  return nvfp4_gemm(ws + fl.x.codes, ws + fl.x.sf, g[1], ws + fl.w.codes, ws + fl.w.sf, g[0], M, N, K, Y, y_dtype, N,
                     cuda_stream);
 }
 
 namespace {
-// dY both ways from one read, then dX = Q(dY) . Q(W^T)^T and dW = Q(dY^T) . Q(X^T)^T.
-int run_bwd(const void* dY, int dtype, int64_t M, int64_t N, int64_t K, const float* g_dy,
-            const nvfp4_rounding* rdy, const nvfp4_rounding* rdyt,
-            const uint8_t* wt_codes, const uint8_t* wt_sf, const float* g_w,
-            const uint8_t* xt_codes, const uint8_t* xt_sf, const float* g_x,
-            void* dX, int dx_dtype, void* dW, int dw_dtype, uint8_t* ws, const BwdLayout& bl, void* stream) {
-  if (int st = nvfp4_quantize_dual(dY, dtype, M, N, N, g_dy, rdy, ws + bl.dy.codes, ws + bl.dy.sf, rdyt,
-                                   ws + bl.dyt.codes, ws + bl.dyt.sf, NVFP4_SF_SWIZZLED_128x4, stream))
-    return st;
+// dX = Q(dY) . Q(W^T)^T and dW = Q(dY^T) . Q(X^T)^T
+int gradients(int64_t M, int64_t N, int64_t K, const float* g_dy, const uint8_t* wt_codes, const uint8_t* wt_sf, const float* g_w,
+              const uint8_t* xt_codes, const uint8_t* xt_sf, const float* g_x,
+              void* dX, int dx_dtype, void* dW, int dw_dtype, const uint8_t* ws, const BwdLayout& bl, void* stream) {
   return gemm_two({ws + bl.dy.codes, ws + bl.dy.sf, g_dy, wt_codes, wt_sf, g_w, M, K, N, dX, dx_dtype, K},
                   {ws + bl.dyt.codes, ws + bl.dyt.sf, g_dy, xt_codes, xt_sf, g_x, N, K, M, dW, dw_dtype, K}, stream);
 }
@@ -170,16 +144,15 @@ extern "C" int nvfp4_linear_bwd_saved(const void* dY, int dtype, int64_t M, int6
   const uint8_t* sv = static_cast<const uint8_t*>(saved);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   if (gscale_mode == NVFP4_G_GIVEN && !gdy) return NVFP4_ERR_NULL;
-  float* sgdy = reinterpret_cast<float*>(ws + bl.gdy);
-  const float* g_dy = scale_source(gscale_mode, sgdy, gdy);
-  const AmaxOperand op = {dY, M, N, sgdy};
-  if (gscale_mode == NVFP4_G_AMAX)
-    if (int st = tensor_amax_scales(&op, 1, dtype, reinterpret_cast<unsigned int*>(ws + bl.scratch), cuda_stream)) return st;
+  const LayerOperand op = {dY, M, N, rdy, ws + bl.dy.codes, ws + bl.dy.sf, rdyt, ws + bl.dyt.codes, ws + bl.dyt.sf, gdy,
+                           scale_slot(ws, bl.gdy, gscale_mode == NVFP4_G_AMAX)};
+  const float* g_dy;
+  if (int st = quantize_operands(&op, 1, dtype, gscale_mode, &g_dy, cuda_stream)) return st;
   const bool scaled = gscale_mode != NVFP4_G_NONE;     // must match the mode nvfp4_linear_fwd_save ran with
   const float* g_x = scaled ? reinterpret_cast<const float*>(sv + sl.gx) : nullptr;
   const float* g_w = scaled ? reinterpret_cast<const float*>(sv + sl.gw) : nullptr;
-  return run_bwd(dY, dtype, M, N, K, g_dy, rdy, rdyt, sv + sl.wt.codes, sv + sl.wt.sf, g_w, sv + sl.xt.codes, sv + sl.xt.sf,
-                 g_x, dX, dx_dtype, dW, dw_dtype, ws, bl, cuda_stream);
+  return gradients(M, N, K, g_dy, sv + sl.wt.codes, sv + sl.wt.sf, g_w, sv + sl.xt.codes, sv + sl.xt.sf, g_x, dX, dx_dtype, dW, dw_dtype,
+                   ws, bl, cuda_stream);
 }
 
 extern "C" int nvfp4_linear_bwd(const void* dY, const void* W, const void* X, int dtype, int64_t M, int64_t N, int64_t K,
@@ -195,15 +168,13 @@ extern "C" int nvfp4_linear_bwd(const void* dY, const void* W, const void* X, in
   if (!buffer_ok(workspace, workspace_bytes, bl.total)) return NVFP4_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   if (gscale_mode == NVFP4_G_GIVEN && (!gdy || !gw || !gx)) return NVFP4_ERR_NULL;
-  float *sgdy = reinterpret_cast<float*>(ws + bl.gdy), *sgw = reinterpret_cast<float*>(ws + bl.gw), *sgx = reinterpret_cast<float*>(ws + bl.gx);
-  const float *g_dy = scale_source(gscale_mode, sgdy, gdy), *g_w = scale_source(gscale_mode, sgw, gw), *g_x = scale_source(gscale_mode, sgx, gx);
-  const AmaxOperand ops[3] = {{dY, M, N, sgdy}, {W, N, K, sgw}, {X, M, K, sgx}};
-  if (gscale_mode == NVFP4_G_AMAX)
-    if (int st = tensor_amax_scales(ops, 3, dtype, reinterpret_cast<unsigned int*>(ws + bl.scratch), cuda_stream)) return st;
-  if (int st = nvfp4_quantize(W, dtype, N, K, K, 1, g_w, rwt, ws + bl.wt.codes, ws + bl.wt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
-    return st;
-  if (int st = nvfp4_quantize(X, dtype, M, K, K, 1, g_x, rxt, ws + bl.xt.codes, ws + bl.xt.sf, NVFP4_SF_SWIZZLED_128x4, cuda_stream))
-    return st;
-  return run_bwd(dY, dtype, M, N, K, g_dy, rdy, rdyt, ws + bl.wt.codes, ws + bl.wt.sf, g_w, ws + bl.xt.codes, ws + bl.xt.sf,
-                 g_x, dX, dx_dtype, dW, dw_dtype, ws, bl, cuda_stream);
+  const bool amax = gscale_mode == NVFP4_G_AMAX;
+  const LayerOperand ops[3] = {
+      {W, N, K, nullptr, nullptr, nullptr, rwt, ws + bl.wt.codes, ws + bl.wt.sf, gw, scale_slot(ws, bl.gw, amax)},
+      {X, M, K, nullptr, nullptr, nullptr, rxt, ws + bl.xt.codes, ws + bl.xt.sf, gx, scale_slot(ws, bl.gx, amax)},
+      {dY, M, N, rdy, ws + bl.dy.codes, ws + bl.dy.sf, rdyt, ws + bl.dyt.codes, ws + bl.dyt.sf, gdy, scale_slot(ws, bl.gdy, amax)}};
+  const float* g[3];
+  if (int st = quantize_operands(ops, 3, dtype, gscale_mode, g, cuda_stream)) return st;
+  return gradients(M, N, K, g[2], ws + bl.wt.codes, ws + bl.wt.sf, g[0], ws + bl.xt.codes, ws + bl.xt.sf, g[1], dX, dx_dtype, dW, dw_dtype,
+                   ws, bl, cuda_stream);
 }

@@ -268,12 +268,6 @@ __device__ __forceinline__ uint32_t absmax_nan_bf16x2(uint32_t a, uint32_t b) {
   return r;
 }
 
-// g of a tensor whose largest |x| has these bits: amax / 2688, 1 for an all-zero tensor.
-__device__ __forceinline__ float amax_to_scale(uint32_t bits) {
-  const float amax = __uint_as_float(bits);
-  return (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 2688.0f);
-}
-
 // 32 bytes at position j, zeros past the end.
 __device__ __forceinline__ void load_vec32(const uint32_t* x, int64_t j, int64_t n_vec32, uint32_t (&w)[8]) {
   if (j < n_vec32) {
@@ -326,19 +320,21 @@ struct AmaxBits {
 constexpr int kSmallAmaxCluster = 8, kSmallAmaxThreads = 1024;
 constexpr int64_t kSmallAmaxBytes = 2 << 20;
 
-template <typename T>
-__device__ __forceinline__ void amax_cluster(const uint32_t* x, int64_t n_vec32, float* g_out, int late, uint32_t rank) {
-  __shared__ uint32_t warp_max[kSmallAmaxThreads / 32];
-  __shared__ uint32_t block_max[kSmallAmaxCluster];            // the first block's copy is used
+// The maximum of what a cluster's blocks (`block` of `blocks` on the tensor) read, in the first block's first thread.
+template <typename T, int THREADS, int CLUSTER>
+__device__ __forceinline__ uint32_t cluster_amax_bits(const uint32_t* x, int64_t n_vec32, int block, int blocks, int late, uint32_t rank) {
+  __shared__ uint32_t warp_max[THREADS / 32];
+  __shared__ uint32_t block_max[CLUSTER];                      // the first block's copy is used
   // The first block's shared memory may be written only once that block runs: every block arrives here and waits behind its
   // loads, which hide the rendezvous (256 x 512 in bf16, back to back: 1.85 -> 1.89 us).
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   if (!late) { grid_dependency_wait(); grid_dependency_trigger(); }
+  const int64_t stride = (int64_t)blocks * THREADS;
   AmaxBits<T> acc;
-  for (int64_t i = (int64_t)rank * kSmallAmaxThreads + threadIdx.x; i < n_vec32; i += 4 * kSmallAmaxCluster * kSmallAmaxThreads) {
+  for (int64_t i = (int64_t)block * THREADS + threadIdx.x; i < n_vec32; i += 4 * stride) {
     uint32_t w[4][8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) load_vec32(x, i + u * kSmallAmaxCluster * kSmallAmaxThreads, n_vec32, w[u]);
+    for (int u = 0; u < 4; ++u) load_vec32(x, i + u * stride, n_vec32, w[u]);
 #pragma unroll
     for (int u = 0; u < 4; ++u) acc.add8(w[u]);
   }
@@ -347,7 +343,7 @@ __device__ __forceinline__ void amax_cluster(const uint32_t* x, int64_t n_vec32,
   __syncthreads();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (threadIdx.x < 32) {
-    bits = __reduce_max_sync(0xFFFFFFFFu, warp_max[threadIdx.x]);
+    bits = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < THREADS / 32 ? warp_max[threadIdx.x] : 0u);
     if (threadIdx.x == 0) {
       const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&block_max[rank]);
       asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, 0;\n\tst.shared::cluster.u32 [a], %1;\n\t}" ::"r"(mine), "r"(bits) : "memory");
@@ -355,12 +351,17 @@ __device__ __forceinline__ void amax_cluster(const uint32_t* x, int64_t n_vec32,
   }
   if (late) { grid_dependency_wait(); grid_dependency_trigger(); }
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  uint32_t m = 0u;
   if (rank == 0 && threadIdx.x == 0) {
-    uint32_t m = 0u;
 #pragma unroll
-    for (int i = 0; i < kSmallAmaxCluster; ++i) m = max(m, block_max[i]);
-    *g_out = amax_to_scale(m);
+    for (int i = 0; i < CLUSTER; ++i) m = max(m, block_max[i]);
   }
+  return m;
+}
+template <typename T>
+__device__ __forceinline__ void amax_cluster(const uint32_t* x, int64_t n_vec32, float* g_out, int late, uint32_t rank) {
+  const uint32_t m = cluster_amax_bits<T, kSmallAmaxThreads, kSmallAmaxCluster>(x, n_vec32, (int)rank, kSmallAmaxCluster, late, rank);
+  if (rank == 0 && threadIdx.x == 0) *g_out = amax_to_scale(m);
 }
 template <typename T>
 __global__ void __cluster_dims__(kSmallAmaxCluster, 1, 1) __launch_bounds__(kSmallAmaxThreads)
@@ -384,6 +385,31 @@ __global__ void __cluster_dims__(kSmallAmaxCluster, 1, 1) __launch_bounds__(kSma
 amax_cluster_batch_kernel(const __grid_constant__ AmaxBatch batch) {
   const AmaxBatch::Op& op = batch.op[blockIdx.x / kSmallAmaxCluster];
   amax_cluster<T>(op.x, op.n_vec32, op.g, 0, blockIdx.x % kSmallAmaxCluster);
+}
+
+// Tensors above that whose quantizer can reduce them (ScaleSource): every cluster leaves the maximum of its share in a word of
+// its own, so that nothing has to be zeroed before and no ticket taken after: 2080 x 2848 with its quantizer 15.4 -> 14.0 us.
+// Two blocks a cluster, one on each multiprocessor: clusters of eight do not all fit on the chip at once, and the last of them
+// then run alone (16384 x 11008: 75 -> 130 us).  63 of them, 126 multiprocessors, is what a scale's slot has words for.
+constexpr int kSweepCluster = 2, kSweepThreads = 1024, kSweepWords = kScaleSlotBytes / 4 - 1;
+struct AmaxSweep {
+  struct Op {
+    const uint32_t* x;
+    int64_t n_vec32;
+    uint32_t* maxima;
+    int first, clusters;           // of the grid
+  } op[kMaxLayerOperands];
+  int n;
+};
+template <typename T>
+__global__ void __cluster_dims__(kSweepCluster, 1, 1) __launch_bounds__(kSweepThreads)
+amax_sweep_kernel(const __grid_constant__ AmaxSweep p) {
+  const int cluster = blockIdx.x / kSweepCluster, rank = blockIdx.x % kSweepCluster;
+  const int which = (p.n > 1 && cluster >= p.op[1].first) + (p.n > 2 && cluster >= p.op[2].first);
+  const AmaxSweep::Op& op = p.op[which];
+  const uint32_t m = cluster_amax_bits<T, kSweepThreads, kSweepCluster>(op.x, op.n_vec32, (cluster - op.first) * kSweepCluster + rank,
+                                                                        op.clusters * kSweepCluster, 0, rank);
+  if (rank == 0 && threadIdx.x == 0) op.maxima[cluster - op.first] = m;
 }
 
 // Strided tensors: 16-byte loads, grid-stride.
@@ -464,6 +490,16 @@ __global__ void amax_finalize_kernel(float* out) {
   grid_dependency_wait();
   grid_dependency_trigger();
   *out = amax_to_scale(__float_as_uint(*out));
+}
+
+struct ScalePairs {
+  const float* from[kMaxLayerOperands];
+  float* to[kMaxLayerOperands];
+};
+__global__ void copy_scales_kernel(const __grid_constant__ ScalePairs p, int n) {
+  grid_dependency_wait();
+  grid_dependency_trigger();
+  if ((int)threadIdx.x < n && p.to[threadIdx.x]) *p.to[threadIdx.x] = load_scale(p.from[threadIdx.x]);
 }
 
 __global__ void zero_words_kernel(unsigned int* words, int n) {
@@ -629,6 +665,7 @@ extern "C" int nvfp4_quantize_dual(const void* x, int dtype, int64_t rows, int64
 }
 
 namespace nvfp4 {
+namespace {
 // Per-tensor scale in one launch where the tensor allows it (dense, 32-byte aligned); `scratch_zeroed` is two
 // zeroed 32-bit words in device memory that the kernel leaves zeroed.  Otherwise the three-step public path.
 int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* g_out,
@@ -649,38 +686,24 @@ int tensor_amax_scale_ws(const void* x, int dtype, int64_t rows, int64_t cols, i
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
-// Together below 64 MB the operands still lie in the level-two cache when their quantizers read them, so nothing is lost by
-// sweeping them all first, and a launch and its latency are saved for each but one: 256-token layer step 36.8 -> 34.9 us,
-// 2080 x 1056 x 2848 62.6 -> 61.7, 3584 x 1440 x 1952 68.6 -> 67.2, 544 x 800 x 8288 fine-tuning step 84.6 -> 81.9; the
-// 350M-class QKV step (39 MB) +-0.5 %.
-bool amax_merge(const AmaxOperand* ops, int n, int dtype) {
-  int64_t total = 0;
-  for (int i = 0; i < n; ++i) {
-    if (!ops[i].x || !amax_flat_ok(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols)) return false;
-    total += ops[i].rows * ops[i].cols * (dtype == NVFP4_BF16 ? 2 : 4);
-  }
-  return n > 1 && total <= (int64_t)64 << 20;
-}
+int64_t operand_bytes(const LayerOperand& op, int dtype) { return op.rows * op.cols * (dtype == NVFP4_BF16 ? 2 : 4); }
+bool needs_scratch(const LayerOperand& op, int dtype) { return operand_bytes(op, dtype) > kSmallAmaxBytes; }
+cudaError_t zero_words(unsigned int* words, int n, cudaStream_t s) { return launch_overlapped(zero_words_kernel, 1, 32, 0, s, words, n); }
+// Two words an operand for the passes that take a ticket, behind the first operand's scale.
+unsigned int* amax_scratch(const LayerOperand* ops, int i) { return reinterpret_cast<unsigned int*>(ops[0].slot) + 16 + 2 * i; }
 
-int tensor_amax_scales(const AmaxOperand* ops, int n, int dtype, unsigned int* scratch, void* cuda_stream) {
-  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  if (int st = check_arch()) return st;
-  bool sweep = false;
-  for (int i = 0; i < n; ++i) sweep = sweep || amax_needs_scratch(dtype, ops[i].rows * ops[i].cols);
-  if (sweep && zero_words(scratch, 2 * n, s) != cudaSuccess) return NVFP4_ERR_CUDA;
-  if (!amax_merge(ops, n, dtype)) {
-    for (int i = 0; i < n; ++i)
-      if (int st = tensor_amax_scale_ws(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols, ops[i].g, scratch + 2 * i, sweep || i > 0, cuda_stream))
-        return st;
-    return NVFP4_OK;
-  }
+// One launch for the amax passes of all operands (dense, 32-byte aligned), which leaves their scales in their slots.
+int amax_together(const LayerOperand* ops, int n, int dtype, cudaStream_t s) {
   AmaxBatch b = {};
   b.n = n;
   int64_t total = 0;
+  bool sweep = false;
   for (int i = 0; i < n; ++i) {
-    b.op[i] = {static_cast<const uint32_t*>(ops[i].x), ops[i].rows * ops[i].cols * (dtype == NVFP4_BF16 ? 2 : 4) / 32, ops[i].g, scratch + 2 * i, 0, 0};
+    b.op[i] = {static_cast<const uint32_t*>(ops[i].x), operand_bytes(ops[i], dtype) / 32, ops[i].slot, amax_scratch(ops, i), 0, 0};
     total += b.op[i].n_vec32;
+    sweep = sweep || needs_scratch(ops[i], dtype);
   }
+  if (sweep && zero_words(amax_scratch(ops, 0), 2 * n, s) != cudaSuccess) return NVFP4_ERR_CUDA;
   int first = 0;
   for (int i = 0; i < n; ++i) {                              // blocks in proportion to the sizes, one wave in all
     const int64_t share = (int64_t)sm_count() * kAmaxBlocksPerSm * b.op[i].n_vec32 / total;
@@ -697,10 +720,87 @@ int tensor_amax_scales(const AmaxOperand* ops, int n, int dtype, unsigned int* s
   return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
-bool amax_needs_scratch(int dtype, int64_t elements) { return elements * (dtype == NVFP4_BF16 ? 2 : 4) > kSmallAmaxBytes; }
+// The same for a quantizer that reduces maxima.
+int amax_sweep(const LayerOperand* ops, int n, int dtype, ScaleSource* src, cudaStream_t s) {
+  AmaxSweep b = {};
+  b.n = n;
+  int64_t total = 0;
+  for (int i = 0; i < n; ++i) total += operand_bytes(ops[i], dtype) / 32;
+  int first = 0;
+  for (int i = 0; i < n; ++i) {                              // clusters in proportion to the sizes, one wave in all
+    const int64_t n32 = operand_bytes(ops[i], dtype) / 32, share = (int64_t)sm_count() / kSweepCluster * n32 / total;
+    const int clusters = (int)std::min<int64_t>({ceil_div(n32, (int64_t)kSweepThreads * 4 * kSweepCluster), std::max<int64_t>(share, 1), kSweepWords});
+    b.op[i] = {static_cast<const uint32_t*>(ops[i].x), n32, reinterpret_cast<uint32_t*>(ops[i].slot) + 1, first, clusters};
+    first += clusters;
+    src[i] = {nullptr, b.op[i].maxima, clusters, ops[i].slot};
+  }
+  const cudaError_t e = dtype == NVFP4_BF16 ? launch_overlapped(amax_sweep_kernel<__nv_bfloat16>, first * kSweepCluster, kSweepThreads, 0, s, b)
+                                            : launch_overlapped(amax_sweep_kernel<float>, first * kSweepCluster, kSweepThreads, 0, s, b);
+  return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
 
-cudaError_t zero_words(unsigned int* words, int n, cudaStream_t s) {
-  return launch_overlapped(zero_words_kernel, 1, 32, 0, s, words, n);
+int quantize_operand(const LayerOperand& op, int dtype, const float* g, void* stream) {
+  constexpr int kLayout = NVFP4_SF_SWIZZLED_128x4;
+  if (op.rr && op.rt)
+    return nvfp4_quantize_dual(op.x, dtype, op.rows, op.cols, op.cols, g, op.rr, op.codes_r, op.scales_r, op.rt, op.codes_t, op.scales_t, kLayout, stream);
+  if (op.rr) return nvfp4_quantize(op.x, dtype, op.rows, op.cols, op.cols, 0, g, op.rr, op.codes_r, op.scales_r, kLayout, stream);
+  return nvfp4_quantize(op.x, dtype, op.rows, op.cols, op.cols, 1, g, op.rt, op.codes_t, op.scales_t, kLayout, stream);
+}
+}  // namespace
+
+// Amax by sweeps that leave maxima, and one quantizer launch for all operands, while they have at most this many bytes together.
+// Beyond it the sweep with a ticket wins, whose small blocks start one by one in the tail of the kernel before, and so do the
+// quantizers made for one tensor.  us, ticket / maxima: 2080 x 2848 (12 MB) with its quantizer 15.5 / 13.8, both operands of
+// 4864 x 1120 x 800 (13 MB) and their step 52.9 / 51.1, 16384 x 1024 (34 MB) 21.4 / 22.2, 16384 x 3072 49.0 / 53.5, fp32 step 16384 x 2816 x 1024
+// (67 MB of dY) 206.7 / 210.4.
+constexpr int64_t kSweepBytes = (int64_t)24 << 20;
+
+int quantize_operands(const LayerOperand* ops, int n, int dtype, int gscale_mode, const float** g, void* cuda_stream) {
+  if (int st = check_arch()) return st;
+  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  const bool amax = gscale_mode == NVFP4_G_AMAX, given = gscale_mode == NVFP4_G_GIVEN;
+  ScaleSource src[kMaxLayerOperands];
+  int64_t bytes = 0;
+  bool flat = true, sweep = false;
+  for (int i = 0; i < n; ++i) {
+    for (const nvfp4_rounding* r : {ops[i].rr, ops[i].rt})
+      if (r && ((r->mode != NVFP4_RTN && r->mode != NVFP4_SR) || r->reserved != 0)) return NVFP4_ERR_ENUM;
+    if (!aligned16(ops[i].x)) return NVFP4_ERR_ALIGN;
+    g[i] = amax ? ops[i].slot : given ? ops[i].given : nullptr;
+    src[i] = {g[i], nullptr, 0, given ? ops[i].slot : nullptr};
+    bytes += operand_bytes(ops[i], dtype);
+    flat = flat && amax_flat_ok(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols);
+    sweep = sweep || needs_scratch(ops[i], dtype);
+  }
+  const bool batch = tile_batch_eligible(ops, n, dtype);
+  if (!amax) {
+    if (batch && n > 1) return tile_quantize_batch(ops, src, n, dtype, s);
+    if (given) {
+      ScalePairs p = {};
+      bool any = false;
+      for (int i = 0; i < n; ++i) { p.from[i] = ops[i].given; p.to[i] = ops[i].slot; any = any || ops[i].slot; }
+      if (any && launch_overlapped(copy_scales_kernel, 1, 32, 0, s, p, n) != cudaSuccess) return NVFP4_ERR_CUDA;
+    }
+  } else if (batch && flat && bytes <= kSweepBytes && (sweep || n > 1)) {
+    if (int st = sweep ? amax_sweep(ops, n, dtype, src, s) : amax_together(ops, n, dtype, s)) return st;
+    return tile_quantize_batch(ops, src, n, dtype, s);
+  } else if (n > 1 && flat && bytes <= (int64_t)64 << 20) {
+    // Together below 64 MB the operands still lie in the level-two cache when their quantizers read them, so nothing is lost by
+    // sweeping them all first, and a launch and its latency are saved for each but one.
+    if (int st = amax_together(ops, n, dtype, s)) return st;
+  } else {
+    // One by one: the pass leaves the end of its tensor in the cache for the quantizer behind it.
+    if (sweep && zero_words(amax_scratch(ops, 0), 2 * n, s) != cudaSuccess) return NVFP4_ERR_CUDA;
+    for (int i = 0; i < n; ++i) {
+      if (int st = tensor_amax_scale_ws(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols, ops[i].slot, amax_scratch(ops, i), sweep || i > 0, cuda_stream))
+        return st;
+      if (int st = quantize_operand(ops[i], dtype, g[i], cuda_stream)) return st;
+    }
+    return NVFP4_OK;
+  }
+  for (int i = 0; i < n; ++i)
+    if (int st = quantize_operand(ops[i], dtype, g[i], cuda_stream)) return st;
+  return NVFP4_OK;
 }
 }  // namespace nvfp4
 
@@ -717,8 +817,8 @@ extern "C" int nvfp4_tensor_amax_scale(const void* x, int dtype, int64_t rows, i
   if (flat && total_bytes <= kSmallAmaxBytes)
     return launch_amax_cluster(x, dtype, total_bytes / 32, global_scale_out, false, s) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
   unsigned int* bits = reinterpret_cast<unsigned int*>(global_scale_out);
-  if (zero_words(bits, 1, s) != cudaSuccess) return NVFP4_ERR_CUDA;
-  cudaError_t e;
+  cudaError_t e = launch_overlapped(zero_words_kernel, 1, 32, 0, s, bits, 1);
+  if (e != cudaSuccess) return NVFP4_ERR_CUDA;
   if (flat) {
     const int64_t n32 = total_bytes / 32;
     const int64_t fb = std::min(ceil_div(n32, (int64_t)kAmaxThreads * 4), (int64_t)sm_count() * kAmaxBlocksPerSm);

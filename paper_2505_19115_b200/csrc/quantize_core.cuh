@@ -22,11 +22,29 @@ struct QuantParams {
   int64_t nsb;      // scale blocks per quantized row: Kq / 16 (NVFP4) or Kq / 32 (MXFP4)
 };
 
+// g of a tensor whose largest |x| has these bits: amax / 2688, 1 for an all-zero tensor.
+__device__ __forceinline__ float amax_to_scale(uint32_t bits) {
+  const float amax = __uint_as_float(bits);
+  return (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 2688.0f);
+}
+
+// The per-tensor scale of a source, in every thread of a warp (behind the wait).
+__device__ __forceinline__ float read_scale(const ScaleSource& s) {
+  if (s.n == 0) return load_scale(s.g);
+  uint32_t m = 0u;
+  for (int i = threadIdx.x & 31; i < s.n; i += 32) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(s.maxima + i) : "memory");
+    m = max(m, v);
+  }
+  return amax_to_scale(__reduce_max_sync(0xFFFFFFFFu, m));
+}
+
 // Reciprocal of every block scale a tensor can have: entry q = 1 / (decode(q) * g), one IEEE
 // division each, 0 for the zero scale.  A block then costs one shared-memory read, not a division.
+__device__ __forceinline__ float inv_scale(uint32_t q, float g) { return (q == 0) ? 0.0f : __fdiv_rn(1.0f, __fmul_rn(e4m3_decode(q), g)); }
 __device__ __forceinline__ void build_inv_table(float* inv_table, float g) {
-  for (int q = threadIdx.x; q < 128; q += blockDim.x)
-    inv_table[q] = (q == 0) ? 0.0f : __fdiv_rn(1.0f, __fmul_rn(e4m3_decode((uint32_t)q), g));
+  for (int q = threadIdx.x; q < 128; q += blockDim.x) inv_table[q] = inv_scale((uint32_t)q, g);
 }
 
 // MXFP4: the same table over the 255 E8M0 codes, entry q = 1 / (2^(q-127) * g), 0 for code 0.

@@ -170,6 +170,35 @@ def test_gradients_of_one_launch_equal_the_single_products(shape, dx_dtype, dw_d
     assert torch.equal(want[0], got[0]) and torch.equal(want[1], got[1])
 
 
+# The layer calls quantize their operands together and take the per-tensor scale from an amax sweep's maxima: below 2 MB (one
+# cluster), above (sweeps, one quantizer launch for both), one operand below and one above, and operands too large for one launch.
+@pytest.mark.parametrize("mode", [nb.G_AMAX, nb.G_GIVEN, nb.G_NONE])
+@pytest.mark.parametrize("shape,dtype", [((64, 32, 96), torch.bfloat16), ((2080, 1056, 2848), torch.bfloat16), ((2080, 1056, 2848), torch.float32),
+                                         ((8224, 160, 224), torch.bfloat16), ((16416, 4128, 32), torch.bfloat16)])
+def test_layer_calls_equal_the_single_calls(shape, dtype, mode):
+    M, K, N = shape
+    X, W, dY = (t.cuda().to(dtype) for t in synth.linear_inputs(M, K, N, seed=34, grad_std=1e-3))
+    r = [nb.Rounding(nb.RTN), nb.Rounding(nb.SR, 7, 0), nb.Rounding(nb.SR, 7, 1), nb.Rounding(nb.SR, 7, 2)]
+    g = [None if mode == nb.G_NONE else nb.nvfp4_tensor_amax_scale(t) for t in (X, W, dY)]
+
+    def product(a, b, out_dtype=torch.float32):             # each operand: tensor, transposed, scale, rounding
+        qa, qb = (nb.nvfp4_quantize(t, tr, s, rr, nb.SF_SWIZZLED) for t, tr, s, rr in (a, b))
+        return nb.nvfp4_gemm(*qa, a[2], *qb, b[2], out_dtype=out_dtype)
+    want = (product((X, False, g[0], r[0]), (W, False, g[1], r[0])), product((dY, False, g[2], r[1]), (W, True, g[1], r[0])),
+            product((dY, True, g[2], r[2]), (X, True, g[0], r[3])))
+    gx, gw, gdy = g if mode == nb.G_GIVEN else (None,) * 3
+    Y, saved = nb.nvfp4_linear_fwd_save(X, W, mode, gx=gx, gw=gw, rx=r[0], rw=r[0], rxt=r[3], rwt=r[0])
+    single = (nb.nvfp4_linear_fwd(X, W, mode, gx=gx, gw=gw, rx=r[0], rw=r[0]), nb.nvfp4_linear_bwd_dx(dY, W, mode, gdy=gdy, gw=gw, rdy=r[1], rw=r[0]),
+              nb.nvfp4_linear_bwd_dw(dY, X, mode, gdy=gdy, gx=gx, rdy=r[2], rx=r[3]))
+    fused = (Y, *nb.nvfp4_linear_bwd_saved(dY, saved, K, mode, gdy=gdy, rdy=r[1], rdyt=r[2]))
+    both = nb.nvfp4_linear_bwd(dY, W, X, mode, gdy=gdy, gw=gw, gx=gx, rdy=r[1], rdyt=r[2], rwt=r[0], rxt=r[3])
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    for i in range(3):
+        assert torch.equal(want[i], single[i]) and torch.equal(want[i], fused[i]), i
+    assert torch.equal(want[1], both[0]) and torch.equal(want[2], both[1])
+
+
 # ---------------------------------------------------------------- non-finite inputs stay visible
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
 def test_non_finite_input_propagates_through_the_per_tensor_scale(bad):
