@@ -4,6 +4,9 @@ Every function has the name of the C entry point it calls (include/nvfp4.h).
 torch tensors are used for device memory and streams; all computation happens
 inside the CUDA library.  There is no CPU fallback: if the library is missing
 or a call fails, an exception is raised.
+
+The calls that launch work go through the extension module _calls (csrc/python_calls.cpp says how it takes its
+arguments), the queries through ctypes.
 """
 import ctypes as C
 import os
@@ -111,6 +114,20 @@ def lib():
     return L
 
 
+_calls = None
+
+
+def _native():
+    """The extension module, bound to the library that lib() loaded."""
+    global _calls
+    if _calls is None:
+        lib()
+        from . import _calls as module
+        module.bind(LIB_PATH)
+        _calls = module
+    return _calls
+
+
 def status_string(status: int) -> str:
     return lib().nvfp4_status_string(status).decode()
 
@@ -166,9 +183,8 @@ def nvfp4_quantize(x: torch.Tensor, transposed: bool = False, global_scale: torc
             scales = torch.empty((Rq, max(Kq // 16, 1)), dtype=torch.uint8, device=x.device)
         else:
             scales = torch.empty(max(nvfp4_sf_bytes(Rq, Kq, sf_layout), 16), dtype=torch.uint8, device=x.device)
-    st = lib().nvfp4_quantize(_ptr(x), _dtype_code(x), rows, cols, x.stride(0), int(transposed),
-                              _ptr(global_scale), C.byref(rounding), _ptr(codes), _ptr(scales), sf_layout,
-                              _stream(stream))
+    st = _native().nvfp4_quantize(x, x, rows, cols, x.stride(0), int(transposed), global_scale, rounding, codes, scales,
+                                  sf_layout, stream)
     _check(st, "nvfp4_quantize")
     return codes, scales
 
@@ -189,9 +205,8 @@ def nvfp4_quantize_dual(x: torch.Tensor, global_scale: torch.Tensor = None, roun
 
     cr, sr = bufs(rows, cols)
     ct, stt = bufs(cols, rows)
-    st = lib().nvfp4_quantize_dual(_ptr(x), _dtype_code(x), rows, cols, x.stride(0), _ptr(global_scale),
-                                   C.byref(rounding_row), _ptr(cr), _ptr(sr), C.byref(rounding_t), _ptr(ct), _ptr(stt),
-                                   sf_layout, _stream(stream))
+    st = _native().nvfp4_quantize_dual(x, x, rows, cols, x.stride(0), global_scale, rounding_row, cr, sr, rounding_t,
+                                       ct, stt, sf_layout, stream)
     _check(st, "nvfp4_quantize_dual")
     return cr, sr, ct, stt
 
@@ -212,8 +227,7 @@ def nvfp4_tensor_amax_scale(x: torch.Tensor, out: torch.Tensor = None, stream=No
     assert x.is_cuda and x.dim() == 2 and x.stride(1) == 1
     if out is None:
         out = torch.empty(1, dtype=torch.float32, device=x.device)
-    st = lib().nvfp4_tensor_amax_scale(_ptr(x), _dtype_code(x), x.shape[0], x.shape[1], x.stride(0), _ptr(out),
-                                       _stream(stream))
+    st = _native().nvfp4_tensor_amax_scale(x, x, x.shape[0], x.shape[1], x.stride(0), out, stream)
     _check(st, "nvfp4_tensor_amax_scale")
     return out
 
@@ -225,8 +239,7 @@ def nvfp4_gemm(a_codes, a_sf, a_g, b_codes, b_sf, b_g, out_dtype=torch.float32, 
     N = b_codes.shape[0]
     if out is None:
         out = torch.empty((M, N), dtype=out_dtype, device=a_codes.device)
-    st = lib().nvfp4_gemm(_ptr(a_codes), _ptr(a_sf), _ptr(a_g), _ptr(b_codes), _ptr(b_sf), _ptr(b_g),
-                          M, N, K, _ptr(out), _dtype_code(out), out.stride(0), _stream(stream))
+    st = _native().nvfp4_gemm(a_codes, a_sf, a_g, b_codes, b_sf, b_g, M, N, K, out, out, out.stride(0), stream)
     _check(st, "nvfp4_gemm")
     return out
 
@@ -242,9 +255,8 @@ def nvfp4_gemm_quantized(a_codes, a_sf, a_g, b_codes, b_sf, b_g, out_global_scal
         scales = torch.empty((M, N // 16), dtype=torch.uint8, device=a_codes.device)
     else:
         scales = torch.empty(max(nvfp4_sf_bytes(M, N, sf_layout), 16), dtype=torch.uint8, device=a_codes.device)
-    st = lib().nvfp4_gemm_quantized(_ptr(a_codes), _ptr(a_sf), _ptr(a_g), _ptr(b_codes), _ptr(b_sf), _ptr(b_g), M, N, K,
-                                    _ptr(out_global_scale), C.byref(rounding), _ptr(codes), _ptr(scales), sf_layout,
-                                    _stream(stream))
+    st = _native().nvfp4_gemm_quantized(a_codes, a_sf, a_g, b_codes, b_sf, b_g, M, N, K, out_global_scale, rounding,
+                                        codes, scales, sf_layout, stream)
     _check(st, "nvfp4_gemm_quantized")
     return codes, scales
 
@@ -263,9 +275,7 @@ def _linear(name, which, a, b, M, N, K, out_shape, gscale_mode, ga, gb, ra, rb, 
     if workspace is None:
         workspace = torch.empty(nvfp4_linear_workspace_bytes(M, N, K, which), dtype=torch.uint8, device=a.device)
     assert a.is_contiguous() and b.is_contiguous() and out.is_contiguous() and a.dtype == b.dtype
-    st = getattr(lib(), name)(_ptr(a), _ptr(b), _dtype_code(a), M, N, K, gscale_mode, _ptr(ga), _ptr(gb),
-                              C.byref(ra), C.byref(rb), _ptr(out), _dtype_code(out), _ptr(workspace),
-                              workspace.numel(), _stream(stream))
+    st = getattr(_native(), name)(a, b, a, M, N, K, gscale_mode, ga, gb, ra, rb, out, out, workspace, workspace, stream)
     _check(st, name)
     return out
 
@@ -308,10 +318,9 @@ def nvfp4_linear_fwd_qout(X, W, gy=None, ry=None, gscale_mode=G_AMAX, gx=None, g
     if workspace is None:
         workspace = torch.empty(nvfp4_linear_workspace_bytes(M, N, K, LINEAR_FWD), dtype=torch.uint8, device=X.device)
     assert X.is_contiguous() and W.is_contiguous() and X.dtype == W.dtype
-    st = lib().nvfp4_linear_fwd_qout(_ptr(X), _ptr(W), _dtype_code(X), M, N, K, gscale_mode, _ptr(gx), _ptr(gw),
-                                     C.byref(rx or Rounding(RTN)), C.byref(rw or Rounding(RTN)), _ptr(gy),
-                                     C.byref(ry or Rounding(RTN)), _ptr(codes), _ptr(scales), sf_layout,
-                                     _ptr(workspace), workspace.numel(), _stream(stream))
+    st = _native().nvfp4_linear_fwd_qout(X, W, X, M, N, K, gscale_mode, gx, gw, rx or Rounding(RTN),
+                                         rw or Rounding(RTN), gy, ry or Rounding(RTN), codes, scales, sf_layout,
+                                         workspace, workspace, stream)
     _check(st, "nvfp4_linear_fwd_qout")
     return codes, scales
 
@@ -326,9 +335,8 @@ def nvfp4_linear_fwd_qin(x_codes, x_scales, gx, W, gscale_mode=G_AMAX, gw=None, 
     if workspace is None:
         workspace = torch.empty(nvfp4_linear_workspace_bytes(M, N, K, LINEAR_FWD), dtype=torch.uint8, device=W.device)
     assert W.is_contiguous() and out.is_contiguous()
-    st = lib().nvfp4_linear_fwd_qin(_ptr(x_codes), _ptr(x_scales), _ptr(gx), _ptr(W), _dtype_code(W), M, N, K, gscale_mode,
-                                    _ptr(gw), C.byref(rw or Rounding(RTN)), _ptr(out), _dtype_code(out), _ptr(workspace),
-                                    workspace.numel(), _stream(stream))
+    st = _native().nvfp4_linear_fwd_qin(x_codes, x_scales, gx, W, W, M, N, K, gscale_mode, gw, rw or Rounding(RTN), out,
+                                        out, workspace, workspace, stream)
     _check(st, "nvfp4_linear_fwd_qin")
     return out
 
@@ -359,11 +367,9 @@ def nvfp4_linear_fwd_save(X, W, gscale_mode=G_AMAX, gx=None, gw=None, rx=None, r
         out = torch.empty((M, N), dtype=out_dtype, device=X.device)
     saved = _scratch(nvfp4_linear_saved_bytes(M, N, K), X.device, saved)
     ws = _scratch(nvfp4_linear_fused_workspace_bytes(M, N, K, FUSED_FWD_SAVE), X.device, workspace)
-    st = lib().nvfp4_linear_fwd_save(_ptr(X), _ptr(W), _dtype_code(X), M, N, K, gscale_mode, _ptr(gx), _ptr(gw),
-                                     C.byref(rx or Rounding(RTN)), C.byref(rw or Rounding(RTN)),
-                                     C.byref(rxt or Rounding(SR, 0, 2)), C.byref(rwt or Rounding(RTN)),
-                                     _ptr(out), _dtype_code(out), _ptr(saved), saved.numel(), _ptr(ws), ws.numel(),
-                                     _stream(stream))
+    st = _native().nvfp4_linear_fwd_save(X, W, X, M, N, K, gscale_mode, gx, gw, rx or Rounding(RTN),
+                                         rw or Rounding(RTN), rxt or Rounding(SR, 0, 2), rwt or Rounding(RTN), out, out,
+                                         saved, saved, ws, ws, stream)
     _check(st, "nvfp4_linear_fwd_save")
     return out, saved
 
@@ -377,10 +383,8 @@ def nvfp4_linear_bwd_saved(dY, saved, K, gscale_mode=G_AMAX, gdy=None, rdy=None,
     if dW is None:
         dW = torch.empty((N, K), dtype=dw_dtype, device=dY.device)
     ws = _scratch(nvfp4_linear_fused_workspace_bytes(M, N, K, FUSED_BWD_SAVED), dY.device, workspace)
-    st = lib().nvfp4_linear_bwd_saved(_ptr(dY), _dtype_code(dY), M, N, K, gscale_mode, _ptr(gdy),
-                                      C.byref(rdy or Rounding(SR, 0, 0)), C.byref(rdyt or Rounding(SR, 0, 1)),
-                                      _ptr(saved), saved.numel(), _ptr(dX), _dtype_code(dX), _ptr(dW), _dtype_code(dW),
-                                      _ptr(ws), ws.numel(), _stream(stream))
+    st = _native().nvfp4_linear_bwd_saved(dY, dY, M, N, K, gscale_mode, gdy, rdy or Rounding(SR, 0, 0),
+                                          rdyt or Rounding(SR, 0, 1), saved, saved, dX, dX, dW, dW, ws, ws, stream)
     _check(st, "nvfp4_linear_bwd_saved")
     return dX, dW
 
@@ -394,10 +398,9 @@ def nvfp4_linear_bwd(dY, W, X, gscale_mode=G_AMAX, gdy=None, gw=None, gx=None, r
     if dW is None:
         dW = torch.empty((N, K), dtype=dw_dtype, device=dY.device)
     ws = _scratch(nvfp4_linear_fused_workspace_bytes(M, N, K, FUSED_BWD), dY.device, workspace)
-    st = lib().nvfp4_linear_bwd(_ptr(dY), _ptr(W), _ptr(X), _dtype_code(dY), M, N, K, gscale_mode, _ptr(gdy), _ptr(gw),
-                                _ptr(gx), C.byref(rdy or Rounding(SR, 0, 0)), C.byref(rdyt or Rounding(SR, 0, 1)),
-                                C.byref(rwt or Rounding(RTN)), C.byref(rxt or Rounding(SR, 0, 2)),
-                                _ptr(dX), _dtype_code(dX), _ptr(dW), _dtype_code(dW), _ptr(ws), ws.numel(), _stream(stream))
+    st = _native().nvfp4_linear_bwd(dY, W, X, dY, M, N, K, gscale_mode, gdy, gw, gx, rdy or Rounding(SR, 0, 0),
+                                    rdyt or Rounding(SR, 0, 1), rwt or Rounding(RTN), rxt or Rounding(SR, 0, 2), dX, dX,
+                                    dW, dW, ws, ws, stream)
     _check(st, "nvfp4_linear_bwd")
     return dX, dW
 
@@ -419,9 +422,8 @@ def nvfp4_quantize_mx(x, transposed: bool = False, global_scale=None, rounding: 
     else:
         scales = torch.empty(max(nvfp4_sf_bytes_mx(Rq, Kq, sf_layout), 16), dtype=torch.uint8, device=x.device)
     def call(ws):
-        return lib().nvfp4_quantize_mx(_ptr(x), _dtype_code(x), rows, cols, x.stride(0), int(transposed), _ptr(global_scale),
-                                       C.byref(rounding), _ptr(codes), _ptr(scales), sf_layout, _ptr(ws),
-                                       ws.numel() if ws is not None else 0, _stream(stream))
+        return _native().nvfp4_quantize_mx(x, x, rows, cols, x.stride(0), int(transposed), global_scale, rounding,
+                                           codes, scales, sf_layout, ws, ws.numel() if ws is not None else 0, stream)
     st = call(None)
     if st == 5 and transposed:          # a shape the tile kernel does not take: the library transposes into a workspace first
         st = call(torch.empty(rows * cols * 2, dtype=torch.uint8, device=x.device))
@@ -435,8 +437,7 @@ def nvfp4_gemm_mx(a_codes, a_sf, a_g, b_codes, b_sf, b_g, out_dtype=torch.float3
     N = b_codes.shape[0]
     if out is None:
         out = torch.empty((M, N), dtype=out_dtype, device=a_codes.device)
-    st = lib().nvfp4_gemm_mx(_ptr(a_codes), _ptr(a_sf), _ptr(a_g), _ptr(b_codes), _ptr(b_sf), _ptr(b_g), M, N, K,
-                             _ptr(out), _dtype_code(out), out.stride(0), _stream(stream))
+    st = _native().nvfp4_gemm_mx(a_codes, a_sf, a_g, b_codes, b_sf, b_g, M, N, K, out, out, out.stride(0), stream)
     _check(st, "nvfp4_gemm_mx")
     return out
 
@@ -447,8 +448,7 @@ def nvfp4_gemm_bf16(A, B, out_dtype=torch.float32, out=None, stream=None):
     (M, K), N = A.shape, B.shape[0]
     if out is None:
         out = torch.empty((M, N), dtype=out_dtype, device=A.device)
-    _check(lib().nvfp4_gemm_bf16(_ptr(A), _ptr(B), M, N, K, _ptr(out), _dtype_code(out), out.stride(0), _stream(stream)),
-           "nvfp4_gemm_bf16")
+    _check(_native().nvfp4_gemm_bf16(A, B, M, N, K, out, out, out.stride(0), stream), "nvfp4_gemm_bf16")
     return out
 
 
@@ -459,8 +459,8 @@ def nvfp4_gemm_bf16_ex(A, a_mn_major, B, b_mn_major, out_dtype=torch.float32, ou
     N = B.shape[1] if b_mn_major else B.shape[0]
     if out is None:
         out = torch.empty((M, N), dtype=out_dtype, device=A.device)
-    _check(lib().nvfp4_gemm_bf16_ex(_ptr(A), int(a_mn_major), _ptr(B), int(b_mn_major), M, N, K, _ptr(out), _dtype_code(out),
-                                    out.stride(0), _stream(stream)), "nvfp4_gemm_bf16_ex")
+    _check(_native().nvfp4_gemm_bf16_ex(A, int(a_mn_major), B, int(b_mn_major), M, N, K, out, out, out.stride(0),
+                                        stream), "nvfp4_gemm_bf16_ex")
     return out
 
 
@@ -478,8 +478,7 @@ def nvfp4_linear_bwd_bf16(dY, W, X, dx_dtype=torch.float32, dw_dtype=torch.float
     dX = torch.empty((M, K), dtype=dx_dtype, device=dY.device)
     dW = torch.empty((N, K), dtype=dw_dtype, device=dY.device)
     ws = _scratch(int(lib().nvfp4_linear_bwd_bf16_workspace_bytes(M, N, K)), dY.device, workspace)
-    _check(lib().nvfp4_linear_bwd_bf16(_ptr(dY), _ptr(W), _ptr(X), M, N, K, _ptr(dX), _dtype_code(dX), _ptr(dW),
-                                       _dtype_code(dW), _ptr(ws), ws.numel(), _stream(stream)), "nvfp4_linear_bwd_bf16")
+    _check(_native().nvfp4_linear_bwd_bf16(dY, W, X, M, N, K, dX, dX, dW, dW, ws, ws, stream), "nvfp4_linear_bwd_bf16")
     return dX, dW
 
 
@@ -497,8 +496,7 @@ def nvfp4_linear_fwd_static(X, W, gscale_mode=G_AMAX, gx=None, gw=None, rx=None,
         out = torch.empty((M, N), dtype=out_dtype, device=X.device)
     rx, rw = rx or Rounding(RTN), rw or Rounding(RTN)
     assert X.is_contiguous() and W.is_contiguous() and out.is_contiguous() and X.dtype == W.dtype
-    st = lib().nvfp4_linear_fwd_static(_ptr(X), _ptr(W), _dtype_code(X), M, N, K, gscale_mode, _ptr(gx), _ptr(gw),
-                                       C.byref(rx), C.byref(rw), _ptr(out), _dtype_code(out), _stream(stream))
+    st = _native().nvfp4_linear_fwd_static(X, W, X, M, N, K, gscale_mode, gx, gw, rx, rw, out, out, stream)
     _check(st, "nvfp4_linear_fwd_static")
     return out
 

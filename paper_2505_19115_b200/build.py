@@ -1,8 +1,9 @@
-"""Compile the CUDA sources into paper_2505_19115_b200/libnvfp4.so (sm_100a only)."""
+"""Compile the CUDA sources into paper_2505_19115_b200/libnvfp4.so (sm_100a only), and the binding's extension module."""
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -31,11 +32,31 @@ def _compile(out: str, srcs, defines=(), verbose: bool = False) -> str:
     return out
 
 
-def _fresh(out: str) -> bool:
-    return os.path.exists(out) and all(os.path.getmtime(out) >= os.path.getmtime(d) for d in _deps())
+def _fresh(out: str, deps=None) -> bool:
+    return os.path.exists(out) and all(os.path.getmtime(out) >= os.path.getmtime(d) for d in deps or _deps())
+
+
+CALLS_OUT = os.path.join(HERE, "_calls.so")
+CALLS_SRC = os.path.join(HERE, "csrc", "python_calls.cpp")
+
+
+def build_calls(force: bool = False) -> str:
+    """The extension module through which binding.py calls the library (host code only)."""
+    if not force and _fresh(CALLS_OUT, [CALLS_SRC, os.path.join(ROOT, "include", "nvfp4.h")]):
+        return CALLS_OUT
+    import torch
+    th = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(NVCC))
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", os.path.join(th, "include"),
+                           "-I", os.path.join(th, "include", "torch", "csrc", "api", "include"),
+                           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), "-I", os.path.join(ROOT, "include"),
+                           CALLS_SRC, "-o", CALLS_OUT, "-L", os.path.join(th, "lib"), "-Wl,-rpath," + os.path.join(th, "lib"),
+                           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-ldl"])
+    return CALLS_OUT
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_calls(force)
     if not force and _fresh(OUT):
         return OUT
     return _compile(OUT, sources(), verbose=verbose)

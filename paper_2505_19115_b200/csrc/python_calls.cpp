@@ -1,0 +1,154 @@
+// The Python binding's way into libnvfp4.so: a call takes tensors, rounding descriptors and numbers as they are and makes the
+// C entry point's arguments of them.  A small call is bound by the host, and fetching the arguments one by one in Python and
+// passing them through ctypes took 2.7 us of its 6 (three calls on kept weights: 18.4 -> 14.2 us, a 256-token step's two 29.1 -> 22.9).
+//
+// Argument rules, by the C parameter's type:
+//   pointer       a tensor (its data), an object with a buffer of the pointed-to struct (Rounding), an address, or None
+//   int           a number, or a tensor (its dtype as an nvfp4_dtype)
+//   int64, size_t a number, or a tensor (its number of elements)
+// The last parameter of every entry point is the stream: a torch.cuda.Stream, or None for the current stream.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <c10/cuda/CUDAStream.h>
+#include <dlfcn.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <tuple>
+#include <type_traits>
+#include <utility>
+
+#include "nvfp4.h"
+
+namespace {
+
+// Thrown with the Python error set.
+struct PythonError {};
+
+template <typename T>
+T convert(PyObject* o) {
+  if constexpr (std::is_pointer_v<T>) {
+    if (o == Py_None) return nullptr;
+    if (THPVariable_Check(o)) return static_cast<T>(THPVariable_Unpack(o).data_ptr());
+    if constexpr (std::is_same_v<T, const nvfp4_rounding*>) {
+      Py_buffer view;
+      if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw PythonError{};
+      void* const p = view.buf;                    // the object outlives the call: the caller holds it
+      const bool fits = view.len == (Py_ssize_t)sizeof(nvfp4_rounding);
+      PyBuffer_Release(&view);
+      if (!fits) {
+        PyErr_SetString(PyExc_TypeError, "expected a Rounding");
+        throw PythonError{};
+      }
+      return static_cast<T>(p);
+    }
+    void* const p = PyLong_AsVoidPtr(o);
+    if (!p && PyErr_Occurred()) throw PythonError{};
+    return static_cast<T>(p);
+  } else {
+    if (THPVariable_Check(o)) {
+      const at::Tensor& t = THPVariable_Unpack(o);
+      if constexpr (!std::is_same_v<T, int>) return (T)t.numel();
+      if (t.scalar_type() == at::kBFloat16) return (T)NVFP4_BF16;
+      if (t.scalar_type() == at::kFloat) return (T)NVFP4_FP32;
+      PyErr_Format(PyExc_TypeError, "unsupported dtype %s", c10::toString(t.scalar_type()));
+      throw PythonError{};
+    }
+    if constexpr (std::is_same_v<T, size_t>) {
+      const size_t v = PyLong_AsSize_t(o);
+      if (v == (size_t)-1 && PyErr_Occurred()) throw PythonError{};
+      return v;
+    }
+    const long long v = PyLong_AsLongLong(o);
+    if (v == -1 && PyErr_Occurred()) throw PythonError{};
+    if constexpr (std::is_same_v<T, int>) {
+      if (v != (int)v) {
+        PyErr_SetString(PyExc_OverflowError, "argument out of the range of int");
+        throw PythonError{};
+      }
+    }
+    return (T)v;
+  }
+}
+
+void* stream_handle(PyObject* o) {
+  if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+  PyObject* const handle = PyObject_GetAttrString(o, "cuda_stream");
+  if (!handle) throw PythonError{};
+  void* const p = PyLong_AsVoidPtr(handle);
+  Py_DECREF(handle);
+  if (!p && PyErr_Occurred()) throw PythonError{};
+  return p;
+}
+
+template <typename... A, size_t... I>
+PyObject* call(int (*f)(A...), PyObject* const* args, std::index_sequence<I...>) {
+  constexpr size_t kLast = sizeof...(A) - 1;
+  std::tuple<A...> a{[&]() -> A {
+    if constexpr (I == kLast) return stream_handle(args[I]);
+    else return convert<A>(args[I]);
+  }()...};
+  int st;
+  Py_BEGIN_ALLOW_THREADS
+  st = std::apply(f, a);
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(st);
+}
+
+template <typename... A>
+PyObject* checked_call(int (*f)(A...), PyObject* const* args, Py_ssize_t n) {
+  if (!f) {
+    PyErr_SetString(PyExc_RuntimeError, "bind() first");
+    return nullptr;
+  }
+  if (n != (Py_ssize_t)sizeof...(A)) {
+    PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", (Py_ssize_t)sizeof...(A), n);
+    return nullptr;
+  }
+  try {
+    return call(f, args, std::index_sequence_for<A...>{});
+  } catch (const PythonError&) {
+    return nullptr;
+  } catch (const std::exception& e) {              // torch's own checks (a tensor without storage, no GPU)
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+
+#define NVFP4_CALLS(X)                                                                                                      \
+  X(nvfp4_quantize) X(nvfp4_quantize_dual) X(nvfp4_quantize_mx) X(nvfp4_tensor_amax_scale) X(nvfp4_gemm)                    \
+  X(nvfp4_gemm_quantized) X(nvfp4_gemm_mx) X(nvfp4_gemm_bf16) X(nvfp4_gemm_bf16_ex) X(nvfp4_linear_fwd)                     \
+  X(nvfp4_linear_bwd_dx) X(nvfp4_linear_bwd_dw) X(nvfp4_linear_fwd_qout) X(nvfp4_linear_fwd_qin) X(nvfp4_linear_fwd_save)   \
+  X(nvfp4_linear_bwd_saved) X(nvfp4_linear_bwd) X(nvfp4_linear_bwd_bf16) X(nvfp4_linear_fwd_static)
+
+#define NVFP4_WRAPPER(name)                                                            \
+  decltype(&::name) fn_##name = nullptr;                                               \
+  PyObject* py_##name(PyObject*, PyObject* const* args, Py_ssize_t n) { return checked_call(fn_##name, args, n); }
+NVFP4_CALLS(NVFP4_WRAPPER)
+
+// bind(path): takes the entry points from the library at `path`.
+PyObject* py_bind(PyObject*, PyObject* path) {
+  const char* file = PyUnicode_AsUTF8(path);
+  if (!file) return nullptr;
+  void* const lib = dlopen(file, RTLD_NOW | RTLD_LOCAL);
+  if (!lib) {
+    PyErr_SetString(PyExc_OSError, dlerror());
+    return nullptr;
+  }
+  bool all = true;
+#define NVFP4_BIND(name) all = (fn_##name = reinterpret_cast<decltype(&::name)>(dlsym(lib, #name))) && all;
+  NVFP4_CALLS(NVFP4_BIND)
+  if (!all) {
+    PyErr_Format(PyExc_OSError, "%s lacks entry points", file);
+    return nullptr;
+  }
+  Py_RETURN_NONE;
+}
+
+#define NVFP4_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(py_##name)), METH_FASTCALL, nullptr},
+PyMethodDef methods[] = {{"bind", py_bind, METH_O, nullptr}, NVFP4_CALLS(NVFP4_METHOD){nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__calls() { return PyModule_Create(&module); }

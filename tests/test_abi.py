@@ -171,3 +171,24 @@ def test_stream_handle_without_the_raw_stream_function(monkeypatch):
     monkeypatch.setattr(nb.torch.cuda, "current_stream", lambda *a: Stream())
     assert nb._stream() == 1234
     assert nb._stream(Stream()) == 1234
+
+
+def test_calls_module_takes_its_arguments_as_declared():
+    import torch
+
+    class Stream:
+        cuda_stream = 0
+    x, codes, r = torch.zeros((64, 64), dtype=torch.bfloat16), torch.zeros(4096, dtype=torch.uint8), nb.Rounding()
+
+    def quantize(rows=0, transposed=0, rounding=r, dtype=x):
+        return nb._native().nvfp4_quantize(x, dtype, rows, 64, x.stride(0), transposed, None, rounding, codes, codes, nb.SF_LINEAR, Stream)
+    assert quantize() == 2                                                 # no rows: refused before any launch
+    assert quantize(transposed=2) == 4 and quantize(rounding=None) == 1    # an enum, a pointer that is required
+    assert nb._native().nvfp4_quantize(x, nb.BF16, 0, 64, 64, 0, codes.data_ptr(), r, codes.data_ptr(), codes, nb.SF_LINEAR, Stream) == 2
+    for bad in (dict(rounding=5), dict(dtype=x.double()), dict(rows=1.5)):
+        with pytest.raises(TypeError):
+            quantize(**bad)
+    with pytest.raises(OverflowError):
+        quantize(transposed=1 << 40)
+    with pytest.raises(TypeError):
+        nb._native().nvfp4_quantize(x)
