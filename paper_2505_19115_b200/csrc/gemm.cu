@@ -547,9 +547,9 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
   cluster_sync_all();                               // both CTAs' barriers exist before any remote signal
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // All of the above overlaps the kernel before this one, and what the two producers do until their first copy: they and the
-  // epilogue wait for it, the other roles touch no global memory.  Against a wait here, for all: 2080 x 1056 x 2848 step 55.9 ->
-  // 53.5 us, 256 x 512 x 512 23.5 -> 22.4, 16 x 11008 x 4096 alone 12.5 -> 11.7.
+  // All of the above overlaps the kernel before this one, and what each role does until its first copy, access or bounded wait
+  // on another role: there it waits for that kernel (the time limit of a wait must not run while that one does).  Against a wait
+  // here, for all: 2080 x 1056 x 2848 step 55.9 -> 53.5 us, 256 x 512 x 512 23.5 -> 22.4, 16 x 11008 x 4096 alone 12.5 -> 11.7.
   if constexpr (Q_OUT) {
     grid_dependency_wait();
     build_inv_table(inv_table, load_scale(p.out_g));
@@ -669,6 +669,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
         int tm_unused, tn;
         tile_coords(t.tile, q.tiles_m, q.tiles_n, tm_unused, tn);
         const uint32_t sfb_off = (uint32_t)((tn * BN) % 128) / 32 + (whole ? 0u : 4u * t.half);   // first scale column of this N tile
+        if (i == 0) grid_dependency_wait();
         ACCOUNT(a_acc, ok = mbar_wait_issuer(tempty_bar(acc), acc_ph ^ 1u, abort_flag, 0x12));
         if (!ok) break;
         const uint32_t d_tmem = tmem_base + acc * BN;
@@ -738,6 +739,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
     TileItem t;
     for (int i = 0; !BF16_IN && ok && tile_at<PAIRED, HALVES>(p.order, pair, num_pairs, i, t); ++i) {
       const int k_stages = p.product[t.product].k_stages;
+      if (i == 0) grid_dependency_wait();
       for (int ks = 0; ks < k_stages; ++ks) {
         ACCOUNT(a_land, ok = mbar_wait_warp_relaxed(sfl_bar(s), ph, abort_flag, 0x16));
         if (!ok) break;
