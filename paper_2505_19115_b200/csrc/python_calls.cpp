@@ -2,10 +2,11 @@
 // C entry point's arguments of them.  A small call is bound by the host, and fetching the arguments one by one in Python and
 // passing them through ctypes took 2.7 us of its 6 (three calls on kept weights: 18.4 -> 14.2 us, a 256-token step's two 29.1 -> 22.9).
 //
-// Argument rules, by the C parameter's type:
+// Argument rules, by what the C parameter is:
 //   pointer       a tensor (its data), an object with a buffer of the pointed-to struct (Rounding), an address, or None
-//   int           a number, or a tensor (its dtype as an nvfp4_dtype)
-//   int64, size_t a number, or a tensor (its number of elements)
+//   dtype         an int, or a tensor (its dtype as an nvfp4_dtype): the parameters that NVFP4_CALLS lists
+//   size_t        an int, or a tensor (its number of elements): the size of the buffer before it
+//   int, int64    an int; a tensor in its place is a misplaced argument and refused
 // The last parameter of every entry point is the stream: a torch.cuda.Stream, or None for the current stream.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
@@ -25,50 +26,59 @@ namespace {
 // Thrown with the Python error set.
 struct PythonError {};
 
+[[noreturn]] void type_error(const char* expected, PyObject* got) {
+  PyErr_Format(PyExc_TypeError, "expected %s, got %s", expected, Py_TYPE(got)->tp_name);
+  throw PythonError{};
+}
+
 template <typename T>
-T convert(PyObject* o) {
-  if constexpr (std::is_pointer_v<T>) {
-    if (o == Py_None) return nullptr;
-    if (THPVariable_Check(o)) return static_cast<T>(THPVariable_Unpack(o).data_ptr());
-    if constexpr (std::is_same_v<T, const nvfp4_rounding*>) {
-      Py_buffer view;
-      if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw PythonError{};
-      void* const p = view.buf;                    // the object outlives the call: the caller holds it
-      const bool fits = view.len == (Py_ssize_t)sizeof(nvfp4_rounding);
-      PyBuffer_Release(&view);
-      if (!fits) {
-        PyErr_SetString(PyExc_TypeError, "expected a Rounding");
-        throw PythonError{};
-      }
-      return static_cast<T>(p);
+T convert_pointer(PyObject* o) {
+  if (o == Py_None) return nullptr;
+  if (THPVariable_Check(o)) return static_cast<T>(THPVariable_Unpack(o).data_ptr());
+  if constexpr (std::is_same_v<T, const nvfp4_rounding*>) {
+    Py_buffer view;
+    if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw PythonError{};
+    void* const p = view.buf;                      // the object outlives the call: the caller holds it
+    const bool fits = view.len == (Py_ssize_t)sizeof(nvfp4_rounding);
+    PyBuffer_Release(&view);
+    if (!fits) {
+      PyErr_SetString(PyExc_TypeError, "expected a Rounding");
+      throw PythonError{};
     }
-    void* const p = PyLong_AsVoidPtr(o);
-    if (!p && PyErr_Occurred()) throw PythonError{};
     return static_cast<T>(p);
-  } else {
+  }
+  void* const p = PyLong_AsVoidPtr(o);
+  if (!p && PyErr_Occurred()) throw PythonError{};
+  return static_cast<T>(p);
+}
+
+template <typename T, bool DTYPE>
+T convert_number(PyObject* o) {
+  if constexpr (DTYPE || std::is_same_v<T, size_t>) {
     if (THPVariable_Check(o)) {
       const at::Tensor& t = THPVariable_Unpack(o);
-      if constexpr (!std::is_same_v<T, int>) return (T)t.numel();
+      if constexpr (!DTYPE) return (T)t.numel();
       if (t.scalar_type() == at::kBFloat16) return (T)NVFP4_BF16;
       if (t.scalar_type() == at::kFloat) return (T)NVFP4_FP32;
       PyErr_Format(PyExc_TypeError, "unsupported dtype %s", c10::toString(t.scalar_type()));
       throw PythonError{};
     }
-    if constexpr (std::is_same_v<T, size_t>) {
-      const size_t v = PyLong_AsSize_t(o);
-      if (v == (size_t)-1 && PyErr_Occurred()) throw PythonError{};
-      return v;
-    }
-    const long long v = PyLong_AsLongLong(o);
-    if (v == -1 && PyErr_Occurred()) throw PythonError{};
-    if constexpr (std::is_same_v<T, int>) {
-      if (v != (int)v) {
-        PyErr_SetString(PyExc_OverflowError, "argument out of the range of int");
-        throw PythonError{};
-      }
-    }
-    return (T)v;
   }
+  if (!PyLong_Check(o)) type_error("an int", o);
+  if constexpr (std::is_same_v<T, size_t>) {
+    const size_t v = PyLong_AsSize_t(o);
+    if (v == (size_t)-1 && PyErr_Occurred()) throw PythonError{};
+    return v;
+  }
+  const long long v = PyLong_AsLongLong(o);
+  if (v == -1 && PyErr_Occurred()) throw PythonError{};
+  if constexpr (std::is_same_v<T, int>) {
+    if (v != (int)v) {
+      PyErr_SetString(PyExc_OverflowError, "argument out of the range of int");
+      throw PythonError{};
+    }
+  }
+  return (T)v;
 }
 
 void* stream_handle(PyObject* o) {
@@ -81,12 +91,17 @@ void* stream_handle(PyObject* o) {
   return p;
 }
 
-template <typename... A, size_t... I>
+template <size_t... S>
+constexpr bool one_of(size_t i) { return ((i == S) || ...); }
+
+// DTYPES: the positions of the dtype parameters.
+template <size_t... DTYPES, typename... A, size_t... I>
 PyObject* call(int (*f)(A...), PyObject* const* args, std::index_sequence<I...>) {
   constexpr size_t kLast = sizeof...(A) - 1;
   std::tuple<A...> a{[&]() -> A {
     if constexpr (I == kLast) return stream_handle(args[I]);
-    else return convert<A>(args[I]);
+    else if constexpr (std::is_pointer_v<A>) return convert_pointer<A>(args[I]);
+    else return convert_number<A, one_of<DTYPES...>(I)>(args[I]);
   }()...};
   int st;
   Py_BEGIN_ALLOW_THREADS
@@ -95,7 +110,7 @@ PyObject* call(int (*f)(A...), PyObject* const* args, std::index_sequence<I...>)
   return PyLong_FromLong(st);
 }
 
-template <typename... A>
+template <size_t... DTYPES, typename... A>
 PyObject* checked_call(int (*f)(A...), PyObject* const* args, Py_ssize_t n) {
   if (!f) {
     PyErr_SetString(PyExc_RuntimeError, "bind() first");
@@ -106,7 +121,7 @@ PyObject* checked_call(int (*f)(A...), PyObject* const* args, Py_ssize_t n) {
     return nullptr;
   }
   try {
-    return call(f, args, std::index_sequence_for<A...>{});
+    return call<DTYPES...>(f, args, std::index_sequence_for<A...>{});
   } catch (const PythonError&) {
     return nullptr;
   } catch (const std::exception& e) {              // torch's own checks (a tensor without storage, no GPU)
@@ -115,15 +130,17 @@ PyObject* checked_call(int (*f)(A...), PyObject* const* args, Py_ssize_t n) {
   }
 }
 
+// The entry points, each with the positions of its dtype parameters.
 #define NVFP4_CALLS(X)                                                                                                      \
-  X(nvfp4_quantize) X(nvfp4_quantize_dual) X(nvfp4_quantize_mx) X(nvfp4_tensor_amax_scale) X(nvfp4_gemm)                    \
-  X(nvfp4_gemm_quantized) X(nvfp4_gemm_mx) X(nvfp4_gemm_bf16) X(nvfp4_gemm_bf16_ex) X(nvfp4_linear_fwd)                     \
-  X(nvfp4_linear_bwd_dx) X(nvfp4_linear_bwd_dw) X(nvfp4_linear_fwd_qout) X(nvfp4_linear_fwd_qin) X(nvfp4_linear_fwd_save)   \
-  X(nvfp4_linear_bwd_saved) X(nvfp4_linear_bwd) X(nvfp4_linear_bwd_bf16) X(nvfp4_linear_fwd_static)
+  X(nvfp4_quantize, 1) X(nvfp4_quantize_dual, 1) X(nvfp4_quantize_mx, 1) X(nvfp4_tensor_amax_scale, 1) X(nvfp4_gemm, 10)    \
+  X(nvfp4_gemm_quantized) X(nvfp4_gemm_mx, 10) X(nvfp4_gemm_bf16, 6) X(nvfp4_gemm_bf16_ex, 8) X(nvfp4_linear_fwd, 2, 12)    \
+  X(nvfp4_linear_bwd_dx, 2, 12) X(nvfp4_linear_bwd_dw, 2, 12) X(nvfp4_linear_fwd_qout, 2) X(nvfp4_linear_fwd_qin, 4, 12)    \
+  X(nvfp4_linear_fwd_save, 2, 14) X(nvfp4_linear_bwd_saved, 1, 12, 14) X(nvfp4_linear_bwd, 3, 16, 18)                       \
+  X(nvfp4_linear_bwd_bf16, 7, 9) X(nvfp4_linear_fwd_static, 2, 12)
 
-#define NVFP4_WRAPPER(name)                                                            \
+#define NVFP4_WRAPPER(name, ...)                                                       \
   decltype(&::name) fn_##name = nullptr;                                               \
-  PyObject* py_##name(PyObject*, PyObject* const* args, Py_ssize_t n) { return checked_call(fn_##name, args, n); }
+  PyObject* py_##name(PyObject*, PyObject* const* args, Py_ssize_t n) { return checked_call<__VA_ARGS__>(fn_##name, args, n); }
 NVFP4_CALLS(NVFP4_WRAPPER)
 
 // bind(path): takes the entry points from the library at `path`.
@@ -136,7 +153,7 @@ PyObject* py_bind(PyObject*, PyObject* path) {
     return nullptr;
   }
   bool all = true;
-#define NVFP4_BIND(name) all = (fn_##name = reinterpret_cast<decltype(&::name)>(dlsym(lib, #name))) && all;
+#define NVFP4_BIND(name, ...) all = (fn_##name = reinterpret_cast<decltype(&::name)>(dlsym(lib, #name))) && all;
   NVFP4_CALLS(NVFP4_BIND)
   if (!all) {
     PyErr_Format(PyExc_OSError, "%s lacks entry points", file);
@@ -145,7 +162,7 @@ PyObject* py_bind(PyObject*, PyObject* path) {
   Py_RETURN_NONE;
 }
 
-#define NVFP4_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(py_##name)), METH_FASTCALL, nullptr},
+#define NVFP4_METHOD(name, ...) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(py_##name)), METH_FASTCALL, nullptr},
 PyMethodDef methods[] = {{"bind", py_bind, METH_O, nullptr}, NVFP4_CALLS(NVFP4_METHOD){nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

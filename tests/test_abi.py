@@ -17,6 +17,15 @@ def _declared_symbols():
     return sorted(set(re.findall(r"\b(nvfp4_[a-z0-9_]+)\s*\(", text)))
 
 
+def _declared_parameters():
+    """Entry point -> [(C type, name)] of the calls that take a stream."""
+    text = open(os.path.join(ROOT, "include", "nvfp4.h")).read()
+    text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
+    calls = re.findall(r"NVFP4_API int (nvfp4_[a-z0-9_]+)\(([^)]*)\)", text)
+    split = {n: [tuple(re.fullmatch(r"(.*?)(\w+)", " ".join(p.split())).groups()) for p in ps.split(",")] for n, ps in calls}
+    return {n: [(t.strip(), p) for t, p in ps] for n, ps in split.items() if ps[-1][1] == "cuda_stream"}
+
+
 def test_library_exports_every_declared_symbol():
     names = _declared_symbols()
     assert {"nvfp4_quantize", "nvfp4_gemm", "nvfp4_linear_fwd", "nvfp4_linear_bwd_dx",
@@ -192,3 +201,37 @@ def test_calls_module_takes_its_arguments_as_declared():
         quantize(transposed=1 << 40)
     with pytest.raises(TypeError):
         nb._native().nvfp4_quantize(x)
+
+
+class _NoStream:
+    cuda_stream = 0
+
+
+_THROUGH_CTYPES = {"nvfp4_quantization_noise", "nvfp4_transpose_bf16", "nvfp4_microbench_mma_peak"}
+
+
+# Every parameter of every call, with the others null or zero (refused before any launch): a tensor stands for a dtype and for a
+# buffer's size and for no other number; what is no int is no number either.
+@pytest.mark.parametrize("name", sorted(set(_declared_parameters()) - _THROUGH_CTYPES))
+def test_calls_module_takes_numbers_as_declared(name):
+    import torch
+    params = _declared_parameters()[name]
+    f, x = getattr(nb._native(), name), torch.zeros(64)
+    args = [None if "*" in t else 0 for t, _ in params[:-1]] + [_NoStream]
+    refused = f(*args)
+    assert refused in (1, 2)
+    for i, (t, p) in enumerate(params[:-1]):
+        if "*" in t:
+            continue
+        for bad in (1.0, "1", None) + (() if p.endswith(("dtype", "_bytes")) else (x, torch.zeros((), dtype=torch.int64))):
+            with pytest.raises(TypeError):
+                f(*args[:i], bad, *args[i + 1:])
+        if p.endswith(("dtype", "_bytes")):
+            assert f(*args[:i], x, *args[i + 1:]) == refused, p
+
+
+def test_scales_in_the_place_of_the_scale_mode_are_refused():
+    import torch
+    X, W, g = torch.zeros((32, 64)), torch.zeros((32, 64)), torch.ones(1)
+    with pytest.raises(TypeError):
+        nb.nvfp4_linear_fwd(X, W, g, g)
