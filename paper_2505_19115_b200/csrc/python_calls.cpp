@@ -3,7 +3,7 @@
 // passing them through ctypes took 2.7 us of its 6 (three calls on kept weights: 18.4 -> 14.2 us, a 256-token step's two 29.1 -> 22.9).
 //
 // Argument rules, by what the C parameter is:
-//   pointer       a tensor (its data), an object with a buffer of the pointed-to struct (Rounding), an address, or None
+//   pointer       a tensor or another object with data_ptr(), or None; an object with a buffer of the struct (Rounding)
 //   dtype         an int, or a tensor (its dtype as an nvfp4_dtype): the parameters that NVFP4_CALLS lists
 //   size_t        an int, or a tensor (its number of elements): the size of the buffer before it
 //   int, int64    an int; a tensor in its place is a misplaced argument and refused
@@ -47,7 +47,11 @@ T convert_pointer(PyObject* o) {
     }
     return static_cast<T>(p);
   }
-  void* const p = PyLong_AsVoidPtr(o);
+  if (!PyObject_HasAttrString(o, "data_ptr")) type_error("a tensor or None", o);
+  PyObject* const address = PyObject_CallMethod(o, "data_ptr", nullptr);   // a storage, say
+  if (!address) throw PythonError{};
+  void* const p = PyLong_AsVoidPtr(address);
+  Py_DECREF(address);
   if (!p && PyErr_Occurred()) throw PythonError{};
   return static_cast<T>(p);
 }

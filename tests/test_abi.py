@@ -193,7 +193,7 @@ def test_calls_module_takes_its_arguments_as_declared():
         return nb._native().nvfp4_quantize(x, dtype, rows, 64, x.stride(0), transposed, None, rounding, codes, codes, nb.SF_LINEAR, Stream)
     assert quantize() == 2                                                 # no rows: refused before any launch
     assert quantize(transposed=2) == 4 and quantize(rounding=None) == 1    # an enum, a pointer that is required
-    assert nb._native().nvfp4_quantize(x, nb.BF16, 0, 64, 64, 0, codes.data_ptr(), r, codes.data_ptr(), codes, nb.SF_LINEAR, Stream) == 2
+    assert nb._native().nvfp4_quantize(x, nb.BF16, 0, 64, 64, 0, codes, r, codes.untyped_storage(), codes, nb.SF_LINEAR, Stream) == 2
     for bad in (dict(rounding=5), dict(dtype=x.double()), dict(rows=1.5)):
         with pytest.raises(TypeError):
             quantize(**bad)
@@ -235,3 +235,21 @@ def test_scales_in_the_place_of_the_scale_mode_are_refused():
     X, W, g = torch.zeros((32, 64)), torch.zeros((32, 64)), torch.ones(1)
     with pytest.raises(TypeError):
         nb.nvfp4_linear_fwd(X, W, g, g)
+
+
+@pytest.mark.parametrize("name", sorted(set(_declared_parameters()) - _THROUGH_CTYPES))
+def test_calls_module_takes_no_bare_addresses(name):
+    params = _declared_parameters()[name]
+    f, args = getattr(nb._native(), name), [None if "*" in t else 0 for t, _ in params[:-1]] + [_NoStream]
+    for i, (t, p) in enumerate(params[:-1]):
+        if "*" in t:
+            for bad in (2, 1 << 40, 0, 1.0):
+                with pytest.raises(TypeError):
+                    f(*args[:i], bad, *args[i + 1:])
+
+
+def test_a_number_in_the_place_of_a_scale_is_refused():
+    import torch
+    X, W = torch.zeros((32, 64)), torch.zeros((32, 64))
+    with pytest.raises(TypeError):
+        nb.nvfp4_linear_fwd(X, W, nb.G_GIVEN, 2, 2)
