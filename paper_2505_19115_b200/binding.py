@@ -123,7 +123,7 @@ def _native():
     if _calls is None:
         lib()
         from . import _calls as module
-        module.bind(LIB_PATH)
+        module.bind(LIB_PATH, Rounding)
         _calls = module
     return _calls
 

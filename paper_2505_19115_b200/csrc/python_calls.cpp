@@ -3,7 +3,8 @@
 // passing them through ctypes took 2.7 us of its 6 (three calls on kept weights: 18.4 -> 14.2 us, a 256-token step's two 29.1 -> 22.9).
 //
 // Argument rules, by what the C parameter is:
-//   pointer       a tensor or another object with data_ptr(), or None; an object with a buffer of the struct (Rounding)
+//   pointer       a tensor or another object with data_ptr(), or None
+//   rounding      a Rounding (the class that bind() was given), or None
 //   dtype         an int, or a tensor (its dtype as an nvfp4_dtype): the parameters that NVFP4_CALLS lists
 //   size_t        an int, or a tensor (its number of elements): the size of the buffer before it
 //   int, int64    an int; a tensor in its place is a misplaced argument and refused
@@ -31,22 +32,23 @@ struct PythonError {};
   throw PythonError{};
 }
 
+PyTypeObject* rounding_type = nullptr;             // binding.py's Rounding, a ctypes.Structure laid out as nvfp4_rounding
+
+// The struct is read on the host: nothing but a Rounding will do.
+const nvfp4_rounding* convert_rounding(PyObject* o) {
+  if (o == Py_None) return nullptr;
+  if (!PyObject_TypeCheck(o, rounding_type)) type_error("a Rounding", o);
+  Py_buffer view;
+  if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw PythonError{};
+  void* const p = view.buf;                        // the object outlives the call: the caller holds it
+  PyBuffer_Release(&view);
+  return static_cast<const nvfp4_rounding*>(p);
+}
+
 template <typename T>
 T convert_pointer(PyObject* o) {
   if (o == Py_None) return nullptr;
   if (THPVariable_Check(o)) return static_cast<T>(THPVariable_Unpack(o).data_ptr());
-  if constexpr (std::is_same_v<T, const nvfp4_rounding*>) {
-    Py_buffer view;
-    if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw PythonError{};
-    void* const p = view.buf;                      // the object outlives the call: the caller holds it
-    const bool fits = view.len == (Py_ssize_t)sizeof(nvfp4_rounding);
-    PyBuffer_Release(&view);
-    if (!fits) {
-      PyErr_SetString(PyExc_TypeError, "expected a Rounding");
-      throw PythonError{};
-    }
-    return static_cast<T>(p);
-  }
   if (!PyObject_HasAttrString(o, "data_ptr")) type_error("a tensor or None", o);
   PyObject* const address = PyObject_CallMethod(o, "data_ptr", nullptr);   // a storage, say
   if (!address) throw PythonError{};
@@ -104,6 +106,7 @@ PyObject* call(int (*f)(A...), PyObject* const* args, std::index_sequence<I...>)
   constexpr size_t kLast = sizeof...(A) - 1;
   std::tuple<A...> a{[&]() -> A {
     if constexpr (I == kLast) return stream_handle(args[I]);
+    else if constexpr (std::is_same_v<A, const nvfp4_rounding*>) return convert_rounding(args[I]);
     else if constexpr (std::is_pointer_v<A>) return convert_pointer<A>(args[I]);
     else return convert_number<A, one_of<DTYPES...>(I)>(args[I]);
   }()...};
@@ -147,10 +150,15 @@ PyObject* checked_call(int (*f)(A...), PyObject* const* args, Py_ssize_t n) {
   PyObject* py_##name(PyObject*, PyObject* const* args, Py_ssize_t n) { return checked_call<__VA_ARGS__>(fn_##name, args, n); }
 NVFP4_CALLS(NVFP4_WRAPPER)
 
-// bind(path): takes the entry points from the library at `path`.
-PyObject* py_bind(PyObject*, PyObject* path) {
-  const char* file = PyUnicode_AsUTF8(path);
-  if (!file) return nullptr;
+// bind(path, Rounding): takes the entry points from the library at `path`, and the class of the rounding descriptors.
+PyObject* py_bind(PyObject*, PyObject* args) {
+  const char* file;
+  PyObject* rounding;
+  if (!PyArg_ParseTuple(args, "sO!", &file, &PyType_Type, &rounding)) return nullptr;
+  if (reinterpret_cast<PyTypeObject*>(rounding) != rounding_type) {
+    Py_XDECREF(rounding_type);
+    rounding_type = reinterpret_cast<PyTypeObject*>(Py_NewRef(rounding));
+  }
   void* const lib = dlopen(file, RTLD_NOW | RTLD_LOCAL);
   if (!lib) {
     PyErr_SetString(PyExc_OSError, dlerror());
@@ -167,7 +175,7 @@ PyObject* py_bind(PyObject*, PyObject* path) {
 }
 
 #define NVFP4_METHOD(name, ...) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(py_##name)), METH_FASTCALL, nullptr},
-PyMethodDef methods[] = {{"bind", py_bind, METH_O, nullptr}, NVFP4_CALLS(NVFP4_METHOD){nullptr, nullptr, 0, nullptr}};
+PyMethodDef methods[] = {{"bind", py_bind, METH_VARARGS, nullptr}, NVFP4_CALLS(NVFP4_METHOD){nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

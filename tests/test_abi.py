@@ -253,3 +253,20 @@ def test_a_number_in_the_place_of_a_scale_is_refused():
     X, W = torch.zeros((32, 64)), torch.zeros((32, 64))
     with pytest.raises(TypeError):
         nb.nvfp4_linear_fwd(X, W, nb.G_GIVEN, 2, 2)
+
+
+@pytest.mark.parametrize("name", sorted(n for n, ps in _declared_parameters().items() if any("nvfp4_rounding" in t for t, _ in ps)))
+def test_calls_module_takes_nothing_but_a_rounding_for_one(name):
+    import torch
+
+    class Mine(nb.Rounding):
+        pass
+    params = _declared_parameters()[name]
+    f, args = getattr(nb._native(), name), [None if "*" in t else 0 for t, _ in params[:-1]] + [_NoStream]
+    size, refused = C.sizeof(nb.Rounding), f(*args)
+    for i, (t, p) in enumerate(params[:-1]):
+        if "nvfp4_rounding" in t:
+            for bad in (torch.zeros(size, dtype=torch.uint8), bytes(size), bytearray(size), (C.c_uint8 * size)(), C.byref(nb.Rounding()), 5):
+                with pytest.raises(TypeError):
+                    f(*args[:i], bad, *args[i + 1:])
+            assert f(*args[:i], nb.Rounding(), *args[i + 1:]) == f(*args[:i], Mine(), *args[i + 1:]) == refused, p
