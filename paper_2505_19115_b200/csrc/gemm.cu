@@ -19,14 +19,13 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "bounded_waits.cuh"
 #include "quantize_core.cuh"
 #include "tc_ptx.cuh"
 #include "tensor_map.cuh"
 
 namespace nvfp4 {
 namespace {
-
-__device__ unsigned int g_error_word = 0;
 
 // Cycle account of the CTA-pair kernel (debug builds only: -DNVFP4_GEMM_ACCOUNT, see microbench.py gemm_account).
 // Each role of pair 0 adds up the clock64() cycles it spends in each of its waits and in its work; the product
@@ -50,7 +49,6 @@ constexpr int BK = 256;
 constexpr int MMA_K = 64;         // values per tcgen05.mma (32 bytes)
 constexpr int kGemmThreads = 192;
 constexpr uint32_t kTmemCols = 512;
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
 
 template <int BN>
 struct Cfg {
@@ -84,81 +82,6 @@ struct GemmParams {
   int a_row_tiles, b_row_tiles;     // ceil(M / 128), ceil(N / 128)
   int d_is_bf16;
 };
-
-// ------------------------------------------------------------------------------------------------
-// Bounded waits (the PTX wrappers are in tc_ptx.cuh)
-// ------------------------------------------------------------------------------------------------
-// Bounded waits.  They return false (and record `site`) if the barrier did not flip within the time
-// limit or another role of this CTA already gave up.
-//
-// mbar_wait spins without pause: for the MMA issuer, whose latency is the kernel's critical path.
-// mbar_wait_relaxed sleeps between polls: every other role waits most of the time, and a dozen
-// warps polling shared memory back to back slow the issuer's own barrier reads several times over.
-__device__ __forceinline__ bool mbar_wait_timeout(uint32_t site, volatile uint32_t* abort_flag, unsigned long long t0) {
-  if (*abort_flag) return true;
-  if (global_timer_ns() - t0 > kWaitLimitNs) {
-    *abort_flag = 1u;
-    atomicOr(&g_error_word, 0x100u | site);
-    return true;
-  }
-  return false;
-}
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
-  for (int i = 0; i < 4096; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_timer_ns();
-  while (true) {
-    for (int i = 0; i < 64; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
-    if (mbar_wait_timeout(site, abort_flag, t0)) return false;
-  }
-}
-__device__ __forceinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_timer_ns();
-  while (true) {
-    for (int i = 0; i < 256; ++i) {
-      __nanosleep(32);
-      if (mbar_try_wait(bar, parity)) return true;
-    }
-    if (mbar_wait_timeout(site, abort_flag, t0)) return false;
-  }
-}
-// Wait of the MMA-issuing warp.  The poll is a relaxed one: with MMAs in flight an acquiring
-// try_wait stalls its thread for ~170 cycles even when the phase is already complete, a relaxed one
-// for ~40, and the issuer has only 512 cycles per stage.  Nothing the issuer does afterwards reads
-// memory through the generic proxy: it issues tcgen05.mma, whose shared-memory operands were written
-// by the bulk copies that completed the phase, and whose tensor-memory scales are ordered by
-// tcgen05.fence::after_thread_sync.
-__device__ __forceinline__ bool mbar_wait_issuer(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
-  for (int i = 0; i < 4096; ++i)
-    if (mbar_try_wait_relaxed(bar, parity)) return true;
-  const unsigned long long t0 = global_timer_ns();
-  while (true) {
-    for (int i = 0; i < 64; ++i)
-      if (mbar_try_wait_relaxed(bar, parity)) return true;
-    if (mbar_wait_timeout(site, abort_flag, t0)) return false;
-  }
-}
-// Whole-warp wait of the scale movers, relaxed polls by every lane: these warps issue tcgen05.st, and
-// next to such operations an acquiring poll costs ~180 cycles even when the phase is complete (see
-// mbar_wait_issuer), which with two waits per stage made the movers the slowest role.  What they read
-// afterwards is shared memory written by the bulk copies that completed the phase, so the successful poll is
-// followed by one acquire fence at CTA scope: relaxed observation + fence is the acquire pattern of the PTX
-// memory model, paid once per wait instead of once per poll (0.3 % of the kernel in a same-process A/B).
-__device__ __forceinline__ bool mbar_wait_warp_relaxed(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
-  const bool ok = mbar_wait_issuer(bar, parity, abort_flag, site);
-  asm volatile("fence.acq_rel.cta;" ::: "memory");
-  return ok;
-}
-// Whole-warp wait: lane 0 polls, then every lane observes the completed phase once itself.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
-  bool ok = true;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait_relaxed(bar, parity, abort_flag, site);
-  ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
-  if (ok) (void)mbar_try_wait(bar, parity);
-  return ok;
-}
 
 // Tile order: panels of kPanel row tiles, column-major inside a panel, so that the CTAs running at
 // the same time share both their A row tiles and their B row tiles (each operand tile is then read
@@ -818,7 +741,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
       tile_coords(t.tile, q.tiles_m, q.tiles_n, tm, tn);
       // Polled without sleeping: the next tile's MMAs wait for this read-out.  Against a lane that sleeps 32 ns between its polls:
       // 16384 x 3072 x 2048 fp32 57.6 -> 56.2 us, 16384 x 4096 x 4096 bf16 109.7 -> 107.0, 1024 x 1024 x 16384 21.2 -> 20.1.
-      ACCOUNT(a_tile, ok = mbar_wait(tfull_bar(acc), acc_ph, abort_flag, 0x14));
+      ACCOUNT(a_tile, ok = mbar_wait_warp_spin(tfull_bar(acc), acc_ph, abort_flag, 0x14));
       if (!ok) break;
 #ifdef NVFP4_GEMM_ACCOUNT
       a_read_t0 = clock64();
