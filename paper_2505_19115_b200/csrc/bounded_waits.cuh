@@ -59,19 +59,20 @@ __device__ __forceinline__ bool mbar_wait_issuer(uint32_t bar, uint32_t parity, 
     if (mbar_wait_timeout(site, abort_flag, t0)) return false;
   }
 }
-// Whole-warp wait of the scale movers, relaxed polls by every lane: these warps issue tcgen05.st, and
-// next to such operations an acquiring poll costs ~180 cycles even when the phase is complete (see
-// mbar_wait_issuer), which with two waits per stage made the movers the slowest role.  What they read
-// afterwards is shared memory written by the bulk copies that completed the phase, so the successful poll is
-// followed by one acquire fence at CTA scope: relaxed observation + fence is the acquire pattern of the PTX
-// memory model, paid once per wait instead of once per poll (0.3 % of the kernel in a same-process A/B).
-__device__ __forceinline__ bool mbar_wait_warp_relaxed(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
-  const bool ok = mbar_wait_issuer(bar, parity, abort_flag, site);
+// A whole-warp wait ends alike for every lane: behind it stand instructions that the whole warp has to execute (tcgen05.ld, .st),
+// and lanes that poll for themselves may see the barrier flip, or the time run out, at different polls.
+//
+// The scale movers' waits are polled as the issuer's by every lane: these warps issue tcgen05.st, and next to such operations an
+// acquiring poll costs ~180 cycles even when the phase is complete (see mbar_wait_issuer), which with two waits per stage made the
+// movers the slowest role.  What they read afterwards is shared memory written by the bulk copies that completed the phase, so
+// the successful polls are followed by one acquire fence at CTA scope: relaxed observation + fence is the acquire pattern of the
+// PTX memory model.  A stage's two waits share the vote and the fence: a product chained to another, 3001 x 4096 x 11008 and
+// 3001 x 11008 x 4096, 171.5 us with a fence for each wait and no vote, 171.7 with a vote for each too, 170.0 so.
+__device__ __forceinline__ bool warp_acquire(bool ok) {
+  ok = __all_sync(0xFFFFFFFFu, ok);
   asm volatile("fence.acq_rel.cta;" ::: "memory");
   return ok;
 }
-// A whole-warp wait ends alike for every lane: behind it stand instructions that the whole warp has to execute (tcgen05.ld, .st),
-// and lanes that poll for themselves may see the barrier flip, or the time run out, at different polls.
 __device__ __forceinline__ bool mbar_wait_warp_spin(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
   return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, site));
 }

@@ -664,14 +664,13 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
       const int k_stages = p.product[t.product].k_stages;
       if (i == 0) grid_dependency_wait();
       for (int ks = 0; ks < k_stages; ++ks) {
-        ACCOUNT(a_land, ok = mbar_wait_warp_relaxed(sfl_bar(s), ph, abort_flag, 0x16));
-        if (!ok) break;
+        ACCOUNT(a_land, ok = mbar_wait_issuer(sfl_bar(s), ph, abort_flag, 0x16));
         if constexpr (!C::kSfFollowsStage) {
-          ACCOUNT(a_free, ok = mbar_wait_warp_relaxed(sfe_bar(b), bph ^ 1u, abort_flag, 0x17));
+          ACCOUNT(a_free, ok = ok && mbar_wait_issuer(sfe_bar(b), bph ^ 1u, abort_flag, 0x17));
         } else {                                    // buffer b == stage s: free once that stage's previous MMAs are done
-          ACCOUNT(a_free, ok = mbar_wait_warp_relaxed(empty_bar(s), ph ^ 1u, abort_flag, 0x17));
+          ACCOUNT(a_free, ok = ok && mbar_wait_issuer(empty_bar(s), ph ^ 1u, abort_flag, 0x17));
         }
-        if (!ok) break;
+        if (!(ok = warp_acquire(ok))) break;
         tc_fence_after();
         const uint8_t* sf = smem_gen + s * C::kStageBytes + C::kABytes + C::kBBytes + lane * 16;
         const uint32_t t_sf = tmem_base + C::kSfaCol + b * C::kSfCols + lane_field;

@@ -24,6 +24,10 @@ __global__ void wait_kernel(int even, int odd, uint32_t aborted, uint32_t site, 
   if (threadIdx.x == 0) *ended_true = votes;
 }
 
+__device__ bool movers_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t site) {
+  return warp_acquire(mbar_wait_issuer(bar, parity, abort_flag, site));
+}
+
 template <Wait WAIT>
 bool ends_as(unsigned int want, unsigned int want_word, int even, int odd, uint32_t aborted, uint32_t site) {
   unsigned int *dev = nullptr, got = 0x5555u, word = 0, zero = 0;
@@ -47,9 +51,10 @@ bool check(uint32_t site) {
 }
 
 int main() {
-  bool ok = check<mbar_wait_warp>(0x04) && check<mbar_wait_warp_spin>(0x14);
+  bool ok = check<mbar_wait_warp>(0x04) && check<mbar_wait_warp_spin>(0x14) && check<movers_wait>(0x16);
   // some lanes see the barrier flip, others give up: none goes on
   ok = ok && ends_as<mbar_wait_warp_spin>(0u, 0u, 0, 1, 1u, 0x14) && ends_as<mbar_wait_warp_spin>(0u, 0x114u, 1, 0, 0u, 0x14);
+  ok = ok && ends_as<movers_wait>(0u, 0u, 0, 1, 1u, 0x16) && ends_as<movers_wait>(0u, 0x116u, 1, 0, 0u, 0x16);
   std::puts(ok ? "ok" : "failed");
   return ok ? 0 : 1;
 }
