@@ -56,10 +56,10 @@ def build_calls(force: bool = False) -> str:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    if force or not _fresh(OUT):       # first: the C library needs no PyTorch, and is there for C callers whatever becomes of the module
+        _compile(OUT, sources(), verbose=verbose)
     build_calls(force)
-    if not force and _fresh(OUT):
-        return OUT
-    return _compile(OUT, sources(), verbose=verbose)
+    return OUT
 
 
 # Debug build of the same sources with the GEMM's per-role cycle account compiled in (microbench.py gemm_account).
