@@ -37,14 +37,23 @@ def _fresh(out: str, deps=None) -> bool:
 
 
 CALLS_OUT = os.path.join(HERE, "_calls.so")
+CALLS_BUILT_FOR = os.path.join(HERE, "_calls.so.built_for")     # the Python and PyTorch whose objects the module knows
 CALLS_SRC = os.path.join(HERE, "csrc", "python_calls.cpp")
+
+
+def _text(path: str) -> str:
+    if not os.path.exists(path):
+        return ""
+    with open(path) as f:
+        return f.read()
 
 
 def build_calls(force: bool = False) -> str:
     """The extension module through which binding.py calls the library (host code only)."""
-    if not force and _fresh(CALLS_OUT, [CALLS_SRC, os.path.join(ROOT, "include", "nvfp4.h")]):
-        return CALLS_OUT
     import torch
+    built_for = f"{sysconfig.get_config_var('SOABI')} torch {torch.__version__}"
+    if not force and _fresh(CALLS_OUT, [CALLS_SRC, os.path.join(ROOT, "include", "nvfp4.h")]) and _text(CALLS_BUILT_FOR) == built_for:
+        return CALLS_OUT
     th = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(NVCC))
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", os.path.join(th, "include"),
@@ -52,6 +61,8 @@ def build_calls(force: bool = False) -> str:
                            "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), "-I", os.path.join(ROOT, "include"),
                            CALLS_SRC, "-o", CALLS_OUT, "-L", os.path.join(th, "lib"), "-Wl,-rpath," + os.path.join(th, "lib"),
                            "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-ldl"])
+    with open(CALLS_BUILT_FOR, "w") as f:
+        f.write(built_for)
     return CALLS_OUT
 
 
