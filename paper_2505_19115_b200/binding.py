@@ -122,7 +122,11 @@ def _native():
     global _calls
     if _calls is None:
         lib()
-        from . import _calls as module
+        try:
+            from . import _calls as module
+        except ImportError as e:
+            raise RuntimeError(f"the extension module _calls cannot be imported ({e}): build it with "
+                               "`python -m paper_2505_19115_b200.build`") from e
         module.bind(LIB_PATH, Rounding)
         _calls = module
     return _calls

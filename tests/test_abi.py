@@ -203,6 +203,17 @@ def test_calls_module_takes_its_arguments_as_declared():
         nb._native().nvfp4_quantize(x)
 
 
+def test_a_missing_calls_module_says_what_to_run(monkeypatch):
+    import sys
+
+    import paper_2505_19115_b200
+    monkeypatch.setattr(nb, "_calls", None)
+    monkeypatch.delattr(paper_2505_19115_b200, "_calls", raising=False)
+    monkeypatch.setitem(sys.modules, "paper_2505_19115_b200._calls", None)
+    with pytest.raises(RuntimeError, match="python -m paper_2505_19115_b200.build"):
+        nb._native()
+
+
 class _NoStream:
     cuda_stream = 0
 
