@@ -199,6 +199,66 @@ def test_layer_calls_equal_the_single_calls(shape, dtype, mode):
     assert torch.equal(want[1], both[0]) and torch.equal(want[2], both[1])
 
 
+# The layer calls' shared quantizer has a pass of its own over the scale padding, for per-tensor scales under which the zeros beyond
+# a tensor do not encode to zero scales.  Rows and columns fill neither a tile nor a scale tile; what a call leaves in its buffers
+# is compared byte for byte, padding included, with the single quantizers.
+@pytest.mark.parametrize("g", [0.0, 1e-40, float("nan"), 1.0])
+@pytest.mark.parametrize("shape,dtype", [((96, 160, 224), torch.bfloat16), ((96, 160, 224), torch.float32), ((2080, 1056, 2848), torch.bfloat16)])
+def test_layer_operands_under_any_given_scale_equal_the_single_quantizers(shape, dtype, g):
+    M, K, N = shape
+    X, W, dY = (t.cuda().to(dtype) for t in synth.linear_inputs(M, K, N, seed=35, grad_std=1e-3))
+    g_t = torch.full((1,), g, device="cuda")
+    r = [nb.Rounding(nb.RTN), nb.Rounding(nb.SR, 8, 0), nb.Rounding(nb.SR, 8, 1), nb.Rounding(nb.SR, 8, 2)]
+
+    def buffer(nbytes):
+        return torch.full((nbytes,), 0xA5, dtype=torch.uint8, device="cuda")
+
+    def assert_holds(buf, *operands):                       # in the buffer's order, each part from a multiple of 256 bytes
+        at = 0
+        for x, transposed, rounding in operands:
+            Rq, Kq = x.shape[::-1] if transposed else x.shape
+            codes, scales = nb.nvfp4_quantize(x, transposed, g_t, rounding, nb.SF_SWIZZLED)
+            for want in (codes.reshape(-1), scales[:nb.nvfp4_sf_bytes(Rq, Kq)]):
+                assert torch.equal(buf[at:at + want.numel()], want), (tuple(x.shape), transposed)
+                at = (at + want.numel() + 255) // 256 * 256
+    saved, ws = buffer(nb.nvfp4_linear_saved_bytes(M, N, K)), buffer(nb.nvfp4_linear_fused_workspace_bytes(M, N, K, nb.FUSED_FWD_SAVE))
+    nb.nvfp4_linear_fwd_save(X, W, nb.G_GIVEN, gx=g_t, gw=g_t, rx=r[0], rw=r[0], rxt=r[3], rwt=r[0], saved=saved, workspace=ws)
+    assert_holds(saved, (W, True, r[0]), (X, True, r[3]))
+    assert_holds(ws, (X, False, r[0]), (W, False, r[0]))
+    ws = buffer(nb.nvfp4_linear_fused_workspace_bytes(M, N, K, nb.FUSED_BWD))
+    nb.nvfp4_linear_bwd(dY, W, X, nb.G_GIVEN, gdy=g_t, gw=g_t, gx=g_t, rdy=r[1], rdyt=r[2], rwt=r[0], rxt=r[3], workspace=ws)
+    assert_holds(ws, (dY, False, r[1]), (dY, True, r[2]), (W, True, r[0]), (X, True, r[3]))
+    ws = buffer(nb.nvfp4_linear_workspace_bytes(M, N, K, nb.LINEAR_BWD_DW))
+    nb.nvfp4_linear_bwd_dw(dY, X, nb.G_GIVEN, gdy=g_t, gx=g_t, rdy=r[2], rx=r[3], workspace=ws)
+    assert_holds(ws, (dY, True, r[2]), (X, True, r[3]))
+    assert nb.nvfp4_device_error_word() == 0
+
+
+# Operands aligned to 16 bytes, but not to the 32 that the amax sweeps load at once: they take the passes for any tensor.
+@pytest.mark.parametrize("moved", [(True, True, True), (True, False, False), (False, True, False)])
+@pytest.mark.parametrize("shape,dtype", [((64, 32, 96), torch.bfloat16), ((2080, 1056, 2848), torch.bfloat16), ((2080, 1056, 2848), torch.float32),
+                                         ((16416, 4128, 32), torch.bfloat16)])
+def test_layer_calls_on_operands_aligned_to_16_bytes(shape, dtype, moved):
+    M, K, N = shape
+    X, W, dY = (t.cuda().to(dtype) for t in synth.linear_inputs(M, K, N, seed=36, grad_std=1e-3))
+
+    def at_16(x):
+        buf = torch.zeros(x.numel() + 16, dtype=x.dtype, device="cuda")
+        view = buf[16 // x.element_size():][:x.numel()].view(x.shape)
+        assert view.data_ptr() % 32 == 16
+        return view.copy_(x)
+
+    def results(X, W, dY):
+        Y, saved = nb.nvfp4_linear_fwd_save(X, W)
+        return (Y, *nb.nvfp4_linear_bwd_saved(dY, saved, K), *nb.nvfp4_linear_bwd(dY, W, X), nb.nvfp4_linear_fwd(X, W))
+    want = results(X, W, dY)
+    got = results(*(at_16(x) if m else x for x, m in zip((X, W, dY), moved)))
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    for i, (a, b) in enumerate(zip(want, got)):
+        assert torch.equal(a, b), i
+
+
 # ---------------------------------------------------------------- non-finite inputs stay visible
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
 def test_non_finite_input_propagates_through_the_per_tensor_scale(bad):
