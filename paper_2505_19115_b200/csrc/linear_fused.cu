@@ -107,6 +107,7 @@ extern "C" int nvfp4_linear_fwd_save(const void* X, const void* W, int dtype, in
   uint8_t* sv = static_cast<uint8_t*>(saved);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   if (gscale_mode == NVFP4_G_GIVEN && (!gx || !gw)) return NVFP4_ERR_NULL;
+  if (!aligned16(Y)) return NVFP4_ERR_ALIGN;             // rejected here, not by the product behind the quantizers
   // The backward pass reads the scales from `saved`, given ones too.  W first: its pass leaves the (smaller) weight tensor in
   // the level-two cache for the quantizer that follows it.
   const bool kept = gscale_mode != NVFP4_G_NONE;
@@ -144,6 +145,7 @@ extern "C" int nvfp4_linear_bwd_saved(const void* dY, int dtype, int64_t M, int6
   const uint8_t* sv = static_cast<const uint8_t*>(saved);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   if (gscale_mode == NVFP4_G_GIVEN && !gdy) return NVFP4_ERR_NULL;
+  if (!aligned16(dX) || !aligned16(dW)) return NVFP4_ERR_ALIGN;
   const LayerOperand op = {dY, M, N, rdy, ws + bl.dy.codes, ws + bl.dy.sf, rdyt, ws + bl.dyt.codes, ws + bl.dyt.sf, gdy,
                            scale_slot(ws, bl.gdy, gscale_mode == NVFP4_G_AMAX)};
   const float* g_dy;
@@ -168,6 +170,7 @@ extern "C" int nvfp4_linear_bwd(const void* dY, const void* W, const void* X, in
   if (!buffer_ok(workspace, workspace_bytes, bl.total)) return NVFP4_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   if (gscale_mode == NVFP4_G_GIVEN && (!gdy || !gw || !gx)) return NVFP4_ERR_NULL;
+  if (!aligned16(dX) || !aligned16(dW)) return NVFP4_ERR_ALIGN;
   const bool amax = gscale_mode == NVFP4_G_AMAX;
   const LayerOperand ops[3] = {
       {W, N, K, nullptr, nullptr, nullptr, rwt, ws + bl.wt.codes, ws + bl.wt.sf, gw, scale_slot(ws, bl.gw, amax)},

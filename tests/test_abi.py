@@ -172,6 +172,15 @@ def test_newer_entry_points_reject_bad_arguments_on_the_host():
     assert gx(a=None) == 1 and gx(am=2) == 4 and gx(am=1, bm=0) == 4 and gx(am=1, bm=1, M=100) == 2
 
 
+def test_fused_layer_calls_reject_misaligned_outputs_before_any_launch():
+    L, r, buf, off = nb.lib(), nb.Rounding(), C.c_void_p(0x1000), C.c_void_p(0x1004)
+    rb, big = C.byref(r), 1 << 30
+    assert L.nvfp4_linear_fwd_save(buf, buf, 0, 256, 512, 512, 0, None, None, rb, rb, rb, rb, off, 1, buf, big, buf, big, None) == 3
+    for dX, dW in ((off, buf), (buf, off)):
+        assert L.nvfp4_linear_bwd_saved(buf, 0, 256, 512, 512, 0, None, rb, rb, buf, big, dX, 1, dW, 1, buf, big, None) == 3
+        assert L.nvfp4_linear_bwd(buf, buf, buf, 0, 256, 512, 512, 0, None, None, None, rb, rb, rb, rb, dX, 1, dW, 1, buf, big, None) == 3
+
+
 def test_stream_handle_without_the_raw_stream_function(monkeypatch):
     # the quick way to the current stream's handle is private to torch: where it is missing, the public one serves
     class Stream:
