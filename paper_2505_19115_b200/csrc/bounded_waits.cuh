@@ -66,8 +66,8 @@ __device__ __forceinline__ bool mbar_wait_issuer(uint32_t bar, uint32_t parity, 
 // acquiring poll costs ~180 cycles even when the phase is complete (see mbar_wait_issuer), which with two waits per stage made the
 // movers the slowest role.  What they read afterwards is shared memory written by the bulk copies that completed the phase, so
 // the successful polls are followed by one acquire fence at CTA scope: relaxed observation + fence is the acquire pattern of the
-// PTX memory model.  A stage's two waits share the vote and the fence: a product chained to another, 3001 x 4096 x 11008 and
-// 3001 x 11008 x 4096, 171.5 us with a fence for each wait and no vote, 171.7 with a vote for each too, 170.0 so.
+// PTX memory model.  A stage's two waits share the vote and the fence: products of 3001 x 4096 x 11008 and 3001 x 11008 x 4096, one
+// chained to the other, took 171.5 us with a fence for each wait and no vote, 171.7 with a vote for each too, and take 170.0 so.
 __device__ __forceinline__ bool warp_acquire(bool ok) {
   ok = __all_sync(0xFFFFFFFFu, ok);
   asm volatile("fence.acq_rel.cta;" ::: "memory");

@@ -472,7 +472,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
   const uint32_t tmem_base = *tmem_slot;
   // All of the above overlaps the kernel before this one, and what each role does until its first copy, access or bounded wait
   // on another role: there it waits for that kernel (the time limit of a wait must not run while that one does).  Against a wait
-  // here, for all: 2080 x 1056 x 2848 step 55.9 -> 53.5 us, 256 x 512 x 512 23.5 -> 22.4, 16 x 11008 x 4096 alone 12.5 -> 11.7.
+  // here, for all: 2080 x 1056 x 2848 step 56.4 -> 54.7 us, 256 x 512 x 512 23.3 -> 22.7, 16 tokens on kept 11008 x 4096 weights 14.3 -> 14.0.
   if constexpr (Q_OUT) {
     grid_dependency_wait();
     build_inv_table(inv_table, load_scale(p.out_g));

@@ -772,7 +772,7 @@ int quantize_operands(const LayerOperand* ops, int n, int dtype, int gscale_mode
     flat = flat && amax_flat_ok(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols);
     sweep = sweep || needs_scratch(ops[i], dtype);
   }
-  const bool batch = tile_batch_eligible(ops, n, dtype);
+  const bool batch = tile_batch_eligible(ops, n);
   if (!amax) {
     if (batch && n > 1) return tile_quantize_batch(ops, src, n, dtype, s);
     if (given) {

@@ -436,7 +436,7 @@ quantize_tile_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
 
 // Several operands of one layer call in one launch: their tiles (128 rows, swizzled NVFP4 scales) in one list, each with the
 // outputs and the roundings of its operand.  Small operands leave most of the chip idle, and each launch costs its latency:
-// one step of 256 x 512 x 512 25.2 -> 23.4 us, 2080 x 1056 x 2848 57.9 -> 55.8, 3680 x 896 x 640 with given scales 36.1 -> 30.0.
+// one step of 256 x 512 x 512 24.9 -> 22.3 us, 2080 x 1056 x 2848 55.6 -> 54.7, 3680 x 896 x 640 with given scales 40.0 -> 34.3.
 struct TileBatch {
   struct Op {
     CUtensorMap x, ct, cr;
@@ -721,8 +721,7 @@ int tile_quantize_row(const void* x, int dtype, int64_t rows, int64_t cols, int6
 
 // Several operands in one launch: tensors that the 128-row tiles take, together small enough (see launch_tile) and with tile
 // counts that tile * magic divides exactly.
-bool tile_batch_eligible(const LayerOperand* ops, int n, int dtype) {
-  (void)dtype;
+bool tile_batch_eligible(const LayerOperand* ops, int n) {
   int64_t elements = 0;
   for (int i = 0; i < n; ++i) {
     const LayerOperand& op = ops[i];
