@@ -755,13 +755,20 @@ int quantize_operand(const LayerOperand& op, int dtype, const float* g, void* st
 // (67 MB of dY) 206.7 / 210.4.
 constexpr int64_t kSweepBytes = (int64_t)24 << 20;
 
+// Where there are no amax passes, bf16 operands of which only the transposed outputs are asked for are quantized apart from this many
+// bytes on: the kernel for all has room for both outputs, the one for a single output has more blocks on a multiprocessor for
+// the random stream's chains.  Weight gradient, us, apart / in one launch: 4096 x 1024 x 1024 (17 MB) 17.7 / 16.7, 8192 x 512 x 1024 (25 MB)
+// 21.8 / 21.6, 2336 x 1024 x 4096 (24 MB) 20.3 / 21.3, 4096 x 4096 x 1024 25.0 / 26.7, 12288 x 4096 x 64 43.0 / 46.9; fp32 operands
+// 4096 x 2048 x 2048 26.7 / 24.7, 8192 x 4096 x 1024 53.0 / 51.2.
+constexpr int64_t kApartBytes = (int64_t)20 << 20;
+
 int quantize_operands(const LayerOperand* ops, int n, int dtype, int gscale_mode, const float** g, void* cuda_stream) {
   if (int st = check_arch()) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const bool amax = gscale_mode == NVFP4_G_AMAX, given = gscale_mode == NVFP4_G_GIVEN;
   ScaleSource src[kMaxLayerOperands];
   int64_t bytes = 0;
-  bool flat = true, sweep = false;
+  bool flat = true, sweep = false, rows = false;
   for (int i = 0; i < n; ++i) {
     for (const nvfp4_rounding* r : {ops[i].rr, ops[i].rt})
       if (r && ((r->mode != NVFP4_RTN && r->mode != NVFP4_SR) || r->reserved != 0)) return NVFP4_ERR_ENUM;
@@ -771,10 +778,12 @@ int quantize_operands(const LayerOperand* ops, int n, int dtype, int gscale_mode
     bytes += operand_bytes(ops[i], dtype);
     flat = flat && amax_flat_ok(ops[i].x, dtype, ops[i].rows, ops[i].cols, ops[i].cols);
     sweep = sweep || needs_scratch(ops[i], dtype);
+    rows = rows || ops[i].rr;
   }
   const bool batch = tile_batch_eligible(ops, n);
   if (!amax) {
-    if (batch && n > 1) return tile_quantize_batch(ops, src, n, dtype, s);
+    const bool apart = !rows && dtype == NVFP4_BF16 && bytes >= kApartBytes;
+    if (batch && n > 1 && !apart) return tile_quantize_batch(ops, src, n, dtype, s);
     if (given) {
       ScalePairs p = {};
       bool any = false;
