@@ -740,7 +740,10 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
       tile_coords(t.tile, q.tiles_m, q.tiles_n, tm, tn);
       // Polled without sleeping: the next tile's MMAs wait for this read-out.  Against a lane that sleeps 32 ns between its polls:
       // 16384 x 3072 x 2048 fp32 57.6 -> 56.2 us, 16384 x 4096 x 4096 bf16 109.7 -> 107.0, 1024 x 1024 x 16384 21.2 -> 20.1.
-      ACCOUNT(a_tile, ok = mbar_wait_warp_spin(tfull_bar(acc), acc_ph, abort_flag, 0x14));
+      // Tiles of a single k-stage are bound by the stores: there the lane that sleeps wins (bf16 output, 16384 x 11008 x 256 68.7 -> 61.2,
+      // 32768 x 4096 x 256 49.7 -> 47.0; fp32 133.9 / 134.1).
+      ACCOUNT(a_tile, ok = q.k_stages > 1 ? mbar_wait_warp_spin(tfull_bar(acc), acc_ph, abort_flag, 0x14)
+                                          : mbar_wait_warp(tfull_bar(acc), acc_ph, abort_flag, 0x14));
       if (!ok) break;
 #ifdef NVFP4_GEMM_ACCOUNT
       a_read_t0 = clock64();
