@@ -42,6 +42,8 @@ inline cudaError_t set_max_dynamic_smem(DeviceFlags& flags, Kernel kernel, int b
 //   * it calls grid_dependency_trigger() only after that wait.  A kernel that follows it directly therefore starts when
 //     everything TWO launches back is finished, and may read that without waiting ("late" kernels), as long as it still waits
 //     before it ends, so that "finished" keeps meaning "and all before it".
+//   * the late one of two products (gemm_two) does not trigger: what follows starts when it and all before it are finished.  Blocks of
+//     the next kernel would take its room (16384 x 11008 x 512 181 -> 182 us, 512 x 11008 x 11008 126.1 -> 128.3).
 // After anything else on the stream (a kernel that does not take part, a copy) the attribute changes nothing.
 // Launched the ordinary way -> this way, us: one step of a 256 x 512 x 512 layer (six kernels) 34.8 -> 22.4, of a 2080 x 1056 x 2848
 // one 67.1 -> 54.6, 16 tokens through kept 11008 x 4096 weights (three kernels) 20.5 -> 14.0.

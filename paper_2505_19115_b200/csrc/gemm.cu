@@ -81,6 +81,7 @@ struct GemmParams {
   int k_mmas;                       // instructions along K
   int a_row_tiles, b_row_tiles;     // ceil(M / 128), ceil(N / 128)
   int d_is_bf16;
+  int late = 0;
 };
 
 // Tile order: panels of kPanel row tiles, column-major inside a panel, so that the CTAs running at
@@ -394,6 +395,7 @@ struct Gemm2Params {
   Gemm2Maps maps[PRODUCTS];
   Gemm2Product product[PRODUCTS];
   TileOrder order;
+  int late = 0;                     // see gemm_two
   // quantized output (OUT == 2): per-tensor scale of the output, rounding, scales destination
   const float* out_g;
   PhiloxStream out_rng;
@@ -473,8 +475,12 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
   // All of the above overlaps the kernel before this one, and what each role does until its first copy, access or bounded wait
   // on another role: there it waits for that kernel (the time limit of a wait must not run while that one does).  Against a wait
   // here, for all: 2080 x 1056 x 2848 step 56.4 -> 54.7 us, 256 x 512 x 512 23.3 -> 22.7, 16 tokens on kept 11008 x 4096 weights 14.3 -> 14.0.
+  // A late product (gemm_two) waits at its end instead: nothing that it reads or writes is the kernel before's.
+  auto follow = [&] {
+    if (!p.late) grid_dependency_wait();
+  };
   if constexpr (Q_OUT) {
-    grid_dependency_wait();
+    follow();
     build_inv_table(inv_table, load_scale(p.out_g));
     __syncthreads();
   }
@@ -509,8 +515,8 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
         const uint32_t st = smem_base + s * C::kStageBytes;
         const uint32_t lead_full = map_to_cta(full_bar(s), 0);
         if (i == 0 && ks == 0) {
-          grid_dependency_wait();
-          grid_dependency_trigger();
+          follow();
+          if (!p.late) grid_dependency_trigger();
         }
         if (issuer) {
           if (rank == 0) mbar_arrive_expect_tx(full_bar(s), operand_tx);
@@ -558,7 +564,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
       for (int ks = 0; ks < q.k_stages; ++ks) {
         if (!(ok = mbar_wait_relaxed(sfx_bar(s), ph ^ 1u, abort_flag, 0x18))) break;
         const uint32_t sf = smem_base + s * C::kStageBytes + C::kABytes + C::kBBytes;
-        if (i == 0 && ks == 0) grid_dependency_wait();
+        if (i == 0 && ks == 0) follow();
         if (issuer) {
           mbar_arrive_expect_tx(sfl_bar(s), kScaleTx);
           tma_load_2d(sf, &m.sfa, sfl_bar(s), 0, a_row + ks * kSfTiles);
@@ -592,7 +598,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
         int tm_unused, tn;
         tile_coords(t.tile, q.tiles_m, q.tiles_n, tm_unused, tn);
         const uint32_t sfb_off = (uint32_t)((tn * BN) % 128) / 32 + (whole ? 0u : 4u * t.half);   // first scale column of this N tile
-        if (i == 0) grid_dependency_wait();
+        if (i == 0) follow();
         ACCOUNT(a_acc, ok = mbar_wait_issuer(tempty_bar(acc), acc_ph ^ 1u, abort_flag, 0x12));
         if (!ok) break;
         const uint32_t d_tmem = tmem_base + acc * BN;
@@ -662,7 +668,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
     TileItem t;
     for (int i = 0; !BF16_IN && ok && tile_at<PAIRED, HALVES>(p.order, pair, num_pairs, i, t); ++i) {
       const int k_stages = p.product[t.product].k_stages;
-      if (i == 0) grid_dependency_wait();
+      if (i == 0) follow();
       for (int ks = 0; ks < k_stages; ++ks) {
         ACCOUNT(a_land, ok = mbar_wait_issuer(sfl_bar(s), ph, abort_flag, 0x16));
         if constexpr (!C::kSfFollowsStage) {
@@ -718,7 +724,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
     // Against four warps that held 3 of 8 chunks and streamed the others through their staging buffers (16384 x 11008 x
     // 4096 with fp32 output: 366 -> 313 us, input gradient of the same layer 293 -> 259; chained bf16 layers 190 -> 182).
     const int quarter = warp & 3, half = (warp >> 2) & 1;
-    grid_dependency_wait();
+    follow();
     float alphas[PAIRED ? 2 : 1];
     for (int w = 0; w < (PAIRED ? 2 : 1); ++w) alphas[w] = load_scale(p.product[w].a_g) * load_scale(p.product[w].b_g);
     [[maybe_unused]] const float cq = Q_OUT ? __fdiv_rn(__fdiv_rn(1.0f, 6.0f), load_scale(p.out_g)) : 0.0f;
@@ -868,6 +874,7 @@ gemm2_nvfp4_kernel(const __grid_constant__ Gemm2Params<PAIRED ? 2 : 1> p) {
     ACCOUNT_STORE(pair == 0 && rank == 0 && warp == 8 && lane == 0, 14, a_total + ACCOUNT_NOW());
   }
 
+  if (p.late) grid_dependency_wait();
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                               // the peer's MMAs and loads are done before anyone frees or exits
@@ -1020,6 +1027,7 @@ int launch_gemm2(const uint8_t* a_codes, const uint8_t* b_codes, const GemmParam
   constexpr bool kHalves = has_halves(BN, OUT, BF16_IN, false);
   Gemm2Params<1> p;
   const int64_t max_pairs = sm_count() / 2;
+  p.late = g.late;
   order_tiles(0, 0, ceil_div(g.M, 256) * ceil_div(g.N, BN), 1, max_pairs, kHalves, &p.order);
   const int64_t pairs = std::min<int64_t>(p.order.n1, max_pairs);
   if (!describe_product<BN, BF16_IN, MX>(g, a_codes, b_codes, MN, p.order.split < p.order.n1, &p.maps[0], &p.product[0])) return NVFP4_ERR_CUDA;
@@ -1085,6 +1093,21 @@ int paired_tile_width(const GemmParams (&p)[2], bool bf16_in) {
   return cycles[0] <= cycles[1] ? 128 : 256;
 }
 
+// Two products, the longer contraction first, that are better launched apart: the shorter one bound by its stores (at most three
+// k-stages, fp32, more output than the level-two cache holds), and more than a third of the pairs without one of the longer one's
+// last tiles.  In one launch those pairs alone store meanwhile, and the tiles of the longer one wait for operands behind their stores.
+// Apart, the shorter one goes first and the longer one is late: a pair that is done with its stores begins with it.  us with the
+// quantizer of dY, one launch / apart: 16384 x 5120 x 512 107.9 / 95.8, 16384 x 11008 x 512 193.9 / 181.2, 4096 x 11008 x 512
+// 60.1 / 54.7, 512 x 11008 x 11008 131.7 / 125.7, 16384 x 11008 x 256 185.7 / 156.5.  On the other side of each line: four k-stages
+// 8192 x 11008 x 1024 119.2 / 123.1; bf16 output 16384 x 11008 x 512 127.2 / 130.4; 92 MB 2048 x 11008 x 512 32.4 / 34.5; 64 of 74
+// pairs busy 512 x 8192 x 8192 72.5 / 74.6, 16384 x 4096 x 512 80.0 / 81.3.
+bool better_apart(const GemmParams (&p)[2], int bn) {
+  constexpr int64_t kBeyondCache = (int64_t)144 << 20;
+  if (p[1].d_is_bf16 || p[1].k_stages > 3 || (int64_t)p[1].M * p[1].N * 4 < kBeyondCache) return false;
+  const int64_t pairs = sm_count() / 2, last = ceil_div(p[0].M, 256) * ceil_div(p[0].N, bn) % pairs;
+  return last != 0 && 3 * (pairs - last) > pairs;
+}
+
 // 0 = automatic.  128 / 256: single-CTA kernel with that tile width.  2128 / 2192 / 2256: CTA-pair
 // kernel with a 256 x {128,192,256} tile.
 int gemm_tile_n_override = 0;
@@ -1123,9 +1146,11 @@ int checked_params(const GemmCall& c, GemmParams* p) {
   p->tiles_m = p->tiles_n = 0;
   return check_arch();
 }
-int gemm(const GemmCall& c, void* cuda_stream) {
+// late: nothing that it reads or writes is the kernel before's, and that one has waited for all before it.
+int gemm(const GemmCall& c, void* cuda_stream, bool late = false) {
   GemmParams p;
   if (int st = checked_params(c, &p)) return st;
+  p.late = late;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const int bn = gemm_tile_n_override ? gemm_tile_n_override : 2000 + pair_tile_width(c.M, c.N);
   switch (bn) {
@@ -1153,6 +1178,10 @@ int nvfp4::gemm_two(const GemmCall& x, const GemmCall& y, void* cuda_stream) {
   const int mn[2] = {0, 0};
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const int bn = gemm_tile_n_override ? gemm_tile_n_override - 2000 : paired_tile_width(p, false);
+  if (!gemm_tile_n_override && better_apart(p, bn)) {
+    if (int st = gemm(*c[1], cuda_stream)) return st;
+    return gemm(*c[0], cuda_stream, /*late=*/true);
+  }
   return bn == 128 ? launch_gemm2_paired<128, false>(p, a, b, mn, s) : launch_gemm2_paired<256, false>(p, a, b, mn, s);
 }
 

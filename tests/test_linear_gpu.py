@@ -170,6 +170,25 @@ def test_gradients_of_one_launch_equal_the_single_products(shape, dx_dtype, dw_d
     assert torch.equal(want[0], got[0]) and torch.equal(want[1], got[1])
 
 
+# Where one of the gradients is bound by its stores, they are launched apart and the other one does not wait for it: three contractions,
+# either gradient being the late one.  Calls follow one another on the same buffers.
+@pytest.mark.parametrize("shape", [(8224, 4736, 96), (96, 4736, 8224), (8224, 4736, 544)])
+@pytest.mark.parametrize("dw_dtype", [torch.float32, torch.bfloat16])
+def test_gradients_launched_apart_equal_the_single_products(shape, dw_dtype):
+    M, K, N = shape
+    X, W, dY = (t.cuda() for t in synth.linear_inputs(M, K, N, seed=37, grad_std=1e-3))
+    grads = [dY, dY.flip(0).contiguous(), (dY * 2).contiguous()]
+    rt, sr0, sr1, sr2 = nb.Rounding(nb.RTN), nb.Rounding(nb.SR, 6, 0), nb.Rounding(nb.SR, 6, 1), nb.Rounding(nb.SR, 6, 2)
+    want = [(nb.nvfp4_linear_bwd_dx(g, W, rdy=sr0, rw=rt), nb.nvfp4_linear_bwd_dw(g, X, rdy=sr1, rx=sr2, out_dtype=dw_dtype)) for g in grads]
+    ws = torch.empty(nb.nvfp4_linear_fused_workspace_bytes(M, N, K, nb.FUSED_BWD), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    got = [nb.nvfp4_linear_bwd(grads[i % 3], W, X, rdy=sr0, rdyt=sr1, rwt=rt, rxt=sr2, dw_dtype=dw_dtype, workspace=ws) for i in range(6)]
+    torch.cuda.synchronize()
+    assert nb.nvfp4_device_error_word() == 0
+    for i, (dX, dW) in enumerate(got):
+        assert torch.equal(want[i % 3][0], dX) and torch.equal(want[i % 3][1], dW), i
+
+
 # The layer calls quantize their operands together and take the per-tensor scale from an amax sweep's maxima: below 2 MB (one
 # cluster), above (sweeps, one quantizer launch for both), one operand below and one above, and operands too large for one launch.
 @pytest.mark.parametrize("mode", [nb.G_AMAX, nb.G_GIVEN, nb.G_NONE])
